@@ -294,12 +294,10 @@ __device__ __forceinline__ void stream_update(const StreamChunk &d, const Stream
     const int32_t qs = sj.sb + a;
     const double *sR = reinterpret_cast<const double *>(side + L.s_R);
     const double *sA = reinterpret_cast<const double *>(side + L.s_avg);
-    double Rn = sR[qs - d.sa] + (double)r;
-    if (rule != kRuleCfr) Rn = Rn > 0.0 ? Rn : 0.0;
+    double Rn, Sn;
+    pf = narrow_pos(slot_terms(sR[qs - d.sa], sA[qs - d.sa], widen(r), widen(m), wt, rule, Rn, Sn));
     Rg[qs] = Rn;
-    avgg[qs] = sA[qs - d.sa] + wt * (double)m;
-    const double x = rule == kRulePcfrPlus ? Rn + (double)r : Rn;
-    pf = (float)(x > 0.0 ? x : 0.0);
+    avgg[qs] = Sn;
   }
   float tot = 0.f;  // positive parts in action order
   for (int b = 0; b < MAXA; ++b) {

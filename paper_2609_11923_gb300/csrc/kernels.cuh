@@ -395,18 +395,63 @@ __device__ __forceinline__ double avg_weight(long long t, int rule) {
   return rule == kRulePcfrPlus ? x * x : x;
 }
 
+// Conversions and comparisons of doubles in integer arithmetic. GB300's FP64
+// pipe takes one warp instruction every 16-19 cycles per SM whatever the
+// number of active lanes, and conversions (cvt.f64.f32, cvt.f32.f64) and
+// compares (setp.f64) run there too, with 100 cycles of latency each
+// (measured; 64 for an add). The slot update is a chain of them on a few
+// lanes of a warp, so only its add and its multiply-add stay on that pipe: five
+// iterations of the 2.8M-node random tree 635 -> 595 us, 50 of a 21k-node
+// endgame 1,291 -> 1,255 us. Same results bit for bit, for every input.
+__device__ __forceinline__ double widen(float x) {  // (double)x
+  const uint32_t u = __float_as_uint(x), e = (u >> 23) & 255u;
+  if (e - 1u < 254u)
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+  if ((u << 1) == 0u) return __hiloint2double((int)u, 0);
+  return (double)x;  // subnormal, infinite or NaN
+}
+
+__device__ __forceinline__ float narrow_pos(double x) {  // (float)x of x >= 0, to nearest, ties to even
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  const uint32_t e = (hi >> 20) - 896u;
+  if (e - 1u < 254u) {
+    const uint32_t m = (e << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
+    const uint32_t rest = lo & 0x1fffffffu;  // bits below the last place
+    return __uint_as_float(m + (rest > 0x10000000u - (m & 1u) ? 1u : 0u));
+  }
+  if ((hi | lo) == 0u) return 0.f;
+  return (float)x;
+}
+
+__device__ __forceinline__ double positive_part(double x) {  // x > 0.0 ? x : 0.0 (NaN and -0 give 0)
+  const long long b = __double_as_longlong(x);
+  return b > 0 && b <= 0x7ff0000000000000ll ? x : 0.0;
+}
+
+// A set total as a double: FP32 totals are widened.
+__device__ __forceinline__ double as_double(float x) { return widen(x); }
+__device__ __forceinline__ double as_double(double x) { return x; }
+
 // One slot's update from its set's totals (instantaneous regret r, average
-// term m): R <- R + r (clamped at 0 except under vanilla CFR), avg += w * m.
-// Returns what regret matching takes the positive part of: the new R, or
-// R + r under PCFR+.
+// term m) and its cumulative regret R and average sum S: Rn = R + r (clamped
+// at 0 except under vanilla CFR) and Sn = S + wt * m. Returns what regret
+// matching takes the positive part of: the new R, or R + r under PCFR+.
+__device__ __forceinline__ double slot_terms(double R, double S, double r, double m, double wt, int rule, double &Rn,
+                                             double &Sn) {
+  Rn = R + r;
+  if (rule != kRuleCfr) Rn = positive_part(Rn);
+  Sn = S + wt * m;
+  return positive_part(rule == kRulePcfrPlus ? Rn + r : Rn);
+}
+
+// The same on the slot's entries in memory.
 __device__ __forceinline__ double slot_update(double *R, double *avg, int32_t q, double r, double m, double wt,
                                               int rule) {
-  double Rn = R[q] + r;
-  if (rule != kRuleCfr) Rn = Rn > 0.0 ? Rn : 0.0;
+  double Rn, Sn;
+  const double pos = slot_terms(R[q], avg[q], r, m, wt, rule, Rn, Sn);
   R[q] = Rn;
-  avg[q] += wt * m;
-  const double x = rule == kRulePcfrPlus ? Rn + r : Rn;
-  return x > 0.0 ? x : 0.0;
+  avg[q] = Sn;
+  return pos;
 }
 
 // ------------------------------------------------------------- backward
@@ -694,40 +739,32 @@ __device__ __forceinline__ void bwd_set(const GameView &g, const StateView<T> &s
     for (int a = 0; a < MAXA; ++a)
       if (a == lane) { r = racc[a]; m = macc[a]; }
     double pos = 0.0;
-    if (lane < na) pos = slot_update(st.R, st.avg, sb + lane, (double)r, (double)m, wt, rule);
+    if (lane < na) pos = slot_update(st.R, st.avg, sb + lane, as_double(r), as_double(m), wt, rule);
     if constexpr (sizeof(T) == 8) {
       double tot = 0.0;
       for (int a = 0; a < na; ++a) tot += __shfl_sync(mask, pos, a, LANES);
       if (lane < na) st.sigma[sb + lane] = tot > 0.0 ? pos / tot : 1.0 / (double)na;
     } else {
-      const float pf = (float)pos;
+      const float pf = narrow_pos(pos);
       float tot = 0.f;
       for (int a = 0; a < na; ++a) tot += __shfl_sync(mask, pf, a, LANES);
       if (lane < na) st.sigma[sb + lane] = tot > 0.f ? pf / tot : 1.f / (float)na;
     }
   } else if (lane == 0) {
-    double pos[MAXA];
-    double tot = 0.0;
+    T pos[MAXA];
+    T tot = T(0);
 #pragma unroll
     for (int a = 0; a < MAXA; ++a) {
       if (a < na) {
-        pos[a] = slot_update(st.R, st.avg, sb + a, (double)racc[a], (double)macc[a], wt, rule);
+        const double x = slot_update(st.R, st.avg, sb + a, as_double(racc[a]), as_double(macc[a]), wt, rule);
+        if constexpr (sizeof(T) == 8) pos[a] = x;
+        else pos[a] = narrow_pos(x);
         tot += pos[a];
       }
     }
-    if constexpr (sizeof(T) == 8) {
 #pragma unroll
-      for (int a = 0; a < MAXA; ++a)
-        if (a < na) st.sigma[sb + a] = tot > 0.0 ? pos[a] / tot : 1.0 / (double)na;
-    } else {
-      float totf = 0.f;
-#pragma unroll
-      for (int a = 0; a < MAXA; ++a)
-        if (a < na) totf += (float)pos[a];
-#pragma unroll
-      for (int a = 0; a < MAXA; ++a)
-        if (a < na) st.sigma[sb + a] = totf > 0.f ? (float)pos[a] / totf : 1.f / (float)na;
-    }
+    for (int a = 0; a < MAXA; ++a)
+      if (a < na) st.sigma[sb + a] = tot > T(0) ? pos[a] / tot : T(1) / (T)na;
   }
 }
 
@@ -815,7 +852,7 @@ __device__ __forceinline__ void bwd_set_block(const GameView &g, const StateView
   // positive parts summed in action order
   double pos = 0.0;
   if (tid < na) {
-    pos = slot_update(st.R, st.avg, sb + tid, (double)r, (double)m, wt, rule);
+    pos = slot_update(st.R, st.avg, sb + tid, as_double(r), as_double(m), wt, rule);
     s_pos[tid] = pos;
   }
   __syncthreads();
@@ -826,8 +863,8 @@ __device__ __forceinline__ void bwd_set_block(const GameView &g, const StateView
       st.sigma[sb + tid] = tot > 0.0 ? pos / tot : 1.0 / (double)na;
     } else {
       float tot = 0.f;
-      for (int a = 0; a < na; ++a) tot += (float)s_pos[a];
-      st.sigma[sb + tid] = tot > 0.f ? (float)pos / tot : 1.f / (float)na;
+      for (int a = 0; a < na; ++a) tot += narrow_pos(s_pos[a]);
+      st.sigma[sb + tid] = tot > 0.f ? narrow_pos(pos) / tot : 1.f / (float)na;
     }
   }
   __syncthreads();  // shared arrays are reused by the block's next set
