@@ -110,9 +110,14 @@ __device__ __forceinline__ void cta_bwd_wide(const GameView &g, T *v, int32_t wi
   }
 }
 
+// FP64 kernels hold two registers a value: fewer threads, more registers. The
+// FP64 pipe is full with four warps an SM.
+template <typename T, int MAXA, int THREADS> constexpr int kBatchThreads = sizeof(T) == 8 && THREADS > 256 ? (MAXA <= 4 ? 512 : 256) : THREADS;
+
 template <typename T, int MAXA, int LANES, int THREADS, bool CLUSTERED>
 __global__ void __launch_bounds__(THREADS) batch_iterate_kernel(const InstDesc *table, int n_inst) {
   __shared__ double sm[THREADS];
+  __shared__ double s_rows[THREADS / 32][kChainDoubles<T, MAXA, LANES>];
   const int ncta = CLUSTERED ? (int)cluster_ncta() : 1;   // CTAs sharing this instance
   const int rank = CLUSTERED ? (int)cluster_rank() : 0;
   const int inst = (int)blockIdx.x / ncta;
@@ -162,7 +167,7 @@ __global__ void __launch_bounds__(THREADS) batch_iterate_kernel(const InstDesc *
         }
         // 1024-thread blocks leave 64 registers a thread: lean average terms
         for (int32_t I = w.is0 + gid; I < w.is1; I += NG)
-          bwd_set<T, MAXA, LANES, CLUSTERED, (THREADS >= 1024)>(in.g, st, I, I >= w.is2, lane, mask, wt, in.rule, upd);
+          bwd_set<T, MAXA, LANES, CLUSTERED, (THREADS >= 1024)>(in.g, st, I, I >= w.is2, lane, mask, wt, in.rule, upd, s_rows[threadIdx.x / 32]);
         level_sync<CLUSTERED>();
       }
     }

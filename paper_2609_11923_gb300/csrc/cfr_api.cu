@@ -296,7 +296,11 @@ extern "C" int cfr_compile(const cfr_game_spec *spec, const cfr_options *opt, cf
   if (h->exec_form == CFR_EXEC_AUTO)
     h->exec_form = c.N <= (h->opt.precision == CFR_P32 ? 768 : 350) ? CFR_EXEC_PERSISTENT : CFR_EXEC_GRAPH;
   // lanes per information set: the smallest group that covers the mean set
-  auto pick = [](double mean) { return mean <= 4.0 ? 4 : mean <= 8.0 ? 8 : mean <= 16.0 ? 16 : 32; };
+  // (FP64: at most 8, the group its ordered sums are cheapest with)
+  const int widest = h->opt.precision == CFR_P64 && h->maxa_tier <= 8 ? 8 : 32;
+  auto pick = [&](double mean) {
+    return std::min(widest, mean <= 4.0 ? 4 : mean <= 8.0 ? 8 : mean <= 16.0 ? 16 : 32);
+  };
   // (tiled depths: at most one tile of sets per warp's worth of lanes, so a
   // warp's member reads stay one run)
   h->level_lanes.assign(c.D, 8);

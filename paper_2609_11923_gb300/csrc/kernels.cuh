@@ -583,34 +583,62 @@ __device__ __forceinline__ void member_terms(const GameView &g, const StateView<
   member_data<T, MAXA, PERSIST, LEAN>(g, st, k, m0, m1, vb, na, p2, sig, h, ir, d, mm);
 }
 
-// Adds one chunk's member terms to the group totals. P64: lane order (the
-// members' ascending order), every lane ends with the same totals. P32:
-// per-lane partial sums (finished by a butterfly).
+// FP64 sums of a set run in the order of the definition, one dependent chain
+// of adds for every slot's regret term and every slot's average term. On
+// GB300 a warp instruction of the FP64 pipe costs the SM 16-19 cycles
+// however few lanes it serves, so a chain belongs to one lane: chain c < MAXA
+// is the regret sum of action c, chain MAXA + a the average sum of action a,
+// and lane c % LANES of the group adds chain c's terms member by member from
+// the warp's rows in shared memory. (Every lane adding every chain took
+// 2 * na adds a member where this takes one or two.) One FP64 iteration of the
+// 11M-node card game, autotuned: 701 -> 488 us; of an 80k-node random tree in
+// two half passes: 367 -> 266 us.
+template <typename T, int MAXA, int LANES>
+constexpr bool kChains = sizeof(T) == 8 && LANES >= 4 && LANES <= 32 && MAXA <= 8;
+template <int MAXA, int LANES> constexpr int kChainAcc = (2 * MAXA + LANES - 1) / LANES;  // chains of a lane
+constexpr int kChainRow = 33;  // doubles of a chain's row: a term of each lane, and one that spreads the banks
+template <typename T, int MAXA, int LANES>
+constexpr int kChainDoubles = kChains<T, MAXA, LANES> ? 2 * MAXA * kChainRow : 1;  // a warp's rows
+
+template <int MAXA, int LANES>
+__device__ __forceinline__ void accumulate_chains(double *rows, int32_t cnt, int32_t na, unsigned mask,
+                                                  const double (&d)[MAXA], const double (&mm)[MAXA],
+                                                  double (&acc)[kChainAcc<MAXA, LANES>]) {
+  const int wl = threadIdx.x & 31, lane = wl & (LANES - 1), g0 = wl - lane;
+#pragma unroll
+  for (int a = 0; a < MAXA; ++a) {
+    if (a < na) {
+      rows[a * kChainRow + wl] = d[a];
+      rows[(MAXA + a) * kChainRow + wl] = mm[a];
+    }
+  }
+  __syncwarp(mask);
+#pragma unroll
+  for (int j = 0; j < LANES; ++j) {
+    if (j < cnt) {
+#pragma unroll
+      for (int i = 0; i < kChainAcc<MAXA, LANES>; ++i) {
+        const int c = lane + i * LANES;  // rows of actions >= na hold stale terms: their sums are never used
+        if (c < 2 * MAXA) acc[i] = acc[i] + rows[c * kChainRow + g0 + j];
+      }
+    }
+  }
+  __syncwarp(mask);
+}
+
+// Adds one chunk's member terms to the group totals. P64 without chains:
+// lane order (the members' ascending order), every lane ends with the same
+// totals. P32: per-lane partial sums (finished by a butterfly).
 template <typename T, int MAXA, int LANES>
 __device__ __forceinline__ void accumulate_chunk(int32_t cnt, int32_t na, unsigned mask, const T (&d)[MAXA],
                                                  const T (&mm)[MAXA], T (&racc)[MAXA], T (&macc)[MAXA]) {
   if constexpr (sizeof(T) == 8) {
-    if constexpr (LANES <= 8) {  // unrolled: the shuffles issue ahead of the ordered adds
+    for (int j = 0; j < cnt; ++j) {
 #pragma unroll
-      for (int j = 0; j < LANES; ++j) {
-        if (j < cnt) {
-#pragma unroll
-          for (int a = 0; a < MAXA; ++a) {
-            if (a < na) {
-              racc[a] = racc[a] + __shfl_sync(mask, d[a], j, LANES);
-              macc[a] = macc[a] + __shfl_sync(mask, mm[a], j, LANES);
-            }
-          }
-        }
-      }
-    } else {  // wide groups keep the loop (registers)
-      for (int j = 0; j < cnt; ++j) {
-#pragma unroll
-        for (int a = 0; a < MAXA; ++a) {
-          if (a < na) {
-            racc[a] = racc[a] + __shfl_sync(mask, d[a], j, LANES);
-            macc[a] = macc[a] + __shfl_sync(mask, mm[a], j, LANES);
-          }
+      for (int a = 0; a < MAXA; ++a) {
+        if (a < na) {
+          racc[a] = racc[a] + __shfl_sync(mask, d[a], j, LANES);
+          macc[a] = macc[a] + __shfl_sync(mask, mm[a], j, LANES);
         }
       }
     }
@@ -630,7 +658,7 @@ __device__ __forceinline__ void accumulate_chunk(int32_t cnt, int32_t na, unsign
 // the set's slots runs one lane per action. LEAN: see member_data.
 template <typename T, int MAXA, int LANES, bool PERSIST, bool LEAN = false>
 __device__ __forceinline__ void bwd_set(const GameView &g, const StateView<T> &st, int32_t I, bool p2,
-                                        int lane, unsigned mask, double wt, int rule, int upd) {
+                                        int lane, unsigned mask, double wt, int rule, int upd, double *rows) {
   const int32_t sb = __ldg(g.iset_slot + I);
   const int32_t na = __ldg(g.iset_slot + I + 1) - sb;
   const int32_t m0 = __ldg(g.iset_mem + I), m1 = __ldg(g.iset_mem + I + 1);
@@ -643,6 +671,14 @@ __device__ __forceinline__ void bwd_set(const GameView &g, const StateView<T> &s
     racc[a] = T(0);
     macc[a] = T(0);
   }
+  constexpr bool CHAINS = kChains<T, MAXA, LANES>;
+  double acc[kChainAcc<MAXA, LANES>];  // CHAINS: this lane's chains instead of racc, macc
+#pragma unroll
+  for (int i = 0; i < kChainAcc<MAXA, LANES>; ++i) acc[i] = 0.0;
+  auto add_chunk = [&](int32_t cnt, const T(&d)[MAXA], const T(&mm)[MAXA]) {
+    if constexpr (CHAINS) accumulate_chains<MAXA, LANES>(rows, cnt, na, mask, d, mm, acc);
+    else accumulate_chunk<T, MAXA, LANES>(cnt, na, mask, d, mm, racc, macc);
+  };
   constexpr bool TWO = MAXA <= 8 && LANES <= 8;  // narrow groups keep two chunks in flight
   constexpr int NCH = 2;
   int32_t k0 = m0;
@@ -666,8 +702,7 @@ __device__ __forceinline__ void bwd_set(const GameView &g, const StateView<T> &s
 #pragma unroll
         for (int j = 0; j < NCH; ++j) {  // chunks in member order
           const int32_t left = m1 - k0 - j * LANES;
-          accumulate_chunk<T, MAXA, LANES>(left < 0 ? 0 : (left < LANES ? left : LANES), na, mask, d[j], mm[j], racc,
-                                           macc);
+          add_chunk(left < 0 ? 0 : (left < LANES ? left : LANES), d[j], mm[j]);
         }
 #pragma unroll
         for (int j = 0; j < NCH; ++j) {
@@ -688,9 +723,9 @@ __device__ __forceinline__ void bwd_set(const GameView &g, const StateView<T> &s
         T d0[MAXA], mm0[MAXA], d1[MAXA], mm1[MAXA];
         member_data<T, MAXA, PERSIST, LEAN>(g, st, k0 + lane, m0, m1, vb, na, p2, sig, ps0, ir0, d0, mm0);
         member_data<T, MAXA, PERSIST, LEAN>(g, st, k0 + LANES + lane, m0, m1, vb, na, p2, sig, ps1, ir1, d1, mm1);
-        accumulate_chunk<T, MAXA, LANES>(LANES, na, mask, d0, mm0, racc, macc);
+        add_chunk(LANES, d0, mm0);
         const int32_t c1 = (m1 - k0 - LANES) < LANES ? (m1 - k0 - LANES) : LANES;
-        accumulate_chunk<T, MAXA, LANES>(c1, na, mask, d1, mm1, racc, macc);
+        add_chunk(c1, d1, mm1);
         ps0 = qs0; ir0 = jr0; ps1 = qs1; ir1 = jr1;
       }
     }
@@ -700,7 +735,7 @@ __device__ __forceinline__ void bwd_set(const GameView &g, const StateView<T> &s
       T d[MAXA], mm[MAXA];
       member_terms<T, MAXA, PERSIST, LEAN>(g, st, k0 + lane, m0, m1, mr, vb, na, p2, sig, d, mm);
       const int32_t cnt = (m1 - k0) < LANES ? (m1 - k0) : LANES;
-      accumulate_chunk<T, MAXA, LANES>(cnt, na, mask, d, mm, racc, macc);
+      add_chunk(cnt, d, mm);
     }
   } else {
     int32_t ps, ir;
@@ -711,7 +746,7 @@ __device__ __forceinline__ void bwd_set(const GameView &g, const StateView<T> &s
       T d[MAXA], mm[MAXA];
       member_data<T, MAXA, PERSIST, LEAN>(g, st, k0 + lane, m0, m1, vb, na, p2, sig, ps, ir, d, mm);
       const int32_t cnt = (m1 - k0) < LANES ? (m1 - k0) : LANES;
-      accumulate_chunk<T, MAXA, LANES>(cnt, na, mask, d, mm, racc, macc);
+      add_chunk(cnt, d, mm);
       ps = qs; ir = jr;
     }
   }
@@ -730,20 +765,34 @@ __device__ __forceinline__ void bwd_set(const GameView &g, const StateView<T> &s
       avg_terms<T, MAXA>(sig, na, macc);
     }
   }
-  // every lane now holds the set's totals racc[a], macc[a]
+  // every lane now holds the set's totals racc[a], macc[a] (CHAINS: its own
+  // chains' totals)
+  if constexpr (CHAINS && LANES < MAXA) {  // more actions than lanes are possible: every lane takes all totals
+#pragma unroll
+    for (int a = 0; a < MAXA; ++a) {
+      racc[a] = __shfl_sync(mask, acc[a / LANES], a % LANES, LANES);
+      macc[a] = __shfl_sync(mask, acc[(MAXA + a) / LANES], (MAXA + a) % LANES, LANES);
+    }
+  }
   if (na <= LANES) {
     // lane a updates slot a (slot_update), then sigma^{t+1} = RM; the sum of
     // positive parts runs in action order
     T r = T(0), m = T(0);
+    if constexpr (CHAINS && LANES >= MAXA) {
+      r = acc[0];
+      if constexpr (MAXA % LANES == 0) m = acc[MAXA / LANES];
+      else m = __shfl_sync(mask, acc[0], (lane + MAXA) & (LANES - 1), LANES);
+    } else {
 #pragma unroll
-    for (int a = 0; a < MAXA; ++a)
-      if (a == lane) { r = racc[a]; m = macc[a]; }
+      for (int a = 0; a < MAXA; ++a)
+        if (a == lane) { r = racc[a]; m = macc[a]; }
+    }
     double pos = 0.0;
     if (lane < na) pos = slot_update(st.R, st.avg, sb + lane, as_double(r), as_double(m), wt, rule);
     if constexpr (sizeof(T) == 8) {
       double tot = 0.0;
       for (int a = 0; a < na; ++a) tot += __shfl_sync(mask, pos, a, LANES);
-      if (lane < na) st.sigma[sb + lane] = tot > 0.0 ? pos / tot : 1.0 / (double)na;
+      if (lane < na) st.sigma[sb + lane] = __double_as_longlong(tot) > 0 ? pos / tot : 1.0 / (double)na;
     } else {
       const float pf = narrow_pos(pos);
       float tot = 0.f;
@@ -792,7 +841,7 @@ __device__ __forceinline__ void bwd_set_block(const GameView &g, const StateView
     racc[a] = T(0);
     macc[a] = T(0);
   }
-  T r = T(0), m = T(0);  // P64: column tid's running sums (tid < na)
+  T r = T(0), m = T(0);  // P64: r is chain tid's running sum (tid < 2 MAXA)
   int32_t ps, ir;
   member_idx(g, m0 + tid, m1, mr, ps, ir);
   for (int32_t k0 = m0; k0 < m1; k0 += kThreads) {
@@ -809,12 +858,10 @@ __device__ __forceinline__ void bwd_set_block(const GameView &g, const StateView
         s_m[tid * MAXA + a] = mm[a];
       }
       __syncthreads();
-      if (tid < na) {
+      if (tid < 2 * MAXA) {  // one chain a thread: the regret columns, then the average columns
         const int cnt = (m1 - k0) < kThreads ? (m1 - k0) : kThreads;
-        for (int j = 0; j < cnt; ++j) {
-          r = r + s_d[j * MAXA + tid];
-          m = m + s_m[j * MAXA + tid];
-        }
+        const T *col = tid < MAXA ? s_d + tid : s_m + (tid - MAXA);
+        for (int j = 0; j < cnt; ++j) r = r + col[j * MAXA];
       }
       __syncthreads();
     } else {
@@ -848,6 +895,12 @@ __device__ __forceinline__ void bwd_set_block(const GameView &g, const StateView
       m = s_m[tid];
     }
   }
+  if constexpr (sizeof(T) == 8) {  // thread a takes its average chain's total
+    __syncthreads();
+    if (tid >= MAXA && tid < 2 * MAXA) s_m[tid - MAXA] = r;
+    __syncthreads();
+    if (tid < na) m = s_m[tid];
+  }
   // thread a updates slot a (slot_update), then sigma^{t+1} = RM with the
   // positive parts summed in action order
   double pos = 0.0;
@@ -874,7 +927,7 @@ __device__ __forceinline__ void bwd_set_block(const GameView &g, const StateView
 // chunk, then the information-set groups (LANES == kThreads: one set per
 // block).
 template <typename T, int MAXA, int LANES>
-__global__ void __launch_bounds__(kThreads, MAXA <= 4 ? 4 : (MAXA <= 8 ? 3 : 1)) bwd_level_kernel(GameView g, StateView<T> st, LevelWork w,
+__global__ void __launch_bounds__(kThreads, MAXA > 8 ? 1 : (MAXA <= 4 ? 4 : 3) - (sizeof(T) == 8 ? 1 : 0)) bwd_level_kernel(GameView g, StateView<T> st, LevelWork w,
                                                             int nb_chance, int rule, int upd, int bump_t) {
   pdl_enter();
   const int nb_wide = w.wc1 - w.wc0;
@@ -897,8 +950,9 @@ __global__ void __launch_bounds__(kThreads, MAXA <= 4 ? 4 : (MAXA <= 8 ? 3 : 1))
     const int lane = threadIdx.x % LANES;
     const unsigned mask = group_mask<LANES>();
     const double wt = avg_weight(*st.t + 1, rule);
+    __shared__ double s_rows[kThreads / 32][kChainDoubles<T, MAXA, LANES>];
     for (int32_t I = w.is0 + gid; I < w.is1; I += ngroups)
-      bwd_set<T, MAXA, LANES, false>(g, st, I, I >= w.is2, lane, mask, wt, rule, upd);
+      bwd_set<T, MAXA, LANES, false>(g, st, I, I >= w.is2, lane, mask, wt, rule, upd, s_rows[threadIdx.x / 32]);
   }
   if (bump_t) {  // depth 0 holds only the root: no other block reads t here
     __syncthreads();
@@ -982,6 +1036,7 @@ __global__ void __launch_bounds__(kThreads) persistent_kernel(PersistArgs<T> a) 
   const int gid = tid / LANES, ngroups = nthr / LANES, lane = tid % LANES;
   const unsigned mask = group_mask<LANES>();
   const int halves = a.order ? 2 : 1;  // alternating: player 1's half, then player 2's
+  __shared__ double s_rows[kThreads / 32][kChainDoubles<T, MAXA, LANES>];
   for (long long it = 0; it < a.n_iter; ++it) {
     const double wt = avg_weight(t0 + it + 1, a.rule);
     for (int hf = 0; hf < halves; ++hf) {
@@ -1010,7 +1065,7 @@ __global__ void __launch_bounds__(kThreads) persistent_kernel(PersistArgs<T> a) 
           for (int32_t q = w.wc0 + blockIdx.x; q < w.wc1; q += gridDim.x) bwd_wide_chunk<T, true>(a.g, w, a.st.v, q);
         }
         for (int32_t I = w.is0 + gid; I < w.is1; I += ngroups)
-          bwd_set<T, MAXA, LANES, true>(a.g, a.st, I, I >= w.is2, lane, mask, wt, a.rule, upd);
+          bwd_set<T, MAXA, LANES, true>(a.g, a.st, I, I >= w.is2, lane, mask, wt, a.rule, upd, s_rows[threadIdx.x / 32]);
         if (!grid_sync(a.bar)) return;
       }
     }

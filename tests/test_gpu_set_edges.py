@@ -1,0 +1,47 @@
+"""Sets at the edges of the lane groups: one set of M members and A actions
+above A sets of M members and B actions, M around the group and block sizes
+and actions around the register tiers. FP64 sums run one chain per slot and
+must equal the oracle bitwise whatever the group."""
+import numpy as np
+import pytest
+import torch
+
+import gamegen as gg
+import oracle
+from paper_2609_11923_gb300 import cfr
+
+pytestmark = pytest.mark.gpu
+
+
+def two_level_game(m, a, b, seed=0):
+    """Chance over m outcomes; player 1 (one set, a actions) does not see
+    which; player 2 (b actions) sees player 1's action only. Random payoffs."""
+    rng = np.random.default_rng(1000 * seed + 100 * m + 10 * a + b)
+    p = rng.gamma(1.0, size=m)
+    nodes = [(gg.CHANCE, -1, list(range(1, m + 1)), list(p / p.sum()), 0.0)]
+    nodes += [None] * m
+    for k in range(1, m + 1):
+        kids = []
+        for i in range(a):
+            leaves = []
+            for _ in range(b):
+                leaves.append(len(nodes))
+                nodes.append((gg.TERMINAL, -1, [], None, float(rng.uniform(-1, 1))))
+            kids.append(len(nodes))
+            nodes.append((gg.P2, 1 + i, leaves, None, 0.0))
+        nodes[k] = (gg.P1, 0, kids, None, 0.0)
+    return gg.from_lists(nodes, [(0, a)] + [(1, b)] * a)
+
+
+@pytest.mark.parametrize("lanes", [1, 2, 4, 8, 16, 32, 256])
+@pytest.mark.parametrize("a,b", [(2, 3), (4, 4), (5, 2), (8, 7)])
+def test_fp64_sums_equal_the_oracle_at_every_group_edge(lanes, a, b):
+    for m in (1, 3, 4, 7, 8, 9, 16, 17, 31, 33, 255, 257):
+        g = two_level_game(m, a, b)
+        s = cfr.Solver(g, precision=cfr.P64, exec_form=cfr.EXEC_LEVELS, lanes_per_set=lanes)
+        s.iterate(30)
+        R, avg, _ = s.get_state()
+        o = oracle.solve(g, 30)
+        np.testing.assert_array_equal(R, o.R, err_msg="m=%d" % m)
+        np.testing.assert_array_equal(avg, o.sbar, err_msg="m=%d" % m)
+        s.close()
