@@ -927,13 +927,14 @@ extern "C" int cfr_current_strategy(cfr_handle *h, double *out, int on_device, v
 
 static int launch_br(cfr_handle *h, int d, cudaStream_t s) {
   const LevelWork &w = h->levels[d];
-  const int L = std::min(h->level_lanes[d], 32);  // best response: lane groups of at most a warp
+  int L = std::min(h->level_lanes[d], 32);  // best response: lane groups of at most a warp
+  if (h->c.level_tiled[d]) L = std::min(L, kTiledLanes);
   const int nch = w.ch1 - w.ch0, nis = w.is1 - w.is0;
   const int nb_ch = nch > 0 ? grid_for(nch, kThreads) : 0;
   const int nb_is = nis > 0 ? grid_for(nis, kThreads / L) : 0;
   const int nb_wide = w.wc1 - w.wc0;
   CK(launch_br_level(h->maxa_tier, L, std::max(1, nb_ch + nb_wide + nb_is), s, game_view(h), h->p<double2>(h->b_reach2),
-                     h->p<double>(h->b_sbs), h->p<double2>(h->b_vb), h->p<double>(h->b_vavg), w, nb_ch));
+                     h->p<double>(h->b_sbs), h->p<double2>(h->b_vb), h->p<double>(h->b_vavg), w, nb_ch, true));
   return CFR_OK;
 }
 
@@ -948,20 +949,20 @@ extern "C" int cfr_exploitability(cfr_handle *h, double *out_expl, double *out_b
                                                                        h->p<double>(h->b_avg), h->p<double>(h->b_sbs));
   CK(cudaGetLastError());
   for (int64_t d = 0; d < c.D; ++d) {
-    int rc = launch_fwd<double>(h, d, s, g, h->p<double>(h->b_sbs), h->p<double2>(h->b_reach2));
+    int rc = launch_fwd<double>(h, d, s, g, h->p<double>(h->b_sbs), h->p<double2>(h->b_reach2), d > 0);
     if (rc) return rc;
   }
   for (int64_t d = c.D - 1; d >= 0; --d) {
     int rc = launch_br(h, (int)d, s);
     if (rc) return rc;
   }
-  double root[3];
-  const int64_t rs = c.N - 1;  // the root's value slot
-  CK(cudaMemcpyAsync(root, h->p<double2>(h->b_vb) + rs, 16, cudaMemcpyDeviceToHost, s));
-  CK(cudaMemcpyAsync(root + 2, h->p<double>(h->b_vavg) + rs, 8, cudaMemcpyDeviceToHost, s));
+  double *res = h->p<double>(h->b_out), root[4];
+  CK(launch_k(br_result_kernel, 1, 1, 0, s, true, (const double2 *)h->p<double2>(h->b_vb),
+              (const double *)h->p<double>(h->b_vavg), (int32_t)(c.N - 1), res));  // N - 1: the root's value slot
+  CK(cudaMemcpyAsync(root, res, sizeof root, cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
-  *out_expl = 0.5 * (root[0] - root[1]);
-  if (out_br) { out_br[0] = root[0]; out_br[1] = root[1]; out_br[2] = root[2]; }
+  *out_expl = root[0];
+  if (out_br) { out_br[0] = root[1]; out_br[1] = root[2]; out_br[2] = root[3]; }
   return CFR_OK;
 }
 

@@ -50,7 +50,7 @@ cudaError_t launch_persistent(int maxa, int lanes, int grid, cudaStream_t s, Per
                               int *query_occupancy);
 
 cudaError_t launch_br_level(int maxa, int lanes, int grid, cudaStream_t s, GameView g, const double2 *reach2,
-                            const double *sbs, double2 *vb, double *vavg, LevelWork w, int nb_chance);
+                            const double *sbs, double2 *vb, double *vavg, LevelWork w, int nb_chance, bool pdl);
 
 }  // namespace cfr
 
