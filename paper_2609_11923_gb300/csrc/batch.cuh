@@ -1,23 +1,70 @@
 // batch.cuh — many independent solves in one launch (batched serving).
 //
-// One CTA owns one instance for the whole call: it runs that instance's n
-// CFR+ iterations with __syncthreads() between depth levels (no grid
-// barrier, no cross-CTA traffic), so a batch of hundreds of uneven
-// subgames is one launch whose CTAs the hardware schedules as SMs free up.
-// Large instances instead get a thread-block cluster of several CTAs (the
-// clustered instances of the kernel, launched with a cluster dimension):
-// the cluster's CTAs share each depth's work and meet at the hardware
-// cluster barrier (barrier.cluster, release/acquire) between depths, and
-// read the state arrays through L2 because their L1s are not coherent.
-// Each instance's arithmetic depends only on its own arrays and on the
-// launch shape (THREADS, LANES, cluster size): a solve gives bitwise the
-// same result alone and inside any mix run with the same shape. The
-// per-level device functions are the ones of kernels.cuh; wide chance nodes
-// are summed by one CTA in a fixed order.
+// One CTA, or one thread-block cluster of up to 16, owns one instance for the
+// whole call: it runs that instance's n CFR+ iterations with a barrier between
+// depth levels (no grid barrier). How many CTAs an instance gets is chosen by
+// plan_clusters from the sizes in the batch; instances of one cluster size
+// are one launch, and the launches of a call run concurrently (chain_enter).
+// The CTAs of a cluster share each depth's work, meet at the hardware cluster
+// barrier (barrier.cluster, release/acquire) between depths, and read the
+// state arrays through L2 because their L1s are not coherent. Each instance's
+// arithmetic depends only on its own arrays and on (THREADS, LANES), not on
+// the number of its CTAs: a solve gives bitwise the same result alone and
+// inside any mix run with the same shape. Wide chance nodes are summed by one
+// CTA in a fixed order.
+//
+// One CTA for every instance left the largest alone on one SM: a round of 64
+// endgames of 1e3 to 2e5 edges (50 iterations, exploitability, strategies)
+// 13.2 -> 5.0 ms; of ten of 2e5 to 1e6 edges, 8 CTAs each before, 11.9 -> 9.2.
 #pragma once
+#include <algorithm>
+#include <queue>
+#include <utility>
+#include <vector>
+
 #include "kernels.cuh"
 
 namespace cfr {
+
+// CTAs for every instance of a batch (host). load: the instance's nodes times
+// the share of the longest run's iterations. Starting from `least` CTAs each,
+// the instance with the most load per CTA takes the next cluster size while
+// SMs are left for it, or its share exceeds an even one of the whole batch;
+// kSplitNodes per CTA and less stay whole, because a cluster barrier costs
+// more than a CTA's (about 1,600 cycles against 300 with stores in flight)
+// and the state is then read through L2. Clusters above 8 CTAs need most of a
+// GPC: at most six of them.
+constexpr int64_t kSplitNodes = 12000;
+inline std::vector<int> plan_clusters(const std::vector<int64_t> &load, int least, int sms) {
+  static const int sizes[] = {1, 2, 3, 4, 6, 8, 12, 16};
+  const int n = (int)load.size();
+  std::vector<int> cta(n, least);
+  std::priority_queue<std::pair<int64_t, int>> most;  // (load per CTA, instance)
+  int64_t all = 0;
+  int used = 0, wide = 0;
+  for (int i = 0; i < n; ++i) {
+    all += load[i];
+    used += least;
+    most.push({load[i] / least, -i});
+  }
+  while (!most.empty()) {
+    const int64_t per = most.top().first;
+    const int i = -most.top().second;
+    most.pop();
+    if (per <= kSplitNodes) break;
+    int next = 0;
+    for (int c : sizes)
+      if (c > cta[i]) { next = c; break; }
+    if (next == 0 || (next > 8 && cta[i] <= 8 && wide == 6)) continue;
+    if (used + next - cta[i] > sms && per <= all / sms) break;
+    if (next > 8 && used + next - cta[i] > sms) continue;
+    if (next > 8 && cta[i] <= 8) ++wide;
+    used += next - cta[i];
+    cta[i] = next;
+    most.push({load[i] / next, -i});
+  }
+  return cta;
+}
 
 // Everything a CTA needs about one bound instance (device pointers into the
 // instance's own arena).
@@ -34,7 +81,8 @@ struct InstDesc {
   double2 *vb;
   double *vavg;
   double *sbs;
-  double *out;      // exploitability result slot (batch_br_kernel)
+  double *out;      // read-out scratch of A doubles (as sbs)
+  double *res;      // four results of batch_br_kernel
   long long n_iter; // iterations this call runs for the instance
   int32_t D;
   int32_t rule;
@@ -110,20 +158,41 @@ __device__ __forceinline__ void cta_bwd_wide(const GameView &g, T *v, int32_t wi
   }
 }
 
+constexpr int kBatchLevels = 32;  // depths whose work descriptors a CTA keeps in shared memory
+
 // FP64 kernels hold two registers a value: fewer threads, more registers. The
 // FP64 pipe is full with four warps an SM.
 template <typename T, int MAXA, int THREADS> constexpr int kBatchThreads = sizeof(T) == 8 && THREADS > 256 ? (MAXA <= 4 ? 512 : 256) : THREADS;
 
+// Every launch of one call's chain may start as soon as the one before it has
+// started (programmatic dependent launch: the instances are independent);
+// the first CTA of each waits, once its own work is done, for the launch
+// before to be complete, so the end of the last launch is the end of all.
+__device__ __forceinline__ void chain_enter() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void chain_leave() {
+  if (blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// What bounds it: a small instance is a chain of dependent steps, 2 D - 1 of
+// them an iteration, each a barrier and two or three dependent loads; a large
+// one is latency of gathers at the occupancy of 64 registers a thread. The
+// slot updates (FP64) wait until the values of all depths are known and then
+// run one thread per set over the whole game: on the way up they would hold
+// every depth back by a dependent chain of FP64 instructions that serve a few
+// lanes each.
 template <typename T, int MAXA, int LANES, int THREADS, bool CLUSTERED>
-__global__ void __launch_bounds__(THREADS) batch_iterate_kernel(const InstDesc *table, int n_inst) {
+__global__ void __launch_bounds__(THREADS) batch_iterate_kernel(const InstDesc *table,
+                                                                const __grid_constant__ InstDesc one, int n_inst) {
   __shared__ double sm[THREADS];
   __shared__ double s_rows[THREADS / 32][kChainDoubles<T, MAXA, LANES>];
+  __shared__ LevelWork s_lw[kBatchLevels];
+  chain_enter();
   const int ncta = CLUSTERED ? (int)cluster_ncta() : 1;   // CTAs sharing this instance
   const int rank = CLUSTERED ? (int)cluster_rank() : 0;
   const int inst = (int)blockIdx.x / ncta;
   if (inst >= n_inst) return;  // the whole cluster leaves together
   const int ct = rank * THREADS + (int)threadIdx.x, NT = ncta * THREADS;
-  const InstDesc in = table[inst];
+  const InstDesc in = table ? table[inst] : one;
   StateView<T> st;
   st.reach = (vec2_t<T> *)in.reach;
   st.v = (T *)in.v;
@@ -131,24 +200,33 @@ __global__ void __launch_bounds__(THREADS) batch_iterate_kernel(const InstDesc *
   st.R = in.R;
   st.avg = in.avg;
   st.t = in.t;
+  T *def_r = (T *)in.sbs, *def_m = (T *)in.out;  // the sets' totals (read-out scratch, idle here)
+  const LevelWork *lw = in.lw;
+  if (in.D <= kBatchLevels) {
+    const int words = in.D * (int)(sizeof(LevelWork) / 4);
+    for (int i = threadIdx.x; i < words; i += THREADS)
+      reinterpret_cast<int *>(s_lw)[i] = reinterpret_cast<const int *>(in.lw)[i];
+    lw = s_lw;
+    __syncthreads();
+  }
   const long long t0 = *in.t;
   const int lane = threadIdx.x % LANES, gid = ct / LANES;
   const int NG = NT / LANES;
   const unsigned mask = group_mask<LANES>();
+  double *rows = s_rows[threadIdx.x / 32];
   const int halves = in.order ? 2 : 1;  // alternating: player 1's half, then player 2's
   for (long long it = 0; it < in.n_iter; ++it) {
     const double wt = avg_weight(t0 + it + 1, in.rule);
     for (int hf = 0; hf < halves; ++hf) {
       const int upd = in.order ? (1 << hf) : 3;
       for (int d = 0; d < in.D; ++d) {
-        const LevelWork w = in.lw[d];
         if (in.g.int_edge) {  // member order: depth d + 1 pulls
-          if (d + 1 < in.D) {
-            const int32_t qe = in.lw[d + 1].ie;
-            for (int32_t q = in.lw[d + 1].ib + ct; q < qe; q += kPull * NT)
-              fwd_pull<T, CLUSTERED>(in.g, st.sigma, st.reach, q, NT, qe);
-          }
+          if (d + 1 >= in.D) break;
+          const int32_t qe = lw[d + 1].ie;
+          for (int32_t q = lw[d + 1].ib + ct; q < qe; q += kPull * NT)
+            fwd_pull<T, CLUSTERED>(in.g, st.sigma, st.reach, q, NT, qe);
         } else {
+          const LevelWork w = lw[d];
           for (int32_t qw = w.ib + rank * THREADS + (threadIdx.x & ~31); qw < w.ie; qw += 4 * NT) {
             if (w.fan) fwd_int4<T, CLUSTERED, true>(in.g, st.sigma, st.reach, qw + (threadIdx.x & 31), NT, w.ie);
             else fwd_int4<T, CLUSTERED, false>(in.g, st.sigma, st.reach, qw + (threadIdx.x & 31), NT, w.ie);
@@ -158,138 +236,106 @@ __global__ void __launch_bounds__(THREADS) batch_iterate_kernel(const InstDesc *
         level_sync<CLUSTERED>();
       }
       for (int d = in.D - 1; d >= 0; --d) {
-        const LevelWork w = in.lw[d];
-        if (d > 0) {  // a chance root's value has no reader in an iteration
+        const LevelWork w = lw[d];
+        if (d == 0 && w.is0 == w.is1) break;  // a chance root's value has no reader in an iteration
+        if (d > 0) {
           for (int32_t i = w.ch0 + ct; i < w.ch1; i += NT)
             bwd_chance<T, CLUSTERED>(in.g, st.v, i);
           if (rank == 0)
             for (int32_t i = w.wd0; i < w.wd1; ++i) cta_bwd_wide<T, THREADS, CLUSTERED>(in.g, st.v, i, sm);
         }
-        // 1024-thread blocks leave 64 registers a thread: lean average terms
         for (int32_t I = w.is0 + gid; I < w.is1; I += NG)
-          bwd_set<T, MAXA, LANES, CLUSTERED, (THREADS >= 1024)>(in.g, st, I, I >= w.is2, lane, mask, wt, in.rule, upd, s_rows[threadIdx.x / 32]);
+          bwd_set<T, MAXA, LANES, CLUSTERED, sizeof(T) == 4, true>(in.g, st, I, I >= w.is2, lane, mask, wt, in.rule,
+                                                                  upd, rows, def_r, def_m);
         level_sync<CLUSTERED>();
       }
+      if (upd == 3) {
+        for (int32_t I = ct; I < in.n_sets; I += NT)
+          update_set<T, MAXA, CLUSTERED>(in.g, st, I, wt, in.rule, def_r, def_m);
+      } else {  // one player's sets
+        for (int d = 0; d < in.D; ++d) {
+          const int32_t i0 = upd == 1 ? lw[d].is0 : lw[d].is2, i1 = upd == 1 ? lw[d].is2 : lw[d].is1;
+          for (int32_t I = i0 + (ct + NT - i0 % NT) % NT; I < i1; I += NT)  // set I: always thread I % NT
+            update_set<T, MAXA, CLUSTERED>(in.g, st, I, wt, in.rule, def_r, def_m);
+        }
+      }
+      level_sync<CLUSTERED>();
     }
   }
   if (ct == 0) *in.t = t0 + in.n_iter;
+  chain_leave();
 }
 
-// Exploitability of every instance's average strategy (FP64), one CTA each:
-// normalise the average, forward reach under it, then both best responses by
-// depth (the same arithmetic as br_level_kernel, with CTA-wide loops).
-template <int MAXA, int LANES, int THREADS>
-__global__ void __launch_bounds__(THREADS) batch_br_kernel(const InstDesc *table, int n_inst) {
+// Exploitability of every instance's average strategy (FP64): normalise the
+// average, forward reach under it, then both best responses by depth (the
+// arithmetic of br_level_kernel). CTAs and clusters as batch_iterate_kernel.
+template <int MAXA, int LANES, int THREADS, bool CLUSTERED>
+__global__ void __launch_bounds__(THREADS) batch_br_kernel(const InstDesc *table, const __grid_constant__ InstDesc one,
+                                                           int n_inst) {
   __shared__ double sm[THREADS];
-  const int inst = blockIdx.x;
+  chain_enter();
+  const int ncta = CLUSTERED ? (int)cluster_ncta() : 1;
+  const int rank = CLUSTERED ? (int)cluster_rank() : 0;
+  const int inst = (int)blockIdx.x / ncta;
   if (inst >= n_inst) return;
-  const InstDesc in = table[inst];
+  const int ct = rank * THREADS + (int)threadIdx.x, NT = ncta * THREADS;
+  const InstDesc in = table ? table[inst] : one;
   const GameView &g = in.g;
   // average strategy, normalised per set
-  for (int32_t I = threadIdx.x; I < in.n_sets; I += THREADS) {
+  for (int32_t I = ct; I < in.n_sets; I += NT) {
     const int32_t sb = __ldg(g.iset_slot + I), na = __ldg(g.iset_slot + I + 1) - sb;
     double tot = 0.0;
     for (int32_t a = 0; a < na; ++a) tot += in.avg[sb + a];
     for (int32_t a = 0; a < na; ++a) in.sbs[sb + a] = tot > 0.0 ? in.avg[sb + a] / tot : 1.0 / (double)na;
   }
-  __syncthreads();
+  level_sync<CLUSTERED>();
   for (int d = 0; d < in.D; ++d) {
-    const LevelWork w = in.lw[d];
     if (g.int_edge) {  // member order: depth d + 1 pulls
-      if (d + 1 < in.D) {
-        const int32_t qe = in.lw[d + 1].ie;
-        for (int32_t q = in.lw[d + 1].ib + (int32_t)threadIdx.x; q < qe; q += kPull * THREADS)
-          fwd_pull<double, false>(g, in.sbs, in.reach2, q, THREADS, qe);
-      }
+      if (d + 1 >= in.D) break;
+      const int32_t qe = in.lw[d + 1].ie;
+      for (int32_t q = in.lw[d + 1].ib + ct; q < qe; q += kPull * NT)
+        fwd_pull<double, CLUSTERED>(g, in.sbs, in.reach2, q, NT, qe);
     } else {
-      for (int32_t qw = w.ib + (threadIdx.x & ~31); qw < w.ie; qw += 4 * THREADS) {
-        if (w.fan) fwd_int4<double, false, true>(g, in.sbs, in.reach2, qw + (threadIdx.x & 31), THREADS, w.ie);
-        else fwd_int4<double, false, false>(g, in.sbs, in.reach2, qw + (threadIdx.x & 31), THREADS, w.ie);
+      const LevelWork w = in.lw[d];
+      for (int32_t qw = w.ib + rank * THREADS + (threadIdx.x & ~31); qw < w.ie; qw += 4 * NT) {
+        if (w.fan) fwd_int4<double, CLUSTERED, true>(g, in.sbs, in.reach2, qw + (threadIdx.x & 31), NT, w.ie);
+        else fwd_int4<double, CLUSTERED, false>(g, in.sbs, in.reach2, qw + (threadIdx.x & 31), NT, w.ie);
       }
-      for (int32_t i = w.wd0; i < w.wd1; ++i) cta_fwd_wide<double, false>(g, in.reach2, i, threadIdx.x, THREADS);
+      for (int32_t i = w.wd0; i < w.wd1; ++i) cta_fwd_wide<double, CLUSTERED>(g, in.reach2, i, ct, NT);
     }
-    __syncthreads();
+    level_sync<CLUSTERED>();
   }
-  const int lane = threadIdx.x % LANES, gid = threadIdx.x / LANES;
-  constexpr int NG = THREADS / LANES;
+  const int lane = threadIdx.x % LANES, gid = ct / LANES;
+  const int NG = NT / LANES;
   const unsigned mask = group_mask<LANES>();
   for (int d = in.D - 1; d >= 0; --d) {
     const LevelWork w = in.lw[d];
-    for (int32_t i = w.ch0 + threadIdx.x; i < w.ch1; i += THREADS) {
-      const int32_t h = __ldg(g.ch_vs + i);
-      const int32_t cb = __ldg(g.ch_vb + i), ce = cb + __ldg(g.ch_nch + i);
-      double sx = 0.0, sy = 0.0, sa = 0.0;
-      for (int32_t c = cb; c < ce; ++c) { const double2 x = in.vb[c]; sx += x.x; sy += x.y; sa += in.vavg[c]; }
-      in.vb[h] = make_double2(sx, sy);
-      in.vavg[h] = sa;
-    }
-    for (int32_t i = w.wd0; i < w.wd1; ++i) {
+    for (int32_t i = w.ch0 + ct; i < w.ch1; i += NT) br_chance<CLUSTERED>(g, in.vb, in.vavg, i);
+    for (int32_t i = w.wd0; i < w.wd1 && rank == 0; ++i) {
       const int32_t h = __ldg(g.wide_vs + i);
       const int32_t cb = __ldg(g.wide_vb + i), ce = cb + __ldg(g.wide_nch + i);
       double sx = 0.0, sy = 0.0, sa = 0.0;
-      for (int32_t c = cb + threadIdx.x; c < ce; c += THREADS) { const double2 x = in.vb[c]; sx += x.x; sy += x.y; sa += in.vavg[c]; }
+      for (int32_t c = cb + threadIdx.x; c < ce; c += THREADS) {
+        const double2 x = ldm<CLUSTERED>(in.vb + c);
+        sx += x.x; sy += x.y; sa += ldm<CLUSTERED>(in.vavg + c);
+      }
       sx = cta_sum<THREADS>(sx, sm);
       sy = cta_sum<THREADS>(sy, sm);
       sa = cta_sum<THREADS>(sa, sm);
       if (threadIdx.x == 0) { in.vb[h] = make_double2(sx, sy); in.vavg[h] = sa; }
     }
-    for (int32_t I = w.is0 + gid; I < w.is1; I += NG) {
-      const int p = I >= w.is2 ? 1 : 0;
-      const int32_t sb = __ldg(g.iset_slot + I), na = __ldg(g.iset_slot + I + 1) - sb;
-      const int32_t m0 = __ldg(g.iset_mem + I), m1 = __ldg(g.iset_mem + I + 1);
-      const MemberRanks mr = member_ranks(g, I, m0);
-      const int32_t vb0 = __ldg(g.iset_vb + I);
-      double sg[MAXA], Q[MAXA];
-#pragma unroll
-      for (int a = 0; a < MAXA; ++a) { sg[a] = a < na ? in.sbs[sb + a] : 0.0; Q[a] = 0.0; }
-      for (int32_t k0 = m0; k0 < m1; k0 += LANES) {
-        const int32_t k = k0 + lane;
-        double q[MAXA];
-#pragma unroll
-        for (int a = 0; a < MAXA; ++a) q[a] = 0.0;
-        if (k < m1) {
-          const int32_t h = __ldg(g.mem_vs + k);
-          const int32_t cb = vb0 + (k - m0), M = m1 - m0;
-          const double2 r = in.reach2[member_rank(g, k, mr)];
-          const double po = p ? r.x : r.y;
-          double oth = 0.0, va = 0.0;
-#pragma unroll
-          for (int a = 0; a < MAXA; ++a) {
-            if (a < na) {
-              const double2 x = in.vb[cb + a * M];
-              q[a] = po * (p ? x.y : x.x);
-              oth += sg[a] * (p ? x.x : x.y);
-              va += sg[a] * in.vavg[cb + a * M];
-            }
-          }
-          reinterpret_cast<double *>(in.vb + h)[1 - p] = oth;
-          in.vavg[h] = va;
-        }
-        const int cnt = (m1 - k0) < LANES ? (m1 - k0) : LANES;
-        for (int j = 0; j < cnt; ++j) {
-#pragma unroll
-          for (int a = 0; a < MAXA; ++a)
-            if (a < na) Q[a] += __shfl_sync(mask, q[a], j, LANES);
-        }
-      }
-      int best = 0;
-      for (int a = 1; a < na; ++a)
-        if (p == 0 ? Q[a] > Q[best] : Q[a] < Q[best]) best = a;
-      for (int32_t k = m0 + lane; k < m1; k += LANES) {
-        const int32_t h = __ldg(g.mem_vs + k);
-        const int32_t cb = vb0 + (k - m0) + best * (m1 - m0);
-        reinterpret_cast<double *>(in.vb + h)[p] = reinterpret_cast<const double *>(in.vb + cb)[p];
-      }
-    }
-    __syncthreads();
+    for (int32_t I = w.is0 + gid; I < w.is1; I += NG)
+      br_set<MAXA, LANES, CLUSTERED>(g, in.reach2, in.sbs, in.vb, in.vavg, I, I >= w.is2 ? 1 : 0, lane, mask);
+    level_sync<CLUSTERED>();
   }
-  if (threadIdx.x == 0) {
-    const double2 root = in.vb[in.root_vs];
-    in.out[0] = 0.5 * (root.x - root.y);
-    in.out[1] = root.x;
-    in.out[2] = root.y;
-    in.out[3] = in.vavg[in.root_vs];
+  if (ct == 0) {
+    const double2 root = ldm<CLUSTERED>(in.vb + in.root_vs);
+    in.res[0] = 0.5 * (root.x - root.y);
+    in.res[1] = root.x;
+    in.res[2] = root.y;
+    in.res[3] = ldm<CLUSTERED>(in.vavg + in.root_vs);
   }
+  chain_leave();
 }
 
 }  // namespace cfr

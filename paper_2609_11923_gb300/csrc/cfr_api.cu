@@ -1499,88 +1499,137 @@ extern "C" int cfr_autotune(cfr_handle *h, int reps, void *stream) {
 }
 
 // ----------------------------------------------------------- batched solves
-static int batch_table(cfr_handle *const *hs, int n, const int64_t *iters, int64_t n_iter, void *table_dev,
-                       size_t table_bytes, int *maxa, int *precision, std::vector<InstDesc> &tab) {
+static InstDesc inst_desc(const cfr_handle *h, int64_t n_iter) {
+  InstDesc d;
+  memset(&d, 0, sizeof d);
+  d.g = game_view(h);
+  d.reach = h->arena + h->b_reach.off;
+  d.v = h->arena + h->b_v.off;
+  d.sigma = h->arena + h->b_sigma.off;
+  d.R = h->p<double>(h->b_R);
+  d.avg = h->p<double>(h->b_avg);
+  d.t = h->p<long long>(h->b_t);
+  d.lw = h->p<LevelWork>(h->b_levels);
+  d.reach2 = h->p<double2>(h->b_reach2);
+  d.vb = h->p<double2>(h->b_vb);
+  d.vavg = h->p<double>(h->b_vavg);
+  d.sbs = h->p<double>(h->b_sbs);
+  d.out = h->p<double>(h->b_out);
+  d.n_iter = n_iter;
+  d.D = (int32_t)h->c.D;
+  d.rule = h->rule;
+  d.n_sets = (int32_t)h->c.I;
+  d.root_vs = (int32_t)(h->c.N - 1);
+  d.order = h->order;
+  return d;
+}
+
+// A batched call's plan: the instances' descriptors ordered by cluster size
+// (largest first, and by load within a size), and one launch for each size.
+struct BatchPlan {
+  std::vector<InstDesc> tab;
+  struct Launch {
+    int first, count, cluster;
+  };
+  std::vector<Launch> launches;
+  int maxa = 4, precision = -1;
+};
+
+static int batch_plan(cfr_handle *const *hs, int n, const int64_t *iters, int64_t n_iter, void *table_dev,
+                      size_t table_bytes, int cluster, BatchPlan &bp) {
   if (!hs || n <= 0) return set_err(CFR_ERR_ARG, "batch: no instances");
-  if (!table_dev || table_bytes < sizeof(InstDesc) * (size_t)n)
-    return set_err(CFR_ERR_ARG, "batch: the descriptor table needs %zu bytes", sizeof(InstDesc) * (size_t)n);
+  if (!table_dev || table_bytes < cfr_batch_table_bytes(n))
+    return set_err(CFR_ERR_ARG, "batch: the descriptor table needs %zu bytes", cfr_batch_table_bytes(n));
   if (reinterpret_cast<uintptr_t>(table_dev) % 16 != 0) return set_err(CFR_ERR_ARG, "batch: table must be 16-byte aligned");
-  tab.resize(n);
-  *maxa = 4;
-  *precision = -1;
+  int64_t longest = 1;
   for (int i = 0; i < n; ++i) {
     cfr_handle *h = hs[i];
     if (!h) return set_err(CFR_ERR_ARG, "batch: null handle %d", i);
     if (!h->bound) return set_err(CFR_ERR_NOT_BOUND, "batch: instance %d is not bound", i);
-    if (*precision < 0) *precision = h->precision;
-    else if (*precision != h->precision) return set_err(CFR_ERR_ARG, "batch: instances mix precisions");
+    if (bp.precision < 0) bp.precision = h->precision;
+    else if (bp.precision != h->precision) return set_err(CFR_ERR_ARG, "batch: instances mix precisions");
     if (h->maxa_tier > 8) return set_err(CFR_ERR_UNSUPPORTED, "batch: instance %d has sets of more than 8 actions", i);
-    *maxa = std::max(*maxa, h->maxa_tier);
-    InstDesc &d = tab[i];
-    memset(&d, 0, sizeof d);
-    d.g = game_view(h);
-    d.reach = h->arena + h->b_reach.off;
-    d.v = h->arena + h->b_v.off;
-    d.sigma = h->arena + h->b_sigma.off;
-    d.R = h->p<double>(h->b_R);
-    d.avg = h->p<double>(h->b_avg);
-    d.t = h->p<long long>(h->b_t);
-    d.lw = h->p<LevelWork>(h->b_levels);
-    d.reach2 = h->p<double2>(h->b_reach2);
-    d.vb = h->p<double2>(h->b_vb);
-    d.vavg = h->p<double>(h->b_vavg);
-    d.sbs = h->p<double>(h->b_sbs);
-    d.out = h->p<double>(h->b_out);
-    d.n_iter = iters ? iters[i] : n_iter;
-    if (d.n_iter < 0) return set_err(CFR_ERR_ARG, "batch: negative iteration count");
-    d.D = (int32_t)h->c.D;
-    d.rule = h->rule;
-    d.n_sets = (int32_t)h->c.I;
-    d.root_vs = (int32_t)(h->c.N - 1);
-    d.order = h->order;
+    bp.maxa = std::max(bp.maxa, h->maxa_tier);
+    const int64_t it = iters ? iters[i] : n_iter;
+    if (it < 0) return set_err(CFR_ERR_ARG, "batch: negative iteration count");
+    longest = std::max(longest, it);
+  }
+  std::vector<int64_t> load(n);
+  for (int i = 0; i < n; ++i) {
+    const double share = iters ? (double)iters[i] / (double)longest : 1.0;
+    load[i] = (int64_t)((double)hs[i]->c.N * share);
+  }
+  const std::vector<int> cta = plan_clusters(load, cluster, device_sms());
+  std::vector<int> at(n);
+  for (int i = 0; i < n; ++i) at[i] = i;
+  std::stable_sort(at.begin(), at.end(), [&](int a, int b) {
+    return cta[a] != cta[b] ? cta[a] > cta[b] : load[a] > load[b];
+  });
+  double *res = reinterpret_cast<double *>((char *)table_dev + sizeof(InstDesc) * (size_t)n);
+  bp.tab.resize(n);
+  for (int k = 0; k < n; ++k) {
+    const int i = at[k];
+    bp.tab[k] = inst_desc(hs[i], iters ? iters[i] : n_iter);
+    bp.tab[k].res = res + 4 * (size_t)i;
+    if (k == 0 || cta[i] != cta[at[k - 1]]) bp.launches.push_back({k, 0, cta[i]});
+    ++bp.launches.back().count;
   }
   return CFR_OK;
 }
 
-extern "C" size_t cfr_batch_table_bytes(int n) { return n > 0 ? sizeof(InstDesc) * (size_t)n : 0; }
+static_assert(sizeof(InstDesc) % 16 == 0, "descriptors and the results behind them are 16-byte aligned");
+
+// n descriptors, then four results of each instance.
+extern "C" size_t cfr_batch_table_bytes(int n) { return n > 0 ? (sizeof(InstDesc) + 4 * sizeof(double)) * (size_t)n : 0; }
+
+static int batch_shape(int *threads, int *lanes) {
+  if (*threads == 0) *threads = 256;
+  if (*lanes == 0) *lanes = 4;
+  if ((*threads != 256 && *threads != 1024) || (*lanes != 2 && *lanes != 4 && *lanes != 8 && *lanes != 32))
+    return set_err(CFR_ERR_ARG, "batch: threads must be 256 or 1024 and lanes 2, 4, 8 or 32");
+  return CFR_OK;
+}
 
 extern "C" int cfr_batch_iterate(cfr_handle *const *hs, int n, const int64_t *iters, int64_t n_iter, void *table_dev,
                                  size_t table_bytes, int threads, int lanes, int cluster, void *stream) {
-  std::vector<InstDesc> tab;
-  int maxa = 4, prec = 0;
-  int rc = batch_table(hs, n, iters, n_iter, table_dev, table_bytes, &maxa, &prec, tab);
-  if (rc) return rc;
-  if (threads == 0) threads = 256;
-  if (lanes == 0) lanes = 4;
-  if ((threads != 256 && threads != 1024) || (lanes != 2 && lanes != 4 && lanes != 8 && lanes != 32))
-    return set_err(CFR_ERR_ARG, "batch: threads must be 256 or 1024 and lanes 2, 4, 8 or 32");
   if (cluster == 0) cluster = 1;
   if (cluster != 1 && cluster != 2 && cluster != 4 && cluster != 8)
     return set_err(CFR_ERR_ARG, "batch: cluster must be 1, 2, 4 or 8 CTAs per instance");
-  if (n == 0) return CFR_OK;
+  int rc = batch_shape(&threads, &lanes);
+  if (rc) return rc;
+  BatchPlan bp;
+  if ((rc = batch_plan(hs, n, iters, n_iter, table_dev, table_bytes, cluster, bp))) return rc;
   cudaStream_t s = (cudaStream_t)stream;
-  CK(cudaMemcpyAsync(table_dev, tab.data(), sizeof(InstDesc) * (size_t)n, cudaMemcpyHostToDevice, s));
-  if (prec == CFR_P64) CK(launch_batch_iterate<double>(maxa, lanes, threads, cluster, n, s, (const InstDesc *)table_dev));
-  else CK(launch_batch_iterate<float>(maxa, lanes, threads, cluster, n, s, (const InstDesc *)table_dev));
-  for (int i = 0; i < n; ++i) hs[i]->iteration_host += tab[i].n_iter;
+  const InstDesc *tab = (const InstDesc *)table_dev;
+  CK(cudaMemcpyAsync(table_dev, bp.tab.data(), sizeof(InstDesc) * (size_t)n, cudaMemcpyHostToDevice, s));
+  bool chained = false;
+  for (const BatchPlan::Launch &l : bp.launches) {
+    if (bp.precision == CFR_P64)
+      CK(launch_batch_iterate<double>(bp.maxa, lanes, threads, l.cluster, chained, l.count, s, tab + l.first, bp.tab[0]));
+    else
+      CK(launch_batch_iterate<float>(bp.maxa, lanes, threads, l.cluster, chained, l.count, s, tab + l.first, bp.tab[0]));
+    chained = true;
+  }
+  for (int i = 0; i < n; ++i) hs[i]->iteration_host += iters ? iters[i] : n_iter;
   return CFR_OK;
 }
 
 extern "C" int cfr_batch_exploitability(cfr_handle *const *hs, int n, double *out, void *table_dev, size_t table_bytes,
                                         int threads, int lanes, void *stream) {
   if (!out) return set_err(CFR_ERR_ARG, "batch: null output");
-  std::vector<InstDesc> tab;
-  int maxa = 4, prec = 0;
-  int rc = batch_table(hs, n, nullptr, 0, table_dev, table_bytes, &maxa, &prec, tab);
+  int rc = batch_shape(&threads, &lanes);
   if (rc) return rc;
-  if (threads == 0) threads = 256;
-  if (lanes == 0) lanes = 4;
-  if ((threads != 256 && threads != 1024) || (lanes != 2 && lanes != 4 && lanes != 8 && lanes != 32))
-    return set_err(CFR_ERR_ARG, "batch: threads must be 256 or 1024 and lanes 2, 4, 8 or 32");
+  BatchPlan bp;
+  if ((rc = batch_plan(hs, n, nullptr, 0, table_dev, table_bytes, 1, bp))) return rc;
   cudaStream_t s = (cudaStream_t)stream;
-  CK(cudaMemcpyAsync(table_dev, tab.data(), sizeof(InstDesc) * (size_t)n, cudaMemcpyHostToDevice, s));
-  CK(launch_batch_br(maxa, lanes, threads, n, s, (const InstDesc *)table_dev));
-  for (int i = 0; i < n; ++i) CK(cudaMemcpyAsync(out + 4 * i, tab[i].out, 4 * sizeof(double), cudaMemcpyDeviceToHost, s));
+  const InstDesc *tab = (const InstDesc *)table_dev;
+  CK(cudaMemcpyAsync(table_dev, bp.tab.data(), sizeof(InstDesc) * (size_t)n, cudaMemcpyHostToDevice, s));
+  bool chained = false;
+  for (const BatchPlan::Launch &l : bp.launches) {
+    CK(launch_batch_br(bp.maxa, lanes, threads, l.cluster, chained, l.count, s, tab + l.first, bp.tab[0]));
+    chained = true;
+  }
+  CK(cudaMemcpyAsync(out, tab + n, 4 * sizeof(double) * (size_t)n, cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
   return CFR_OK;
 }

@@ -1,12 +1,17 @@
 // Batched best-response kernel instances (see batch.cuh).
 #include "k_batch.cuh"
 namespace cfr {
-cudaError_t launch_batch_br(int maxa, int lanes, int threads, int n, cudaStream_t s, const InstDesc *table) {
-#define BR_CASE(MA, L, TH)                                                   \
-  if (maxa == MA && lanes == L && threads == TH) {                           \
-    batch_br_kernel<MA, L, TH><<<n, TH, 0, s>>>(table, n);                   \
-    return cudaGetLastError();                                               \
-  }
+template <int MA, int L, int TH>
+static cudaError_t br_one(int cluster, bool chained, int n, cudaStream_t s, const InstDesc *table, const InstDesc &one) {
+  constexpr int NT = kBatchThreads<double, MA, TH>;
+  if (cluster == 1) return launch_batch_any(batch_br_kernel<MA, L, NT, false>, NT, 1, chained, n, s, table, one);
+  return launch_batch_any(batch_br_kernel<MA, L, NT, true>, NT, cluster, chained, n, s, table, one);
+}
+
+cudaError_t launch_batch_br(int maxa, int lanes, int threads, int cluster, bool chained, int n, cudaStream_t s,
+                            const InstDesc *table, const InstDesc &one) {
+#define BR_CASE(MA, L, TH) \
+  if (maxa == MA && lanes == L && threads == TH) return br_one<MA, L, TH>(cluster, chained, n, s, table, one);
   CFR_BATCH_ALL(BR_CASE)
 #undef BR_CASE
   return cudaErrorInvalidValue;

@@ -682,10 +682,13 @@ __device__ __forceinline__ void accumulate_chunk(int32_t cnt, int32_t na, unsign
 // in chunks of LANES (two chunks per step for narrow groups); each step loads
 // the next step's member indices while its own reach and child values are in
 // flight, so a step waits for one memory round trip, not two. The update of
-// the set's slots runs one lane per action. LEAN: see member_data.
-template <typename T, int MAXA, int LANES, bool PERSIST, bool LEAN = false>
+// the set's slots runs one lane per action. LEAN: see member_data. DEFER: the
+// set's totals go to def_r (and def_m: FP32 the set's sum of own reach at its
+// first slot, FP64 every slot's average term) for update_set to take up later.
+template <typename T, int MAXA, int LANES, bool PERSIST, bool LEAN = false, bool DEFER = false>
 __device__ __forceinline__ void bwd_set(const GameView &g, const StateView<T> &st, int32_t I, bool p2,
-                                        int lane, unsigned mask, double wt, int rule, int upd, double *rows) {
+                                        int lane, unsigned mask, double wt, int rule, int upd, double *rows,
+                                        T *def_r = nullptr, T *def_m = nullptr) {
   const int32_t sb = __ldg(g.iset_slot + I);
   const int32_t na = __ldg(g.iset_slot + I + 1) - sb;
   const int32_t m0 = __ldg(g.iset_mem + I), m1 = __ldg(g.iset_mem + I + 1);
@@ -779,6 +782,31 @@ __device__ __forceinline__ void bwd_set(const GameView &g, const StateView<T> &s
   }
   // alternating updates: the other player's sets only pass their values up
   if (!(upd & (p2 ? 2 : 1))) return;
+  if constexpr (DEFER) {
+    if constexpr (CHAINS) {
+#pragma unroll
+      for (int i = 0; i < kChainAcc<MAXA, LANES>; ++i) {
+        const int c = lane + i * LANES;
+        if (c < na) def_r[sb + c] = acc[i];
+        else if (c >= MAXA && c - MAXA < na) def_m[sb + c - MAXA] = acc[i];
+      }
+    } else {
+      static_assert(sizeof(T) == 4 && LEAN && MAXA <= 8, "deferred updates: FP64 needs chains, FP32 lean average terms");
+      macc[0] = group_sum_butterfly<LANES>(macc[0], mask);
+      if (lane == 0) def_m[sb] = macc[0];
+      group_sum_scatter<LANES, MAXA>(racc, lane, mask);
+      if constexpr (MAXA <= LANES) {
+        constexpr int STEP = LANES / MAXA;
+        if (lane % STEP == 0 && lane / STEP < na) def_r[sb + lane / STEP] = racc[0];
+      } else {
+        constexpr int PER = MAXA / LANES;
+#pragma unroll
+        for (int i = 0; i < PER; ++i)
+          if (lane * PER + i < na) def_r[sb + lane * PER + i] = racc[i];
+      }
+    }
+    return;
+  }
   if constexpr (sizeof(T) == 4) {
 #pragma unroll
     for (int a = 0; a < MAXA; ++a) {
@@ -842,6 +870,52 @@ __device__ __forceinline__ void bwd_set(const GameView &g, const StateView<T> &s
     for (int a = 0; a < MAXA; ++a)
       if (a < na) st.sigma[sb + a] = tot > T(0) ? pos[a] / tot : T(1) / (T)na;
   }
+}
+
+// The slot updates of set I from its deferred totals, by one thread: a warp's
+// FP64 instructions then serve 32 sets at once instead of the few lanes of a
+// group. Every slot's loads are issued before the first is used.
+template <typename T, int MAXA, bool PERSIST>
+__device__ __forceinline__ void update_set(const GameView &g, const StateView<T> &st, int32_t I, double wt, int rule,
+                                           const T *def_r, const T *def_m) {
+  const int32_t sb = __ldg(g.iset_slot + I);
+  const int32_t na = __ldg(g.iset_slot + I + 1) - sb;
+  constexpr int W = 4;  // slots in flight
+  T pos[MAXA];
+  T tot = T(0), spw = T(0);
+  if constexpr (sizeof(T) == 4) spw = ldm<PERSIST>(def_m + sb);
+#pragma unroll
+  for (int a0 = 0; a0 < MAXA; a0 += W) {
+    double R[W], S[W];
+    T r[W], m[W];
+#pragma unroll
+    for (int j = 0; j < W; ++j) {
+      if (a0 + j < na) {
+        const int32_t q = sb + a0 + j;
+        R[j] = st.R[q];
+        S[j] = st.avg[q];
+        r[j] = ldm<PERSIST>(def_r + q);
+        if constexpr (sizeof(T) == 4) m[j] = st.sigma[q] * spw;  // written by this thread the iteration before
+        else m[j] = ldm<PERSIST>(def_m + q);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < W; ++j) {
+      if (a0 + j < na) {
+        const int32_t q = sb + a0 + j;
+        double Rn, Sn;
+        const double x = slot_terms(R[j], S[j], as_double(r[j]), as_double(m[j]), wt, rule, Rn, Sn);
+        st.R[q] = Rn;
+        st.avg[q] = Sn;
+        if constexpr (sizeof(T) == 8) pos[a0 + j] = x;
+        else pos[a0 + j] = narrow_pos(x);
+        tot += pos[a0 + j];
+      }
+    }
+  }
+#pragma unroll
+  for (int a = 0; a < MAXA; ++a)
+    if (a < na) st.sigma[sb + a] = tot > T(0) ? pos[a] / tot : T(1) / (T)na;
 }
 
 // One information set per block, for depths with few sets of hundreds of

@@ -246,3 +246,86 @@ def test_server_answers_an_invalid_spec_with_an_error_result():
     srv.close()
     assert res[0].status == "error" and "CFR_ERR_INVALID_SPEC" in res[0].message
     assert res[1].status in ("solved", "capped")
+
+
+def chain_game(depth):
+    """`depth` decision nodes in a row (players in turn), each with a way out:
+    more depths than a CTA keeps work descriptors for."""
+    rng = np.random.default_rng(depth)
+    nodes = []
+    for d in range(depth):
+        nxt = 2 * (d + 1)
+        nodes.append((gg.P1 if d % 2 == 0 else gg.P2, d, [2 * d + 1, nxt], None, 0.0))
+        nodes.append((gg.TERMINAL, -1, [], None, float(rng.uniform(-1, 1))))
+    nodes.append((gg.TERMINAL, -1, [], None, float(rng.uniform(-1, 1))))
+    return gg.from_lists(nodes, [(d % 2, 2) for d in range(depth)])
+
+
+@pytest.mark.parametrize("order", [cfr.ORDER_SIMULTANEOUS, cfr.ORDER_ALTERNATING])
+@pytest.mark.parametrize("depth", [1, 31, 32, 33, 60])
+def test_batched_deep_games_match_oracle(depth, order):
+    g = chain_game(depth)
+    opts = cfr.make_options(precision=cfr.P64, order=order)
+    h = cfr.cfr_compile(g, opts)
+    n = cfr.cfr_plan(h)
+    pool = serve.DevicePool(n + 4096)
+    s = int(torch.cuda.current_stream().cuda_stream)
+    cfr.cfr_bind(h, pool.ptr(pool.alloc(n)), n, s)
+    tb = cfr.cfr_batch_table_bytes(1)
+    table = torch.empty(tb + 16, dtype=torch.uint8, device="cuda")
+    for cluster in (1, 2):
+        cfr.cfr_reset(h, s)
+        cfr.cfr_batch_iterate([h], 50, (table.data_ptr() + 15) & ~15, tb, 256, 4, s, cluster=cluster)
+        out = np.empty(cfr.cfr_get_counts(h)["n_slots"])
+        cfr.cfr_avg_strategy(h, out, False, s)
+        np.testing.assert_array_equal(out, oracle.solve(g, 50, order=order).avg_strategy())
+    cfr.cfr_destroy(h)
+
+
+@pytest.mark.parametrize("precision,threads,lanes", [(cfr.P32, 1024, 8), (cfr.P32, 256, 32), (cfr.P32, 256, 2),
+                                                     (cfr.P64, 1024, 8), (cfr.P64, 256, 2)])
+def test_results_do_not_depend_on_how_ctas_are_shared_out(precision, threads, lanes):
+    # alone, the large games get 16 CTAs; in the mix of 170 instances fewer,
+    # and the small ones one: the results are the same bits
+    big = [gg.endgame(21, 300000), gg.endgame(22, 60000), gg.random_tree(5, depth=11)]
+    specs = big + [gg.endgame(900 + i, 1500) for i in range(4)]
+    copies = specs + [specs[3 + i % 4] for i in range(163)]
+    pool, hs, table, tp, tb, s = bound(copies, precision)
+    cfr.cfr_batch_iterate(hs, 12, tp, tb, threads, lanes, s)
+    ex = cfr.cfr_batch_exploitability(hs, tp, tb, threads, lanes, s)
+    for i in (0, 1, 2, 3, 6, 169):
+        p2, h2, t2, tp2, tb2, _ = bound([copies[i]], precision)
+        cfr.cfr_batch_iterate(h2, 12, tp2, tb2, threads, lanes, s)
+        e2 = cfr.cfr_batch_exploitability(h2, tp2, tb2, threads, lanes, s)
+        n = cfr.cfr_get_counts(h2[0])["n_slots"]
+        a, b = cfr.cfr_get_state(hs[i], n, s), cfr.cfr_get_state(h2[0], n, s)
+        np.testing.assert_array_equal(a[0], b[0])
+        np.testing.assert_array_equal(a[1], b[1])
+        np.testing.assert_array_equal(ex[i], e2[0])
+        cfr.cfr_destroy(h2[0])
+    for h in hs:
+        cfr.cfr_destroy(h)
+
+
+@pytest.mark.parametrize("a,b", [(1, 2), (4, 4), (5, 8), (8, 3)])
+def test_best_response_at_group_edges_matches_oracle(a, b):
+    from tests.test_gpu_set_edges import two_level_game
+
+    specs = [two_level_game(m, a, b, seed=1) for m in (1, 2, 3, 4, 5, 7, 8, 9, 31, 32, 33, 65)]
+    pool, hs, table, tp, tb, s = bound(specs)
+    for lanes in (2, 4, 8, 32):
+        for threads in (256, 1024):
+            for h in hs:
+                cfr.cfr_reset(h, s)
+            cfr.cfr_batch_iterate(hs, 7, tp, tb, threads, lanes, s)
+            ex = cfr.cfr_batch_exploitability(hs, tp, tb, threads, lanes, s)
+            for sp, row, h in zip(specs, ex, hs):
+                sig = np.empty(cfr.cfr_get_counts(h)["n_slots"])
+                cfr.cfr_avg_strategy(h, sig, False, s)
+                o = oracle.Oracle(sp)
+                want = o.best_response(sig)
+                # payoffs in [-1, 1]: sums of at most 65 x 64 terms of 1/M each in another order
+                np.testing.assert_allclose(row[1:3], want[:2], rtol=0, atol=1e-14)
+                np.testing.assert_allclose(cfr.cfr_exploitability(h, s)[1:3], want[:2], rtol=0, atol=1e-14)
+    for h in hs:
+        cfr.cfr_destroy(h)
