@@ -10,6 +10,7 @@
  */
 #ifndef CFR_MLP_H
 #define CFR_MLP_H
+#include <stddef.h>
 #include <stdint.h>
 
 #ifdef __cplusplus
@@ -46,6 +47,37 @@ int mlp_adam(float *w, const float *g, float *m, float *v, long n, float lr, flo
 int mlp_to_bf16(const float *x, void *y, long n, void *stream);
 
 const char *mlp_last_error(void);
+
+/* A network of three hidden ReLU layers of 256 and 8 logits, in_dim inputs (a
+ * multiple of 4, at most 256), as a few kernels: weights W_l [fan_in x
+ * fan_out] and biases b_l in FP32 (l = 0..3), the same numerics as the calls
+ * above layer by layer. `img` holds the weights packed as tensor-core
+ * operands: mlp_net_image_bytes(in_dim) bytes (0: the shape is not taken),
+ * zeroed once by the caller, written by mlp_net_adam. Returns as above, with
+ * mlp_net_last_error(). */
+size_t mlp_net_image_bytes(int in_dim);
+/* Bytes of the workspace of mlp_net_grad for a batch of `rows`. */
+size_t mlp_net_work_bytes(int in_dim, int rows);
+
+/* prob [rows x 8] = the masked softmax of the logits of X [rows x in_dim].
+ * err (device int) is set to 1 if a wait inside the kernel gave up. */
+int mlp_net_predict(const float *X, int in_dim, int rows, const void *img, const float *const *b, const int32_t *nact,
+                    float *prob, int *err, void *stream);
+
+/* Loss and every gradient of a batch (mlp_softmax_xent's loss and weights).
+ * *loss (set on return) is a device address in `work`: the summed loss of the
+ * rows, then an int that is 1 if a wait inside a kernel gave up. */
+int mlp_net_grad(const float *X, int in_dim, int rows, const void *img, const float *const *b, const int32_t *nact,
+                 const float *target, const float *weight, float *const *gW, float *const *gb, void *work,
+                 size_t work_bytes, float **loss, void *stream);
+
+/* One Adam step on all of a network's tensors (w, g, m, v: W_0, b_0, W_1,
+ * ...), which also writes the BF16 copies wb[l] of the weights and, when img
+ * is non-NULL, their images. step = 0 writes only the copies and images. */
+int mlp_net_adam(float *const *w, const float *const *g, float *const *m, float *const *v, void *const *wb, void *img,
+                 int in_dim, float lr, float b1, float b2, float eps, long step, void *stream);
+
+const char *mlp_net_last_error(void);
 
 #ifdef __cplusplus
 }

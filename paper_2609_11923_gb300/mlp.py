@@ -25,6 +25,17 @@ _lib.mlp_colsum.argtypes = [_vp, _i, _i, _vp, _vp]
 _lib.mlp_adam.argtypes = [_vp, _vp, _vp, _vp, _l, ctypes.c_float, ctypes.c_float, ctypes.c_float, ctypes.c_float, _l,
                           _vp, _vp]
 _lib.mlp_to_bf16.argtypes = [_vp, _vp, _l, _vp]
+_pp, _f32 = ctypes.POINTER(_vp), ctypes.c_float
+_lib.mlp_net_predict.argtypes = [_vp, _i, _i, _vp, _pp, _vp, _vp, _vp, _vp]
+_lib.mlp_net_grad.argtypes = [_vp, _i, _i, _vp, _pp, _vp, _vp, _vp, _pp, _pp, _vp, ctypes.c_size_t,
+                              ctypes.POINTER(_vp), _vp]
+_lib.mlp_net_adam.argtypes = [_pp, _pp, _pp, _pp, _pp, _vp, _i, _f32, _f32, _f32, _f32, _l, _vp]
+for _f in ("mlp_net_predict", "mlp_net_grad", "mlp_net_adam"):
+    getattr(_lib, _f).restype = ctypes.c_int
+_lib.mlp_net_image_bytes.argtypes = [_i]
+_lib.mlp_net_work_bytes.argtypes = [_i, _i]
+_lib.mlp_net_image_bytes.restype = _lib.mlp_net_work_bytes.restype = ctypes.c_size_t
+_lib.mlp_net_last_error.restype = ctypes.c_char_p
 for _f in ("mlp_gemm", "mlp_softmax_xent", "mlp_relu_grad", "mlp_colsum", "mlp_adam", "mlp_to_bf16"):
     getattr(_lib, _f).restype = ctypes.c_int
 _lib.mlp_last_error.restype = ctypes.c_char_p
@@ -37,8 +48,17 @@ def _ck(rc):
         raise RuntimeError("mlp: " + (_lib.mlp_last_error() or b"").decode())
 
 
+def _net_ck(rc):
+    if rc != 0:
+        raise RuntimeError("mlp: " + (_lib.mlp_net_last_error() or b"").decode())
+
+
 def _p(t) -> int:
     return 0 if t is None else int(t.data_ptr())
+
+
+def _ptrs(ts):
+    return (_vp * len(ts))(*[t.data_ptr() for t in ts])
 
 
 class MLP:
@@ -63,14 +83,49 @@ class MLP:
         self.mb = [torch.zeros_like(b) for b in self.b]
         self.vb = [torch.zeros_like(b) for b in self.b]
         self.step_no = 0
+        self._acts, self._X = None, None
+        # networks of the warm start's shape run through the fused kernels
+        # (mlp_net_*), from packed images of the weights; any other shape
+        # runs layer by layer through mlp_gemm
+        self.fused = (self.dims[1:] == [256, 256, 256, N_OUT] and self.dev.type == "cuda"
+                      and _lib.mlp_net_image_bytes(in_dim) > 0)
+        self.img = self.work = None
+        if self.fused:
+            self.img = torch.zeros(_lib.mlp_net_image_bytes(in_dim), dtype=torch.uint8, device=self.dev)
+            self._err = torch.zeros(1, dtype=torch.int32, device=self.dev)
         self.sync_bf16()
 
     def _s(self) -> int:
         return int(self.torch.cuda.current_stream(self.dev).cuda_stream)
 
+    @property
+    def acts(self):
+        """The input, every hidden layer's output and the logits of the last
+        forward pass in FP32. The fused passes keep none: after one of them
+        they are computed here."""
+        if self._acts is None and self._X is not None:
+            self.forward(self._X)
+        return self._acts
+
+    @acts.setter
+    def acts(self, value):
+        self._acts = value
+
     def sync_bf16(self):
+        if self.fused:
+            _net_ck(_lib.mlp_net_adam(self._all(self.W, self.b), None, None, None, _ptrs(self.Wb), _p(self.img),
+                                      self.dims[0], 0.0, 0.0, 0.0, 0.0, 0, self._s()))
+            return
         for w, wb in zip(self.W, self.Wb):
             _ck(_lib.mlp_to_bf16(_p(w), _p(wb), w.numel(), self._s()))
+
+    @staticmethod
+    def _all(weights, biases):
+        return _ptrs([t for pair in zip(weights, biases) for t in pair])
+
+    def _rows_ok(self, X) -> bool:
+        return (self.fused and X.dtype == self.torch.float32 and X.dim() == 2 and X.shape[0] > 0
+                and X.shape[1] == self.dims[0])
 
     # ---------------------------------------------------------------- passes
     def forward(self, X) -> "torch.Tensor":
@@ -112,8 +167,22 @@ class MLP:
 
     def loss_and_grad(self, X, nact, target, weight=None) -> float:
         torch = self.torch
-        logits = self.forward(X)
         B = X.shape[0]
+        if self._rows_ok(X):
+            need = _lib.mlp_net_work_bytes(self.dims[0], B)
+            if self.work is None or self.work.numel() < need:
+                self.work = torch.empty(need, dtype=torch.uint8, device=self.dev)
+            loss = _vp()
+            _net_ck(_lib.mlp_net_grad(_p(X), self.dims[0], B, _p(self.img), _ptrs(self.b), _p(nact), _p(target),
+                                      _p(weight), _ptrs(self.gW), _ptrs(self.gb), _p(self.work), self.work.numel(),
+                                      ctypes.byref(loss), self._s()))
+            self._acts, self._X = None, X
+            at = loss.value - self.work.data_ptr()
+            got = self.work[at:at + 8].cpu()
+            if int(got.view(torch.int32)[1]) != 0:
+                raise RuntimeError("mlp: a bounded wait of the training kernels gave up")
+            return float(got.view(torch.float32)[0]) / B
+        logits = self.forward(X)
         dlog = torch.empty_like(logits)
         rows = torch.empty(B, dtype=torch.float32, device=self.dev)
         _ck(_lib.mlp_softmax_xent(_p(logits), N_OUT, _p(nact), _p(target), _p(weight), B, None, _p(dlog), _p(rows),
@@ -123,6 +192,11 @@ class MLP:
 
     def adam_step(self, lr=1e-3, b1=0.9, b2=0.999, eps=1e-8) -> None:
         self.step_no += 1
+        if self.fused:
+            _net_ck(_lib.mlp_net_adam(self._all(self.W, self.b), self._all(self.gW, self.gb),
+                                      self._all(self.mW, self.mb), self._all(self.vW, self.vb), _ptrs(self.Wb),
+                                      _p(self.img), self.dims[0], lr, b1, b2, eps, self.step_no, self._s()))
+            return
         for w, g, m, v, wb in zip(self.W, self.gW, self.mW, self.vW, self.Wb):
             _ck(_lib.mlp_adam(_p(w), _p(g), _p(m), _p(v), w.numel(), lr, b1, b2, eps, self.step_no, _p(wb), self._s()))
         for b, g, m, v in zip(self.b, self.gb, self.mb, self.vb):
@@ -130,6 +204,12 @@ class MLP:
 
     def predict(self, X, nact) -> "torch.Tensor":
         torch = self.torch
+        if self._rows_ok(X):
+            prob = torch.empty((X.shape[0], N_OUT), dtype=torch.float32, device=self.dev)
+            _net_ck(_lib.mlp_net_predict(_p(X), self.dims[0], X.shape[0], _p(self.img), _ptrs(self.b), _p(nact),
+                                         _p(prob), _p(self._err), self._s()))
+            self._acts, self._X = None, X
+            return prob
         logits = self.forward(X)
         prob = torch.empty_like(logits)
         _ck(_lib.mlp_softmax_xent(_p(logits), N_OUT, _p(nact), None, None, X.shape[0], _p(prob), None, None,

@@ -69,3 +69,83 @@ def test_training_lowers_the_loss_on_a_fixed_task():
 
     net = warmstart.train(np.pad(X, ((0, 0), (0, warmstart.F_IN - F))), nact, T, epochs=4, batch=1024, lr=3e-3)
     assert net.history[-1] < 0.6 * net.history[0]
+
+
+def _batch(rows, dim, seed=0):
+    rng = np.random.default_rng(seed * 1000003 + rows * 257 + dim)
+    X = rng.standard_normal((rows, dim)).astype(np.float32)
+    nact = rng.integers(1, M.N_OUT + 1, size=rows).astype(np.int32)
+    T = rng.random((rows, M.N_OUT)).astype(np.float32) * (np.arange(M.N_OUT) < nact[:, None])
+    return X, nact, T / T.sum(1, keepdims=True)
+
+
+# Fused network at the edges of its tiles (128 rows), operand groups (64
+# rows), row splits and input blocks (64 features), against the FP64 reference
+# with BF16-rounded operands; the bounds are those of the layer-by-layer test
+# above (activations whose BF16 rounding flips on the last bit, 2^-8 of a term).
+@pytest.mark.parametrize("dim", [4, 60, 64, 192, 196, 256])
+@pytest.mark.parametrize("rows", [1, 63, 127, 128, 129, 2049])
+def test_fused_network_matches_fp64_reference(rows, dim):
+    X, nact, T = _batch(rows, dim)
+    weight = np.random.default_rng(rows).random(rows).astype(np.float32) + 0.5
+    net = M.MLP(dim, seed=3)
+    assert net.fused
+    for b in net.b:
+        b.copy_(torch.randn(b.shape, generator=torch.Generator(device="cuda").manual_seed(dim), device="cuda"))
+    put = lambda x: torch.tensor(x, device="cuda")  # noqa: E731
+    W, b = net.numpy_params()
+    z = mlp_ref.forward(W, b, X.astype(np.float64), bf16=True)[-1]
+    z = np.where(np.arange(M.N_OUT) < nact[:, None], z, -np.inf)
+    p = np.exp(z - z.max(1, keepdims=True))
+    p /= p.sum(1, keepdims=True)
+    got = net.predict(put(X), put(nact)).cpu().numpy()
+    np.testing.assert_allclose(got, p, rtol=0, atol=2e-2)
+    np.testing.assert_array_equal(got[np.arange(M.N_OUT) >= nact[:, None]], 0.0)
+    for w in (None, weight):
+        loss = net.loss_and_grad(put(X), put(nact), put(T), None if w is None else put(w))
+        rl, rW, rb = mlp_ref.loss_and_grads(W, b, X.astype(np.float64), nact, T.astype(np.float64),
+                                            None if w is None else w.astype(np.float64), bf16=True)
+        assert loss == pytest.approx(rl, rel=1e-3)
+        gW, gb = net.numpy_grads()
+        for g, r in zip(gW + gb, rW + rb):
+            np.testing.assert_allclose(g, r, rtol=2e-2, atol=(5e-3 if rows > 128 else 2e-2) * np.abs(r).max())
+
+
+def test_fused_network_takes_unaligned_rows_and_keeps_the_activations_available():
+    X, nact, T = _batch(300, 192, seed=1)
+    net = M.MLP(192, seed=5)
+    base = torch.zeros(300 * 192 + 1, device="cuda")
+    view = base[1:].view(300, 192)  # 4-byte aligned only
+    view.copy_(torch.tensor(X))
+    n = torch.tensor(nact, device="cuda")
+    a, b = net.predict(view, n), net.predict(torch.tensor(X, device="cuda"), n)
+    assert torch.equal(a, b)
+    acts = net.acts
+    assert len(acts) == 5 and acts[0].data_ptr() != 0 and torch.equal(acts[0].cpu(), torch.tensor(X))
+    assert torch.allclose(torch.softmax(acts[-1].masked_fill(
+        torch.arange(8, device="cuda") >= n[:, None], -torch.inf), 1), a, atol=1e-2)
+
+
+def test_adam_steps_agree_between_the_fused_and_the_layer_by_layer_network():
+    X, nact, T = (torch.tensor(x, device="cuda") for x in _batch(500, 192, seed=2))
+    a, b = M.MLP(192, seed=7), M.MLP(192, seed=7)
+    b.fused = False
+    for _ in range(3):
+        la, lb = a.loss_and_grad(X, nact, T), b.loss_and_grad(X, nact, T)
+        assert la == pytest.approx(lb, rel=1e-4)
+        for x, y in zip(a.gW + a.gb, b.gW + b.gb):  # the same gradients into both updates
+            y.copy_(x)
+        a.adam_step(1e-3)
+        b.adam_step(1e-3)
+        for x, y in zip(a.W + a.b + a.Wb + a.mW + a.vW, b.W + b.b + b.Wb + b.mW + b.vW):
+            assert torch.equal(x, y)  # one formula, one rounding
+
+
+def test_other_shapes_run_layer_by_layer():
+    X, nact, T = _batch(70, 20, seed=4)
+    net = M.MLP(20, hidden=(32, 48), seed=1)
+    assert not net.fused
+    loss = net.loss_and_grad(*(torch.tensor(x, device="cuda") for x in (X, nact, T)))
+    W, b = net.numpy_params()
+    rl, _, _ = mlp_ref.loss_and_grads(W, b, X.astype(np.float64), nact, T.astype(np.float64), bf16=True)
+    assert loss == pytest.approx(rl, rel=1e-3)
