@@ -16,6 +16,9 @@
 // One CTA for every instance left the largest alone on one SM: a round of 64
 // endgames of 1e3 to 2e5 edges (50 iterations, exploitability, strategies)
 // 13.2 -> 5.0 ms; of ten of 2e5 to 1e6 edges, 8 CTAs each before, 11.9 -> 9.2.
+// Small solves in shared memory, loads issued together, slot updates by lanes
+// and enough registers: 5.0 -> 2.9 and 9.2 -> 5.4 ms; an iteration of 10,400
+// nodes in one CTA 28 -> 13 us (33 with the updates inside the depths).
 #pragma once
 #include <algorithm>
 #include <queue>
@@ -27,15 +30,16 @@
 namespace cfr {
 
 // CTAs for every instance of a batch (host). load: the instance's nodes times
-// the share of the longest run's iterations. Starting from `least` CTAs each,
-// the instance with the most load per CTA takes the next cluster size while
-// SMs are left for it, or its share exceeds an even one of the whole batch;
-// kSplitNodes per CTA and less stay whole, because a cluster barrier costs
-// more than a CTA's (about 1,600 cycles against 300 with stores in flight)
-// and the state is then read through L2. Clusters above 8 CTAs need most of a
-// GPC: at most six of them.
-constexpr int64_t kSplitNodes = 12000;
-inline std::vector<int> plan_clusters(const std::vector<int64_t> &load, int least, int sms) {
+// the share of the longest run's iterations; alone[i]: it is as fast in one
+// CTA. Starting from `least` CTAs each, the instance with the most load per
+// CTA takes the next cluster size while SMs are left for it, or its share
+// exceeds an even one of the whole batch. kSplitNodes per CTA and less stay as
+// they are: a cluster barrier costs 1,600 cycles with stores in flight, a
+// CTA's 300 (an endgame of 21,000 nodes: 29 us an iteration on 2 CTAs, 18 on
+// 8). Clusters above 8 CTAs need most of a GPC: at most six of them.
+constexpr int64_t kSplitNodes = 3000;
+inline std::vector<int> plan_clusters(const std::vector<int64_t> &load, const std::vector<char> &alone, int least,
+                                      int sms) {
   static const int sizes[] = {1, 2, 3, 4, 6, 8, 12, 16};
   const int n = (int)load.size();
   std::vector<int> cta(n, least);
@@ -52,6 +56,7 @@ inline std::vector<int> plan_clusters(const std::vector<int64_t> &load, int leas
     const int i = -most.top().second;
     most.pop();
     if (per <= kSplitNodes) break;
+    if (alone[i] && cta[i] == 1) continue;
     int next = 0;
     for (int c : sizes)
       if (c > cta[i]) { next = c; break; }
@@ -89,7 +94,7 @@ struct InstDesc {
   int32_t n_sets;
   int32_t root_vs;  // the root's value slot (N - 1)
   int32_t order;    // 0 simultaneous, 1 alternating updates
-  int32_t pad;
+  int32_t n_nodes, n_int, n_dec, n_slots, n_chance;  // value slots, internal nodes, members, slots, narrow chance nodes
 };
 
 template <int THREADS>
@@ -160,9 +165,247 @@ __device__ __forceinline__ void cta_bwd_wide(const GameView &g, T *v, int32_t wi
 
 constexpr int kBatchLevels = 32;  // depths whose work descriptors a CTA keeps in shared memory
 
-// FP64 kernels hold two registers a value: fewer threads, more registers. The
-// FP64 pipe is full with four warps an SM.
-template <typename T, int MAXA, int THREADS> constexpr int kBatchThreads = sizeof(T) == 8 && THREADS > 256 ? (MAXA <= 4 ? 512 : 256) : THREADS;
+// Where a solve's arrays are while a batched kernel runs.
+//   kSolo      one CTA, in global memory: its L1 holds what fits
+//   kCluster   several CTAs: state is read through L2, L1s are not coherent
+//   kResident  one CTA, copied into shared memory for the whole call
+constexpr int kSolo = 0, kCluster = 1, kResident = 2;
+
+// Threads of a CTA. The caller's 1,024 become 512 with twice the registers
+// (64 spilled; results do not depend on it); FP64 holds two registers a value,
+// and its pipe is full with four warps an SM.
+template <typename T, int MAXA, int THREADS>
+constexpr int kBatchThreads = THREADS <= 256 || (sizeof(T) == 8 && MAXA > 4) ? 256 : 512;
+
+template <int MODE, typename X>
+__device__ __forceinline__ X ldk(const X *p) {  // the compiled game: never written
+  if constexpr (MODE == kResident) return *p;
+  else return __ldg(p);
+}
+
+// Byte offsets of a resident solve's arrays in shared memory (16-byte
+// aligned; the state that goes back to global memory is sigma, R and avg:
+// reach and the inner values are recomputed by every iteration).
+struct ResidentLayout {
+  uint32_t iset_slot, iset_mem, iset_vb, iset_rank, mem_vs, int_edge, ch_vb, ch_nch, ch_vs;
+  uint32_t reach, v, sigma, R, avg, def_r, def_m, total;
+};
+
+__host__ __device__ inline ResidentLayout resident_layout(const InstDesc &in, uint32_t T) {
+  ResidentLayout L;
+  uint32_t at = 0;
+  auto take = [&](uint32_t n, uint32_t size) {
+    const uint32_t o = at;
+    at += (n * size + 15u) & ~15u;
+    return o;
+  };
+  const uint32_t I = (uint32_t)in.n_sets, A = (uint32_t)in.n_slots;
+  L.iset_slot = take(I + 1, 4);
+  L.iset_mem = take(I + 1, 4);
+  L.iset_vb = take(I, 4);
+  L.iset_rank = take(I, 8);
+  L.mem_vs = take((uint32_t)in.n_dec, 4);
+  L.int_edge = take((uint32_t)in.n_int, 8);
+  L.ch_vb = take((uint32_t)in.n_chance, 4);
+  L.ch_nch = take((uint32_t)in.n_chance, 4);
+  L.ch_vs = take((uint32_t)in.n_chance, 4);
+  L.reach = take((uint32_t)in.n_int, 2 * T);
+  L.v = take((uint32_t)in.n_nodes, T);
+  L.sigma = take(A, T);
+  L.R = take(A, 8);
+  L.avg = take(A, 8);
+  L.def_r = take(A, T);
+  L.def_m = take(A, T);
+  L.total = at;
+  return L;
+}
+
+// Games of at most this many nodes may be resident (32-bit offsets above
+// cannot overflow below it; the byte count decides).
+constexpr int64_t kResidentNodes = 1 << 16;
+constexpr uint32_t kResidentBytes = 190 * 1024;
+
+// The arrays that a batched iteration works on (member order).
+template <typename T> struct GroupView {
+  const int32_t *iset_slot, *iset_mem, *iset_vb, *mem_vs, *ch_vb, *ch_nch, *ch_vs;
+  const int2 *iset_rank, *int_edge;
+  vec2_t<T> *reach;
+  T *v, *sigma, *def_r, *def_m;
+  double *R, *avg;
+};
+
+// Internal nodes q, q + stride, ... of one depth pull their reach from their
+// parents' (as fwd_pull): kPullFar in flight while that many are left, then
+// two.
+constexpr int kPullFar = 4;
+template <typename T, int MODE>
+__device__ __forceinline__ void group_pull(const GroupView<T> &g, int32_t q, int32_t stride, int32_t qe) {
+  constexpr bool C = MODE == kCluster;
+  if constexpr (MODE != kResident) {
+    for (; q + (kPullFar - 1) * stride < qe; q += kPullFar * stride) {
+      int2 e[kPullFar];
+      vec2_t<T> r[kPullFar];
+      T s[kPullFar];
+#pragma unroll
+      for (int u = 0; u < kPullFar; ++u) e[u] = ldk<MODE>(g.int_edge + q + u * stride);
+#pragma unroll
+      for (int u = 0; u < kPullFar; ++u) {
+        r[u] = ldm<C>(g.reach + e[u].x);
+        s[u] = e[u].y >= 0 ? ldm<C>(g.sigma + (e[u].y & kMask)) : T(1);
+      }
+#pragma unroll
+      for (int u = 0; u < kPullFar; ++u) {
+        if (e[u].y >= 0) {
+          if (e[u].y & kP2Bit) r[u].y = r[u].y * s[u];
+          else r[u].x = r[u].x * s[u];
+        }
+        g.reach[q + u * stride] = r[u];
+      }
+    }
+  }
+  for (; q < qe; q += 2 * stride) {
+    const bool two = q + stride < qe;
+    const int2 e0 = ldk<MODE>(g.int_edge + q), e1 = two ? ldk<MODE>(g.int_edge + q + stride) : e0;
+    vec2_t<T> r0 = ldm<C>(g.reach + e0.x), r1 = two ? ldm<C>(g.reach + e1.x) : r0;
+    const T s0 = e0.y >= 0 ? ldm<C>(g.sigma + (e0.y & kMask)) : T(1);
+    const T s1 = two && e1.y >= 0 ? ldm<C>(g.sigma + (e1.y & kMask)) : T(1);
+    if (e0.y >= 0) {
+      if (e0.y & kP2Bit) r0.y = r0.y * s0;
+      else r0.x = r0.x * s0;
+    }
+    if (e1.y >= 0) {
+      if (e1.y & kP2Bit) r1.y = r1.y * s1;
+      else r1.x = r1.x * s1;
+    }
+    g.reach[q] = r0;
+    if (two) g.reach[q + stride] = r1;
+  }
+}
+
+// FP32: sets averaging this many members at a depth take a warp each (eight
+// lanes walk them in many dependent steps, and there are few of them).
+constexpr int kLongSet = 32;
+
+// One set by the LANES lanes of a group: its members' values, and the set's
+// totals into def_r and def_m (see bwd_set, whose sums these are). Every load
+// of a step is issued before the first value is used.
+template <typename T, int MAXA, int LANES, int MODE>
+__device__ __forceinline__ void group_set(const GroupView<T> &g, int32_t I, bool p2, int lane, unsigned mask, int upd,
+                                          double *rows) {
+  constexpr bool C = MODE == kCluster, CHAINS = sizeof(T) == 8;
+  constexpr int U = LANES <= 8 ? 2 : 1;  // members of a lane in flight
+  const int32_t sb = ldk<MODE>(g.iset_slot + I), se = ldk<MODE>(g.iset_slot + I + 1);
+  const int32_t m0 = ldk<MODE>(g.iset_mem + I), m1 = ldk<MODE>(g.iset_mem + I + 1);
+  const int32_t vb = ldk<MODE>(g.iset_vb + I);
+  const int2 rk = ldk<MODE>(g.iset_rank + I);
+  const int32_t na = se - sb, M = m1 - m0;
+  T sig[MAXA], racc[MAXA], spw = T(0);
+  double acc[kChainAcc<MAXA, LANES>];
+#pragma unroll
+  for (int a = 0; a < MAXA; ++a) {
+    sig[a] = a < na ? ldm<C>(g.sigma + sb + a) : T(0);
+    racc[a] = T(0);
+  }
+#pragma unroll
+  for (int i = 0; i < kChainAcc<MAXA, LANES>; ++i) acc[i] = 0.0;
+  for (int32_t k0 = 0; k0 < M; k0 += U * LANES) {
+    int32_t h[U];
+    vec2_t<T> r[U];
+    T vc[U][MAXA];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int32_t k = k0 + u * LANES + lane;
+      const bool in = k < M;
+      h[u] = in ? ldk<MODE>(g.mem_vs + m0 + k) : -1;
+      r[u].x = r[u].y = T(0);
+      if (in) r[u] = ldm<C>(g.reach + rk.x + k * rk.y);
+      const T *v = g.v + vb + k;
+#pragma unroll
+      for (int a = 0; a < MAXA; ++a) vc[u][a] = in && a < na ? ldm<C>(v + a * M) : T(0);
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (k0 + u * LANES >= M) break;  // the same for the whole group
+      T vh = T(0);
+#pragma unroll
+      for (int a = 0; a < MAXA; ++a)
+        if (a < na) vh = vh + sig[a] * vc[u][a];
+      if (h[u] >= 0) g.v[h[u]] = vh;
+      const T po = p2 ? r[u].x : r[u].y;  // opponent's reach (chance is inside v)
+      const T pw = p2 ? r[u].y : r[u].x;  // own reach
+      const T f = (p2 ? T(-1) : T(1)) * po;
+      if constexpr (CHAINS) {
+        T d[MAXA], mm[MAXA];
+#pragma unroll
+        for (int a = 0; a < MAXA; ++a) {
+          d[a] = T(0);
+          mm[a] = T(0);
+          if (a < na) {
+            d[a] = f * (vc[u][a] - vh);
+            mm[a] = pw * sig[a];
+          }
+        }
+        const int32_t left = M - k0 - u * LANES;
+        accumulate_chains<MAXA, LANES>(rows, left < LANES ? left : LANES, na, mask, d, mm, acc);
+      } else {
+#pragma unroll
+        for (int a = 0; a < MAXA; ++a)
+          if (a < na) racc[a] += f * (vc[u][a] - vh);  // 0 for lanes without a member
+        spw += pw;
+      }
+    }
+  }
+  if (!(upd & (p2 ? 2 : 1))) return;  // alternating updates: the other player's sets only pass their values up
+  if constexpr (CHAINS) {
+#pragma unroll
+    for (int i = 0; i < kChainAcc<MAXA, LANES>; ++i) {
+      const int c = lane + i * LANES;
+      if (c < na) g.def_r[sb + c] = acc[i];
+      else if (c >= MAXA && c - MAXA < na) g.def_m[sb + c - MAXA] = acc[i];
+    }
+  } else {
+    spw = group_sum_butterfly<LANES>(spw, mask);
+    if (lane == 0) g.def_m[sb] = spw;
+    group_sum_scatter<LANES, MAXA>(racc, lane, mask);
+    constexpr int STEP = MAXA <= LANES ? LANES / MAXA : 1, PER = MAXA <= LANES ? 1 : MAXA / LANES;
+    if (lane % STEP == 0) {
+#pragma unroll
+      for (int i = 0; i < PER; ++i)
+        if (lane / STEP * PER + i < na) g.def_r[sb + lane / STEP * PER + i] = racc[i];
+    }
+  }
+}
+
+// The slot updates of set I from its totals, by MAXA lanes, one for each slot:
+// FP64 instructions then serve most lanes of a warp, and the chain of a set is
+// one slot's.
+template <typename T, int MAXA, int MODE>
+__device__ __forceinline__ void group_update(const GroupView<T> &g, int32_t I, int a, unsigned mask, double wt,
+                                             int rule) {
+  constexpr bool C = MODE == kCluster;
+  const int32_t sb = ldk<MODE>(g.iset_slot + I), na = ldk<MODE>(g.iset_slot + I + 1) - sb, q = sb + a;
+  T pos = T(0);
+  if (a < na) {
+    const double R = g.R[q], S = g.avg[q];
+    const T r = ldm<C>(g.def_r + q);
+    T m;
+    if constexpr (sizeof(T) == 4) m = g.sigma[q] * ldm<C>(g.def_m + sb);  // this thread wrote sigma the iteration before
+    else m = ldm<C>(g.def_m + q);
+    double Rn, Sn;
+    const double x = slot_terms(R, S, as_double(r), as_double(m), wt, rule, Rn, Sn);
+    g.R[q] = Rn;
+    g.avg[q] = Sn;
+    if constexpr (sizeof(T) == 8) pos = x;
+    else pos = narrow_pos(x);
+  }
+  T tot = T(0);  // positive parts in action order
+#pragma unroll
+  for (int b = 0; b < MAXA; ++b) {
+    const T x = __shfl_sync(mask, pos, b, MAXA);
+    if (b < na) tot += x;
+  }
+  if (a < na) g.sigma[q] = match(pos, tot, na);
+}
 
 // Every launch of one call's chain may start as soon as the one before it has
 // started (programmatic dependent launch: the instances are independent);
@@ -174,25 +417,174 @@ __device__ __forceinline__ void chain_leave() {
 }
 
 // What bounds it: a small instance is a chain of dependent steps, 2 D - 1 of
-// them an iteration, each a barrier and two or three dependent loads; a large
-// one is latency of gathers at the occupancy of 64 registers a thread. The
-// slot updates (FP64) wait until the values of all depths are known and then
-// run one thread per set over the whole game: on the way up they would hold
-// every depth back by a dependent chain of FP64 instructions that serve a few
-// lanes each.
-template <typename T, int MAXA, int LANES, int THREADS, bool CLUSTERED>
-__global__ void __launch_bounds__(THREADS) batch_iterate_kernel(const InstDesc *table,
-                                                                const __grid_constant__ InstDesc one, int n_inst) {
-  __shared__ double sm[THREADS];
-  __shared__ double s_rows[THREADS / 32][kChainDoubles<T, MAXA, LANES>];
+// them an iteration, each a barrier and two or three dependent loads, so the
+// smallest games run from shared memory; a large one is the latency of its
+// gathers. The slot updates (FP64) wait until the values of all depths are
+// known and then run over the whole game at once: on the way up they would
+// hold every depth back by a dependent chain of FP64 instructions that serve
+// a few lanes each.
+template <typename T, int MAXA, int LANES, int NT, int MODE>
+__global__ void __launch_bounds__(NT, 1) batch_iterate_kernel(const InstDesc *table, const __grid_constant__ InstDesc one,
+                                                           int n_inst) {
+  constexpr bool CLUSTERED = MODE == kCluster;
+  extern __shared__ __align__(128) unsigned char s_solve[];
+  __shared__ double sm[MODE == kResident ? 1 : NT];
+  __shared__ double s_rows[NT / 32][kChainDoubles<T, MAXA, LANES>];
   __shared__ LevelWork s_lw[kBatchLevels];
+  __shared__ InstDesc s_in;
+  __shared__ unsigned char s_long[64];  // depths (modulo 64) whose sets average kLongSet members or more
   chain_enter();
   const int ncta = CLUSTERED ? (int)cluster_ncta() : 1;   // CTAs sharing this instance
   const int rank = CLUSTERED ? (int)cluster_rank() : 0;
   const int inst = (int)blockIdx.x / ncta;
   if (inst >= n_inst) return;  // the whole cluster leaves together
-  const int ct = rank * THREADS + (int)threadIdx.x, NT = ncta * THREADS;
-  const InstDesc in = table ? table[inst] : one;
+  const int tid = threadIdx.x, ct = rank * NT + tid, all = ncta * NT;
+  {
+    const int *src = reinterpret_cast<const int *>(table ? table + inst : &one);
+    for (int i = tid; i < (int)(sizeof(InstDesc) / 4); i += NT) reinterpret_cast<int *>(&s_in)[i] = src[i];
+  }
+  __syncthreads();
+  const InstDesc &in = s_in;
+  const int D = in.D, rule = in.rule;
+  const LevelWork *lw = in.lw;
+  if (D <= kBatchLevels) {
+    const int words = D * (int)(sizeof(LevelWork) / 4);
+    for (int i = tid; i < words; i += NT)
+      reinterpret_cast<int *>(s_lw)[i] = reinterpret_cast<const int *>(in.lw)[i];
+    lw = s_lw;
+  }
+  GroupView<T> g;
+  if constexpr (MODE == kResident) {
+    const ResidentLayout L = resident_layout(in, sizeof(T));
+    auto stage = [&](uint32_t off, const void *src, uint32_t bytes) {  // arena arrays are padded to 256 bytes
+      const uint32_t dst = (uint32_t)__cvta_generic_to_shared(s_solve + off);
+      for (uint32_t i = tid * 16u; i < bytes; i += NT * 16u)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + i), "l"((const char *)src + i) : "memory");
+      return s_solve + off;
+    };
+    const uint32_t I = (uint32_t)in.n_sets, A = (uint32_t)in.n_slots;
+    g.iset_slot = (const int32_t *)stage(L.iset_slot, in.g.iset_slot, 4 * (I + 1));
+    g.iset_mem = (const int32_t *)stage(L.iset_mem, in.g.iset_mem, 4 * (I + 1));
+    g.iset_vb = (const int32_t *)stage(L.iset_vb, in.g.iset_vb, 4 * I);
+    g.iset_rank = (const int2 *)stage(L.iset_rank, in.g.iset_rank, 8 * I);
+    g.mem_vs = (const int32_t *)stage(L.mem_vs, in.g.mem_vs, 4 * (uint32_t)in.n_dec);
+    g.int_edge = (const int2 *)stage(L.int_edge, in.g.int_edge, 8 * (uint32_t)in.n_int);
+    g.ch_vb = (const int32_t *)stage(L.ch_vb, in.g.ch_vb, 4 * (uint32_t)in.n_chance);
+    g.ch_nch = (const int32_t *)stage(L.ch_nch, in.g.ch_nch, 4 * (uint32_t)in.n_chance);
+    g.ch_vs = (const int32_t *)stage(L.ch_vs, in.g.ch_vs, 4 * (uint32_t)in.n_chance);
+    g.reach = (vec2_t<T> *)stage(L.reach, in.reach, 2 * (uint32_t)sizeof(T));  // the root's
+    g.v = (T *)stage(L.v, in.v, (uint32_t)sizeof(T) * (uint32_t)in.n_nodes);
+    g.sigma = (T *)stage(L.sigma, in.sigma, (uint32_t)sizeof(T) * A);
+    g.R = (double *)stage(L.R, in.R, 8 * A);
+    g.avg = (double *)stage(L.avg, in.avg, 8 * A);
+    g.def_r = (T *)(s_solve + L.def_r);
+    g.def_m = (T *)(s_solve + L.def_m);
+    asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+  } else {
+    g.iset_slot = in.g.iset_slot;
+    g.iset_mem = in.g.iset_mem;
+    g.iset_vb = in.g.iset_vb;
+    g.iset_rank = in.g.iset_rank;
+    g.mem_vs = in.g.mem_vs;
+    g.int_edge = in.g.int_edge;
+    g.ch_vb = in.g.ch_vb;
+    g.ch_nch = in.g.ch_nch;
+    g.ch_vs = in.g.ch_vs;
+    g.reach = (vec2_t<T> *)in.reach;
+    g.v = (T *)in.v;
+    g.sigma = (T *)in.sigma;
+    g.R = in.R;
+    g.avg = in.avg;
+    g.def_r = (T *)in.sbs;  // the sets' totals (read-out scratch, idle here)
+    g.def_m = (T *)in.out;
+  }
+  const long long t0 = *in.t, n_iter = in.n_iter;
+  const int n_sets = in.n_sets;
+  if (tid < 64) s_long[tid] = 0;
+  __syncthreads();
+  if (D <= 64 && tid < D) {  // a property of the game alone: the sums' shape does not depend on the batch
+    const int n = lw[tid].is1 - lw[tid].is0;
+    if (n > 0) s_long[tid] = in.g.iset_mem[lw[tid].is1] - in.g.iset_mem[lw[tid].is0] >= kLongSet * n;
+  }
+  __syncthreads();
+  const int lane = tid % LANES, gid = ct / LANES, ngroups = all / LANES;
+  const unsigned mask = group_mask<LANES>();
+  // slot updates: set I always by the same threads (their L1 holds its R and avg)
+  const int ua = tid % MAXA, ugid = ct / MAXA, ugroups = all / MAXA;
+  const unsigned umask = group_mask<MAXA>();
+  double *rows = s_rows[tid / 32];
+  const int halves = in.order ? 2 : 1;  // alternating: player 1's half, then player 2's
+  for (long long it = 0; it < n_iter; ++it) {
+    const double wt = avg_weight(t0 + it + 1, rule);
+    for (int hf = 0; hf < halves; ++hf) {
+      const int upd = halves == 2 ? (1 << hf) : 3;
+      for (int d = 1; d < D; ++d) {
+        group_pull<T, MODE>(g, lw[d].ib + ct, all, lw[d].ie);
+        level_sync<CLUSTERED>();
+      }
+      for (int d = D - 1; d >= 0; --d) {
+        const LevelWork &w = lw[d];
+        const int is0 = w.is0, is2 = w.is2, is1 = w.is1;
+        if (d == 0 && is0 == is1) break;  // a chance root's value has no reader in an iteration
+        if (d > 0) {
+          for (int32_t i = w.ch0 + ct; i < w.ch1; i += all) {  // narrow chance nodes: left to right
+            const int32_t cb = ldk<MODE>(g.ch_vb + i), n = ldk<MODE>(g.ch_nch + i);
+            T s = T(0);
+            for (int32_t c = 0; c < n; ++c) s = s + ldm<CLUSTERED>(g.v + cb + c);
+            g.v[ldk<MODE>(g.ch_vs + i)] = s;
+          }
+          if constexpr (MODE != kResident) {
+            if (rank == 0)
+              for (int32_t i = w.wd0; i < w.wd1; ++i) cta_bwd_wide<T, NT, CLUSTERED>(in.g, g.v, i, sm);
+          }
+        }
+        if (sizeof(T) == 4 && LANES < 32 && s_long[d & 63] != 0) {  // a warp for every set
+          for (int32_t I = is0 + ct / 32; I < is1; I += all / 32)
+            group_set<T, MAXA, 32, MODE>(g, I, I >= is2, tid & 31, 0xffffffffu, upd, rows);
+        } else {
+          for (int32_t I = is0 + gid; I < is1; I += ngroups)
+            group_set<T, MAXA, LANES, MODE>(g, I, I >= is2, lane, mask, upd, rows);
+        }
+        level_sync<CLUSTERED>();
+      }
+      if (upd == 3) {
+        for (int32_t I = ugid; I < n_sets; I += ugroups) group_update<T, MAXA, MODE>(g, I, ua, umask, wt, rule);
+      } else {  // one player's sets
+        for (int d = 0; d < D; ++d) {
+          const int32_t i0 = upd == 1 ? lw[d].is0 : lw[d].is2, i1 = upd == 1 ? lw[d].is2 : lw[d].is1;
+          for (int32_t I = i0 + (ugid + ugroups - i0 % ugroups) % ugroups; I < i1; I += ugroups)
+            group_update<T, MAXA, MODE>(g, I, ua, umask, wt, rule);
+        }
+      }
+      level_sync<CLUSTERED>();
+    }
+  }
+  if constexpr (MODE == kResident) {
+    for (int q = tid; q < in.n_slots; q += NT) {
+      ((T *)in.sigma)[q] = g.sigma[q];
+      in.R[q] = g.R[q];
+      in.avg[q] = g.avg[q];
+    }
+  }
+  if (ct == 0) *in.t = t0 + n_iter;
+  chain_leave();
+}
+
+// Breadth-first and value-slot reach orders (layout options): the same
+// iteration with the pushing forward of kernels.cuh.
+template <typename T, int MAXA, int LANES, int NT, int MODE>
+__global__ void __launch_bounds__(NT) batch_iterate_push_kernel(const InstDesc *table,
+                                                                const __grid_constant__ InstDesc one, int n_inst) {
+  constexpr bool CLUSTERED = MODE == kCluster;
+  __shared__ double sm[NT];
+  __shared__ double s_rows[NT / 32][kChainDoubles<T, MAXA, LANES>];
+  chain_enter();
+  const int ncta = CLUSTERED ? (int)cluster_ncta() : 1;
+  const int rank = CLUSTERED ? (int)cluster_rank() : 0;
+  const int inst = (int)blockIdx.x / ncta;
+  if (inst >= n_inst) return;
+  const int ct = rank * NT + (int)threadIdx.x, all = ncta * NT;
+  const InstDesc &in = table ? table[inst] : one;
   StateView<T> st;
   st.reach = (vec2_t<T> *)in.reach;
   st.v = (T *)in.v;
@@ -200,66 +592,35 @@ __global__ void __launch_bounds__(THREADS) batch_iterate_kernel(const InstDesc *
   st.R = in.R;
   st.avg = in.avg;
   st.t = in.t;
-  T *def_r = (T *)in.sbs, *def_m = (T *)in.out;  // the sets' totals (read-out scratch, idle here)
-  const LevelWork *lw = in.lw;
-  if (in.D <= kBatchLevels) {
-    const int words = in.D * (int)(sizeof(LevelWork) / 4);
-    for (int i = threadIdx.x; i < words; i += THREADS)
-      reinterpret_cast<int *>(s_lw)[i] = reinterpret_cast<const int *>(in.lw)[i];
-    lw = s_lw;
-    __syncthreads();
-  }
   const long long t0 = *in.t;
-  const int lane = threadIdx.x % LANES, gid = ct / LANES;
-  const int NG = NT / LANES;
+  const int lane = threadIdx.x % LANES, gid = ct / LANES, ngroups = all / LANES;
   const unsigned mask = group_mask<LANES>();
   double *rows = s_rows[threadIdx.x / 32];
-  const int halves = in.order ? 2 : 1;  // alternating: player 1's half, then player 2's
+  const int halves = in.order ? 2 : 1;
   for (long long it = 0; it < in.n_iter; ++it) {
     const double wt = avg_weight(t0 + it + 1, in.rule);
     for (int hf = 0; hf < halves; ++hf) {
       const int upd = in.order ? (1 << hf) : 3;
       for (int d = 0; d < in.D; ++d) {
-        if (in.g.int_edge) {  // member order: depth d + 1 pulls
-          if (d + 1 >= in.D) break;
-          const int32_t qe = lw[d + 1].ie;
-          for (int32_t q = lw[d + 1].ib + ct; q < qe; q += kPull * NT)
-            fwd_pull<T, CLUSTERED>(in.g, st.sigma, st.reach, q, NT, qe);
-        } else {
-          const LevelWork w = lw[d];
-          for (int32_t qw = w.ib + rank * THREADS + (threadIdx.x & ~31); qw < w.ie; qw += 4 * NT) {
-            if (w.fan) fwd_int4<T, CLUSTERED, true>(in.g, st.sigma, st.reach, qw + (threadIdx.x & 31), NT, w.ie);
-            else fwd_int4<T, CLUSTERED, false>(in.g, st.sigma, st.reach, qw + (threadIdx.x & 31), NT, w.ie);
-          }
-          for (int32_t i = w.wd0; i < w.wd1; ++i) cta_fwd_wide<T, CLUSTERED>(in.g, st.reach, i, ct, NT);
+        const LevelWork w = in.lw[d];
+        for (int32_t qw = w.ib + rank * NT + (threadIdx.x & ~31); qw < w.ie; qw += 4 * all) {
+          if (w.fan) fwd_int4<T, CLUSTERED, true>(in.g, st.sigma, st.reach, qw + (threadIdx.x & 31), all, w.ie);
+          else fwd_int4<T, CLUSTERED, false>(in.g, st.sigma, st.reach, qw + (threadIdx.x & 31), all, w.ie);
         }
+        for (int32_t i = w.wd0; i < w.wd1; ++i) cta_fwd_wide<T, CLUSTERED>(in.g, st.reach, i, ct, all);
         level_sync<CLUSTERED>();
       }
       for (int d = in.D - 1; d >= 0; --d) {
-        const LevelWork w = lw[d];
-        if (d == 0 && w.is0 == w.is1) break;  // a chance root's value has no reader in an iteration
+        const LevelWork w = in.lw[d];
         if (d > 0) {
-          for (int32_t i = w.ch0 + ct; i < w.ch1; i += NT)
-            bwd_chance<T, CLUSTERED>(in.g, st.v, i);
+          for (int32_t i = w.ch0 + ct; i < w.ch1; i += all) bwd_chance<T, CLUSTERED>(in.g, st.v, i);
           if (rank == 0)
-            for (int32_t i = w.wd0; i < w.wd1; ++i) cta_bwd_wide<T, THREADS, CLUSTERED>(in.g, st.v, i, sm);
+            for (int32_t i = w.wd0; i < w.wd1; ++i) cta_bwd_wide<T, NT, CLUSTERED>(in.g, st.v, i, sm);
         }
-        for (int32_t I = w.is0 + gid; I < w.is1; I += NG)
-          bwd_set<T, MAXA, LANES, CLUSTERED, sizeof(T) == 4, true>(in.g, st, I, I >= w.is2, lane, mask, wt, in.rule,
-                                                                  upd, rows, def_r, def_m);
+        for (int32_t I = w.is0 + gid; I < w.is1; I += ngroups)
+          bwd_set<T, MAXA, LANES, CLUSTERED>(in.g, st, I, I >= w.is2, lane, mask, wt, in.rule, upd, rows);
         level_sync<CLUSTERED>();
       }
-      if (upd == 3) {
-        for (int32_t I = ct; I < in.n_sets; I += NT)
-          update_set<T, MAXA, CLUSTERED>(in.g, st, I, wt, in.rule, def_r, def_m);
-      } else {  // one player's sets
-        for (int d = 0; d < in.D; ++d) {
-          const int32_t i0 = upd == 1 ? lw[d].is0 : lw[d].is2, i1 = upd == 1 ? lw[d].is2 : lw[d].is1;
-          for (int32_t I = i0 + (ct + NT - i0 % NT) % NT; I < i1; I += NT)  // set I: always thread I % NT
-            update_set<T, MAXA, CLUSTERED>(in.g, st, I, wt, in.rule, def_r, def_m);
-        }
-      }
-      level_sync<CLUSTERED>();
     }
   }
   if (ct == 0) *in.t = t0 + in.n_iter;

@@ -304,7 +304,7 @@ __device__ __forceinline__ void stream_update(const StreamChunk &d, const Stream
     const float x = __shfl_sync(0xffffffffu, pf, (b * G + jj) & 31);
     if (b < sj.na) tot += x;
   }
-  if (live) sigma[sj.sb + a] = tot > 0.f ? pf / tot : 1.f / (float)sj.na;
+  if (live) sigma[sj.sb + a] = match(pf, tot, sj.na);
 }
 
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {

@@ -904,10 +904,15 @@ extern "C" int cfr_avg_strategy(cfr_handle *h, double *out, int on_device, void 
   cudaStream_t s = (cudaStream_t)stream;
   const Compiled &c = h->c;
   if (c.I == 0) return CFR_OK;
-  avg_normalize_kernel<<<grid_for(c.I, kThreads), kThreads, 0, s>>>(h->p<int32_t>(h->b_iset_slot), (int32_t)c.I,
-                                                                     h->p<double>(h->b_avg), h->p<double>(h->b_sbs));
+  double *dst = on_device ? out : h->p<double>(h->b_out);
+  avg_spec_kernel<<<grid_for(c.I, kThreads), kThreads, 0, s>>>(h->p<int32_t>(h->b_iset_slot), (int32_t)c.I,
+                                                                h->p<double>(h->b_avg), h->p<int32_t>(h->b_spec_slot), dst);
   CK(cudaGetLastError());
-  return deliver(h, h->p<double>(h->b_sbs), out, on_device, s);
+  if (!on_device) {
+    CK(cudaMemcpyAsync(out, dst, 8 * c.A, cudaMemcpyDeviceToHost, s));
+    CK(cudaStreamSynchronize(s));
+  }
+  return CFR_OK;
 }
 
 extern "C" int cfr_current_strategy(cfr_handle *h, double *out, int on_device, void *stream) {
@@ -1521,22 +1526,35 @@ static InstDesc inst_desc(const cfr_handle *h, int64_t n_iter) {
   d.n_sets = (int32_t)h->c.I;
   d.root_vs = (int32_t)(h->c.N - 1);
   d.order = h->order;
+  d.n_nodes = (int32_t)h->c.N;
+  d.n_int = (int32_t)h->c.n_int;
+  d.n_dec = (int32_t)h->c.n_dec;
+  d.n_slots = (int32_t)h->c.A;
+  d.n_chance = (int32_t)h->c.ch_vb.size();
   return d;
+}
+
+// Bytes of shared memory that a solve of this game takes when it is resident
+// in one CTA, 0 if it cannot be.
+static uint32_t resident_bytes(const cfr_handle *h, const InstDesc &d) {
+  const Compiled &c = h->c;
+  if (c.int_edge.empty() || c.N > kResidentNodes) return 0;
+  for (int64_t l = 1; l < c.D; ++l)
+    if (c.level_wide[l + 1] != c.level_wide[l]) return 0;  // wide chance nodes are summed from global memory
+  const uint32_t n = resident_layout(d, h->precision == CFR_P64 ? 8u : 4u).total;
+  return n <= kResidentBytes ? std::max(n, 16u) : 0;
 }
 
 // A batched call's plan: the instances' descriptors ordered by cluster size
 // (largest first, and by load within a size), and one launch for each size.
 struct BatchPlan {
   std::vector<InstDesc> tab;
-  struct Launch {
-    int first, count, cluster;
-  };
-  std::vector<Launch> launches;
+  std::vector<BatchLaunch> launches;
   int maxa = 4, precision = -1;
 };
 
 static int batch_plan(cfr_handle *const *hs, int n, const int64_t *iters, int64_t n_iter, void *table_dev,
-                      size_t table_bytes, int cluster, BatchPlan &bp) {
+                      size_t table_bytes, int cluster, bool iterate, BatchPlan &bp) {
   if (!hs || n <= 0) return set_err(CFR_ERR_ARG, "batch: no instances");
   if (!table_dev || table_bytes < cfr_batch_table_bytes(n))
     return set_err(CFR_ERR_ARG, "batch: the descriptor table needs %zu bytes", cfr_batch_table_bytes(n));
@@ -1559,20 +1577,51 @@ static int batch_plan(cfr_handle *const *hs, int n, const int64_t *iters, int64_
     const double share = iters ? (double)iters[i] / (double)longest : 1.0;
     load[i] = (int64_t)((double)hs[i]->c.N * share);
   }
-  const std::vector<int> cta = plan_clusters(load, cluster, device_sms());
-  std::vector<int> at(n);
-  for (int i = 0; i < n; ++i) at[i] = i;
-  std::stable_sort(at.begin(), at.end(), [&](int a, int b) {
-    return cta[a] != cta[b] ? cta[a] > cta[b] : load[a] > load[b];
+  // one launch for each kind: push or pull, cluster size, resident or not
+  struct Entry {
+    int inst, push, mode;
+    uint32_t smem;
+    InstDesc d;
+  };
+  std::vector<Entry> e(n);
+  std::vector<char> alone(n, 0);
+  for (int i = 0; i < n; ++i) {
+    e[i].inst = i;
+    e[i].push = iterate && hs[i]->c.int_edge.empty();
+    e[i].d = inst_desc(hs[i], iters ? iters[i] : n_iter);
+    e[i].smem = iterate && cluster == 1 ? resident_bytes(hs[i], e[i].d) : 0;
+    // FP32: as fast resident in one CTA as in a cluster of 8 (10,400 nodes: 16 us an iteration either way)
+    alone[i] = e[i].smem > 0 && bp.precision == CFR_P32;
+  }
+  const std::vector<int> cta = plan_clusters(load, alone, cluster, device_sms());
+  for (int i = 0; i < n; ++i) {
+    if (cta[i] > 1) e[i].smem = 0;
+    e[i].mode = cta[i] > 1 ? kCluster : e[i].smem > 0 ? kResident : kSolo;
+  }
+  std::stable_sort(e.begin(), e.end(), [&](const Entry &a, const Entry &b) {
+    const int ca = cta[a.inst], cb = cta[b.inst];
+    if (ca != cb) return ca > cb;
+    if (a.push != b.push) return a.push > b.push;
+    if (a.mode != b.mode) return a.mode < b.mode;
+    return load[a.inst] > load[b.inst];
   });
   double *res = reinterpret_cast<double *>((char *)table_dev + sizeof(InstDesc) * (size_t)n);
   bp.tab.resize(n);
   for (int k = 0; k < n; ++k) {
-    const int i = at[k];
-    bp.tab[k] = inst_desc(hs[i], iters ? iters[i] : n_iter);
-    bp.tab[k].res = res + 4 * (size_t)i;
-    if (k == 0 || cta[i] != cta[at[k - 1]]) bp.launches.push_back({k, 0, cta[i]});
+    const Entry &x = e[k];
+    bp.tab[k] = x.d;
+    bp.tab[k].res = res + 4 * (size_t)x.inst;
+    if (k == 0 || cta[x.inst] != cta[e[k - 1].inst] || x.push != e[k - 1].push || x.mode != e[k - 1].mode) {
+      BatchLaunch l;
+      l.first = k;
+      l.cluster = cta[x.inst];
+      l.mode = x.mode;
+      l.push = x.push;
+      l.chained = k > 0;
+      bp.launches.push_back(l);
+    }
     ++bp.launches.back().count;
+    bp.launches.back().smem = std::max(bp.launches.back().smem, x.smem);
   }
   return CFR_OK;
 }
@@ -1598,17 +1647,15 @@ extern "C" int cfr_batch_iterate(cfr_handle *const *hs, int n, const int64_t *it
   int rc = batch_shape(&threads, &lanes);
   if (rc) return rc;
   BatchPlan bp;
-  if ((rc = batch_plan(hs, n, iters, n_iter, table_dev, table_bytes, cluster, bp))) return rc;
+  if ((rc = batch_plan(hs, n, iters, n_iter, table_dev, table_bytes, cluster, true, bp))) return rc;
   cudaStream_t s = (cudaStream_t)stream;
   const InstDesc *tab = (const InstDesc *)table_dev;
   CK(cudaMemcpyAsync(table_dev, bp.tab.data(), sizeof(InstDesc) * (size_t)n, cudaMemcpyHostToDevice, s));
-  bool chained = false;
-  for (const BatchPlan::Launch &l : bp.launches) {
+  for (const BatchLaunch &l : bp.launches) {
     if (bp.precision == CFR_P64)
-      CK(launch_batch_iterate<double>(bp.maxa, lanes, threads, l.cluster, chained, l.count, s, tab + l.first, bp.tab[0]));
+      CK(launch_batch_iterate<double>(bp.maxa, lanes, threads, l, s, tab + l.first, bp.tab[0]));
     else
-      CK(launch_batch_iterate<float>(bp.maxa, lanes, threads, l.cluster, chained, l.count, s, tab + l.first, bp.tab[0]));
-    chained = true;
+      CK(launch_batch_iterate<float>(bp.maxa, lanes, threads, l, s, tab + l.first, bp.tab[0]));
   }
   for (int i = 0; i < n; ++i) hs[i]->iteration_host += iters ? iters[i] : n_iter;
   return CFR_OK;
@@ -1620,15 +1667,11 @@ extern "C" int cfr_batch_exploitability(cfr_handle *const *hs, int n, double *ou
   int rc = batch_shape(&threads, &lanes);
   if (rc) return rc;
   BatchPlan bp;
-  if ((rc = batch_plan(hs, n, nullptr, 0, table_dev, table_bytes, 1, bp))) return rc;
+  if ((rc = batch_plan(hs, n, nullptr, 0, table_dev, table_bytes, 1, false, bp))) return rc;
   cudaStream_t s = (cudaStream_t)stream;
   const InstDesc *tab = (const InstDesc *)table_dev;
   CK(cudaMemcpyAsync(table_dev, bp.tab.data(), sizeof(InstDesc) * (size_t)n, cudaMemcpyHostToDevice, s));
-  bool chained = false;
-  for (const BatchPlan::Launch &l : bp.launches) {
-    CK(launch_batch_br(bp.maxa, lanes, threads, l.cluster, chained, l.count, s, tab + l.first, bp.tab[0]));
-    chained = true;
-  }
+  for (const BatchLaunch &l : bp.launches) CK(launch_batch_br(bp.maxa, lanes, threads, l, s, tab + l.first, bp.tab[0]));
   CK(cudaMemcpyAsync(out, tab + n, 4 * sizeof(double) * (size_t)n, cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
   return CFR_OK;

@@ -1,5 +1,5 @@
 // Batched-iteration kernel instances, FP64 (see batch.cuh).
 #include "k_batch.cuh"
 namespace cfr {
-template cudaError_t launch_batch_iterate<double>(int, int, int, int, bool, int, cudaStream_t, const InstDesc *, const InstDesc &);
+template cudaError_t launch_batch_iterate<double>(int, int, int, const BatchLaunch &, cudaStream_t, const InstDesc *, const InstDesc &);
 }

@@ -2,16 +2,16 @@
 #include "k_batch.cuh"
 namespace cfr {
 template <int MA, int L, int TH>
-static cudaError_t br_one(int cluster, bool chained, int n, cudaStream_t s, const InstDesc *table, const InstDesc &one) {
+static cudaError_t br_one(const BatchLaunch &l, cudaStream_t s, const InstDesc *table, const InstDesc &one) {
   constexpr int NT = kBatchThreads<double, MA, TH>;
-  if (cluster == 1) return launch_batch_any(batch_br_kernel<MA, L, NT, false>, NT, 1, chained, n, s, table, one);
-  return launch_batch_any(batch_br_kernel<MA, L, NT, true>, NT, cluster, chained, n, s, table, one);
+  if (l.mode == kCluster) return launch_batch_any(batch_br_kernel<MA, L, NT, true>, NT, l, s, table, one);
+  return launch_batch_any(batch_br_kernel<MA, L, NT, false>, NT, l, s, table, one);
 }
 
-cudaError_t launch_batch_br(int maxa, int lanes, int threads, int cluster, bool chained, int n, cudaStream_t s,
+cudaError_t launch_batch_br(int maxa, int lanes, int threads, const BatchLaunch &l, cudaStream_t s,
                             const InstDesc *table, const InstDesc &one) {
 #define BR_CASE(MA, L, TH) \
-  if (maxa == MA && lanes == L && threads == TH) return br_one<MA, L, TH>(cluster, chained, n, s, table, one);
+  if (maxa == MA && lanes == L && threads == TH) return br_one<MA, L, TH>(l, s, table, one);
   CFR_BATCH_ALL(BR_CASE)
 #undef BR_CASE
   return cudaErrorInvalidValue;

@@ -424,19 +424,24 @@ __device__ __forceinline__ double avg_weight(long long t, int rule) {
 
 // Conversions and comparisons of doubles in integer arithmetic. GB300's FP64
 // pipe takes one warp instruction every 16-19 cycles per SM whatever the
-// number of active lanes, and conversions (cvt.f64.f32, cvt.f32.f64) and
-// compares (setp.f64) run there too, with 100 cycles of latency each
-// (measured; 64 for an add). The slot update is a chain of them on a few
-// lanes of a warp, so only its add and its multiply-add stay on that pipe: five
-// iterations of the 2.8M-node random tree 635 -> 595 us, 50 of a 21k-node
-// endgame 1,291 -> 1,255 us. Same results bit for bit, for every input.
+// number of active lanes (an instruction whose predicate is off in all of
+// them included), and conversions (cvt.f64.f32, cvt.f32.f64) and compares
+// (setp.f64) run there too, with 100 cycles of latency each (measured; 64
+// for an add). The slot update is a chain of them on a few lanes of a warp, so
+// only its add and its multiply-add stay on that pipe, and what is rarely
+// needed is a function of its own, or the compiler runs it always, predicated
+// off: a round of 16 warps 2,372 -> 609 cycles, of one warp 645 -> 304. Same
+// results bit for bit (NaNs stay NaNs).
 __device__ __forceinline__ double widen(float x) {  // (double)x
-  const uint32_t u = __float_as_uint(x), e = (u >> 23) & 255u;
-  if (e - 1u < 254u)
-    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
-  if ((u << 1) == 0u) return __hiloint2double((int)u, 0);
-  return (double)x;  // subnormal, infinite or NaN
+  const uint32_t e = (__float_as_uint(x) >> 23) & 255u;
+  const bool sub = e == 0u;  // zero or subnormal: scaled into the normal range first
+  const uint32_t u = __float_as_uint(sub ? x * 18446744073709551616.f : x);
+  uint32_t hi = ((u & 0x7fffffffu) >> 3) + (sub ? 0x34000000u : 0x38000000u) + (e == 255u ? 0x38000000u : 0u);
+  if ((u << 1) == 0u) hi = 0u;
+  return __hiloint2double((int)((u & 0x80000000u) | hi), (int)(u << 29));
 }
+
+static __device__ __noinline__ float narrow_rare(double x) { return (float)x; }
 
 __device__ __forceinline__ float narrow_pos(double x) {  // (float)x of x >= 0, to nearest, ties to even
   const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
@@ -447,7 +452,7 @@ __device__ __forceinline__ float narrow_pos(double x) {  // (float)x of x >= 0, 
     return __uint_as_float(m + (rest > 0x10000000u - (m & 1u) ? 1u : 0u));
   }
   if ((hi | lo) == 0u) return 0.f;
-  return (float)x;
+  return narrow_rare(x);  // to a subnormal or infinite float
 }
 
 __device__ __forceinline__ double positive_part(double x) {  // x > 0.0 ? x : 0.0 (NaN and -0 give 0)
@@ -459,6 +464,21 @@ __device__ __forceinline__ double positive_part(double x) {  // x > 0.0 ? x : 0.
 __device__ __forceinline__ double as_double(float x) { return widen(x); }
 __device__ __forceinline__ double as_double(double x) { return x; }
 
+// PCFR+ matches against R + r.
+static __device__ __noinline__ double predicted(double R, double r) { return R + r; }
+
+// sigma of a slot from its positive part and the set's sum of them (uniform
+// where the sum is zero), with one division.
+__device__ __forceinline__ float match(float pos, float tot, int32_t na) {
+  const bool some = tot > 0.f;
+  return (some ? pos : 1.f) / (some ? tot : (float)na);
+}
+__device__ __forceinline__ double match(double pos, double tot, int32_t na) {
+  const long long b = __double_as_longlong(tot);
+  const bool some = b > 0 && b <= 0x7ff0000000000000ll;
+  return (some ? pos : 1.0) / (some ? tot : widen((float)na));
+}
+
 // One slot's update from its set's totals (instantaneous regret r, average
 // term m) and its cumulative regret R and average sum S: Rn = R + r (clamped
 // at 0 except under vanilla CFR) and Sn = S + wt * m. Returns what regret
@@ -468,7 +488,9 @@ __device__ __forceinline__ double slot_terms(double R, double S, double r, doubl
   Rn = R + r;
   if (rule != kRuleCfr) Rn = positive_part(Rn);
   Sn = S + wt * m;
-  return positive_part(rule == kRulePcfrPlus ? Rn + r : Rn);
+  double x = Rn;
+  if (rule == kRulePcfrPlus) x = predicted(Rn, r);
+  return positive_part(x);
 }
 
 // The same on the slot's entries in memory.
@@ -555,11 +577,8 @@ __device__ __forceinline__ void member_idx(const GameView &g, int32_t k, int32_t
 // already known, or zeros. The member's child a is slot vb + a * M + (k -
 // m0) of the set's block (M = m1 - m0 members): for each action the group's
 // lanes read consecutive members' children as one run. The average-strategy terms are
-// pw * sigma(a). LEAN (FP32 only): only pw is carried (mm[0]) and the set's
-// sum of pw is multiplied by sigma(a) once (avg_terms), which frees
-// registers where the budget is tight; otherwise each product is added, in
-// member order in FP64, as the definition does.
-template <typename T, int MAXA, bool PERSIST, bool LEAN = false>
+// pw * sigma(a), each added, in member order in FP64, as the definition does.
+template <typename T, int MAXA, bool PERSIST>
 __device__ __forceinline__ void member_data(const GameView &g, const StateView<T> &st, int32_t k, int32_t m0,
                                             int32_t m1, int32_t vb, int32_t na, bool p2, const T (&sig)[MAXA],
                                             int32_t h, int32_t ir, T (&d)[MAXA], T (&mm)[MAXA]) {
@@ -585,29 +604,19 @@ __device__ __forceinline__ void member_data(const GameView &g, const StateView<T
   for (int a = 0; a < MAXA; ++a) {
     if (a < na) {
       d[a] = f * (vc[a] - vh);
-      if constexpr (!LEAN || sizeof(T) == 8) mm[a] = pw * sig[a];
+      mm[a] = pw * sig[a];
     }
   }
-  if constexpr (LEAN && sizeof(T) == 4) mm[0] = pw;
-}
-
-// LEAN FP32: the set's average terms sigma(a) * (sum of the members' own
-// reach), from the sum carried in macc[0].
-template <typename T, int MAXA>
-__device__ __forceinline__ void avg_terms(const T (&sig)[MAXA], int32_t na, T (&macc)[MAXA]) {
-  const T spw = macc[0];
-#pragma unroll
-  for (int a = 0; a < MAXA; ++a) macc[a] = a < na ? sig[a] * spw : T(0);
 }
 
 // Indices, loads and per-member terms of one member (k < m1), or zeros.
-template <typename T, int MAXA, bool PERSIST, bool LEAN = false>
+template <typename T, int MAXA, bool PERSIST>
 __device__ __forceinline__ void member_terms(const GameView &g, const StateView<T> &st, int32_t k, int32_t m0,
                                              int32_t m1, MemberRanks mr, int32_t vb, int32_t na, bool p2,
                                              const T (&sig)[MAXA], T (&d)[MAXA], T (&mm)[MAXA]) {
   int32_t h, ir;
   member_idx(g, k, m1, mr, h, ir);
-  member_data<T, MAXA, PERSIST, LEAN>(g, st, k, m0, m1, vb, na, p2, sig, h, ir, d, mm);
+  member_data<T, MAXA, PERSIST>(g, st, k, m0, m1, vb, na, p2, sig, h, ir, d, mm);
 }
 
 // FP64 sums of a set run in the order of the definition, one dependent chain
@@ -682,13 +691,10 @@ __device__ __forceinline__ void accumulate_chunk(int32_t cnt, int32_t na, unsign
 // in chunks of LANES (two chunks per step for narrow groups); each step loads
 // the next step's member indices while its own reach and child values are in
 // flight, so a step waits for one memory round trip, not two. The update of
-// the set's slots runs one lane per action. LEAN: see member_data. DEFER: the
-// set's totals go to def_r (and def_m: FP32 the set's sum of own reach at its
-// first slot, FP64 every slot's average term) for update_set to take up later.
-template <typename T, int MAXA, int LANES, bool PERSIST, bool LEAN = false, bool DEFER = false>
+// the set's slots runs one lane per action.
+template <typename T, int MAXA, int LANES, bool PERSIST>
 __device__ __forceinline__ void bwd_set(const GameView &g, const StateView<T> &st, int32_t I, bool p2,
-                                        int lane, unsigned mask, double wt, int rule, int upd, double *rows,
-                                        T *def_r = nullptr, T *def_m = nullptr) {
+                                        int lane, unsigned mask, double wt, int rule, int upd, double *rows) {
   const int32_t sb = __ldg(g.iset_slot + I);
   const int32_t na = __ldg(g.iset_slot + I + 1) - sb;
   const int32_t m0 = __ldg(g.iset_mem + I), m1 = __ldg(g.iset_mem + I + 1);
@@ -710,38 +716,8 @@ __device__ __forceinline__ void bwd_set(const GameView &g, const StateView<T> &s
     else accumulate_chunk<T, MAXA, LANES>(cnt, na, mask, d, mm, racc, macc);
   };
   constexpr bool TWO = MAXA <= 8 && LANES <= 8;  // narrow groups keep two chunks in flight
-  constexpr int NCH = 2;
   int32_t k0 = m0;
-  // The two forms below compute the same; the one with chunk arrays
-  // compiles to fewer spills in LEAN kernels (64 registers a thread), the
-  // one with named chunks runs faster with a larger register budget.
-  if constexpr (TWO && LEAN) {
-    if (k0 + (NCH - 1) * LANES < m1) {
-      int32_t ps[NCH], ir[NCH];
-#pragma unroll
-      for (int j = 0; j < NCH; ++j) member_idx(g, k0 + j * LANES + lane, m1, mr, ps[j], ir[j]);
-      for (; k0 + (NCH - 1) * LANES < m1; k0 += NCH * LANES) {
-        int32_t qs[NCH], jr[NCH];  // the next step's indices
-#pragma unroll
-        for (int j = 0; j < NCH; ++j) member_idx(g, k0 + (NCH + j) * LANES + lane, m1, mr, qs[j], jr[j]);
-        T d[NCH][MAXA], mm[NCH][MAXA];
-#pragma unroll
-        for (int j = 0; j < NCH; ++j)
-          member_data<T, MAXA, PERSIST, LEAN>(g, st, k0 + j * LANES + lane, m0, m1, vb, na, p2, sig, ps[j], ir[j],
-                                              d[j], mm[j]);
-#pragma unroll
-        for (int j = 0; j < NCH; ++j) {  // chunks in member order
-          const int32_t left = m1 - k0 - j * LANES;
-          add_chunk(left < 0 ? 0 : (left < LANES ? left : LANES), d[j], mm[j]);
-        }
-#pragma unroll
-        for (int j = 0; j < NCH; ++j) {
-          ps[j] = qs[j];
-          ir[j] = jr[j];
-        }
-      }
-    }
-  } else if constexpr (TWO) {
+  if constexpr (TWO) {
     if (k0 + LANES < m1) {
       int32_t ps0, ir0, ps1, ir1;
       member_idx(g, k0 + lane, m1, mr, ps0, ir0);
@@ -751,8 +727,8 @@ __device__ __forceinline__ void bwd_set(const GameView &g, const StateView<T> &s
         member_idx(g, k0 + 2 * LANES + lane, m1, mr, qs0, jr0);
         member_idx(g, k0 + 3 * LANES + lane, m1, mr, qs1, jr1);
         T d0[MAXA], mm0[MAXA], d1[MAXA], mm1[MAXA];
-        member_data<T, MAXA, PERSIST, LEAN>(g, st, k0 + lane, m0, m1, vb, na, p2, sig, ps0, ir0, d0, mm0);
-        member_data<T, MAXA, PERSIST, LEAN>(g, st, k0 + LANES + lane, m0, m1, vb, na, p2, sig, ps1, ir1, d1, mm1);
+        member_data<T, MAXA, PERSIST>(g, st, k0 + lane, m0, m1, vb, na, p2, sig, ps0, ir0, d0, mm0);
+        member_data<T, MAXA, PERSIST>(g, st, k0 + LANES + lane, m0, m1, vb, na, p2, sig, ps1, ir1, d1, mm1);
         add_chunk(LANES, d0, mm0);
         const int32_t c1 = (m1 - k0 - LANES) < LANES ? (m1 - k0 - LANES) : LANES;
         add_chunk(c1, d1, mm1);
@@ -763,7 +739,7 @@ __device__ __forceinline__ void bwd_set(const GameView &g, const StateView<T> &s
   if constexpr (TWO) {  // the last chunk
     for (; k0 < m1; k0 += LANES) {
       T d[MAXA], mm[MAXA];
-      member_terms<T, MAXA, PERSIST, LEAN>(g, st, k0 + lane, m0, m1, mr, vb, na, p2, sig, d, mm);
+      member_terms<T, MAXA, PERSIST>(g, st, k0 + lane, m0, m1, mr, vb, na, p2, sig, d, mm);
       const int32_t cnt = (m1 - k0) < LANES ? (m1 - k0) : LANES;
       add_chunk(cnt, d, mm);
     }
@@ -774,7 +750,7 @@ __device__ __forceinline__ void bwd_set(const GameView &g, const StateView<T> &s
       int32_t qs, jr;  // the next step's indices
       member_idx(g, k0 + LANES + lane, m1, mr, qs, jr);
       T d[MAXA], mm[MAXA];
-      member_data<T, MAXA, PERSIST, LEAN>(g, st, k0 + lane, m0, m1, vb, na, p2, sig, ps, ir, d, mm);
+      member_data<T, MAXA, PERSIST>(g, st, k0 + lane, m0, m1, vb, na, p2, sig, ps, ir, d, mm);
       const int32_t cnt = (m1 - k0) < LANES ? (m1 - k0) : LANES;
       add_chunk(cnt, d, mm);
       ps = qs; ir = jr;
@@ -782,42 +758,13 @@ __device__ __forceinline__ void bwd_set(const GameView &g, const StateView<T> &s
   }
   // alternating updates: the other player's sets only pass their values up
   if (!(upd & (p2 ? 2 : 1))) return;
-  if constexpr (DEFER) {
-    if constexpr (CHAINS) {
-#pragma unroll
-      for (int i = 0; i < kChainAcc<MAXA, LANES>; ++i) {
-        const int c = lane + i * LANES;
-        if (c < na) def_r[sb + c] = acc[i];
-        else if (c >= MAXA && c - MAXA < na) def_m[sb + c - MAXA] = acc[i];
-      }
-    } else {
-      static_assert(sizeof(T) == 4 && LEAN && MAXA <= 8, "deferred updates: FP64 needs chains, FP32 lean average terms");
-      macc[0] = group_sum_butterfly<LANES>(macc[0], mask);
-      if (lane == 0) def_m[sb] = macc[0];
-      group_sum_scatter<LANES, MAXA>(racc, lane, mask);
-      if constexpr (MAXA <= LANES) {
-        constexpr int STEP = LANES / MAXA;
-        if (lane % STEP == 0 && lane / STEP < na) def_r[sb + lane / STEP] = racc[0];
-      } else {
-        constexpr int PER = MAXA / LANES;
-#pragma unroll
-        for (int i = 0; i < PER; ++i)
-          if (lane * PER + i < na) def_r[sb + lane * PER + i] = racc[i];
-      }
-    }
-    return;
-  }
   if constexpr (sizeof(T) == 4) {
 #pragma unroll
     for (int a = 0; a < MAXA; ++a) {
       if (a < na) {
         racc[a] = group_sum_butterfly<LANES>(racc[a], mask);
-        if constexpr (!LEAN) macc[a] = group_sum_butterfly<LANES>(macc[a], mask);
+        macc[a] = group_sum_butterfly<LANES>(macc[a], mask);
       }
-    }
-    if constexpr (LEAN) {
-      macc[0] = group_sum_butterfly<LANES>(macc[0], mask);
-      avg_terms<T, MAXA>(sig, na, macc);
     }
   }
   // every lane now holds the set's totals racc[a], macc[a] (CHAINS: its own
@@ -847,12 +794,12 @@ __device__ __forceinline__ void bwd_set(const GameView &g, const StateView<T> &s
     if constexpr (sizeof(T) == 8) {
       double tot = 0.0;
       for (int a = 0; a < na; ++a) tot += __shfl_sync(mask, pos, a, LANES);
-      if (lane < na) st.sigma[sb + lane] = __double_as_longlong(tot) > 0 ? pos / tot : 1.0 / (double)na;
+      if (lane < na) st.sigma[sb + lane] = match(pos, tot, na);
     } else {
       const float pf = narrow_pos(pos);
       float tot = 0.f;
       for (int a = 0; a < na; ++a) tot += __shfl_sync(mask, pf, a, LANES);
-      if (lane < na) st.sigma[sb + lane] = tot > 0.f ? pf / tot : 1.f / (float)na;
+      if (lane < na) st.sigma[sb + lane] = match(pf, tot, na);
     }
   } else if (lane == 0) {
     T pos[MAXA];
@@ -868,54 +815,8 @@ __device__ __forceinline__ void bwd_set(const GameView &g, const StateView<T> &s
     }
 #pragma unroll
     for (int a = 0; a < MAXA; ++a)
-      if (a < na) st.sigma[sb + a] = tot > T(0) ? pos[a] / tot : T(1) / (T)na;
+      if (a < na) st.sigma[sb + a] = match(pos[a], tot, na);
   }
-}
-
-// The slot updates of set I from its deferred totals, by one thread: a warp's
-// FP64 instructions then serve 32 sets at once instead of the few lanes of a
-// group. Every slot's loads are issued before the first is used.
-template <typename T, int MAXA, bool PERSIST>
-__device__ __forceinline__ void update_set(const GameView &g, const StateView<T> &st, int32_t I, double wt, int rule,
-                                           const T *def_r, const T *def_m) {
-  const int32_t sb = __ldg(g.iset_slot + I);
-  const int32_t na = __ldg(g.iset_slot + I + 1) - sb;
-  constexpr int W = 4;  // slots in flight
-  T pos[MAXA];
-  T tot = T(0), spw = T(0);
-  if constexpr (sizeof(T) == 4) spw = ldm<PERSIST>(def_m + sb);
-#pragma unroll
-  for (int a0 = 0; a0 < MAXA; a0 += W) {
-    double R[W], S[W];
-    T r[W], m[W];
-#pragma unroll
-    for (int j = 0; j < W; ++j) {
-      if (a0 + j < na) {
-        const int32_t q = sb + a0 + j;
-        R[j] = st.R[q];
-        S[j] = st.avg[q];
-        r[j] = ldm<PERSIST>(def_r + q);
-        if constexpr (sizeof(T) == 4) m[j] = st.sigma[q] * spw;  // written by this thread the iteration before
-        else m[j] = ldm<PERSIST>(def_m + q);
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < W; ++j) {
-      if (a0 + j < na) {
-        const int32_t q = sb + a0 + j;
-        double Rn, Sn;
-        const double x = slot_terms(R[j], S[j], as_double(r[j]), as_double(m[j]), wt, rule, Rn, Sn);
-        st.R[q] = Rn;
-        st.avg[q] = Sn;
-        if constexpr (sizeof(T) == 8) pos[a0 + j] = x;
-        else pos[a0 + j] = narrow_pos(x);
-        tot += pos[a0 + j];
-      }
-    }
-  }
-#pragma unroll
-  for (int a = 0; a < MAXA; ++a)
-    if (a < na) st.sigma[sb + a] = tot > T(0) ? pos[a] / tot : T(1) / (T)na;
 }
 
 // One information set per block, for depths with few sets of hundreds of
@@ -1014,11 +915,11 @@ __device__ __forceinline__ void bwd_set_block(const GameView &g, const StateView
     if constexpr (sizeof(T) == 8) {
       double tot = 0.0;
       for (int a = 0; a < na; ++a) tot += s_pos[a];
-      st.sigma[sb + tid] = tot > 0.0 ? pos / tot : 1.0 / (double)na;
+      st.sigma[sb + tid] = match(pos, tot, na);
     } else {
       float tot = 0.f;
       for (int a = 0; a < na; ++a) tot += narrow_pos(s_pos[a]);
-      st.sigma[sb + tid] = tot > 0.f ? narrow_pos(pos) / tot : 1.f / (float)na;
+      st.sigma[sb + tid] = match(narrow_pos(pos), tot, na);
     }
   }
   __syncthreads();  // shared arrays are reused by the block's next set
@@ -1224,6 +1125,18 @@ __global__ void rm_kernel(const int32_t *iset_slot, int32_t n_sets, const double
 }
 
 // ------------------------------------------------------------- read-out
+// The average strategy in spec slot order (the two kernels below in one).
+static __global__ void avg_spec_kernel(const int32_t *iset_slot, int32_t n_sets, const double *avg,
+                                       const int32_t *spec_slot_of, double *out) {
+  const int32_t stride = gridDim.x * blockDim.x;
+  for (int32_t I = blockIdx.x * blockDim.x + threadIdx.x; I < n_sets; I += stride) {
+    const int32_t sb = iset_slot[I], na = iset_slot[I + 1] - sb;
+    double tot = 0.0;
+    for (int32_t a = 0; a < na; ++a) tot += avg[sb + a];
+    for (int32_t a = 0; a < na; ++a) out[spec_slot_of[sb + a]] = tot > 0.0 ? avg[sb + a] / tot : 1.0 / (double)na;
+  }
+}
+
 static __global__ void avg_normalize_kernel(const int32_t *iset_slot, int32_t n_sets, const double *avg, double *out) {
   const int32_t stride = gridDim.x * blockDim.x;
   for (int32_t I = blockIdx.x * blockDim.x + threadIdx.x; I < n_sets; I += stride) {

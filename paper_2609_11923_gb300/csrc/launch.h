@@ -57,9 +57,20 @@ cudaError_t launch_br_level(int maxa, int lanes, int grid, cudaStream_t s, GameV
 #include "batch.cuh"
 
 namespace cfr {
+// One launch of a batched call: `count` instances from `first` of the table,
+// `cluster` CTAs each, their arrays where `mode` says (kSolo, kCluster,
+// kResident with `smem` bytes of them). push: the pushing forward (reach
+// orders other than member order). chained: the launch before in the stream
+// is the same call's and need not be complete (chain_enter).
+struct BatchLaunch {
+  int first = 0, count = 0, cluster = 1, mode = kSolo;
+  uint32_t smem = 0;
+  bool push = false, chained = false;
+};
+
 template <typename T>
-cudaError_t launch_batch_iterate(int maxa, int lanes, int threads, int cluster, bool chained, int n, cudaStream_t s,
+cudaError_t launch_batch_iterate(int maxa, int lanes, int threads, const BatchLaunch &l, cudaStream_t s,
                                  const InstDesc *table, const InstDesc &one);
-cudaError_t launch_batch_br(int maxa, int lanes, int threads, int cluster, bool chained, int n, cudaStream_t s,
+cudaError_t launch_batch_br(int maxa, int lanes, int threads, const BatchLaunch &l, cudaStream_t s,
                             const InstDesc *table, const InstDesc &one);
 }  // namespace cfr
