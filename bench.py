@@ -474,6 +474,7 @@ def run_ours(args):
     # the timed region; the game's arena is released first)
     batched = None
     arena_gb = solver.arena_bytes / 1e9
+    graph_kernels = solver.counts_now()["graph_kernels"]
     if rank == 0 and args.batched_requests > 0 and args.workload == "large_card":
         solver.close()
         del solver
@@ -481,10 +482,11 @@ def run_ours(args):
         batched = serving_leg(args.batched_requests, args.max_iters, args.batched_baseline)
     barrier()
 
-    # per depth one forward and one backward launch; in member order the
-    # deepest depth has no forward launch (no internal node below it pulls)
+    # kernels of the captured iteration (graph form); otherwise per depth one
+    # forward and one backward launch (in member order the deepest depth has
+    # no forward launch: no internal node below it pulls)
     fwd_launches = D - 1 if args.reach_order == "members" else D
-    per_iter_launches = {cfr.EXEC_GRAPH: fwd_launches + D, cfr.EXEC_LEVELS: fwd_launches + D}.get(counts["exec_form"], 0)
+    per_iter_launches = graph_kernels or {cfr.EXEC_LEVELS: fwd_launches + D}.get(counts["exec_form"], 0)
     gpu_launches = args.steps * per_iter_launches if per_iter_launches else 1
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,

@@ -86,7 +86,13 @@ typedef struct cfr_options {
    * CFR_EXEC_PERSISTENT: one kernel per cfr_iterate call with a grid-wide
    * barrier between depth levels; CFR_EXEC_AUTO picks by game size: the
    * persistent form up to 768 nodes in CFR_P32 and 350 in CFR_P64 (where
-   * it was measured faster than graph replay), the graph form above. */
+   * it was measured faster than graph replay), the graph form above.
+   * Under CFR_EXEC_AUTO with lanes_per_set, persistent_ctas, graph_iters and
+   * launch_overlap at their defaults, games whose arrays fit one CTA's shared
+   * memory (about 14,000 nodes in CFR_P32; up to 4,000 in CFR_P64) run all
+   * iterations of a call there instead. In the level and graph forms with
+   * lanes_per_set 0, the small depths near the root are one launch of one CTA
+   * that also starts the next iteration's forward pass. */
   int exec_form;
   /* Update rule (Section 3, update rules): CFR_RULE_CFR_PLUS (regret clamped
    * at zero, linear averaging w_t = t), CFR_RULE_CFR (no clamp, linear
@@ -372,25 +378,27 @@ int cfr_pin_host(cfr_handle *h, int pin);
 
 /* Batched solves (many independent games in one launch). Every handle must
  * be bound (each to its own arena) and use the same precision, with sets of
- * at most 8 actions. One CTA of `threads` threads (256 or 1024; 0 = 256)
- * runs all iterations of one instance with `lanes` lanes per information set
- * (2, 4, 8 or 32; 0 = 4); cfr_batch_iterate can instead give every instance
- * a thread-block cluster of `cluster` CTAs (2, 4 or 8) that share its work
- * and meet at the hardware cluster barrier between depths (for large
- * instances). A solve's result depends only on its own data and on
- * (threads, lanes, cluster): it is bitwise the same alone and in any mix.
+ * at most 8 actions. One CTA, or a thread-block cluster of up to 16 that
+ * share its work and meet at the hardware cluster barrier between depths,
+ * runs all iterations of one instance; the library picks the CTAs of every
+ * instance by the sizes in the batch (cfr_batch_iterate: at least `cluster`
+ * each). threads (256 or 1024; 0 = 256): small or large CTAs; lanes (2, 4, 8
+ * or 32; 0 = 4) per information set, where CFR_P32 gives sets that average 32
+ * members at a depth a whole warp. A solve's result depends only on its own
+ * data and on (threads, lanes), not on its CTAs: it is bitwise the same alone
+ * and in any mix.
  * table_dev: caller-owned device buffer of at least cfr_batch_table_bytes(n)
  * bytes (16-byte aligned) for the instance descriptors; it must stay
  * untouched until the launch completes. */
 size_t cfr_batch_table_bytes(int n);
 
 /* Runs iters[i] iterations of instance i (iters may be NULL: every
- * instance runs n_iter), asynchronously on `stream`. cluster: CTAs per
- * instance (0 or 1 = one CTA; 2, 4 or 8 = a thread-block cluster). */
+ * instance runs n_iter), asynchronously on `stream`. cluster: the CTAs that
+ * every instance gets at least (0 or 1, 2, 4 or 8). */
 int cfr_batch_iterate(cfr_handle *const *handles, int n, const int64_t *iters, int64_t n_iter, void *table_dev,
                       size_t table_bytes, int threads, int lanes, int cluster, void *stream);
 
-/* Exploitability of every instance's average strategy in one launch; out
+/* Exploitability of every instance's average strategy; out
  * (host, [4n]) receives per instance (NashConv/2, br1, br2, u). Synchronises
  * `stream`. */
 int cfr_batch_exploitability(cfr_handle *const *handles, int n, double *out, void *table_dev, size_t table_bytes,

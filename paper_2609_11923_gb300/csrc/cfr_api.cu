@@ -70,6 +70,12 @@ struct cfr_handle {
   std::vector<StreamChunk> stream_chunks;
   std::vector<int32_t> stream_c0, stream_ok;
   Buf b_set_info, b_stream_chunks;
+  // CFR_EXEC_AUTO, small games: the whole game resident in one CTA (0: not)
+  uint32_t solo_smem = 0;
+  int solo_threads = 256, solo_lanes = 8;
+  // per-level forms: depths 0 .. top_k near the root as one launch (-1: none)
+  int top_k = -1, top_lanes = 8;
+  uint32_t top_smem = 0;
   size_t plan_bytes = 0;
   char *arena = nullptr;
   bool bound = false;
@@ -88,6 +94,10 @@ struct cfr_handle {
   int64_t iteration_host = 0;  // iterations enqueued since bind/reset (bookkeeping)
   template <typename X> X *p(const Buf &b) const { return reinterpret_cast<X *>(arena + b.off); }
 };
+
+static InstDesc inst_desc(const cfr_handle *h, int64_t n_iter);
+static uint32_t resident_bytes(const cfr_handle *h, const InstDesc &d);
+static void choose_top(cfr_handle *h);
 
 static size_t align_up(size_t x) { return (x + 255) & ~size_t(255); }
 
@@ -342,6 +352,19 @@ extern "C" int cfr_compile(const cfr_game_spec *spec, const cfr_options *opt, cf
     }
   }
   plan(h);
+  choose_top(h);
+  // AUTO with default options: a game that fits one CTA's shared memory runs
+  // there for the whole call (301 nodes: 4.1 us an iteration in FP32, 11.6 in
+  // the persistent form; 4,213: 6.6, 28.8 as a graph; FP64 above about 4,000
+  // nodes is bound by one SM's FP64 pipe and runs as a graph)
+  if (h->opt.exec_form == CFR_EXEC_AUTO && lp == 0 && h->opt.persistent_ctas == 0 && h->opt.graph_iters <= 1 &&
+      h->opt.launch_overlap == CFR_OVERLAP_AUTO && h->maxa_tier <= 8 && c.D > 0 &&
+      (h->precision == CFR_P32 || c.N <= 4000)) {
+    h->solo_smem = resident_bytes(h, inst_desc(h, 0));
+    h->solo_threads = c.N <= 600 ? 256 : 1024;
+    const double mean = c.I > 0 ? tot_mem / (double)c.I : 1.0;
+    h->solo_lanes = h->precision == CFR_P32 && mean <= 4.0 ? 4 : 8;
+  }
   *out = h;
   return CFR_OK;
 }
@@ -418,6 +441,89 @@ template <typename T> static StateView<T> state_view(const cfr_handle *h) {
   s.avg = h->p<double>(h->b_avg);
   s.t = h->p<long long>(h->b_t);
   return s;
+}
+
+static InstDesc inst_desc(const cfr_handle *h, int64_t n_iter) {
+  InstDesc d;
+  memset(&d, 0, sizeof d);
+  d.g = game_view(h);
+  d.reach = h->arena + h->b_reach.off;
+  d.v = h->arena + h->b_v.off;
+  d.sigma = h->arena + h->b_sigma.off;
+  d.R = h->p<double>(h->b_R);
+  d.avg = h->p<double>(h->b_avg);
+  d.t = h->p<long long>(h->b_t);
+  d.lw = h->p<LevelWork>(h->b_levels);
+  d.reach2 = h->p<double2>(h->b_reach2);
+  d.vb = h->p<double2>(h->b_vb);
+  d.vavg = h->p<double>(h->b_vavg);
+  d.sbs = h->p<double>(h->b_sbs);
+  d.out = h->p<double>(h->b_out);
+  d.n_iter = n_iter;
+  d.D = (int32_t)h->c.D;
+  d.rule = h->rule;
+  d.n_sets = (int32_t)h->c.I;
+  d.root_vs = (int32_t)(h->c.N - 1);
+  d.order = h->order;
+  d.n_nodes = (int32_t)h->c.N;
+  d.n_int = (int32_t)h->c.n_int;
+  d.n_dec = (int32_t)h->c.n_dec;
+  d.n_slots = (int32_t)h->c.A;
+  d.n_chance = (int32_t)h->c.ch_vb.size();
+  return d;
+}
+
+// Bytes of shared memory that a solve of this game takes when it is resident
+// in one CTA, 0 if it cannot be.
+static uint32_t resident_bytes(const cfr_handle *h, const InstDesc &d) {
+  const Compiled &c = h->c;
+  if (c.int_edge.empty() || c.N > kResidentNodes) return 0;
+  for (int64_t l = 1; l < c.D; ++l)
+    if (c.level_wide[l + 1] != c.level_wide[l]) return 0;  // wide chance nodes are summed from global memory
+  const uint32_t n = resident_layout(d, h->precision == CFR_P64 ? 8u : 4u).total;
+  return n <= kResidentBytes ? std::max(n, 16u) : 0;
+}
+
+// The part of a game that the near-root kernel holds: depths 0 .. K.
+static InstDesc top_desc(const cfr_handle *h, int64_t K) {
+  const Compiled &c = h->c;
+  InstDesc d = inst_desc(h, 1);
+  d.n_sets = c.level_iset[2 * K + 2];
+  d.n_slots = c.iset_slot[d.n_sets];
+  d.n_dec = c.iset_mem[d.n_sets];
+  d.n_int = c.level_int[K + 1];
+  d.n_chance = c.level_chance[K + 1];
+  d.n_nodes = c.level_begin[K + 2] - 1;  // the children of these depths have value slots 0 .. n_nodes - 1
+  return d;
+}
+
+// Depths that go into the near-root kernel: as long as one CTA passes a depth
+// in four rounds of its groups (FP64: one, its pipe is slow) and the arrays
+// fit its shared memory. Iterations in us without, and with 1, 4 and 8 rounds:
+// random trees of depth 10 and 14 in FP32 52.5, 31.1, 27.1, 27.1 and 107.8,
+// 86.5, 84.5, 84.4; of depth 10 and 12 in FP64 104.5, 82.4, 96.8, 96.7 and
+// 149.7, 127.4, 139.8, 139.8; an endgame of 22,000 nodes in FP32 24.7, 20.8.
+// With lanes_per_set given every depth keeps its own launches, which sum in
+// that shape.
+static void choose_top(cfr_handle *h) {
+  const Compiled &c = h->c;
+  h->top_k = -1;
+  if (c.int_edge.empty() || h->maxa_tier > 8 || h->opt.lanes_per_set != 0 || c.D < 3) return;
+  const uint32_t T = h->precision == CFR_P64 ? 8u : 4u;
+  const int threads = h->precision == CFR_P64 && h->maxa_tier > 4 ? 256 : 512;
+  const int rounds = h->precision == CFR_P64 ? 1 : 4;
+  h->top_lanes = c.I > 0 && (double)c.n_dec / (double)c.I <= 4.0 ? 4 : 8;
+  for (int64_t K = 0; K + 1 < c.D && K + 1 < kBatchLevels; ++K) {
+    if (K > 0 && c.level_wide[K + 1] != c.level_wide[K]) break;  // wide chance nodes: the per-level kernel
+    const int64_t sets = c.level_iset[2 * K + 2] - c.level_iset[2 * K];
+    if (sets * h->top_lanes > rounds * threads || c.level_int[K + 1] - c.level_int[K] > 4 * threads) break;
+    const uint32_t n = resident_layout(top_desc(h, K), T).total;
+    if (n > kResidentBytes) break;
+    if (K > 0) {  // depth 0 alone saves nothing
+      h->top_k = (int)K;
+      h->top_smem = std::max(n, 16u);
+    }
+  }
 }
 
 static int grid_for(int64_t work, int per_block) {
@@ -613,6 +719,7 @@ extern "C" int cfr_bind(cfr_handle *h, void *arena, size_t bytes, void *stream) 
   if ((rc = up(h->b_set_info, h->set_info.data(), sizeof(SetInfo) * h->set_info.size()))) return rc;
   if ((rc = up(h->b_stream_chunks, h->stream_chunks.data(), sizeof(StreamChunk) * h->stream_chunks.size()))) return rc;
   if (!h->stream_chunks.empty()) CK(prepare_bwd_stream());
+  if (h->top_k >= 0) CK(h->precision == CFR_P64 ? prepare_top<double>(h->maxa_tier, h->top_lanes) : prepare_top<float>(h->maxa_tier, h->top_lanes));
   if ((rc = h->precision == CFR_P64 ? default_pull_grids<double>(h) : default_pull_grids<float>(h))) return rc;
   if (c.n_wide) CK(cudaMemsetAsync(h->arena + h->b_wide_cnt.off, 0, 4 * c.n_wide, s));
   CK(cudaMemsetAsync(h->arena + h->b_bar.off, 0, 16, s));
@@ -687,6 +794,21 @@ static bool overlap_on(const cfr_handle *h) {
   return h->opt.launch_overlap == CFR_OVERLAP_ON;
 }
 
+template <typename T>
+static int launch_top_part(cfr_handle *h, cudaStream_t s, int phase, int upd, bool pdl) {
+  const InstDesc d = top_desc(h, h->top_k);
+  CK(launch_top<T>(h->maxa_tier, h->top_lanes, h->top_smem, s, d, h->top_k, h->c.level_begin[h->top_k + 1] - 1, phase, upd,
+                   pdl));
+  return CFR_OK;
+}
+
+// Before the first iteration of a call: the forward pass of the depths that
+// the near-root kernel holds (each iteration ends with the next one's).
+template <typename T>
+static int enqueue_start(cfr_handle *h, cudaStream_t s) {
+  return h->top_k >= 0 ? launch_top_part<T>(h, s, kTopForward, 3, false) : CFR_OK;
+}
+
 // One iteration's launches. Every launch but the first of the iteration may
 // overlap its predecessor's tail (programmatic dependent launch).
 template <typename T>
@@ -698,16 +820,20 @@ static int enqueue_iteration(cfr_handle *h, cudaStream_t s, bool first_overlaps 
   bool pdl = ov && first_overlaps;
   for (int hf = 0; hf < halves; ++hf) {
     const int upd = halves == 2 ? (1 << hf) : 3;
-    for (int64_t d = 0; d < c.D; ++d) {
+    for (int64_t d = std::max(h->top_k, 0); d < c.D; ++d) {
       if (g.int_edge && d + 1 >= c.D) continue;  // member order: no launch for the deepest depth
       int rc = launch_fwd<T>(h, d, s, g, h->p<T>(h->b_sigma), h->p<vec2_t<T>>(h->b_reach), pdl);
       if (rc) return rc;
       pdl = ov;
     }
-    for (int64_t d = c.D - 1; d >= 0; --d) {
+    for (int64_t d = c.D - 1; d > h->top_k; --d) {
       int rc = launch_bwd<T>(h, (int)d, s, upd, pdl);
       if (rc) return rc;
       pdl = ov;
+    }
+    if (h->top_k >= 0) {
+      int rc = launch_top_part<T>(h, s, kTopBackward | kTopForward, upd, pdl);
+      if (rc) return rc;
     }
   }
   return CFR_OK;
@@ -826,9 +952,19 @@ static int iterate_t(cfr_handle *h, int64_t n, cudaStream_t s) {
     CK(cudaGetLastError());
     return CFR_OK;
   }
+  if (h->solo_smem > 0) {
+    BatchLaunch l;
+    l.count = 1;
+    l.mode = kResident;
+    l.smem = h->solo_smem;
+    CK(launch_batch_iterate<T>(h->maxa_tier, h->solo_lanes, h->solo_threads, l, s, nullptr, inst_desc(h, n)));
+    return CFR_OK;
+  }
   if (h->exec_form == CFR_EXEC_LEVELS) {
+    int rc = enqueue_start<T>(h, s);
+    if (rc) return rc;
     for (int64_t i = 0; i < n; ++i) {
-      int rc = enqueue_iteration<T>(h, s, i > 0);
+      rc = enqueue_iteration<T>(h, s, i > 0 || h->top_k >= 0);
       if (rc) return rc;
     }
     return CFR_OK;
@@ -853,6 +989,7 @@ static int iterate_t(cfr_handle *h, int64_t n, cudaStream_t s) {
     h->exec_form = CFR_EXEC_LEVELS;
     return iterate_t<T>(h, n, s);
   }
+  if (int rc = enqueue_start<T>(h, s)) return rc;
   for (int64_t i = 0; i < nk; ++i) CK(cudaGraphLaunch(h->gexec_k, s));
   for (int64_t i = 0; i < n1; ++i) CK(cudaGraphLaunch(h->gexec, s));
   return CFR_OK;
@@ -1354,17 +1491,18 @@ extern "C" int cfr_launch_floor(cfr_handle *h, int64_t n, void *stream, double *
   if (c.D == 0) return CFR_OK;
   cudaStream_t s = (cudaStream_t)stream;
   std::vector<int> grids;
-  for (int64_t d = 0; d < c.D; ++d) {
+  for (int64_t d = std::max(h->top_k, 0); d < c.D; ++d) {
     const LevelWork &w = h->levels[d];
     if (c.int_edge.empty()) grids.push_back(grid_for((w.ie - w.ib + 3) / 4, kThreads) + (w.wc1 - w.wc0));
     else if (d + 1 < c.D)  // member order: the launch of depth d pulls depth d + 1
       grids.push_back(h->pull_grid[d] > 0 ? h->pull_grid[d] : pull_need(h, d));
   }
-  for (int64_t d = c.D - 1; d >= 0; --d) {
+  for (int64_t d = c.D - 1; d > h->top_k; --d) {
     int nb_ch, nb_wide, nb_is;
     bwd_blocks(h, (int)d, &nb_ch, &nb_wide, &nb_is);
     grids.push_back(std::max(1, nb_ch + nb_wide + nb_is));
   }
+  if (h->top_k >= 0) grids.push_back(1);
   if (!h->cap_stream) CK(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t ge = nullptr;
@@ -1449,8 +1587,9 @@ extern "C" int cfr_autotune(cfr_handle *h, int reps, void *stream) {
   auto run_iter = [&]() -> int {
     return h->precision == CFR_P64 ? enqueue_iteration<double>(h, s) : enqueue_iteration<float>(h, s);
   };
-  rc = run_iter();  // realistic reach and values for the trials
-  for (int64_t d = c.D - 1; d >= 0 && rc == CFR_OK; --d) {
+  rc = h->precision == CFR_P64 ? enqueue_start<double>(h, s) : enqueue_start<float>(h, s);
+  if (rc == CFR_OK) rc = run_iter();  // realistic reach and values for the trials
+  for (int64_t d = c.D - 1; d > h->top_k && rc == CFR_OK; --d) {  // the near-root kernel has one shape
     int best = h->level_lanes[d];
     float best_ms = 1e30f;
     std::vector<int> cd = cand;
@@ -1504,47 +1643,6 @@ extern "C" int cfr_autotune(cfr_handle *h, int reps, void *stream) {
 }
 
 // ----------------------------------------------------------- batched solves
-static InstDesc inst_desc(const cfr_handle *h, int64_t n_iter) {
-  InstDesc d;
-  memset(&d, 0, sizeof d);
-  d.g = game_view(h);
-  d.reach = h->arena + h->b_reach.off;
-  d.v = h->arena + h->b_v.off;
-  d.sigma = h->arena + h->b_sigma.off;
-  d.R = h->p<double>(h->b_R);
-  d.avg = h->p<double>(h->b_avg);
-  d.t = h->p<long long>(h->b_t);
-  d.lw = h->p<LevelWork>(h->b_levels);
-  d.reach2 = h->p<double2>(h->b_reach2);
-  d.vb = h->p<double2>(h->b_vb);
-  d.vavg = h->p<double>(h->b_vavg);
-  d.sbs = h->p<double>(h->b_sbs);
-  d.out = h->p<double>(h->b_out);
-  d.n_iter = n_iter;
-  d.D = (int32_t)h->c.D;
-  d.rule = h->rule;
-  d.n_sets = (int32_t)h->c.I;
-  d.root_vs = (int32_t)(h->c.N - 1);
-  d.order = h->order;
-  d.n_nodes = (int32_t)h->c.N;
-  d.n_int = (int32_t)h->c.n_int;
-  d.n_dec = (int32_t)h->c.n_dec;
-  d.n_slots = (int32_t)h->c.A;
-  d.n_chance = (int32_t)h->c.ch_vb.size();
-  return d;
-}
-
-// Bytes of shared memory that a solve of this game takes when it is resident
-// in one CTA, 0 if it cannot be.
-static uint32_t resident_bytes(const cfr_handle *h, const InstDesc &d) {
-  const Compiled &c = h->c;
-  if (c.int_edge.empty() || c.N > kResidentNodes) return 0;
-  for (int64_t l = 1; l < c.D; ++l)
-    if (c.level_wide[l + 1] != c.level_wide[l]) return 0;  // wide chance nodes are summed from global memory
-  const uint32_t n = resident_layout(d, h->precision == CFR_P64 ? 8u : 4u).total;
-  return n <= kResidentBytes ? std::max(n, 16u) : 0;
-}
-
 // A batched call's plan: the instances' descriptors ordered by cluster size
 // (largest first, and by load within a size), and one launch for each size.
 struct BatchPlan {

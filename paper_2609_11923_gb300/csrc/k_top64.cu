@@ -1,0 +1,6 @@
+// Near-root kernel instances, FP64 (see top.cuh).
+#include "k_top.cuh"
+namespace cfr {
+template cudaError_t prepare_top<double>(int, int);
+template cudaError_t launch_top<double>(int, int, uint32_t, cudaStream_t, const InstDesc &, int, int, int, int, bool);
+}

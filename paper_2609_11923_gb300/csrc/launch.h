@@ -55,6 +55,7 @@ cudaError_t launch_br_level(int maxa, int lanes, int grid, cudaStream_t s, GameV
 }  // namespace cfr
 
 #include "batch.cuh"
+#include "top.cuh"
 
 namespace cfr {
 // One launch of a batched call: `count` instances from `first` of the table,
@@ -73,4 +74,11 @@ cudaError_t launch_batch_iterate(int maxa, int lanes, int threads, const BatchLa
                                  const InstDesc *table, const InstDesc &one);
 cudaError_t launch_batch_br(int maxa, int lanes, int threads, const BatchLaunch &l, cudaStream_t s,
                             const InstDesc *table, const InstDesc &one);
+
+// The depths near the root as one launch (top_kernel). smem: the bytes of its
+// arrays (prepare_top first, outside any capture).
+template <typename T> cudaError_t prepare_top(int maxa, int lanes);
+template <typename T>
+cudaError_t launch_top(int maxa, int lanes, uint32_t smem, cudaStream_t s, const InstDesc &in, int K, int v_new, int phase,
+                       int upd, bool pdl);
 }  // namespace cfr
