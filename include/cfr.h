@@ -147,9 +147,9 @@ typedef struct cfr_options {
    * but its launch and block scheduling overlap the previous kernel's tail
    * (and the FP32 streaming backward copies its first inputs before that
    * wait). CFR_OVERLAP_OFF: plain stream order. CFR_OVERLAP_AUTO (default):
-   * on in CFR_P32, off in CFR_P64 (measured on one GB300: the FP64 card
-   * game takes 8.5 ms per iteration without it and 10.4 ms with it; FP32
-   * gains 1-2%). Results are bitwise the same. */
+   * on in CFR_P32, and in CFR_P64 up to 100,000 nodes (measured on one
+   * GB300: the FP64 card game takes 8.5 ms per iteration without it and
+   * 10.4 ms with it). Results are bitwise the same. */
   int launch_overlap;
   /* Graph form: iterations recorded into one CUDA graph (the paper's
    * alternative-execution table records 1, 10 and 100); 0 or 1 = one.

@@ -571,13 +571,13 @@ static int default_pull_grids(cfr_handle *h) {
 // nodes take the form that writes those children warp-wide.
 template <typename T>
 static int launch_fwd(const cfr_handle *h, int64_t d, cudaStream_t s, const GameView &g, const T *sigma,
-                      vec2_t<T> *reach, bool pdl = false) {
+                      vec2_t<T> *reach, bool pdl = false, bool after_fwd = false) {
   const LevelWork &w = h->levels[d];
   if (g.int_edge) {  // member order: the next depth's internal nodes pull their reach
     if (d + 1 >= h->c.D) return CFR_OK;
     const LevelWork &n = h->levels[d + 1];
     const int nb = h->pull_grid[d] > 0 ? h->pull_grid[d] : pull_need(h, d);
-    CK(launch_k(fwd_pull_kernel<T>, nb, kThreads, 0, s, pdl, g, sigma, reach, n.ib, n.ie));
+    CK(launch_k(fwd_pull_kernel<T>, nb, kThreads, 0, s, pdl, g, sigma, reach, n.ib, n.ie, pdl && after_fwd ? 1 : 0));
     return CFR_OK;
   }
   const int nb = grid_for((w.ie - w.ib + 3) / 4, kThreads);
@@ -782,15 +782,18 @@ static int launch_bwd(cfr_handle *h, int d, cudaStream_t s, int upd = 3, bool pd
   }
   // at least one block: the depth-0 launch also advances t
   CK(launch_bwd_level<T>(h->maxa_tier, lanes, std::max(1, nb_ch + nb_wide + nb_is), s, game_view(h), state_view<T>(h),
-                         w, nb_ch, h->rule, upd, (d == 0 && (upd & 2)) ? 1 : 0, pdl));
+                         w, nb_ch, h->rule, upd, (d == 0 && (upd & 2)) ? 1 : 0, pdl,
+                         pdl && h->c.D > 1));  // (with one depth the launch before may be this one's own)
   return CFR_OK;
 }
 
 // Programmatic dependent launch between the per-level kernels: on by
-// choice, or by default in FP32 only (in FP64 the overlapped graph ran the
-// card game 22% slower on one GB300, 10.4 against 8.5 ms per iteration).
+// choice, or by default in FP32 and in FP64 up to 100,000 nodes, where the
+// launches' latency counts (iterations in us with and without, FP64: random
+// trees of 33k, 300k and 2.8M nodes 76 / 82, 130 / 125, 352 / 340; a card game
+// of 81k 68 / 78; of 264M 10,400 / 8,500).
 static bool overlap_on(const cfr_handle *h) {
-  if (h->opt.launch_overlap == CFR_OVERLAP_AUTO) return h->precision == CFR_P32;
+  if (h->opt.launch_overlap == CFR_OVERLAP_AUTO) return h->precision == CFR_P32 || h->c.N <= 100000;
   return h->opt.launch_overlap == CFR_OVERLAP_ON;
 }
 
@@ -822,7 +825,8 @@ static int enqueue_iteration(cfr_handle *h, cudaStream_t s, bool first_overlaps 
     const int upd = halves == 2 ? (1 << hf) : 3;
     for (int64_t d = std::max(h->top_k, 0); d < c.D; ++d) {
       if (g.int_edge && d + 1 >= c.D) continue;  // member order: no launch for the deepest depth
-      int rc = launch_fwd<T>(h, d, s, g, h->p<T>(h->b_sigma), h->p<vec2_t<T>>(h->b_reach), pdl);
+      int rc = launch_fwd<T>(h, d, s, g, h->p<T>(h->b_sigma), h->p<vec2_t<T>>(h->b_reach), pdl,
+                             d > std::max(h->top_k, 0));
       if (rc) return rc;
       pdl = ov;
     }
@@ -1091,7 +1095,7 @@ extern "C" int cfr_exploitability(cfr_handle *h, double *out_expl, double *out_b
                                                                        h->p<double>(h->b_avg), h->p<double>(h->b_sbs));
   CK(cudaGetLastError());
   for (int64_t d = 0; d < c.D; ++d) {
-    int rc = launch_fwd<double>(h, d, s, g, h->p<double>(h->b_sbs), h->p<double2>(h->b_reach2), d > 0);
+    int rc = launch_fwd<double>(h, d, s, g, h->p<double>(h->b_sbs), h->p<double2>(h->b_reach2), d > 0, d > 0);
     if (rc) return rc;
   }
   for (int64_t d = c.D - 1; d >= 0; --d) {
