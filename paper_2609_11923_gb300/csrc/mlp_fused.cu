@@ -46,7 +46,9 @@ constexpr int kBlkK = 64;                     // contraction elements of a block
 constexpr uint32_t kWBlk = 256 * 128;         // bytes of a block of 256 rows
 constexpr uint32_t kABlk = kTile * 128;       // bytes of a block of a tile's rows
 constexpr uint32_t kOBlk = 16 * 128;          // bytes of a block of the output layer (8 logits and 8 rows of zeros)
-constexpr int kRing = 4;                      // weight blocks in flight
+// Tiles of a CTA in flight and weight blocks in flight (64 KB of activations a
+// tile, 32 KB a block).
+template <int PIPES> constexpr int kRing = PIPES == 1 ? 4 : 2;
 constexpr int kEpi = 256;                     // epilogue threads: 8 warps
 constexpr int kThreads = kEpi + 64;           // and a loading and an issuing warp
 constexpr int kStagesPredict = 4, kStagesTrain = 7;
@@ -190,39 +192,49 @@ template <bool TRAIN> struct Stage {
 };
 
 struct RowSmem {  // after the operand blocks
-  uint64_t full[kRing], empty[kRing], acc, act;
+  uint64_t full[4], empty[4], acc[2], act[2];
   uint32_t tmem;
   int stop;
   float bias[4][kH];
   float col[4][kH];  // column sums of the tile's four 32-row parts
 };
 
-// What bounds it: at 200,000 rows the tensor cores' 74 GFLOP and the epilogues
-// between dependent layers, which one tile a CTA does not overlap; the rows'
+// What bounds it: at 200,000 rows the tensor cores' 74 GFLOP (40 us) and the
+// epilogues between dependent layers, which one tile a CTA does not overlap; the rows'
 // features are the only traffic to speak of (160 MB; the layers one after
 // another with FP32 activations moved ten times that). 200,000 rows: 2,781 us
-// as one mma.sync product a layer, 166 here. A training step of 4,096 rows:
-// 2,500 us as 30 launches, 159 here with the host's share.
-template <bool TRAIN>
+// as one mma.sync product a layer, 166 here with one tile a CTA, 128 with two.
+// A training step of 4,096 rows: 2,500 us as 30 launches, 159 here with the
+// host's share.
+//
+// PIPES = 2 (inference with more tiles than SMs): two tiles a CTA in turn, the
+// epilogue of one under the products of the other. Each has its own operand
+// blocks, accumulators and four epilogue warps; every layer's weights are
+// loaded once for each.
+template <bool TRAIN, int PIPES>
 __global__ void __launch_bounds__(kThreads, 1) mlp_rows_kernel(const RowArgs a) {
+  static_assert(!TRAIN || PIPES == 1, "a training tile takes all epilogue warps");
   extern __shared__ __align__(1024) unsigned char s_dyn[];
   using S = Stage<TRAIN>;
-  unsigned char *s_act = s_dyn, *s_ring = s_dyn + 4 * kABlk;
-  RowSmem &sm = *reinterpret_cast<RowSmem *>(s_ring + kRing * kWBlk);
+  constexpr int R = kRing<PIPES>, PT = kEpi / PIPES;  // ring blocks, epilogue threads of a tile
+  unsigned char *s_ring = s_dyn + PIPES * 4 * kABlk;
+  RowSmem &sm = *reinterpret_cast<RowSmem *>(s_ring + R * kWBlk);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
-    for (int i = 0; i < kRing; ++i) {
+    for (int i = 0; i < R; ++i) {
       mbar_init(smem_u32(&sm.full[i]), 1);
       mbar_init(smem_u32(&sm.empty[i]), 1);
     }
-    mbar_init(smem_u32(&sm.acc), 1);
-    mbar_init(smem_u32(&sm.act), kEpi);
+    for (int p = 0; p < PIPES; ++p) {
+      mbar_init(smem_u32(&sm.acc[p]), 1);
+      mbar_init(smem_u32(&sm.act[p]), PT);
+    }
     sm.stop = (smem_u32(s_dyn) & 1023u) != 0u;  // the swizzle needs 1,024-byte aligned blocks
     if (sm.stop) atomicExch(a.err, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_smem();
   }
-  if (warp == 8) tmem_alloc(smem_u32(&sm.tmem), 256);
+  if (warp == 8) tmem_alloc(smem_u32(&sm.tmem), 256 * PIPES);
   for (int i = tid; i < 4 * kH; i += kThreads) {
     const int l = i / kH, c = i % kH;
     sm.bias[l][c] = l < 3 || c < kOut ? a.b[l][c] : 0.f;
@@ -240,49 +252,55 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_rows_kernel(const RowArgs a) 
       if (lane == 0) {
         int n = 0;  // ring entries issued
         bool ok = true;
-        for (int t = blockIdx.x; t < a.tiles && ok; t += gridDim.x)
-          for (int s = 0; s < S::kCount && ok; ++s)
+        for (int t = blockIdx.x; t < a.tiles && ok; t += PIPES * gridDim.x)
+          for (int sp = 0; sp < S::kCount * PIPES && ok; ++sp) {
+            const int s = sp / PIPES, p = sp % PIPES;
+            if (t + p * (int)gridDim.x >= a.tiles) continue;
             for (int e = 0; e < S::entries(s, a.in_blocks); ++e, ++n) {
-              const int slot = n % kRing;
-              if (n >= kRing && !mbar_wait(smem_u32(&sm.empty[slot]), (uint32_t)((n / kRing - 1) & 1))) { ok = false; break; }
+              const int slot = n % R;
+              if (n >= R && !mbar_wait(smem_u32(&sm.empty[slot]), (uint32_t)((n / R - 1) & 1))) { ok = false; break; }
               if (*stop) { ok = false; break; }
               const uint32_t bytes = S::bytes(s);
               mbar_expect_tx(smem_u32(&sm.full[slot]), bytes);
               bulk_g2s(smem_u32(s_ring + slot * kWBlk), a.img + S::offset(im, s, e), bytes, smem_u32(&sm.full[slot]));
             }
+          }
         if (!ok) {
           *stop = 1;
           atomicExch(a.err, 1);
         }
-        for (int i = n > kRing ? n - kRing : 0; i < n; ++i)  // no copy is in flight when the CTA leaves
-          mbar_wait(smem_u32(&sm.full[i % kRing]), (uint32_t)((i / kRing) & 1));
+        for (int i = n > R ? n - R : 0; i < n; ++i)  // no copy is in flight when the CTA leaves
+          mbar_wait(smem_u32(&sm.full[i % R]), (uint32_t)((i / R) & 1));
       }
     } else if (warp == 9) {
       // the issuing thread
       if (lane == 0) {
-        int n = 0, turn = 0;
+        int n = 0, turn[2] = {0, 0};
         bool ok = true;
-        for (int t = blockIdx.x; t < a.tiles && ok; t += gridDim.x)
-          for (int s = 0; s < S::kCount && ok; ++s, ++turn) {
-            if (!mbar_wait(smem_u32(&sm.act), (uint32_t)(turn & 1)) || *stop) { ok = false; break; }
+        for (int t = blockIdx.x; t < a.tiles && ok; t += PIPES * gridDim.x)
+          for (int sp = 0; sp < S::kCount * PIPES && ok; ++sp) {
+            const int s = sp / PIPES, p = sp % PIPES;
+            if (t + p * (int)gridDim.x >= a.tiles) continue;
+            if (!mbar_wait(smem_u32(&sm.act[p]), (uint32_t)(turn[p] & 1)) || *stop) { ok = false; break; }
+            ++turn[p];
             fence_after();
             const uint32_t idesc = s == 3 ? op_idesc(kTile, 16) : op_idesc(kTile, kH);
             for (int e = 0; e < S::entries(s, a.in_blocks); ++e, ++n) {
-              const int slot = n % kRing;
-              if (!mbar_wait(smem_u32(&sm.full[slot]), (uint32_t)((n / kRing) & 1)) || *stop) { ok = false; break; }
+              const int slot = n % R;
+              if (!mbar_wait(smem_u32(&sm.full[slot]), (uint32_t)((n / R) & 1)) || *stop) { ok = false; break; }
               fence_after();
-              const uint32_t wb = smem_u32(s_ring + slot * kWBlk), ab = smem_u32(s_act);
+              const uint32_t wb = smem_u32(s_ring + slot * kWBlk), ab = smem_u32(s_dyn + p * 4 * kABlk);
               // 16 elements of the contraction (32 bytes of a row) an instruction
               const int steps = s == 3 ? 16 : s == 4 ? 1 : 4;
               for (int k = 0; k < steps; ++k) {
                 const uint32_t blk = s == 3 ? (uint32_t)(k >> 2) : (uint32_t)e, in = (uint32_t)(k & 3) * 32u;
                 const uint64_t da = op_desc(ab + blk * kABlk + in);
                 const uint64_t db = op_desc(wb + (s == 3 ? blk * kOBlk : 0u) + in);
-                mma_f16(tmem, da, db, idesc, (e | k) ? 1u : 0u);
+                mma_f16(tmem + (uint32_t)p * 256u, da, db, idesc, (e | k) ? 1u : 0u);
               }
               mma_commit(smem_u32(&sm.empty[slot]));
             }
-            if (ok) mma_commit(smem_u32(&sm.acc));
+            if (ok) mma_commit(smem_u32(&sm.acc[p]));
           }
         if (!ok) {
           *stop = 1;
@@ -290,12 +308,15 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_rows_kernel(const RowArgs a) 
         }
       }
     } else {
-      // epilogue: thread = row of the tile, the warpgroups share the columns
-      const int wg = warp >> 2, part = warp & 3, row = part * 32 + lane;
-      const uint32_t acc = tmem + ((uint32_t)(part * 32) << 16);
+      // epilogue: thread = row of the tile; with one tile the warpgroups share
+      // the columns, with two each has its own tile
+      const int p = PIPES == 2 ? warp >> 2 : 0, wg = PIPES == 2 ? 0 : warp >> 2;
+      const int part = warp & 3, row = part * 32 + lane, ptid = tid % PT;
+      unsigned char *s_act = s_dyn + p * 4 * kABlk;
+      const uint32_t acc = tmem + (uint32_t)p * 256u + ((uint32_t)(part * 32) << 16);
       const uint32_t in_pad = (uint32_t)a.in_blocks * kBlkK;
       int turn = 0;
-      for (int t = blockIdx.x; t < a.tiles; t += gridDim.x) {
+      for (int t = blockIdx.x + p * gridDim.x; t < a.tiles; t += PIPES * gridDim.x) {
         const int r0 = t * kTile;
         unsigned char *grp = TRAIN ? a.groups + (size_t)(2 * t + (row >> 6)) * kGroup : nullptr;
         const uint32_t gk = (uint32_t)(row & 63);  // this row's place in its group's contraction
@@ -303,18 +324,18 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_rows_kernel(const RowArgs a) 
         // columns past the features are zeros)
         if (a.vec) {
           const int nv = (int)in_pad / 4, items = kTile * nv;
-          for (int i0 = tid; i0 < items; i0 += 8 * kEpi) {
+          for (int i0 = ptid; i0 < items; i0 += 8 * PT) {
             float4 x[8];
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
-              const int i = i0 + u * kEpi, r = i / nv, c = i % nv * 4;
+              const int i = i0 + u * PT, r = i / nv, c = i % nv * 4;
               x[u] = make_float4(0.f, 0.f, 0.f, 0.f);
               if (i < items && r0 + r < a.B && c < a.in_dim)
                 x[u] = __ldg(reinterpret_cast<const float4 *>(a.X + (size_t)(r0 + r) * a.in_dim + c));
             }
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
-              const int i = i0 + u * kEpi, r = i / nv, c = i % nv * 4;
+              const int i = i0 + u * PT, r = i / nv, c = i % nv * 4;
               if (i < items) {
                 uint2 w;
                 w.x = pack2(x[u].x, x[u].y);
@@ -325,7 +346,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_rows_kernel(const RowArgs a) 
           }
         } else {
           const int items = kTile * (int)in_pad;
-          for (int i = tid; i < items; i += kEpi) {
+          for (int i = ptid; i < items; i += PT) {
             const int r = i / (int)in_pad, c = i % (int)in_pad;
             const float x = r0 + r < a.B && c < a.in_dim ? a.X[(size_t)(r0 + r) * a.in_dim + c] : 0.f;
             *reinterpret_cast<__nv_bfloat16 *>(s_act + (c / kBlkK) * kABlk + blk_off((uint32_t)r, (uint32_t)(c % kBlkK))) =
@@ -333,7 +354,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_rows_kernel(const RowArgs a) 
           }
         }
         fence_smem();
-        mbar_arrive(smem_u32(&sm.act));
+        mbar_arrive(smem_u32(&sm.act[p]));
         if constexpr (TRAIN) {  // the features' operand block: every epilogue thread has to have written its part
           asm volatile("bar.sync 1, 256;" ::: "memory");
           for (uint32_t c = (uint32_t)wg * 8u; c < in_pad; c += 16u) {  // 8 columns at a time
@@ -347,7 +368,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_rows_kernel(const RowArgs a) 
         uint32_t live[3][4];  // which of this thread's hidden values are positive
 #pragma unroll
         for (int s = 0; s < S::kCount; ++s) {
-          wait_or_go_on(smem_u32(&sm.acc), (uint32_t)(turn & 1), stop, a.err);
+          wait_or_go_on(smem_u32(&sm.acc[p]), (uint32_t)(turn & 1), stop, a.err);
           ++turn;
           fence_after();
           if (s == 3) {
@@ -415,7 +436,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_rows_kernel(const RowArgs a) 
             }
           } else {
             const int l = s < 3 ? s : 6 - s;  // the hidden layer this stage writes (its values, or their gradient)
-            for (int q = 0; q < 4; ++q) {
+            for (int q = 0; q < 4 * PIPES; ++q) {
               const uint32_t c0 = (uint32_t)(wg * 128 + q * 32);
               float x[32];
               tmem_ld32(acc + c0, x);
@@ -473,7 +494,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_rows_kernel(const RowArgs a) 
           fence_before();
           if (s != S::kCount - 1) {
             fence_smem();
-            mbar_arrive(smem_u32(&sm.act));
+            mbar_arrive(smem_u32(&sm.act[p]));
           }
         }
       }
@@ -483,7 +504,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_rows_kernel(const RowArgs a) 
   fence_before();
   __syncthreads();
   fence_after();
-  if (warp == 8) tmem_free(tmem, 256);
+  if (warp == 8) tmem_free(tmem, 256 * PIPES);
 }
 
 // ------------------------------------------------------- weight gradients
@@ -729,7 +750,7 @@ static Work work_of(int in_dim, int rows) {
   return w;
 }
 
-constexpr size_t kRowSmem = 4 * (size_t)kABlk + kRing * (size_t)kWBlk + sizeof(RowSmem);
+template <int PIPES> constexpr size_t kRowSmem = PIPES * 4 * (size_t)kABlk + kRing<PIPES> * (size_t)kWBlk + sizeof(RowSmem);
 constexpr size_t kGradSmem = kGradRing * (size_t)kGradSlot + sizeof(GradSmem);
 
 static thread_local std::string g_err;
@@ -790,8 +811,12 @@ int mlp_net_predict(const float *X, int in_dim, int rows, const void *img, const
   if (!prob || (reinterpret_cast<uintptr_t>(prob) & 15u)) return fail(-1, "mlp_net_predict: prob must be 16-byte aligned");
   if ((rc = sm_count(&sms))) return rc;
   a.prob = prob;
-  NET_CK(cudaFuncSetAttribute(mlp_rows_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowSmem));
-  mlp_rows_kernel<false><<<a.tiles < sms ? a.tiles : sms, mlpf::kThreads, kRowSmem, (cudaStream_t)stream>>>(a);
+  // more tiles than SMs: two in turn on each
+  const bool two = a.tiles > sms;
+  auto kern = two ? mlp_rows_kernel<false, 2> : mlp_rows_kernel<false, 1>;
+  const size_t smem = two ? kRowSmem<2> : kRowSmem<1>;
+  NET_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  kern<<<a.tiles < sms ? a.tiles : sms, mlpf::kThreads, smem, (cudaStream_t)stream>>>(a);
   NET_CK(cudaGetLastError());
   return 0;
 }
@@ -814,10 +839,10 @@ int mlp_net_grad(const float *X, int in_dim, int rows, const void *img, const fl
   a.groups = ws + w.groups;
   a.colsum = (float *)(ws + w.colsum);
   *loss = (float *)(ws + w.loss);
-  NET_CK(cudaFuncSetAttribute(mlp_rows_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowSmem));
+  NET_CK(cudaFuncSetAttribute(mlp_rows_kernel<true, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowSmem<1>));
   NET_CK(cudaFuncSetAttribute(mlp_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGradSmem));
   NET_CK(cudaMemsetAsync(ws + w.loss, 0, 8, s));
-  mlp_rows_kernel<true><<<a.tiles < sms ? a.tiles : sms, mlpf::kThreads, kRowSmem, s>>>(a);
+  mlp_rows_kernel<true, 1><<<a.tiles < sms ? a.tiles : sms, mlpf::kThreads, kRowSmem<1>, s>>>(a);
   NET_CK(cudaGetLastError());
   float *part = (float *)(ws + w.part);
   mlp_wgrad_kernel<<<dim3((unsigned)w.splits, 4), mlpf::kThreads, kGradSmem, s>>>(a.groups, w.n_groups, w.per_split, in_dim,
