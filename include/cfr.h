@@ -383,8 +383,7 @@ int cfr_pin_host(cfr_handle *h, int pin);
  * runs all iterations of one instance; the library picks the CTAs of every
  * instance by the sizes in the batch (cfr_batch_iterate: at least `cluster`
  * each). threads (256 or 1024; 0 = 256): small or large CTAs; lanes (2, 4, 8
- * or 32; 0 = 4) per information set, where CFR_P32 gives sets that average 32
- * members at a depth a whole warp. A solve's result depends only on its own
+ * or 32; 0 = 4) per information set: the shape of its sums. A solve's result depends only on its own
  * data and on (threads, lanes), not on its CTAs: it is bitwise the same alone
  * and in any mix.
  * table_dev: caller-owned device buffer of at least cfr_batch_table_bytes(n)

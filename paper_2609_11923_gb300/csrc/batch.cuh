@@ -282,8 +282,16 @@ __device__ __forceinline__ void group_pull(const GroupView<T> &g, int32_t q, int
   }
 }
 
-// FP32: sets averaging this many members at a depth take a warp each (eight
-// lanes walk them in many dependent steps, and there are few of them).
+// The regret terms are rounded before they are added (no fused multiply-add),
+// in every form of the sum below.
+__device__ __forceinline__ float times(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float plus(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double times(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double plus(double a, double b) { return __dadd_rn(a, b); }
+
+// FP32: sets averaging this many members at a depth take a warp each: eight
+// lanes walk them in many dependent steps, and there are few of them. The
+// sums are those of eight lanes, bit for bit (group_set_long).
 constexpr int kLongSet = 32;
 
 // One set by the LANES lanes of a group: its members' values, and the set's
@@ -350,7 +358,7 @@ __device__ __forceinline__ void group_set(const GroupView<T> &g, int32_t I, bool
       } else {
 #pragma unroll
         for (int a = 0; a < MAXA; ++a)
-          if (a < na) racc[a] += f * (vc[u][a] - vh);  // 0 for lanes without a member
+          if (a < na) racc[a] = plus(racc[a], times(f, vc[u][a] - vh));  // 0 for lanes without a member
         spw += pw;
       }
     }
@@ -374,6 +382,71 @@ __device__ __forceinline__ void group_set(const GroupView<T> &g, int32_t I, bool
         if (lane / STEP * PER + i < na) g.def_r[sb + lane / STEP * PER + i] = racc[i];
     }
   }
+}
+
+// One long set by a warp with the sums of group_set<.., 8, ..>: lane l of
+// eight adds members l, l + 8, l + 16, ... in turn. The warp's lanes compute 32
+// members' terms at once, then every lane adds the four of its column (its
+// lane modulo 8) in that order. FP32.
+template <int MAXA, int MODE>
+__device__ __forceinline__ void group_set_long(const GroupView<float> &g, int32_t I, bool p2, int upd) {
+  constexpr bool C = MODE == kCluster;
+  constexpr int U = 2;  // members of a lane in flight
+  const int lane = threadIdx.x & 31, col = lane & 7;
+  const int32_t sb = ldk<MODE>(g.iset_slot + I), se = ldk<MODE>(g.iset_slot + I + 1);
+  const int32_t m0 = ldk<MODE>(g.iset_mem + I), m1 = ldk<MODE>(g.iset_mem + I + 1);
+  const int32_t vb = ldk<MODE>(g.iset_vb + I);
+  const int2 rk = ldk<MODE>(g.iset_rank + I);
+  const int32_t na = se - sb, M = m1 - m0;
+  float sig[MAXA], racc[MAXA], spw = 0.f;
+#pragma unroll
+  for (int a = 0; a < MAXA; ++a) {
+    sig[a] = a < na ? ldm<C>(g.sigma + sb + a) : 0.f;
+    racc[a] = 0.f;
+  }
+  for (int32_t k0 = 0; k0 < M; k0 += U * 32) {
+    int32_t h[U];
+    float2 r[U];
+    float vc[U][MAXA];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int32_t k = k0 + u * 32 + lane;
+      const bool in = k < M;
+      h[u] = in ? ldk<MODE>(g.mem_vs + m0 + k) : -1;
+      r[u] = make_float2(0.f, 0.f);
+      if (in) r[u] = ldm<C>(g.reach + rk.x + k * rk.y);
+      const float *v = g.v + vb + k;
+#pragma unroll
+      for (int a = 0; a < MAXA; ++a) vc[u][a] = in && a < na ? ldm<C>(v + a * M) : 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (k0 + u * 32 >= M) break;
+      float vh = 0.f;
+#pragma unroll
+      for (int a = 0; a < MAXA; ++a)
+        if (a < na) vh = vh + sig[a] * vc[u][a];
+      if (h[u] >= 0) g.v[h[u]] = vh;
+      const float po = p2 ? r[u].x : r[u].y, pw = p2 ? r[u].y : r[u].x;
+      const float f = (p2 ? -1.f : 1.f) * po;
+#pragma unroll
+      for (int a = 0; a < MAXA; ++a) {
+        if (a < na) {  // the same for the whole warp
+          const float d = times(f, vc[u][a] - vh);
+#pragma unroll
+          for (int c = 0; c < 4; ++c) racc[a] = plus(racc[a], __shfl_sync(0xffffffffu, d, c * 8 + col));
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < 4; ++c) spw = plus(spw, __shfl_sync(0xffffffffu, pw, c * 8 + col));
+    }
+  }
+  if (!(upd & (p2 ? 2 : 1))) return;
+  spw = group_sum_butterfly<8>(spw, 0xffffffffu);
+  group_sum_scatter<8, MAXA>(racc, col, 0xffffffffu);
+  if (lane == 0) g.def_m[sb] = spw;
+  constexpr int STEP = 8 / MAXA;
+  if (lane < 8 && lane % STEP == 0 && lane / STEP < na) g.def_r[sb + lane / STEP] = racc[0];
 }
 
 // The slot updates of set I from its totals, by MAXA lanes, one for each slot:
@@ -502,7 +575,7 @@ __global__ void __launch_bounds__(NT, 1) batch_iterate_kernel(const InstDesc *ta
   const int n_sets = in.n_sets;
   if (tid < 64) s_long[tid] = 0;
   __syncthreads();
-  if (D <= 64 && tid < D) {  // a property of the game alone: the sums' shape does not depend on the batch
+  if (D <= 64 && tid < D) {
     const int n = lw[tid].is1 - lw[tid].is0;
     if (n > 0) s_long[tid] = in.g.iset_mem[lw[tid].is1] - in.g.iset_mem[lw[tid].is0] >= kLongSet * n;
   }
@@ -538,10 +611,13 @@ __global__ void __launch_bounds__(NT, 1) batch_iterate_kernel(const InstDesc *ta
               for (int32_t i = w.wd0; i < w.wd1; ++i) cta_bwd_wide<T, NT, CLUSTERED>(in.g, g.v, i, sm);
           }
         }
-        if (sizeof(T) == 4 && LANES < 32 && s_long[d & 63] != 0) {  // a warp for every set
-          for (int32_t I = is0 + ct / 32; I < is1; I += all / 32)
-            group_set<T, MAXA, 32, MODE>(g, I, I >= is2, tid & 31, 0xffffffffu, upd, rows);
-        } else {
+        bool by_warp = false;
+        if constexpr (sizeof(T) == 4 && LANES == 8) {
+          by_warp = s_long[d & 63] != 0;
+          if (by_warp)
+            for (int32_t I = is0 + ct / 32; I < is1; I += all / 32) group_set_long<MAXA, MODE>(g, I, I >= is2, upd);
+        }
+        if (!by_warp) {
           for (int32_t I = is0 + gid; I < is1; I += ngroups)
             group_set<T, MAXA, LANES, MODE>(g, I, I >= is2, lane, mask, upd, rows);
         }
@@ -631,7 +707,7 @@ __global__ void __launch_bounds__(NT) batch_iterate_push_kernel(const InstDesc *
 // average, forward reach under it, then both best responses by depth (the
 // arithmetic of br_level_kernel). CTAs and clusters as batch_iterate_kernel.
 template <int MAXA, int LANES, int THREADS, bool CLUSTERED>
-__global__ void __launch_bounds__(THREADS) batch_br_kernel(const InstDesc *table, const __grid_constant__ InstDesc one,
+__global__ void __launch_bounds__(THREADS, 1) batch_br_kernel(const InstDesc *table, const __grid_constant__ InstDesc one,
                                                            int n_inst) {
   __shared__ double sm[THREADS];
   chain_enter();
@@ -647,7 +723,7 @@ __global__ void __launch_bounds__(THREADS) batch_br_kernel(const InstDesc *table
     const int32_t sb = __ldg(g.iset_slot + I), na = __ldg(g.iset_slot + I + 1) - sb;
     double tot = 0.0;
     for (int32_t a = 0; a < na; ++a) tot += in.avg[sb + a];
-    for (int32_t a = 0; a < na; ++a) in.sbs[sb + a] = tot > 0.0 ? in.avg[sb + a] / tot : 1.0 / (double)na;
+    for (int32_t a = 0; a < na; ++a) in.sbs[sb + a] = match(in.avg[sb + a], tot, na);
   }
   level_sync<CLUSTERED>();
   for (int d = 0; d < in.D; ++d) {

@@ -1026,16 +1026,25 @@ extern "C" int cfr_synchronize(cfr_handle *h, void *stream) {
 }
 
 // ------------------------------------------------------------- read-out
-static int deliver(cfr_handle *h, const double *dev_compiled, double *out, int on_device, cudaStream_t s) {
+// The average strategy into dst, in spec slot order (to_spec) or slot order.
+static int launch_avg(const cfr_handle *h, double *dst, bool to_spec, cudaStream_t s) {
   const Compiled &c = h->c;
-  if (c.A == 0) return CFR_OK;
-  double *dst = on_device ? out : h->p<double>(h->b_out);
-  permute_kernel<<<grid_for(c.A, kThreads), kThreads, 0, s>>>(h->p<int32_t>(h->b_spec_slot), dev_compiled, dst, (int32_t)c.A);
+  const int32_t *slots = h->p<int32_t>(h->b_iset_slot), *to = to_spec ? h->p<int32_t>(h->b_spec_slot) : nullptr;
+  const double *avg = h->p<double>(h->b_avg);
+  const int32_t I = (int32_t)c.I;
+  if (h->maxa_tier == 4) avg_strategy_kernel<4><<<grid_for(4 * c.I, kThreads), kThreads, 0, s>>>(slots, I, avg, to, dst);
+  else if (h->maxa_tier == 8) avg_strategy_kernel<8><<<grid_for(8 * c.I, kThreads), kThreads, 0, s>>>(slots, I, avg, to, dst);
+  else avg_strategy_kernel<1><<<grid_for(c.I, kThreads), kThreads, 0, s>>>(slots, I, avg, to, dst);
   CK(cudaGetLastError());
-  if (!on_device) {
-    CK(cudaMemcpyAsync(out, dst, 8 * c.A, cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
-  }
+  return CFR_OK;
+}
+
+// Where a strategy is read out to: the caller's device array, or the staging
+// buffer that finish_read_out copies to the caller's host array.
+static int finish_read_out(cfr_handle *h, const double *dst, double *out, int on_device, cudaStream_t s) {
+  if (on_device) return CFR_OK;
+  CK(cudaMemcpyAsync(out, dst, 8 * h->c.A, cudaMemcpyDeviceToHost, s));
+  CK(cudaStreamSynchronize(s));
   return CFR_OK;
 }
 
@@ -1043,17 +1052,10 @@ extern "C" int cfr_avg_strategy(cfr_handle *h, double *out, int on_device, void 
   if (!h || (!out && h->c.A > 0)) return set_err(CFR_ERR_ARG, "cfr_avg_strategy: null argument");
   if (!h->bound) return set_err(CFR_ERR_NOT_BOUND, "cfr_avg_strategy: not bound");
   cudaStream_t s = (cudaStream_t)stream;
-  const Compiled &c = h->c;
-  if (c.I == 0) return CFR_OK;
+  if (h->c.I == 0) return CFR_OK;
   double *dst = on_device ? out : h->p<double>(h->b_out);
-  avg_spec_kernel<<<grid_for(c.I, kThreads), kThreads, 0, s>>>(h->p<int32_t>(h->b_iset_slot), (int32_t)c.I,
-                                                                h->p<double>(h->b_avg), h->p<int32_t>(h->b_spec_slot), dst);
-  CK(cudaGetLastError());
-  if (!on_device) {
-    CK(cudaMemcpyAsync(out, dst, 8 * c.A, cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
-  }
-  return CFR_OK;
+  const int rc = launch_avg(h, dst, true, s);
+  return rc ? rc : finish_read_out(h, dst, out, on_device, s);
 }
 
 extern "C" int cfr_current_strategy(cfr_handle *h, double *out, int on_device, void *stream) {
@@ -1062,19 +1064,23 @@ extern "C" int cfr_current_strategy(cfr_handle *h, double *out, int on_device, v
   cudaStream_t s = (cudaStream_t)stream;
   const Compiled &c = h->c;
   if (c.A == 0) return CFR_OK;
-  double *tmp = h->p<double>(h->b_sbs);
-  if (h->precision == CFR_P64) CK(cudaMemcpyAsync(tmp, h->p<double>(h->b_sigma), 8 * c.A, cudaMemcpyDeviceToDevice, s));
-  else {
-    to_double_kernel<float><<<grid_for(c.A, kThreads), kThreads, 0, s>>>(h->p<float>(h->b_sigma), tmp, (int32_t)c.A);
-    CK(cudaGetLastError());
-  }
-  return deliver(h, tmp, out, on_device, s);
+  double *dst = on_device ? out : h->p<double>(h->b_out);
+  const int32_t *to = h->p<int32_t>(h->b_spec_slot);
+  const int nb = grid_for(c.A, kThreads);
+  if (h->precision == CFR_P64)
+    current_strategy_kernel<double><<<nb, kThreads, 0, s>>>(h->p<double>(h->b_sigma), to, dst, (int32_t)c.A);
+  else
+    current_strategy_kernel<float><<<nb, kThreads, 0, s>>>(h->p<float>(h->b_sigma), to, dst, (int32_t)c.A);
+  CK(cudaGetLastError());
+  return finish_read_out(h, dst, out, on_device, s);
 }
 
 static int launch_br(cfr_handle *h, int d, cudaStream_t s) {
   const LevelWork &w = h->levels[d];
-  int L = std::min(h->level_lanes[d], 32);  // best response: lane groups of at most a warp
-  if (h->c.level_tiled[d]) L = std::min(L, kTiledLanes);
+  // lane groups of at most a warp; a warp where a lane can keep its members
+  // (the sets of a tile are neighbouring warps, which share its reach in L1)
+  int L = std::min(h->level_lanes[d], 32);
+  if (h->c.level_mean_members[d] > 32.0) L = 32;
   const int nch = w.ch1 - w.ch0, nis = w.is1 - w.is0;
   const int nb_ch = nch > 0 ? grid_for(nch, kThreads) : 0;
   const int nb_is = nis > 0 ? grid_for(nis, kThreads / L) : 0;
@@ -1090,10 +1096,10 @@ extern "C" int cfr_exploitability(cfr_handle *h, double *out_expl, double *out_b
   cudaStream_t s = (cudaStream_t)stream;
   const Compiled &c = h->c;
   GameView g = game_view(h);
-  if (c.I > 0)
-    avg_normalize_kernel<<<grid_for(c.I, kThreads), kThreads, 0, s>>>(h->p<int32_t>(h->b_iset_slot), (int32_t)c.I,
-                                                                       h->p<double>(h->b_avg), h->p<double>(h->b_sbs));
-  CK(cudaGetLastError());
+  if (c.I > 0) {
+    const int rc = launch_avg(h, h->p<double>(h->b_sbs), false, s);
+    if (rc) return rc;
+  }
   for (int64_t d = 0; d < c.D; ++d) {
     int rc = launch_fwd<double>(h, d, s, g, h->p<double>(h->b_sbs), h->p<double2>(h->b_reach2), d > 0, d > 0);
     if (rc) return rc;

@@ -151,18 +151,30 @@ __device__ __forceinline__ int32_t wide_of_chunk(const GameView &g, const LevelW
   return lo;
 }
 
-// Fixed-shape block reduction (all threads call it; the result is valid in thread 0).
-__device__ __forceinline__ double block_sum(double x) {
-  __shared__ double sm[kThreads];
-  __syncthreads();
-  sm[threadIdx.x] = x;
-  __syncthreads();
+// Fixed-shape block reduction of N values at once (all threads call it; the
+// results are valid in thread 0): butterflies within the warps, then one
+// across them.
+template <int N>
+__device__ __forceinline__ void block_sum(double (&x)[N]) {
+  __shared__ double sm[N][kThreads / 32];
+  const int warp = threadIdx.x / 32, lane = threadIdx.x & 31;
 #pragma unroll
-  for (int s = kThreads / 2; s > 0; s >>= 1) {
-    if ((int)threadIdx.x < s) sm[threadIdx.x] += sm[threadIdx.x + s];
-    __syncthreads();
+  for (int off = 16; off > 0; off >>= 1)
+#pragma unroll
+    for (int i = 0; i < N; ++i) x[i] += __shfl_xor_sync(0xffffffffu, x[i], off);
+  __syncthreads();  // the array may still be read from the call before
+  if (lane == 0)
+#pragma unroll
+    for (int i = 0; i < N; ++i) sm[i][warp] = x[i];
+  __syncthreads();
+  if (warp == 0) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) x[i] = lane < kThreads / 32 ? sm[i][lane] : 0.0;
+#pragma unroll
+    for (int off = kThreads / 64; off > 0; off >>= 1)
+#pragma unroll
+      for (int i = 0; i < N; ++i) x[i] += __shfl_xor_sync(0xffffffffu, x[i], off);
   }
-  return sm[0];
 }
 
 // The sum of v[cb, ce) strictly left to right (the FP64 parity order), for
@@ -569,23 +581,23 @@ __device__ __forceinline__ void bwd_wide_chunk(const GameView &g, const LevelWor
     return;
   } else {
     const int32_t c0 = cb + (q - q0) * kWideChunkK, c1 = min(ce, c0 + kWideChunkK);
-    double x = 0.0;
-    for (int32_t c = c0 + threadIdx.x; c < c1; c += blockDim.x) x += (double)ldm<PERSIST>(v + c);
-    x = block_sum(x);
+    double x[1] = {0.0};
+    for (int32_t c = c0 + threadIdx.x; c < c1; c += blockDim.x) x[0] += (double)ldm<PERSIST>(v + c);
+    block_sum(x);
     __shared__ unsigned s_ticket;
     if (threadIdx.x == 0) {
-      g.wide_part[q] = x;
+      g.wide_part[q] = x[0];
       __threadfence();
       s_ticket = atomicAdd(g.wide_cnt + wi, 1u);
     }
     __syncthreads();
     if (s_ticket == (unsigned)(nq - 1)) {  // the last chunk's block adds the partials (fixed shape)
       __threadfence();
-      double y = 0.0;
-      for (int32_t k = threadIdx.x; k < nq; k += blockDim.x) y += __ldcg(g.wide_part + q0 + k);
-      y = block_sum(y);
+      double y[1] = {0.0};
+      for (int32_t k = threadIdx.x; k < nq; k += blockDim.x) y[0] += __ldcg(g.wide_part + q0 + k);
+      block_sum(y);
       if (threadIdx.x == 0) {
-        v[h] = (T)y;
+        v[h] = (T)y[0];
         g.wide_cnt[wi] = 0u;
       }
     }
@@ -1172,7 +1184,8 @@ __global__ void init_state_kernel(const int32_t *iset_slot, int32_t n_sets, T *s
   for (int32_t q = tid; q < A; q += stride) { R[q] = 0.0; avg[q] = 0.0; }
   for (int32_t I = tid; I < n_sets; I += stride) {
     const int32_t sb = iset_slot[I], na = iset_slot[I + 1] - sb;
-    for (int32_t a = 0; a < na; ++a) sigma[sb + a] = (T)(1.0 / (double)na);  // RM of zero regret
+    const T u = T(1) / (T)na;  // RM of zero regret
+    for (int32_t a = 0; a < na; ++a) sigma[sb + a] = u;
   }
   if (tid == 0) {
     *t = 0;
@@ -1213,38 +1226,40 @@ __global__ void rm_kernel(const int32_t *iset_slot, int32_t n_sets, const double
 }
 
 // ------------------------------------------------------------- read-out
-// The average strategy in spec slot order (the two kernels below in one).
-static __global__ void avg_spec_kernel(const int32_t *iset_slot, int32_t n_sets, const double *avg,
-                                       const int32_t *spec_slot_of, double *out) {
-  const int32_t stride = gridDim.x * blockDim.x;
-  for (int32_t I = blockIdx.x * blockDim.x + threadIdx.x; I < n_sets; I += stride) {
+// The average strategy of every set (uniform where its sum is zero) into
+// out[to[q]] for slot q, or out[q] without `to`. A lane a slot: what bounds it
+// is the FP64 division (137 cycles a warp and SM), so each slot has one. LANES
+// = 1: one thread a set, for sets of more than 8 actions.
+template <int LANES>
+__global__ void __launch_bounds__(kThreads) avg_strategy_kernel(const int32_t *iset_slot, int32_t n_sets,
+                                                                const double *avg, const int32_t *to, double *out) {
+  const int32_t groups = gridDim.x * blockDim.x / LANES;
+  const int lane = threadIdx.x % LANES;
+  for (int32_t I = (blockIdx.x * blockDim.x + threadIdx.x) / LANES; I < n_sets; I += groups) {
     const int32_t sb = iset_slot[I], na = iset_slot[I + 1] - sb;
-    double tot = 0.0;
-    for (int32_t a = 0; a < na; ++a) tot += avg[sb + a];
-    for (int32_t a = 0; a < na; ++a) out[spec_slot_of[sb + a]] = tot > 0.0 ? avg[sb + a] / tot : 1.0 / (double)na;
+    if constexpr (LANES > 1) {
+      const double x = lane < na ? avg[sb + lane] : 0.0;
+      double tot = 0.0;  // in action order
+#pragma unroll
+      for (int a = 0; a < LANES; ++a) {
+        const double y = __shfl_sync(group_mask<LANES>(), x, a, LANES);
+        if (a < na) tot += y;
+      }
+      if (lane < na) out[to ? to[sb + lane] : sb + lane] = match(x, tot, na);
+    } else {
+      double tot = 0.0;
+      for (int32_t a = 0; a < na; ++a) tot += avg[sb + a];
+      for (int32_t a = 0; a < na; ++a) out[to ? to[sb + a] : sb + a] = match(avg[sb + a], tot, na);
+    }
   }
 }
 
-static __global__ void avg_normalize_kernel(const int32_t *iset_slot, int32_t n_sets, const double *avg, double *out) {
-  const int32_t stride = gridDim.x * blockDim.x;
-  for (int32_t I = blockIdx.x * blockDim.x + threadIdx.x; I < n_sets; I += stride) {
-    const int32_t sb = iset_slot[I], na = iset_slot[I + 1] - sb;
-    double tot = 0.0;
-    for (int32_t a = 0; a < na; ++a) tot += avg[sb + a];
-    for (int32_t a = 0; a < na; ++a) out[sb + a] = tot > 0.0 ? avg[sb + a] / tot : 1.0 / (double)na;
-  }
-}
-
+// The current strategy in spec slot order: out[to[q]] = sigma[q].
 template <typename T>
-__global__ void to_double_kernel(const T *in, double *out, int32_t n) {
+__global__ void __launch_bounds__(kThreads) current_strategy_kernel(const T *sigma, const int32_t *to, double *out,
+                                                                    int32_t A) {
   const int32_t stride = gridDim.x * blockDim.x;
-  for (int32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += stride) out[q] = (double)in[q];
-}
-
-// out[spec_slot_of[q]] = in[q]: compiled slot order -> spec slot order
-static __global__ void permute_kernel(const int32_t *spec_slot_of, const double *in, double *out, int32_t A) {
-  const int32_t stride = gridDim.x * blockDim.x;
-  for (int32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < A; q += stride) out[spec_slot_of[q]] = in[q];
+  for (int32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < A; q += stride) out[to[q]] = as_double(sigma[q]);
 }
 
 // ------------------------------------------------ exact best response (FP64)
@@ -1262,35 +1277,29 @@ __device__ __forceinline__ void br_wide_chunk(const GameView &g, const LevelWork
   const int32_t cb = __ldg(g.wide_vb + wi), ce = cb + __ldg(g.wide_nch + wi);
   const int32_t q0 = __ldg(g.wide_chunk + wi), nq = __ldg(g.wide_chunk + wi + 1) - q0;
   const int32_t c0 = cb + (q - q0) * kWideChunkK, c1 = min(ce, c0 + kWideChunkK);
-  double sx = 0.0, sy = 0.0, sa = 0.0;
+  double x[3] = {0.0, 0.0, 0.0};
   for (int32_t c = c0 + threadIdx.x; c < c1; c += blockDim.x) {
-    const double2 x = vb[c];
-    sx += x.x; sy += x.y; sa += vavg[c];
+    const double2 y = vb[c];
+    x[0] += y.x; x[1] += y.y; x[2] += vavg[c];
   }
-  sx = block_sum(sx);
-  sy = block_sum(sy);
-  sa = block_sum(sa);
+  block_sum(x);
   __shared__ unsigned s_ticket;
   if (threadIdx.x == 0) {
-    g.wide_part[3 * q] = sx; g.wide_part[3 * q + 1] = sy; g.wide_part[3 * q + 2] = sa;
+    g.wide_part[3 * q] = x[0]; g.wide_part[3 * q + 1] = x[1]; g.wide_part[3 * q + 2] = x[2];
     __threadfence();
     s_ticket = atomicAdd(g.wide_cnt + wi, 1u);
   }
   __syncthreads();
   if (s_ticket == (unsigned)(nq - 1)) {  // the last chunk's block adds the partials (fixed shape)
     __threadfence();
-    double tx = 0.0, ty = 0.0, ta = 0.0;
-    for (int32_t k = threadIdx.x; k < nq; k += blockDim.x) {
-      tx += __ldcg(g.wide_part + 3 * (q0 + k));
-      ty += __ldcg(g.wide_part + 3 * (q0 + k) + 1);
-      ta += __ldcg(g.wide_part + 3 * (q0 + k) + 2);
-    }
-    tx = block_sum(tx);
-    ty = block_sum(ty);
-    ta = block_sum(ta);
+    double y[3] = {0.0, 0.0, 0.0};
+    for (int32_t k = threadIdx.x; k < nq; k += blockDim.x)
+#pragma unroll
+      for (int i = 0; i < 3; ++i) y[i] += __ldcg(g.wide_part + 3 * (q0 + k) + i);
+    block_sum(y);
     if (threadIdx.x == 0) {
-      vb[h] = make_double2(tx, ty);
-      vavg[h] = ta;
+      vb[h] = make_double2(y[0], y[1]);
+      vavg[h] = y[2];
       g.wide_cnt[wi] = 0u;
     }
   }
@@ -1321,47 +1330,74 @@ __device__ __forceinline__ void br_chance(const GameView &g, double2 *vb, double
 // FP64 pipe (a warp instruction every 16-19 cycles an SM) bounds it: every
 // member and action takes three fused multiply-adds, each lane sums its own
 // members' action values, and the group's sums are finished by a shared-out
-// butterfly, so nothing is added twice. The members of the last chunk keep
-// their best action's value in a register and write both lanes at once.
-// Best responses to a strategy of the 11M-node card game: 893 -> 294 us
-// (every lane used to add every member's value, and the launches to wait for
-// one another's end).
+// butterfly, so nothing is added twice. A lane keeps its last kBrKeep members'
+// action values in registers until the best action is known and writes both
+// of a member's values at once; members before those write the other lane's
+// value on the way and take a second pass over the best action's children.
+// Best responses to a strategy of the 11M-node card game: 893 -> 269 us (every
+// lane used to add every member's value, and the launches to wait for one
+// another's end; 285 with one member kept).
+template <int MAXA> constexpr int kBrKeep = MAXA <= 4 ? 4 : (MAXA <= 8 ? 2 : 1);
+
 template <int MAXA, int LANES, bool PERSIST>
 __device__ __forceinline__ void br_set(const GameView &g, const double2 *reach2, const double *sbs, double2 *vb,
                                        double *vavg, int32_t I, int p, int lane, unsigned mask) {
+  constexpr int KEEP = kBrKeep<MAXA>;
   const int32_t sb = __ldg(g.iset_slot + I), na = __ldg(g.iset_slot + I + 1) - sb;
-  const int32_t m0 = __ldg(g.iset_mem + I), m1 = __ldg(g.iset_mem + I + 1), M = m1 - m0;
+  const int32_t m0 = __ldg(g.iset_mem + I), M = __ldg(g.iset_mem + I + 1) - m0;
   const MemberRanks mr = member_ranks(g, I, m0);
   const int32_t vb0 = __ldg(g.iset_vb + I);
-  double sg[MAXA], Q[MAXA], own[MAXA];
+  double sg[MAXA], Q[MAXA];
 #pragma unroll
-  for (int a = 0; a < MAXA; ++a) { sg[a] = a < na ? ldm<PERSIST>(sbs + sb + a) : 0.0; Q[a] = 0.0; own[a] = 0.0; }
-  const int32_t last = m0 + (M - 1) / LANES * LANES;  // first member of the last chunk
-  int32_t h = -1;
-  double oth = 0.0;
-  for (int32_t k0 = m0; k0 <= last; k0 += LANES) {
-    const int32_t k = k0 + lane;
-    h = -1;
-    if (k < m1) {
-      h = __ldg(g.mem_vs + k);
-      const int32_t cb = vb0 + (k - m0);
-      const double2 r = ldm<PERSIST>(reach2 + member_rank(g, k, mr));
-      const double po = p ? r.x : r.y;
-      double va = 0.0;
-      oth = 0.0;
+  for (int a = 0; a < MAXA; ++a) { sg[a] = a < na ? ldm<PERSIST>(sbs + sb + a) : 0.0; Q[a] = 0.0; }
+  // one member (k < M): its value slot, the other lane's value, and its own
+  // player's values of the actions
+  auto member = [&](int32_t k, double (&own)[MAXA], double &oth) {
+    const int32_t h = __ldg(g.mem_vs + m0 + k);
+    const double2 r = ldm<PERSIST>(reach2 + member_rank(g, m0 + k, mr));
+    constexpr int W = MAXA <= 8 ? MAXA : 4;  // actions whose loads are issued together
+    const double po = p ? r.x : r.y;
+    double va = 0.0;
+    oth = 0.0;
 #pragma unroll
-      for (int a = 0; a < MAXA; ++a) {
-        if (a < na) {
-          const double2 x = ldm<PERSIST>(vb + cb + a * M);
-          own[a] = p ? x.y : x.x;
-          Q[a] = fma(po, own[a], Q[a]);
-          oth = fma(sg[a], p ? x.x : x.y, oth);
-          va = fma(sg[a], ldm<PERSIST>(vavg + cb + a * M), va);
+    for (int a0 = 0; a0 < MAXA; a0 += W) {
+      double2 x[W];
+      double y[W];
+#pragma unroll
+      for (int j = 0; j < W; ++j) {
+        if (a0 + j < na) {
+          x[j] = ldm<PERSIST>(vb + vb0 + k + (a0 + j) * M);
+          y[j] = ldm<PERSIST>(vavg + vb0 + k + (a0 + j) * M);
         }
       }
-      if (k0 < last) reinterpret_cast<double *>(vb + h)[1 - p] = oth;
-      vavg[h] = va;
+#pragma unroll
+      for (int j = 0; j < W; ++j) {
+        const int a = a0 + j;
+        if (a < na) {
+          own[a] = p ? x[j].y : x[j].x;
+          Q[a] = fma(po, own[a], Q[a]);
+          oth = fma(sg[a], p ? x[j].x : x[j].y, oth);
+          va = fma(sg[a], y[j], va);
+        }
+      }
     }
+    vavg[h] = va;
+    return h;
+  };
+  const int32_t chunks = (M + LANES - 1) / LANES;
+  const int32_t kept = chunks > KEEP ? (chunks - KEEP) * LANES : 0;  // first member that is kept
+  for (int32_t k = lane; k < kept; k += LANES) {
+    double own[MAXA], oth;
+    const int32_t h = member(k, own, oth);
+    reinterpret_cast<double *>(vb + h)[1 - p] = oth;
+  }
+  double own[KEEP][MAXA], oth[KEEP];
+  int32_t h[KEEP];
+#pragma unroll
+  for (int c = 0; c < KEEP; ++c) {
+    const int32_t k = kept + c * LANES + lane;
+    h[c] = -1;
+    if (k < M) h[c] = member(k, own[c], oth[c]);
   }
   int best = 0;
   if constexpr (MAXA <= 8) {
@@ -1386,17 +1422,20 @@ __device__ __forceinline__ void br_set(const GameView &g, const double2 *reach2,
     }
   }
   // the group's lanes hold the same sums, so best agrees across it
-  for (int32_t k = m0 + lane; k < last; k += LANES) {
-    const int32_t hk = __ldg(g.mem_vs + k);
-    const double2 x = ldm<PERSIST>(vb + vb0 + (k - m0) + best * M);
+  for (int32_t k = lane; k < kept; k += LANES) {
+    const int32_t hk = __ldg(g.mem_vs + m0 + k);
+    const double2 x = ldm<PERSIST>(vb + vb0 + k + best * M);
     reinterpret_cast<double *>(vb + hk)[p] = p ? x.y : x.x;
   }
-  if (h >= 0) {
-    double mine = own[0];
 #pragma unroll
-    for (int a = 1; a < MAXA; ++a)
-      if (a == best) mine = own[a];
-    vb[h] = p ? make_double2(oth, mine) : make_double2(mine, oth);
+  for (int c = 0; c < KEEP; ++c) {
+    if (h[c] >= 0) {
+      double mine = own[c][0];
+#pragma unroll
+      for (int a = 1; a < MAXA; ++a)
+        if (a == best) mine = own[c][a];
+      vb[h[c]] = p ? make_double2(oth[c], mine) : make_double2(mine, oth[c]);
+    }
   }
 }
 
