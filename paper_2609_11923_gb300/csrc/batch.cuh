@@ -297,16 +297,28 @@ constexpr int kLongSet = 32;
 // One set by the LANES lanes of a group: its members' values, and the set's
 // totals into def_r and def_m (see bwd_set, whose sums these are). Every load
 // of a step is issued before the first value is used.
+struct GroupSet {  // a set's record
+  int32_t sb, na, m0, M, vb;
+  int2 rk;
+};
+template <typename T, int MODE> __device__ __forceinline__ GroupSet group_record(const GroupView<T> &g, int32_t I) {
+  GroupSet s;
+  s.sb = ldk<MODE>(g.iset_slot + I);
+  s.na = ldk<MODE>(g.iset_slot + I + 1) - s.sb;
+  s.m0 = ldk<MODE>(g.iset_mem + I);
+  s.M = ldk<MODE>(g.iset_mem + I + 1) - s.m0;
+  s.vb = ldk<MODE>(g.iset_vb + I);
+  s.rk = ldk<MODE>(g.iset_rank + I);
+  return s;
+}
+
 template <typename T, int MAXA, int LANES, int MODE>
-__device__ __forceinline__ void group_set(const GroupView<T> &g, int32_t I, bool p2, int lane, unsigned mask, int upd,
-                                          double *rows) {
+__device__ __forceinline__ void group_members(const GroupView<T> &g, const GroupSet &s, bool p2, int lane, unsigned mask,
+                                              int upd, double *rows) {
   constexpr bool C = MODE == kCluster, CHAINS = sizeof(T) == 8;
   constexpr int U = LANES <= 8 ? 2 : 1;  // members of a lane in flight
-  const int32_t sb = ldk<MODE>(g.iset_slot + I), se = ldk<MODE>(g.iset_slot + I + 1);
-  const int32_t m0 = ldk<MODE>(g.iset_mem + I), m1 = ldk<MODE>(g.iset_mem + I + 1);
-  const int32_t vb = ldk<MODE>(g.iset_vb + I);
-  const int2 rk = ldk<MODE>(g.iset_rank + I);
-  const int32_t na = se - sb, M = m1 - m0;
+  const int32_t sb = s.sb, na = s.na, m0 = s.m0, M = s.M, vb = s.vb;
+  const int2 rk = s.rk;
   T sig[MAXA], racc[MAXA], spw = T(0);
   double acc[kChainAcc<MAXA, LANES>];
 #pragma unroll
@@ -384,20 +396,34 @@ __device__ __forceinline__ void group_set(const GroupView<T> &g, int32_t I, bool
   }
 }
 
+// The work of a set, in games of more than four actions in code for two, four
+// or MAXA: what bounds a small game is the instructions of its groups, and most
+// sets of an endgame have two actions where its largest has seven (64 endgames
+// of 1e3 to 2e5 edges 2,916 -> 2,591 us, ten of 2e5 to 1e6 5,774 -> 4,954; one-
+// card poker and random trees, whose warps mix two to four actions, 3-6%
+// slower that way).
+template <typename T, int MAXA, int LANES, int MODE>
+__device__ __forceinline__ void group_set(const GroupView<T> &g, int32_t I, bool p2, int lane, unsigned mask, int upd,
+                                          double *rows) {
+  const GroupSet s = group_record<T, MODE>(g, I);
+  if constexpr (MAXA > 4) {
+    if (s.na <= 2) return group_members<T, 2, LANES, MODE>(g, s, p2, lane, mask, upd, rows);
+    if (s.na <= 4) return group_members<T, 4, LANES, MODE>(g, s, p2, lane, mask, upd, rows);
+  }
+  group_members<T, MAXA, LANES, MODE>(g, s, p2, lane, mask, upd, rows);
+}
+
 // One long set by a warp with the sums of group_set<.., 8, ..>: lane l of
 // eight adds members l, l + 8, l + 16, ... in turn. The warp's lanes compute 32
 // members' terms at once, then every lane adds the four of its column (its
 // lane modulo 8) in that order. FP32.
 template <int MAXA, int MODE>
-__device__ __forceinline__ void group_set_long(const GroupView<float> &g, int32_t I, bool p2, int upd) {
+__device__ __forceinline__ void group_members_long(const GroupView<float> &g, const GroupSet &s, bool p2, int upd) {
   constexpr bool C = MODE == kCluster;
   constexpr int U = 2;  // members of a lane in flight
   const int lane = threadIdx.x & 31, col = lane & 7;
-  const int32_t sb = ldk<MODE>(g.iset_slot + I), se = ldk<MODE>(g.iset_slot + I + 1);
-  const int32_t m0 = ldk<MODE>(g.iset_mem + I), m1 = ldk<MODE>(g.iset_mem + I + 1);
-  const int32_t vb = ldk<MODE>(g.iset_vb + I);
-  const int2 rk = ldk<MODE>(g.iset_rank + I);
-  const int32_t na = se - sb, M = m1 - m0;
+  const int32_t sb = s.sb, na = s.na, m0 = s.m0, M = s.M, vb = s.vb;
+  const int2 rk = s.rk;
   float sig[MAXA], racc[MAXA], spw = 0.f;
 #pragma unroll
   for (int a = 0; a < MAXA; ++a) {
@@ -449,33 +475,68 @@ __device__ __forceinline__ void group_set_long(const GroupView<float> &g, int32_
   if (lane < 8 && lane % STEP == 0 && lane / STEP < na) g.def_r[sb + lane / STEP] = racc[0];
 }
 
-// The slot updates of set I from its totals, by MAXA lanes, one for each slot:
-// FP64 instructions then serve most lanes of a warp, and the chain of a set is
-// one slot's.
+template <int MAXA, int MODE>
+__device__ __forceinline__ void group_set_long(const GroupView<float> &g, int32_t I, bool p2, int upd) {
+  const GroupSet s = group_record<float, MODE>(g, I);
+  if constexpr (MAXA > 4) {
+    if (s.na <= 2) return group_members_long<2, MODE>(g, s, p2, upd);
+    if (s.na <= 4) return group_members_long<4, MODE>(g, s, p2, upd);
+  }
+  group_members_long<MAXA, MODE>(g, s, p2, upd);
+}
+
+// The slot updates from the sets' totals, four lanes a set, a slot each (and
+// slots 4 to 7 in a second step where a set has them): FP64 instructions then
+// serve most lanes of a warp, and the chain of a set is one slot's.
+constexpr int kUpdateLanes = 4;
+template <typename T> struct SlotTotals {
+  double R, S;
+  T r, m;
+};
+
+template <typename T, int MODE>
+__device__ __forceinline__ SlotTotals<T> slot_totals(const GroupView<T> &g, int32_t sb, int32_t q) {
+  constexpr bool C = MODE == kCluster;
+  SlotTotals<T> t;
+  t.R = g.R[q];
+  t.S = g.avg[q];
+  t.r = ldm<C>(g.def_r + q);
+  if constexpr (sizeof(T) == 4) t.m = g.sigma[q] * ldm<C>(g.def_m + sb);  // this thread wrote sigma the iteration before
+  else t.m = ldm<C>(g.def_m + q);
+  return t;
+}
+
+template <typename T>
+__device__ __forceinline__ T slot_write(const GroupView<T> &g, int32_t q, const SlotTotals<T> &t, double wt, int rule) {
+  double Rn, Sn;
+  const double x = slot_terms(t.R, t.S, as_double(t.r), as_double(t.m), wt, rule, Rn, Sn);
+  g.R[q] = Rn;
+  g.avg[q] = Sn;
+  if constexpr (sizeof(T) == 8) return x;
+  else return narrow_pos(x);
+}
+
 template <typename T, int MAXA, int MODE>
 __device__ __forceinline__ void group_update(const GroupView<T> &g, int32_t I, int a, unsigned mask, double wt,
                                              int rule) {
-  constexpr bool C = MODE == kCluster;
+  constexpr int L = kUpdateLanes;
   const int32_t sb = ldk<MODE>(g.iset_slot + I), na = ldk<MODE>(g.iset_slot + I + 1) - sb, q = sb + a;
-  T pos = T(0);
-  if (a < na) {
-    const double R = g.R[q], S = g.avg[q];
-    const T r = ldm<C>(g.def_r + q);
-    T m;
-    if constexpr (sizeof(T) == 4) m = g.sigma[q] * ldm<C>(g.def_m + sb);  // this thread wrote sigma the iteration before
-    else m = ldm<C>(g.def_m + q);
-    double Rn, Sn;
-    const double x = slot_terms(R, S, as_double(r), as_double(m), wt, rule, Rn, Sn);
-    g.R[q] = Rn;
-    g.avg[q] = Sn;
-    if constexpr (sizeof(T) == 8) pos = x;
-    else pos = narrow_pos(x);
-  }
+  T pos = T(0), more = T(0);
+  if (a < na) pos = slot_write(g, q, slot_totals<T, MODE>(g, sb, q), wt, rule);
   T tot = T(0);  // positive parts in action order
 #pragma unroll
-  for (int b = 0; b < MAXA; ++b) {
-    const T x = __shfl_sync(mask, pos, b, MAXA);
+  for (int b = 0; b < L; ++b) {
+    const T x = __shfl_sync(mask, pos, b, L);
     if (b < na) tot += x;
+  }
+  if (MAXA > L && na > L) {  // the same for the whole group
+    if (a + L < na) more = slot_write(g, q + L, slot_totals<T, MODE>(g, sb, q + L), wt, rule);
+#pragma unroll
+    for (int b = 0; b < L; ++b) {
+      const T x = __shfl_sync(mask, more, b, L);
+      if (b + L < na) tot += x;
+    }
+    if (a + L < na) g.sigma[q + L] = match(more, tot, na);
   }
   if (a < na) g.sigma[q] = match(pos, tot, na);
 }
@@ -583,8 +644,8 @@ __global__ void __launch_bounds__(NT, 1) batch_iterate_kernel(const InstDesc *ta
   const int lane = tid % LANES, gid = ct / LANES, ngroups = all / LANES;
   const unsigned mask = group_mask<LANES>();
   // slot updates: set I always by the same threads (their L1 holds its R and avg)
-  const int ua = tid % MAXA, ugid = ct / MAXA, ugroups = all / MAXA;
-  const unsigned umask = group_mask<MAXA>();
+  const int ua = tid % kUpdateLanes, ugid = ct / kUpdateLanes, ugroups = all / kUpdateLanes;
+  const unsigned umask = group_mask<kUpdateLanes>();
   double *rows = s_rows[tid / 32];
   const int halves = in.order ? 2 : 1;  // alternating: player 1's half, then player 2's
   for (long long it = 0; it < n_iter; ++it) {

@@ -495,13 +495,12 @@ static __device__ __noinline__ float narrow_rare(double x) { return (float)x; }
 __device__ __forceinline__ float narrow_pos(double x) {  // (float)x of x >= 0, to nearest, ties to even
   const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
   const uint32_t e = (hi >> 20) - 896u;
-  if (e - 1u < 254u) {
-    const uint32_t m = (e << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
-    const uint32_t rest = lo & 0x1fffffffu;  // bits below the last place
-    return __uint_as_float(m + (rest > 0x10000000u - (m & 1u) ? 1u : 0u));
-  }
-  if ((hi | lo) == 0u) return 0.f;
-  return narrow_rare(x);  // to a subnormal or infinite float
+  const uint32_t m = (e << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
+  const uint32_t rest = lo & 0x1fffffffu;  // bits below the last place
+  const bool zero = (hi | lo) == 0u;
+  float y = zero ? 0.f : __uint_as_float(m + (rest > 0x10000000u - (m & 1u) ? 1u : 0u));
+  if (!zero && e - 1u >= 254u) y = narrow_rare(x);  // to a subnormal or infinite float
+  return y;
 }
 
 __device__ __forceinline__ double positive_part(double x) {  // x > 0.0 ? x : 0.0 (NaN and -0 give 0)

@@ -108,12 +108,12 @@ __global__ void __launch_bounds__(kTopThreads<T, MAXA>, 1) top_kernel(const __gr
         group_set<T, MAXA, LANES, kResident>(g, J, J >= is2, lane, mask, upd, rows);
       __syncthreads();
     }
-    const int ua = tid % MAXA, ugid = tid / MAXA;
-    const unsigned umask = group_mask<MAXA>();
+    const int ua = tid % kUpdateLanes, ugid = tid / kUpdateLanes;
+    const unsigned umask = group_mask<kUpdateLanes>();
     for (int d = 0; d <= K; ++d) {
       const int32_t i0 = upd & 1 ? s_lw[d].is0 : s_lw[d].is2, i1 = upd & 2 ? s_lw[d].is1 : s_lw[d].is2;
       if (upd == 3 && d > 0) break;  // both players' sets: all depths at once
-      for (int32_t J = i0 + ugid; J < (upd == 3 ? (int32_t)I : i1); J += NT / MAXA)
+      for (int32_t J = i0 + ugid; J < (upd == 3 ? (int32_t)I : i1); J += NT / kUpdateLanes)
         group_update<T, MAXA, kResident>(g, J, ua, umask, wt, in.rule);
     }
     __syncthreads();
