@@ -29,44 +29,64 @@
 
 namespace cfr {
 
-// CTAs for every instance of a batch (host). load: the instance's nodes times
-// the share of the longest run's iterations; alone[i]: it is as fast in one
-// CTA. Starting from `least` CTAs each, the instance with the most load per
-// CTA takes the next cluster size while SMs are left for it, or its share
-// exceeds an even one of the whole batch. kSplitNodes per CTA and less stay as
-// they are: a cluster barrier costs 1,600 cycles with stores in flight, a
-// CTA's 300 (an endgame of 21,000 nodes: 29 us an iteration on 2 CTAs, 18 on
-// 8). Clusters above 8 CTAs need most of a GPC: at most six of them.
-constexpr int64_t kSplitNodes = 3000;
-inline std::vector<int> plan_clusters(const std::vector<int64_t> &load, const std::vector<char> &alone, int least,
-                                      int sms) {
-  static const int sizes[] = {1, 2, 3, 4, 6, 8, 12, 16};
+// How many CTAs, and clusters of 4, 8 and 16 CTAs, run at the same time at one
+// CTA an SM (a cluster lies in one GPC, and how many SMs each has differs from
+// one GPU to the next).
+struct ClusterRoom {
+  int sms = 0, four = 0, eight = 0, sixteen = 0;
+};
+
+// CTAs for every instance of a batch (host): 1, 2, 4, 8 or 16, at least
+// `least`. Estimated cycles of an iteration, from solves of endgames: in one
+// CTA 8,000 + 1.6 a node from shared memory (`alone`), 12,000 + 2 a node from
+// global memory; in a cluster 45,000 (2 D - 1 barriers of 1,900 with stores in
+// flight, and every read through L2) + 1.5 a node and CTA. The instance that
+// takes longest gets twice its CTAs as long as all of them run at the same
+// time (a cluster too many waits for a whole instance: ten large endgames with
+// six of 16 took 89 us an iteration, with four 64); a batch that does not run
+// at the same time anyway, while it takes longer than an even share of it.
+struct BatchLoad {
+  int64_t nodes;
+  double share;  // of the longest run's iterations
+  bool alone;
+};
+inline std::vector<int> plan_clusters(const std::vector<BatchLoad> &load, int least, const ClusterRoom &room) {
   const int n = (int)load.size();
+  auto cycles = [&](int i, int c) {
+    const double N = (double)load[i].nodes;
+    const double t = c > 1 ? 45000.0 + 1.5 * N / c : load[i].alone ? 8000.0 + 1.6 * N : 12000.0 + 2.0 * N;
+    return t * load[i].share;
+  };
   std::vector<int> cta(n, least);
-  std::priority_queue<std::pair<int64_t, int>> most;  // (load per CTA, instance)
-  int64_t all = 0;
-  int used = 0, wide = 0;
+  int count[17] = {0};  // instances by CTAs
+  double work = 0.0;    // CTA cycles
+  std::priority_queue<std::pair<double, int>> longest;  // (cycles, instance)
   for (int i = 0; i < n; ++i) {
-    all += load[i];
-    used += least;
-    most.push({load[i] / least, -i});
+    ++count[least];
+    work += least * cycles(i, least);
+    longest.push({cycles(i, least), -i});
   }
-  while (!most.empty()) {
-    const int64_t per = most.top().first;
-    const int i = -most.top().second;
-    most.pop();
-    if (per <= kSplitNodes) break;
-    if (alone[i] && cta[i] == 1) continue;
-    int next = 0;
-    for (int c : sizes)
-      if (c > cta[i]) { next = c; break; }
-    if (next == 0 || (next > 8 && cta[i] <= 8 && wide == 6)) continue;
-    if (used + next - cta[i] > sms && per <= all / sms) break;
-    if (next > 8 && used + next - cta[i] > sms) continue;
-    if (next > 8 && cta[i] <= 8) ++wide;
-    used += next - cta[i];
-    cta[i] = next;
-    most.push({load[i] / next, -i});
+  auto fits = [&]() {
+    const int eights = 2 * count[16] + count[8];
+    return count[16] <= room.sixteen && eights <= room.eight && 2 * eights + count[4] <= room.four &&
+           8 * eights + 4 * count[4] + 2 * count[2] + count[1] <= room.sms;
+  };
+  const bool waves = !fits();
+  while (!longest.empty()) {
+    const double t = longest.top().first;
+    const int i = -longest.top().second, c = cta[i];
+    longest.pop();
+    if (c == 16 || cycles(i, 2 * c) >= t) continue;
+    --count[c];
+    ++count[2 * c];
+    if (!fits() && !(waves && t > work / room.sms)) {
+      ++count[c];
+      --count[2 * c];
+      continue;
+    }
+    work += 2 * c * cycles(i, 2 * c) - c * t;
+    cta[i] = 2 * c;
+    longest.push({cycles(i, 2 * c), -i});
   }
   return cta;
 }

@@ -1653,6 +1653,28 @@ extern "C" int cfr_autotune(cfr_handle *h, int reps, void *stream) {
 }
 
 // ----------------------------------------------------------- batched solves
+// Clusters that the current device runs at the same time (asked for once per
+// device: the answer is a property of the GPU).
+static int cluster_room(ClusterRoom *out) {
+  static std::mutex mu;
+  static ClusterRoom known[64];
+  int dev = 0;
+  CK(cudaGetDevice(&dev));
+  std::lock_guard<std::mutex> lock(mu);
+  ClusterRoom r;
+  if (dev >= 0 && dev < 64 && known[dev].sms > 0) {
+    *out = known[dev];
+    return CFR_OK;
+  }
+  CK(cudaDeviceGetAttribute(&r.sms, cudaDevAttrMultiProcessorCount, dev));
+  CK(batch_cluster_room(4, &r.four));
+  CK(batch_cluster_room(8, &r.eight));
+  CK(batch_cluster_room(16, &r.sixteen));
+  if (dev >= 0 && dev < 64) known[dev] = r;
+  *out = r;
+  return CFR_OK;
+}
+
 // A batched call's plan: the instances' descriptors ordered by cluster size
 // (largest first, and by load within a size), and one launch for each size.
 struct BatchPlan {
@@ -1680,11 +1702,7 @@ static int batch_plan(cfr_handle *const *hs, int n, const int64_t *iters, int64_
     if (it < 0) return set_err(CFR_ERR_ARG, "batch: negative iteration count");
     longest = std::max(longest, it);
   }
-  std::vector<int64_t> load(n);
-  for (int i = 0; i < n; ++i) {
-    const double share = iters ? (double)iters[i] / (double)longest : 1.0;
-    load[i] = (int64_t)((double)hs[i]->c.N * share);
-  }
+  std::vector<BatchLoad> load(n);
   // one launch for each kind: push or pull, cluster size, resident or not
   struct Entry {
     int inst, push, mode;
@@ -1692,16 +1710,19 @@ static int batch_plan(cfr_handle *const *hs, int n, const int64_t *iters, int64_
     InstDesc d;
   };
   std::vector<Entry> e(n);
-  std::vector<char> alone(n, 0);
   for (int i = 0; i < n; ++i) {
     e[i].inst = i;
     e[i].push = iterate && hs[i]->c.int_edge.empty();
     e[i].d = inst_desc(hs[i], iters ? iters[i] : n_iter);
     e[i].smem = iterate && cluster == 1 ? resident_bytes(hs[i], e[i].d) : 0;
-    // FP32: as fast resident in one CTA as in a cluster of 8 (10,400 nodes: 16 us an iteration either way)
-    alone[i] = e[i].smem > 0 && bp.precision == CFR_P32;
+    load[i].nodes = hs[i]->c.N;
+    load[i].share = iters ? (double)iters[i] / (double)longest : 1.0;
+    load[i].alone = e[i].smem > 0 && bp.precision == CFR_P32;
   }
-  const std::vector<int> cta = plan_clusters(load, alone, cluster, device_sms());
+  ClusterRoom room;
+  int rc = cluster_room(&room);
+  if (rc) return rc;
+  const std::vector<int> cta = plan_clusters(load, cluster, room);
   for (int i = 0; i < n; ++i) {
     if (cta[i] > 1) e[i].smem = 0;
     e[i].mode = cta[i] > 1 ? kCluster : e[i].smem > 0 ? kResident : kSolo;
@@ -1711,7 +1732,7 @@ static int batch_plan(cfr_handle *const *hs, int n, const int64_t *iters, int64_
     if (ca != cb) return ca > cb;
     if (a.push != b.push) return a.push > b.push;
     if (a.mode != b.mode) return a.mode < b.mode;
-    return load[a.inst] > load[b.inst];
+    return load[a.inst].nodes > load[b.inst].nodes;
   });
   double *res = reinterpret_cast<double *>((char *)table_dev + sizeof(InstDesc) * (size_t)n);
   bp.tab.resize(n);

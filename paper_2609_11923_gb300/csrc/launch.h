@@ -70,6 +70,10 @@ struct BatchLaunch {
   bool push = false, chained = false;
 };
 
+// Clusters of `cluster` CTAs of the batched kernel (one CTA an SM) that run at
+// the same time.
+cudaError_t batch_cluster_room(int cluster, int *clusters);
+
 template <typename T>
 cudaError_t launch_batch_iterate(int maxa, int lanes, int threads, const BatchLaunch &l, cudaStream_t s,
                                  const InstDesc *table, const InstDesc &one);
