@@ -100,7 +100,7 @@ typedef struct cfr_options {
    * R + r, the iteration's instantaneous regret as the prediction; quadratic
    * averaging w_t = t^2). */
   int rule;
-  int lanes_per_set;   /* 0 = by mean set size (see cfr_autotune); else 1, 2, 4, 8, 16 or 32 lanes per set,
+  int lanes_per_set;   /* 0 = by mean set size, long sets in FP32 streaming (see cfr_autotune); else 1, 2, 4, 8, 16 or 32 lanes per set,
                           or 256 = one thread block per set in the per-level kernels (sets of at most 8
                           actions; the persistent kernel then uses 32), or 512 = the streaming backward
                           (CFR_P32 in member order, sets of at most 8 actions): each depth's sets go in
@@ -333,7 +333,8 @@ int cfr_export_array(const cfr_handle *h, int which, void *out, int64_t capacity
  * (1, 2, 4, 8, 16, 32, and 256 = one block per set when sets have at most 8
  * actions, and 512 = the streaming backward at depths that can stream;
  * `reps` launches each; 512 only where sets have at least 32 members on
- * average) and keeps the fastest; in the
+ * average) and takes the fastest where `reps` whole iterations are faster with
+ * it than with the present choice; in the
  * persistent form it also times whole persistent iterations per lane count.
  * Trial launches overwrite the solver state, so the call ends by resetting it
  * (as cfr_reset) and dropping a captured graph. The chosen counts are
@@ -469,10 +470,9 @@ int cfr_iterate_noalloc(cfr_handle *h, int64_t n, void *stream);
  * stderr per handle, then per-level launches of the same kernels in the same
  * order.
  * CFR_DEBUG_STREAM_STALL = 1 (a bound handle; cleared by cfr_reset): the
- * streaming backward's copy warp issues no copies beyond each CTA's first
- * chunks, so the compute threads' and the update warp's waits for the next
- * chunk run out (about a second each) and cfr_synchronize reports
- * CFR_ERR_TIMEOUT. Nothing faults or hangs: every wait is bounded. */
+ * streaming backward issues no copies beyond each team's first chunks, so
+ * the waits for the next chunk run out (about a second each) and
+ * cfr_synchronize reports CFR_ERR_TIMEOUT. Nothing faults or hangs: every wait is bounded. */
 enum { CFR_DEBUG_BARRIER_MISSING_ARRIVALS = 1, CFR_DEBUG_FAIL_GRAPH_CAPTURE = 2, CFR_DEBUG_STREAM_STALL = 3 };
 int cfr_debug_set(cfr_handle *h, int key, int64_t value);
 

@@ -8,44 +8,61 @@
 // interleaved inside it), their members' children's values (one run of value
 // slots), their members' own value slots, their slots' strategy, regret and
 // average, and their set descriptors. The host cuts each depth's sets into
-// chunks of whole groups (a tile of four sets, or one untiled set) whose
-// staged bytes fit one pipeline stage; the depth's narrow chance nodes
-// follow as chance chunks (consecutive nodes, whose children are one run of
-// value slots, and their entries of the chance arrays), summed in the same
-// pipeline. Every CTA walks the chunks c = blockIdx, blockIdx + grid, ...
-// through a ring of kStreamStages stages. Its kStreamCompute compute threads
-// do the members' (or chance nodes') work; the copy warp issues each chunk's
-// cp.async.bulk copies into a stage and a side slot (their mbarriers count
-// the bytes), and the update warp runs every group's slot update.
-// The loads in flight cost no registers, so the memory pipe stays full at a
-// low warp count, and the compute warps never wait for a slot update (they
-// hand each group's partial sums over through a double-buffered array and a
-// pair of mbarriers); the one scattered access left is each member's value
-// write into its parent set's block.
+// chunks of whole groups (a tile of four sets, or one untiled set); the
+// depth's narrow chance nodes follow as chance chunks (consecutive nodes,
+// whose children are one run of value slots, and their entries of the chance
+// arrays). A CTA's warps form teams (StreamShape), and every team walks its
+// own chunks through its own ring of kStreamStages stages: as soon as its
+// threads are done with a chunk, its first warp starts the cp.async.bulk
+// copies of the next chunk but one into the same stage. No team waits for
+// another, so the copies of some teams are in flight while others compute;
+// the loads in flight cost no registers; the one scattered access left is
+// each member's value write into its parent set's block.
 //
-// Work inside a chunk: the compute threads take one group at a time: thread
-// t serves set j = t % G of the group (G = 4 for a tile, 1 otherwise) and
-// members q = t / G, t / G + 256 / G, ... of that set, so a warp reads a
-// tile's reach as one contiguous run. Per-thread FP32 partial sums are
-// finished by a fixed-shape butterfly within the warp and, in the update
-// warp, a sum over the warps in warp order (deterministic run to run); the
-// update warp then updates the group's slots (one lane per slot) and writes
-// sigma^{t+1}. The form pays where sets are long (hundreds of members).
+// What bounds it: the largest depths are near what DRAM gives (a depth of 3.7M
+// members, 93 MB: 31 us -> 26 with 8 warps on one group -> with teams), the
+// others spend their time in the latencies of a group's few hundred
+// instructions, which only independent warps hide. A set of 153 members is 5
+// steps of one warp (19 for a tile of four); over eight warps it was one step
+// that most lanes sat out, and the sums' shuffles cost more than the members.
+// All depths of the 27M-node card game: an iteration of 230 us -> 131 (202 by
+// lane groups, 161 with the best form of each depth); of the 11M-node one
+// 110 by lane groups, 80 here.
+//
+// Work inside a chunk: the team takes one group at a time: thread t serves
+// set j = t % G of the group (G = 4 for a tile, 1 otherwise) and members
+// q = t / G, t / G + n / G, ... of that set (n threads in the team), so a
+// warp reads a tile's reach as one contiguous run. Per-thread FP32 partial
+// sums are finished by a fixed-shape butterfly within the warp and, in the
+// team's first warp, a sum over the team's warps in order (deterministic run
+// to run); that warp then updates the group's slots (one lane per slot) and
+// writes sigma^{t+1}. The form pays where sets are long.
 #pragma once
+#include <algorithm>
+
 #include "kernels.cuh"
 
 namespace cfr {
 
 constexpr int kStreamLanes = 512;                 // lanes_per_set code of this form
-constexpr int kStreamStages = 2;                  // pipeline depth
-constexpr int kStreamStageBytes = 48 * 1024;      // bytes one chunk may stage for the compute threads
-constexpr int kStreamSideSlots = 4;               // ring of the update warp's per-chunk data
-constexpr int kStreamSideBytes = 2048;            // bytes of one side slot
-constexpr int kStreamDynSmem = kStreamStages * kStreamStageBytes + kStreamSideSlots * kStreamSideBytes;
-constexpr int kStreamCompute = 256;               // compute threads of a streaming CTA (two CTAs per SM)
-constexpr int kStreamWarps = kStreamCompute / 32;
+constexpr int kStreamStages = 2;                  // a team's ring
+constexpr int kStreamStageBytes = 48 * 1024;      // bytes one chunk may stage at most
+constexpr int kStreamPackBytes = 6 * 1024;        // groups are packed into a chunk up to this size,
+constexpr int kStreamSpread = 16 * 152;           // as long as the depth makes this many chunks (one for each of a GB300's warps)
+constexpr int kStreamChanceBytes = 1024;          // chance nodes are packed up to this size in any case
+constexpr int kStreamSideBytes = 2048;            // bytes of a chunk's R and average sums, and descriptors, at most
+constexpr int kStreamMaxWarps = 16;               // warps of a streaming CTA (one CTA per SM)
+constexpr int kStreamMinWarps = 6;                // of a CTA, unless its stages are so large that even the largest teams are fewer
+constexpr int kStreamDynSmem = 216 * 1024;        // bytes of all teams' rings
 constexpr int kStreamMinMembers = 32;             // mean members per set below which the autotuner does not try it
-constexpr int kStreamChanceMax = 4 * kStreamCompute;  // chance nodes per chance chunk at most
+// Mean members per set from which a depth streams by default: of an untiled
+// depth, and of a tiled one, which lane groups read worse. Iterations by lane
+// groups / streamed from fewer members on: card games of 36 members a set
+// 39 / 46 us, of 66-78 untiled 54 / 64, of 78 (tiled in the large depths) 62 /
+// 54 with those depths streamed, of 105-120 105 / 80, of 153-171 202 / 131; an
+// endgame of 97-99 33 / 27.
+constexpr int kStreamAutoMembers = 96, kStreamAutoTiled = 64;
+constexpr int kStreamChanceMax = 1024;            // chance nodes per chance chunk at most
 
 // Per information set (member order), 32 bytes, read by the streaming form.
 struct SetInfo {
@@ -78,12 +95,13 @@ struct StreamChunk {
 static_assert(sizeof(SetInfo) == 32, "SetInfo is staged in 32-byte records");
 static_assert(sizeof(StreamChunk) == 64, "StreamChunk is 64 bytes");
 
-// Byte offsets of the staged arrays: in a stage (what the compute threads
-// read) and in a side slot (what the update warp reads for the slot
-// updates, so that the stage can be refilled while it still works).
+// Byte offsets of the staged arrays: what the members' work reads, then
+// (from total on) what the slot updates read besides: R, then the average
+// sums, 8 bytes a slot each. (s_*: the latter's sizes together with the
+// descriptors', which kStreamSideBytes bounds.)
 struct StreamLayout {
-  uint32_t reach, val, mem, info, sig, total;  // stage
-  uint32_t s_info, s_R, s_avg, s_total;        // side slot
+  uint32_t reach, val, mem, info, sig, total;
+  uint32_t s_info, s_R, s_avg, s_total;
 };
 
 __host__ __device__ inline StreamLayout stream_layout(const StreamChunk &c) {
@@ -106,8 +124,13 @@ __host__ __device__ inline bool stream_fits(const StreamLayout &L) {
   return L.total <= (uint32_t)kStreamStageBytes && L.s_total <= (uint32_t)kStreamSideBytes;
 }
 
+// Bytes of a set chunk's stage.
+__host__ __device__ inline uint32_t stream_bytes(const StreamChunk &c) {
+  return stream_layout(c).total + 16u * (uint32_t)c.nsa;
+}
+
 // A chance chunk's stage: the children's values, then its entries of the
-// three chance arrays (nothing in the side slot).
+// three chance arrays.
 struct ChanceLayout {
   uint32_t vb, nch, vs, total;  // offsets of ch_vb, ch_nch, ch_vs entries; bytes
 };
@@ -148,7 +171,7 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t
 // Bounded wait for the phase of the given parity: false when it gave up
 // (about a second of polling).
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-  const long long t0 = clock64();
+  long long t0 = 0;
   for (int it = 0; it < (1 << 26); ++it) {
     uint32_t ok;
     asm volatile(
@@ -157,382 +180,410 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
         : "r"(bar), "r"(parity)
         : "memory");
     if (ok) return true;
+    if (it == 0) t0 = clock64();
     if (clock64() - t0 > 2000000000ll) break;  // about a second at the boost clock
   }
   return false;
-}
-
-// Issues the copies of chunk d into a stage and a side slot (one thread):
-// the stage's copies counted on its mbarrier bar, the side slot's on sbar (a
-// chance chunk puts nothing in the side slot: its phase of sbar completes
-// with no bytes). Returns false (and issues nothing) if the chunk does not
-// fit. parts: kIssueRest the expected byte counts and every copy but the
-// children's values, kIssueValues the children's values (of everything a
-// backward launch reads, the one input the backward launch before it
-// writes).
-constexpr int kIssueRest = 1, kIssueValues = 2, kIssueAll = 3;
-__device__ __forceinline__ bool stream_issue(const StreamChunk &d, unsigned char *stage, unsigned char *side,
-                                             uint32_t bar, uint32_t sbar, const float2 *reach, const float *v,
-                                             const int32_t *mem_vs, const SetInfo *info, const float *sigma,
-                                             const double *R, const double *avg, const GameView &g, int parts) {
-  if (d.kind == kChunkChance) {
-    if (!chance_fits(d)) return false;
-    const ChanceLayout C = chance_layout(d);
-    const uint32_t s = smem_u32(stage);
-    if (parts & kIssueRest) {
-      mbar_expect_tx(sbar, 0);  // nothing in the side slot: its phase completes at once
-      mbar_expect_tx(bar, C.total);  // the four sizes below add up to this
-      bulk_g2s(s + C.vb, g.ch_vb + d.ka, C.nch - C.vb, bar);
-      bulk_g2s(s + C.nch, g.ch_nch + d.ka, C.vs - C.nch, bar);
-      bulk_g2s(s + C.vs, g.ch_vs + d.ka, C.total - C.vs, bar);
-    }
-    if (parts & kIssueValues) bulk_g2s(s, v + d.va, C.vb, bar);
-    return true;
-  }
-  if (d.kind != kChunkSets) return false;
-  const StreamLayout L = stream_layout(d);
-  if (!stream_fits(L) || d.nra <= 0 || d.nva <= 0 || d.nka <= 0 || d.I1 <= d.I0 || d.nsa <= 0) return false;
-  const uint32_t s = smem_u32(stage), t = smem_u32(side);
-  if (parts & kIssueRest) {
-    mbar_expect_tx(sbar, L.s_total);  // the side slot's three copies
-    bulk_g2s(t + L.s_info, info + d.I0, L.s_R - L.s_info, sbar);
-    bulk_g2s(t + L.s_R, R + d.sa, L.s_avg - L.s_R, sbar);
-    bulk_g2s(t + L.s_avg, avg + d.sa, L.s_total - L.s_avg, sbar);
-    mbar_expect_tx(bar, L.total);  // the stage's five copies
-    bulk_g2s(s + L.reach, reach + d.ra, L.val - L.reach, bar);
-    bulk_g2s(s + L.mem, mem_vs + d.ka, L.info - L.mem, bar);
-    bulk_g2s(s + L.info, info + d.I0, L.sig - L.info, bar);
-    bulk_g2s(s + L.sig, sigma + d.sa, L.total - L.sig, bar);
-  }
-  if (parts & kIssueValues) bulk_g2s(s + L.val, v + d.va, L.mem - L.val, bar);
-  return true;
-}
-
-// The member work of one group of sets (G = 1 or 4) of a staged chunk, by
-// the kStreamCompute compute threads: thread t serves set j = t % G and
-// members t / G, t / G + kStreamCompute / G, ...; writes each member's value and leaves
-// the thread's partial regret and average sums, finished by a butterfly over
-// the warp's lanes that serve the same set, in racc / macc.
-template <int MAXA>
-__device__ __forceinline__ void stream_members(const StreamChunk &d, const StreamLayout &L, const unsigned char *stage,
-                                               int32_t I, int G, float *v, float (&racc)[MAXA],
-                                               float (&macc)[MAXA]) {
-  const int tid = threadIdx.x;
-  const SetInfo *sinfo = reinterpret_cast<const SetInfo *>(stage + L.info);
-  const int gs = G == 4 ? 2 : 0;
-  const int j = tid & (G - 1);
-  const int LPS = kStreamCompute >> gs;
-  const SetInfo si = sinfo[I + j - d.I0];
-  const bool p2 = (si.flags >> 8) & 1;
-  const float2 *sr = reinterpret_cast<const float2 *>(stage + L.reach);
-  const float *sv = reinterpret_cast<const float *>(stage + L.val);
-  const int32_t *sm = reinterpret_cast<const int32_t *>(stage + L.mem);
-  const float *ss = reinterpret_cast<const float *>(stage + L.sig);
-  float sig[MAXA];
-#pragma unroll
-  for (int a = 0; a < MAXA; ++a) {
-    sig[a] = a < si.na ? ss[si.sb - d.sa + a] : 0.f;
-    racc[a] = 0.f;
-    macc[a] = 0.f;
-  }
-  const int32_t rb = si.rank0 - d.ra, kb = si.m0 - d.ka, cbase = si.vb - d.va;
-  for (int32_t q = tid >> gs; q < si.nm; q += LPS) {
-    const float2 r = sr[rb + q * si.rstep];
-    const int32_t h = sm[kb + q];
-    const int32_t cb = cbase + q;  // child a at cb + a * nm (action-major block)
-    float vc[MAXA];
-    float vh = 0.f;
-#pragma unroll
-    for (int a = 0; a < MAXA; ++a) {
-      if (a < si.na) {
-        vc[a] = sv[cb + a * si.nm];
-        vh = vh + sig[a] * vc[a];
-      }
-    }
-    v[h] = vh;
-    const float po = p2 ? r.x : r.y;  // opponent's reach (chance is inside v)
-    const float pw = p2 ? r.y : r.x;  // own reach
-    const float f = (p2 ? -1.f : 1.f) * po;
-#pragma unroll
-    for (int a = 0; a < MAXA; ++a) {
-      if (a < si.na) {
-        racc[a] += f * (vc[a] - vh);
-        macc[a] += pw * sig[a];
-      }
-    }
-  }
-#pragma unroll
-  for (int a = 0; a < MAXA; ++a) {
-    for (int off = G; off < 32; off <<= 1) {
-      racc[a] += __shfl_xor_sync(0xffffffffu, racc[a], off);
-      macc[a] += __shfl_xor_sync(0xffffffffu, macc[a], off);
-    }
-  }
-}
-
-// The slot update of one group by the update warp: lane = a * G + j
-// updates slot a of set j (the warps' partial sums added in warp order),
-// then writes sigma^{t+1} of the group's sets.
-template <int MAXA>
-__device__ __forceinline__ void stream_update(const StreamChunk &d, const StreamLayout &L, const unsigned char *side,
-                                              int32_t I, int G, float *sigma, double *Rg, double *avgg, double wt,
-                                              int rule, int upd, const float (*red)[4][2 * MAXA]) {
-  const int lane = threadIdx.x & 31;
-  const SetInfo *sinfo = reinterpret_cast<const SetInfo *>(side + L.s_info);
-  const int gs = G == 4 ? 2 : 0;
-  const int jj = lane & (G - 1), a = lane >> gs;
-  const SetInfo sj = sinfo[I + jj - d.I0];
-  const bool q2 = (sj.flags >> 8) & 1;
-  const bool live = a < MAXA && a < sj.na && (upd & (q2 ? 2 : 1));
-  float pf = 0.f;
-  if (live) {
-    float r = 0.f, m = 0.f;
-    for (int w = 0; w < kStreamWarps; ++w) {  // warps in order
-      r += red[w][jj][a];
-      m += red[w][jj][MAXA + a];
-    }
-    const int32_t qs = sj.sb + a;
-    const double *sR = reinterpret_cast<const double *>(side + L.s_R);
-    const double *sA = reinterpret_cast<const double *>(side + L.s_avg);
-    double Rn, Sn;
-    pf = narrow_pos(slot_terms(sR[qs - d.sa], sA[qs - d.sa], widen(r), widen(m), wt, rule, Rn, Sn));
-    Rg[qs] = Rn;
-    avgg[qs] = Sn;
-  }
-  float tot = 0.f;  // positive parts in action order
-  for (int b = 0; b < MAXA; ++b) {
-    const float x = __shfl_sync(0xffffffffu, pf, (b * G + jj) & 31);
-    if (b < sj.na) tot += x;
-  }
-  if (live) sigma[sj.sb + a] = match(pf, tot, sj.na);
 }
 
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
-// The compute threads' work on a staged chance chunk: thread t sums the
-// children of nodes I0 + t, I0 + t + kStreamCompute, ... left to right (as
-// bwd_chance does: the same value bit for bit) and writes the node's value.
-__device__ __forceinline__ void stream_chance_chunk(const StreamChunk &d, const unsigned char *stage, float *v) {
+// How a depth's teams are laid out: teams of `warps` warps, `teams` of them in
+// a CTA, stages of `bytes` bytes (at least the depth's largest chunk).
+struct StreamShape {
+  int32_t teams, warps, bytes;
+};
+
+// The stages take kStreamDynSmem bytes at most. Teams are as small as they can
+// be with kStreamMinWarps warps in a CTA, and larger where the depth has too
+// few chunks to give every team one. (Two warps a team, 14 warps, instead of
+// seven teams of one at depths of 13 KB tiles: 134 us an iteration instead of
+// 131; groups packed into chunks of 6 KB at depths with fewer chunks than
+// teams: 35 us instead of 27 for an endgame of a million edges.)
+inline StreamShape stream_shape(int64_t largest, int64_t chunks, int sms) {
+  StreamShape z;
+  z.bytes = (int32_t)((largest + 127) / 128 * 128);
+  const int fit = std::max(1, std::min(kStreamMaxWarps, kStreamDynSmem / (kStreamStages * z.bytes)));
+  auto teams = [&](int t) { return std::min(fit, kStreamMaxWarps / t); };
+  int t = 1;
+  while (t < 8 && (t * teams(t) < kStreamMinWarps || chunks <= (int64_t)sms * teams(2 * t))) t *= 2;
+  z.warps = t;
+  z.teams = teams(t);
+  return z;
+}
+
+// What lane `lane` of a team's first warp copies of every chunk: copy lane of
+// the stage, in the stage's order (set chunks: reach, values, members,
+// descriptors, strategy, R, average sums; chance chunks: values, first slots,
+// child counts, own slots). w: the chunk's words with the first element and
+// the count (the descriptors': the end); shift: log2 of an element's bytes.
+struct StreamCopy {
+  const void *base;
+  int32_t w, shift;
+};
+
+constexpr int kIssueRest = 1, kIssueValues = 2, kIssueAll = 3;
+
+// Issues the copies of a chunk into a stage, by all lanes of one warp, each of
+// which passes word `lane` of the chunk and its copy of a set and of a chance
+// chunk. Returns false (and issues nothing) if the chunk does not fit. parts:
+// kIssueRest the expected byte count and every copy but the children's
+// values, kIssueValues the children's values (of everything a backward launch
+// reads, the one input the backward launch before it writes).
+__device__ __forceinline__ bool stream_issue(int32_t word, const StreamCopy &sets, const StreamCopy &chance,
+                                             unsigned char *stage, uint32_t bytes, uint32_t bar, int parts) {
+  const int lane = threadIdx.x & 31;
+  const int32_t kind = __shfl_sync(0xffffffffu, word, 10);
+  const StreamCopy c = kind == kChunkChance ? chance : sets;
+  const int32_t e = __shfl_sync(0xffffffffu, word, c.w), x = __shfl_sync(0xffffffffu, word, c.w + 1);
+  const int32_t cnt = c.w == 0 ? x - e : x;
+  const uint32_t n = c.base ? (uint32_t)cnt << c.shift : 0u;
+  uint32_t end = n;  // of this copy in the stage
+#pragma unroll
+  for (int off = 1; off < 8; off <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, end, off);
+    if (lane >= off) end += y;
+  }
+  const uint32_t total = __shfl_sync(0xffffffffu, end, 7);
+  if ((kind != kChunkSets && kind != kChunkChance) || __any_sync(0xffffffffu, c.base && cnt <= 0) || total > bytes)
+    return false;
+  if (lane == 0 && (parts & kIssueRest)) mbar_expect_tx(bar, total);
+  __syncwarp();
+  if (n > 0 && (parts & (lane == (kind == kChunkChance ? 0 : 1) ? kIssueValues : kIssueRest)))
+    bulk_g2s(smem_u32(stage) + end - n, static_cast<const unsigned char *>(c.base) + ((size_t)e << c.shift), n, bar);
+  return true;
+}
+
+__device__ __forceinline__ StreamChunk stream_chunk(int32_t word) {  // from its words, one a lane
+  StreamChunk d;
+  int32_t *w = reinterpret_cast<int32_t *>(&d);
+#pragma unroll
+  for (int i = 0; i < 11; ++i) w[i] = __shfl_sync(0xffffffffu, word, i);
+  return d;
+}
+
+// The members q0, q0 + step, ... of one staged set of NA actions (0: na, at
+// most MAXA): writes their values and adds their terms to racc (the regret
+// sums, player 2's with the sign still to be turned) and own (the sum of the
+// set's own reach, which times the strategy is the average sum). Two members
+// a step, every load before the first use.
+template <int MAXA, int NA>
+__device__ __forceinline__ void stream_sum(const float2 *sr, int32_t rstep, const int32_t *sm, const float *sv,
+                                           const float (&sig)[MAXA], int32_t nm, int32_t na, bool p2, int32_t q0,
+                                           int32_t step, float *v, float (&racc)[MAXA], float &own) {
+  constexpr int A = NA ? NA : MAXA;
+  auto member = [&](const float2 &r, int32_t h, const float(&vc)[A]) {
+    float vh = 0.f;
+#pragma unroll
+    for (int a = 0; a < A; ++a)
+      if (NA || a < na) vh = vh + sig[a] * vc[a];
+    v[h] = vh;
+    const float po = p2 ? r.x : r.y;  // opponent's reach (chance is inside v)
+    own += p2 ? r.y : r.x;
+#pragma unroll
+    for (int a = 0; a < A; ++a)
+      if (NA || a < na) racc[a] += po * (vc[a] - vh);
+  };
+  int32_t q = q0;
+  for (; q + step < nm; q += 2 * step) {
+    const float2 r0 = sr[q * rstep], r1 = sr[(q + step) * rstep];
+    const int32_t h0 = sm[q], h1 = sm[q + step];
+    float c0[A], c1[A];
+#pragma unroll
+    for (int a = 0; a < A; ++a) {
+      c0[a] = NA || a < na ? sv[q + a * nm] : 0.f;  // an action-major block
+      c1[a] = NA || a < na ? sv[q + step + a * nm] : 0.f;
+    }
+    member(r0, h0, c0);
+    member(r1, h1, c1);
+  }
+  if (q < nm) {
+    const float2 r0 = sr[q * rstep];
+    const int32_t h0 = sm[q];
+    float c0[A];
+#pragma unroll
+    for (int a = 0; a < A; ++a) c0[a] = NA || a < na ? sv[q + a * nm] : 0.f;
+    member(r0, h0, c0);
+  }
+}
+
+// The member work of one group of sets (G = 1 or 4) of a staged chunk by the
+// n threads of a team: thread t serves set j = t % G and members t / G,
+// t / G + n / G, ...; writes each member's value and leaves the thread's
+// partial sums, finished by a butterfly over the warp's lanes that serve the
+// same set, in racc (regret) and own (own reach). Sets of two or three
+// actions, as all of a warp's usually are, take code of their own: predicates
+// over MAXA actions doubled a member's instructions, and the members'
+// instructions are what a large depth's time goes into.
+template <int MAXA>
+__device__ __forceinline__ void stream_members(const StreamChunk &d, const StreamLayout &L, const unsigned char *stage,
+                                               int32_t I, int G, int t, int n, float *v, float (&racc)[MAXA],
+                                               float &own) {
+  const SetInfo *sinfo = reinterpret_cast<const SetInfo *>(stage + L.info);
+  const int gs = G == 4 ? 2 : 0;
+  const SetInfo si = sinfo[I + (t & (G - 1)) - d.I0];
+  const bool p2 = (si.flags >> 8) & 1;
+  const float2 *sr = reinterpret_cast<const float2 *>(stage + L.reach) + (si.rank0 - d.ra);
+  const float *sv = reinterpret_cast<const float *>(stage + L.val) + (si.vb - d.va);
+  const int32_t *sm = reinterpret_cast<const int32_t *>(stage + L.mem) + (si.m0 - d.ka);
+  const float *ss = reinterpret_cast<const float *>(stage + L.sig) + (si.sb - d.sa);
+  float sig[MAXA];
+#pragma unroll
+  for (int a = 0; a < MAXA; ++a) {
+    sig[a] = a < si.na ? ss[a] : 0.f;
+    racc[a] = 0.f;
+  }
+  own = 0.f;
+  const int32_t q0 = t >> gs, step = n >> gs;
+  int na = MAXA;
+  if (__all_sync(0xffffffffu, si.na == 2)) {
+    na = 2;
+    stream_sum<MAXA, 2>(sr, si.rstep, sm, sv, sig, si.nm, 2, p2, q0, step, v, racc, own);
+  } else if (__all_sync(0xffffffffu, si.na == 3)) {
+    na = 3;
+    stream_sum<MAXA, 3>(sr, si.rstep, sm, sv, sig, si.nm, 3, p2, q0, step, v, racc, own);
+  } else {
+    stream_sum<MAXA, 0>(sr, si.rstep, sm, sv, sig, si.nm, si.na, p2, q0, step, v, racc, own);
+  }
+  __syncwarp();
+  for (int off = G; off < 32; off <<= 1) {
+    own += __shfl_xor_sync(0xffffffffu, own, off);
+#pragma unroll
+    for (int a = 0; a < MAXA; ++a)
+      if (a < na) racc[a] += __shfl_xor_sync(0xffffffffu, racc[a], off);
+  }
+}
+
+// What lane a * G + j of the updating warp needs of slot a of set j; read
+// before the stage is refilled.
+struct StreamSlot {
+  double R, S;
+  float sig, sign;  // the strategy; of the regret terms
+  int32_t q, na;    // the slot, the set's actions
+  bool live;
+};
+
+__device__ __forceinline__ StreamSlot stream_slot(const StreamChunk &d, const StreamLayout &L,
+                                                  const unsigned char *stage, int32_t I, int G, int maxa, int upd) {
+  const int lane = threadIdx.x & 31;
+  const int gs = G == 4 ? 2 : 0;
+  const int j = lane & (G - 1), a = lane >> gs;
+  const SetInfo si = reinterpret_cast<const SetInfo *>(stage + L.info)[I + j - d.I0];
+  StreamSlot z;
+  z.na = si.na;
+  z.q = si.sb + a;
+  z.live = a < maxa && a < si.na && (upd & ((si.flags >> 8) & 1 ? 2 : 1));
+  z.R = z.S = 0.0;
+  z.sig = 0.f;
+  z.sign = (si.flags >> 8) & 1 ? -1.f : 1.f;
+  if (z.live) {
+    const double *sR = reinterpret_cast<const double *>(stage + L.total);
+    z.sig = reinterpret_cast<const float *>(stage + L.sig)[z.q - d.sa];
+    z.R = sR[z.q - d.sa];
+    z.S = sR[d.nsa + z.q - d.sa];
+  }
+  return z;
+}
+
+// The slot update of one group by one warp: lane = a * G + j updates slot a of
+// set j with its regret total r and the set's own reach, then writes sigma^{t+1} of the group's sets.
+template <int MAXA>
+__device__ __forceinline__ void stream_update(const StreamSlot &z, int G, float r, float own, float *sigma, double *Rg,
+                                              double *avgg, double wt, int rule) {
+  const int j = threadIdx.x & (G - 1);
+  float pf = 0.f;
+  if (z.live) {
+    double Rn, Sn;
+    pf = narrow_pos(slot_terms(z.R, z.S, widen(z.sign * r), widen(own * z.sig), wt, rule, Rn, Sn));
+    Rg[z.q] = Rn;
+    avgg[z.q] = Sn;
+  }
+  float tot = 0.f;  // positive parts in action order
+#pragma unroll
+  for (int b = 0; b < MAXA; ++b) {
+    const float x = __shfl_sync(0xffffffffu, pf, (b * G + j) & 31);
+    if (b < z.na) tot += x;
+  }
+  if (z.live) sigma[z.q] = match(pf, tot, z.na);
+}
+
+// A team's work on a staged chance chunk: its thread t of n sums the children
+// of nodes I0 + t, I0 + t + n, ... left to right (as bwd_chance does: the same
+// value bit for bit) and writes the node's value.
+__device__ __forceinline__ void stream_chance_chunk(const StreamChunk &d, const unsigned char *stage, int t, int n,
+                                                    float *v) {
   const ChanceLayout C = chance_layout(d);
   const float *sv = reinterpret_cast<const float *>(stage);
   const int32_t *svb = reinterpret_cast<const int32_t *>(stage + C.vb);
   const int32_t *snc = reinterpret_cast<const int32_t *>(stage + C.nch);
   const int32_t *svs = reinterpret_cast<const int32_t *>(stage + C.vs);
-  for (int32_t i = d.I0 + (int32_t)threadIdx.x; i < d.I1; i += kStreamCompute) {
+  for (int32_t i = d.I0 + t; i < d.I1; i += n) {
     const int32_t k = i - d.ka;
     const float *p = sv + (svb[k] - d.va);
-    const int32_t n = snc[k];
+    const int32_t nc = snc[k];
     float sum = 0.f;
-    for (int32_t c = 0; c < n; ++c) sum = sum + p[c];
+    for (int32_t c = 0; c < nc; ++c) sum = sum + p[c];
     v[svs[k]] = sum;
   }
 }
 
-// Threads of a streaming CTA: kStreamCompute compute threads, the copy warp
-// (its first lane issues every bulk copy) and the update warp (the slot
-// updates).
-constexpr int kStreamThreads = kStreamCompute + 64;
-
-// Grid: the streaming CTAs over chunks [c0, c1) of this depth (its set
+// Grid: CTAs of shape.teams teams over chunks [c0, c1) of this depth (its set
 // chunks, then its chance chunks; a depth with wide chance nodes does not
-// stream). Chunk i of a CTA uses stage i % kStreamStages (the compute
-// threads' data) and side slot i % kStreamSideSlots (set records, R and
-// average for the update warp). Barriers of a streaming CTA (every wait
-// bounded):
-//   full[s]   the copies of the chunk in stage s have landed (bytes counted)
-//   empty[s]  the compute threads are done with stage s
-//   sfull[k]  the copies of the chunk in side slot k have landed
-//   sfree[k]  the update warp is done with side slot k
-//   rfull[p]  the compute threads have written the partial sums red[p]
-//   rempty[p] the update warp has consumed red[p]
-// The copy warp refills stage s with chunk i + kStreamStages as soon as the
-// compute threads are done with chunk i and the update warp is done with
-// the side slot's previous chunk; the compute warps never wait for a slot
-// update, and the update warp, which works through the chunks in order,
-// never holds up a refill of a stage. Each barrier's phases are waited for
-// in order and a phase cannot complete twice before its waiter sees it: a
-// stage is refilled only after its chunk was consumed, a side slot only
-// after the update warp released it.
+// stream). Chunk i of a team uses stage i % kStreamStages. Barriers of a team
+// (every wait bounded):
+//   full[s]  the copies of the chunk in stage s have landed (bytes counted)
+//   sync     teams of several warps: all threads are done with a group (or a
+//            chance chunk) and have left their partial sums in red
+// A stage is refilled only after every thread of the team is done with its
+// chunk, so a phase cannot complete twice before its waiters see it. red is
+// double-buffered: the first warp has read red[p] of a group before it
+// arrives at the next group's sync, which the others pass before they write
+// red[p] again.
 template <int MAXA>
-__global__ void __launch_bounds__(kStreamThreads, 2)
+__global__ void __launch_bounds__(32 * kStreamMaxWarps, 1)
     bwd_stream_kernel(GameView g, StateView<float> st, const SetInfo *info, const StreamChunk *chunks, int32_t c0,
-                      int32_t c1, int rule, int upd, int *err, int early) {
-  static_assert(kStreamSideSlots >= 2 * kStreamStages, "side slots must outlast the stages by a full ring");
-  constexpr int S = kStreamStages, K = kStreamSideSlots;
-  extern __shared__ __align__(128) unsigned char s_stage[];  // stages, then side slots
-  __shared__ __align__(8) uint64_t s_full[S], s_empty[S], s_sfull[K], s_sfree[K], s_rfull[2], s_rempty[2];
-  __shared__ StreamChunk s_desc[S], s_sdesc[K];
-  __shared__ float s_red[2][kStreamWarps][4][2 * MAXA];
+                      int32_t c1, int rule, int upd, int *err, int early, StreamShape shape) {
+  constexpr int S = kStreamStages;
+  static_assert(S == 2, "the descriptors in flight are the current chunk's, the next one's and the one's after");
+  extern __shared__ __align__(128) unsigned char s_stage[];  // [team][stage]
+  __shared__ __align__(8) uint64_t s_full[kStreamMaxWarps][S], s_sync[kStreamMaxWarps];
+  __shared__ float s_red[2][kStreamMaxWarps][4][MAXA + 1];
   if (!early) pdl_enter();
-  const int32_t b = (int32_t)blockIdx.x;
-  const int32_t nb = (int32_t)gridDim.x;
-  const int tid = threadIdx.x, lane = tid & 31;
-  const int role = tid < kStreamCompute ? 0 : (tid < kStreamCompute + 32 ? 1 : 2);  // compute, copy, update
-  const bool producer = tid == kStreamCompute;
-  unsigned char *s_side = s_stage + S * kStreamStageBytes;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int team = warp / shape.warps, tw = warp - team * shape.warps;  // warp tw of the team
+  const int n = 32 * shape.warps, t = 32 * tw + lane;                   // thread t of n
+  const int32_t stride = (int32_t)gridDim.x * shape.teams;
+  const int32_t first = c0 + (int32_t)blockIdx.x + team * (int32_t)gridDim.x;
+  const uint32_t full0 = smem_u32(&s_full[team][0]), sync = smem_u32(&s_sync[team]);
+  unsigned char *ring = s_stage + (size_t)team * S * shape.bytes;
   if ((smem_u32(s_stage) & 15u) != 0u) {  // bulk copies need 16-byte aligned destinations
-    if (tid == 0) atomicExch(err, 1);
+    if (threadIdx.x == 0) atomicExch(err, 1);
     return;
   }
-  auto issue = [&](int32_t i, const StreamChunk &dsc, int parts) {
-    const int s = i % S, k = i % K;
-    if (parts & kIssueRest) {  // before the copies whose barriers publish them
-      s_desc[s] = dsc;
-      s_sdesc[k] = dsc;
-    }
-    return stream_issue(dsc, s_stage + s * kStreamStageBytes, s_side + k * kStreamSideBytes, smem_u32(&s_full[s]),
-                        smem_u32(&s_sfull[k]), st.reach, st.v, g.mem_vs, info, st.sigma, st.R, st.avg, g, parts);
-  };
-  int32_t issued = 0;  // chunks issued (copy thread)
-  if (producer) {
-    for (int s = 0; s < S; ++s) {
-      mbar_init(smem_u32(&s_full[s]), 1);
-      mbar_init(smem_u32(&s_empty[s]), kStreamCompute);
-    }
-    for (int k = 0; k < K; ++k) {
-      mbar_init(smem_u32(&s_sfull[k]), 1);
-      mbar_init(smem_u32(&s_sfree[k]), 32);
-    }
-    for (int p = 0; p < 2; ++p) {
-      mbar_init(smem_u32(&s_rfull[p]), kStreamCompute);
-      mbar_init(smem_u32(&s_rempty[p]), 32);
-    }
+  if (t == 0) {
+    for (int s = 0; s < S; ++s) mbar_init(full0 + 8 * s, 1);
+    mbar_init(sync, n);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    // the first chunks of this CTA. early: the launch before this one is
-    // the backward launch of the next depth, which writes only values of
-    // this depth's children (and its own slots), so everything else is
-    // copied before waiting for that launch to finish (programmatic
-    // dependent launch), and the children's values after
-    for (int i = 0; i < S; ++i) {
-      const int32_t c = c0 + b + i * nb;
-      if (c >= c1) break;
-      if (!issue(i, chunks[c], early ? kIssueRest : kIssueAll)) {
-        atomicExch(err, 1);  // a chunk larger than a stage: never issued, every wait below gives up
-        break;
-      }
-      ++issued;
-    }
-    if (early) {
-      pdl_enter();
-      for (int i = 0; i < issued; ++i) issue(i, chunks[c0 + b + i * nb], kIssueValues);
+  }
+  __syncthreads();  // barriers initialised (the only CTA-wide barrier)
+  auto word = [&](int32_t c) {  // word `lane` of chunk c
+    return lane < 16 && c < c1 ? __ldg(reinterpret_cast<const int32_t *>(chunks + c) + lane) : 0;
+  };
+  StreamCopy sets{nullptr, 0, 0}, chance{nullptr, 0, 0};  // this lane's copies
+  if (lane == 0) { sets = {st.reach, 2, 3}; chance = {st.v, 4, 2}; }
+  if (lane == 1) { sets = {st.v, 4, 2}; chance = {g.ch_vb, 6, 2}; }
+  if (lane == 2) { sets = {g.mem_vs, 6, 2}; chance = {g.ch_nch, 6, 2}; }
+  if (lane == 3) { sets = {info, 0, 5}; chance = {g.ch_vs, 6, 2}; }
+  if (lane == 4) sets = {st.sigma, 8, 2};
+  if (lane == 5) sets = {st.R, 8, 3};
+  if (lane == 6) sets = {st.avg, 8, 3};
+  auto issue = [&](int32_t i, int32_t w, int parts) {
+    return stream_issue(w, sets, chance, ring + (i % S) * shape.bytes, (uint32_t)shape.bytes, full0 + 8 * (i % S),
+                        parts);
+  };
+  int32_t w0 = word(first), w1 = word(first + stride);
+  // fault-injection hook (err[1], set on the host): issue no copy after the
+  // first ones, so that the waits for the next chunk run out
+  const bool stall = reinterpret_cast<volatile const int *>(err)[1] != 0;
+  int32_t issued = 0;  // chunks whose copies have been issued (the team's first warp)
+  bool ok = true;
+  // the first chunks of the team. early: the launch before this one is the
+  // backward launch of the next depth, which writes only values of this
+  // depth's children (and its own slots), so everything else is copied before
+  // waiting for that launch to finish (programmatic dependent launch), and
+  // the children's values after
+  if (tw == 0) {
+    for (int i = 0; i < S && ok && first + i * stride < c1; ++i) {
+      ok = issue(i, i ? w1 : w0, early ? kIssueRest : kIssueAll);  // a chunk larger than a stage: the waits give up
+      if (ok) ++issued;
     }
   }
-  if (early && !producer) pdl_enter();
-  __syncthreads();  // barriers initialised, first copies issued (the only CTA-wide barrier)
-
-  if (role == 1) {
-    if (!producer) return;
-    // fault-injection hook (err[1], set on the host): issue nothing more, so
-    // the other roles' bounded waits for the next chunk run out; the chunks
-    // already issued land and are consumed before the CTA leaves
-    if (reinterpret_cast<volatile const int *>(err)[1] != 0) return;
-    // refill stage i % S with chunk i + S once chunk i is consumed and the
-    // side slot's previous chunk released
-    int32_t seen = 0;  // chunks known to have landed
-    bool ok = issued == S || c0 + b + issued * nb >= c1;
-    for (int32_t i = 0; ok; ++i) {
-      const int32_t cn = c0 + b + (i + S) * nb;
-      if (cn >= c1) break;
-      const StreamChunk nd = chunks[cn];  // its latency overlaps the waits
-      const int s = i % S;
-      if (!mbar_wait(smem_u32(&s_empty[s]), (uint32_t)((i / S) & 1))) { ok = false; break; }
-      seen = i + 1;
-      const int32_t j = i + S - K;  // the side slot's previous chunk
-      if (j >= 0 && !mbar_wait(smem_u32(&s_sfree[(i + S) % K]), (uint32_t)((j / K) & 1))) { ok = false; break; }
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      if (!issue(i + S, nd, kIssueAll)) { ok = false; break; }
-      issued = i + S + 1;
-    }
-    if (!ok) {
-      atomicExch(err, 1);
-      // let every copy in flight land before the thread leaves (bounded):
-      // the last chunks issued into each stage and side slot
-      for (int32_t i = max(seen, issued - S); i < issued; ++i)
-        mbar_wait(smem_u32(&s_full[i % S]), (uint32_t)((i / S) & 1));
-      for (int32_t i = max(0, issued - K); i < issued; ++i)
-        mbar_wait(smem_u32(&s_sfull[i % K]), (uint32_t)((i / K) & 1));
-    }
-    return;
+  if (early) {
+    pdl_enter();
+    if (tw == 0)
+      for (int i = 0; i < issued; ++i) issue(i, i ? w1 : w0, kIssueValues);
   }
-
-  if (role == 2) {
-    const double wt = avg_weight(*st.t + 1, rule);
-    int32_t grp = 0;  // groups done by this CTA (selects red[grp & 1] and the barrier phases)
-    for (int32_t i = 0;; ++i) {
-      const int32_t c = c0 + b + i * nb;
-      if (c >= c1) break;
-      const int k = i % K;
-      if (!mbar_wait(smem_u32(&s_sfull[k]), (uint32_t)((i / K) & 1))) {
-        atomicExch(err, 1);
-        return;
-      }
-      const StreamChunk d = s_sdesc[k];  // written before the side slot's copies were issued
-      if (d.kind == kChunkSets) {
-        const StreamLayout L = stream_layout(d);
-        const unsigned char *side = s_side + k * kStreamSideBytes;
-        const SetInfo *sinfo = reinterpret_cast<const SetInfo *>(side + L.s_info);
-        for (int32_t I = d.I0; I < d.I1; ++grp) {
-          const int G = sinfo[I - d.I0].flags & 7;
-          const int p = grp & 1;
-          if (!mbar_wait(smem_u32(&s_rfull[p]), (uint32_t)((grp >> 1) & 1))) {
-            atomicExch(err, 1);
-            return;
-          }
-          stream_update<MAXA>(d, L, side, I, G, st.sigma, st.R, st.avg, wt, rule, upd, s_red[p]);
-          mbar_arrive(smem_u32(&s_rempty[p]));
-          I += G;
-        }
-      }
-      mbar_arrive(smem_u32(&s_sfree[k]));
-    }
-    return;
-  }
-
-  int32_t grp = 0;
-  for (int32_t i = 0;; ++i) {
-    const int32_t c = c0 + b + i * nb;
+  const double wt = avg_weight(*st.t + 1, rule);
+  uint32_t phase = 0;  // of sync: groups and chance chunks done
+  int32_t i = 0;
+  for (; ok; ++i) {
+    const int32_t c = first + i * stride;
     if (c >= c1) break;
+    const int32_t w2 = word(c + 2 * stride);  // its latency overlaps this chunk's work
     const int s = i % S;
-    if (!mbar_wait(smem_u32(&s_full[s]), (uint32_t)((i / S) & 1))) {
-      atomicExch(err, 1);
-      return;
-    }
-    const StreamChunk d = s_desc[s];
-    const unsigned char *stage = s_stage + s * kStreamStageBytes;
+    ok = __all_sync(0xffffffffu, mbar_wait(full0 + 8 * s, (uint32_t)((i / S) & 1)));
+    if (!ok) break;
+    const StreamChunk d = stream_chunk(w0);
+    const unsigned char *stage = ring + s * shape.bytes;
+    auto refill = [&]() {  // every thread of the team is done with the stage
+      if (tw == 0 && c + 2 * stride < c1 && !stall) {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        if (issue(i + S, w2, kIssueAll)) issued = i + S + 1;
+        else ok = false;
+      }
+    };
+    auto team_sync = [&]() {
+      __syncwarp();
+      if (shape.warps > 1) {
+        mbar_arrive(sync);
+        ok = __all_sync(0xffffffffu, mbar_wait(sync, phase & 1));
+        ++phase;
+      }
+    };
     if (d.kind == kChunkChance) {
-      stream_chance_chunk(d, stage, st.v);
-      mbar_arrive(smem_u32(&s_empty[s]));
-      continue;
-    }
-    const StreamLayout L = stream_layout(d);
-    const SetInfo *sinfo = reinterpret_cast<const SetInfo *>(stage + L.info);
-    for (int32_t I = d.I0; I < d.I1; ++grp) {
-      const int G = sinfo[I - d.I0].flags & 7;
-      const int p = grp & 1;
-      float racc[MAXA], macc[MAXA];
-      stream_members<MAXA>(d, L, stage, I, G, st.v, racc, macc);
-      // red[p] is free once the update warp consumed it two groups ago
-      if (grp >= 2 && !mbar_wait(smem_u32(&s_rempty[p]), (uint32_t)(((grp >> 1) & 1) ^ 1u))) {
-        atomicExch(err, 1);
-        return;
-      }
-      if (lane < G) {
+      stream_chance_chunk(d, stage, t, n, st.v);
+      team_sync();
+      if (ok) refill();
+    } else {
+      const StreamLayout L = stream_layout(d);
+      const SetInfo *sinfo = reinterpret_cast<const SetInfo *>(stage + L.info);
+      for (int32_t I = d.I0; I < d.I1 && ok;) {
+        const int G = sinfo[I - d.I0].flags & 7;
+        float racc[MAXA], own;
+        stream_members<MAXA>(d, L, stage, I, G, t, n, st.v, racc, own);
+        StreamSlot z;
+        if (tw == 0) z = stream_slot(d, L, stage, I, G, MAXA, upd);
+        const int a = lane >> (G == 4 ? 2 : 0), j = lane & (G - 1);
+        float r = 0.f;
+        if (shape.warps > 1) {
+          float(*red)[4][MAXA + 1] = s_red[phase & 1];
+          if (lane < G) {
 #pragma unroll
-        for (int a = 0; a < MAXA; ++a) {
-          s_red[p][tid >> 5][lane][a] = racc[a];
-          s_red[p][tid >> 5][lane][MAXA + a] = macc[a];
+            for (int b = 0; b < MAXA; ++b) red[warp][lane][b] = racc[b];
+            red[warp][lane][MAXA] = own;
+          }
+          team_sync();
+          if (ok && tw == 0 && a < MAXA) {
+            own = 0.f;
+            for (int w = 0; w < shape.warps; ++w) {  // warps in order
+              r += red[warp + w][j][a];
+              own += red[warp + w][j][MAXA];
+            }
+          }
+        } else {
+          __syncwarp();
+#pragma unroll
+          for (int b = 0; b < MAXA; ++b)
+            if (a == b) r = racc[b];
         }
+        if (!ok) break;
+        I += G;
+        if (I >= d.I1) refill();
+        if (tw == 0) stream_update<MAXA>(z, G, r, own, st.sigma, st.R, st.avg, wt, rule);
       }
-      mbar_arrive(smem_u32(&s_rfull[p]));
-      if (I + G >= d.I1) mbar_arrive(smem_u32(&s_empty[s]));  // this thread is done with stage s
-      I += G;
     }
+    w0 = w1;
+    w1 = w2;
   }
-  // every chunk issued was waited on (full[s]) by the compute threads and
-  // (sfull[k]) by the update warp before they left
+  if (!ok) {
+    atomicExch(err, 1);
+    // let every copy in flight land before the warp leaves (bounded)
+    for (int32_t k = max(0, issued - S); k < issued; ++k)
+      if (k >= i) mbar_wait(full0 + 8 * (k % S), (uint32_t)((k / S) & 1));
+  }
 }
 
 }  // namespace cfr

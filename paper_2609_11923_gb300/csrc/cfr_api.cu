@@ -69,6 +69,7 @@ struct cfr_handle {
   std::vector<SetInfo> set_info;
   std::vector<StreamChunk> stream_chunks;
   std::vector<int32_t> stream_c0, stream_ok;
+  std::vector<int64_t> stream_bytes;  // per depth: bytes of the largest chunk's stage
   Buf b_set_info, b_stream_chunks;
   // CFR_EXEC_AUTO, small games: the whole game resident in one CTA (0: not)
   uint32_t solo_smem = 0;
@@ -159,14 +160,15 @@ static void plan(cfr_handle *h) {
 // Set descriptors and chunks of the streaming backward (FP32, member order,
 // sets of at most 8 actions). A group is a tile of kTileSets sets (members'
 // reach interleaved) or one untiled set; a chunk is a run of whole groups of
-// one depth whose staged bytes (stream_layout) fit one stage. A depth whose
-// largest group does not fit cannot stream.
+// one depth whose staged bytes fit kStreamPackBytes, or one group that is
+// larger. A depth whose largest group does not fit a stage cannot stream.
 static void build_stream(cfr_handle *h) {
   const Compiled &c = h->c;
   h->set_info.clear();
   h->stream_chunks.clear();
   h->stream_c0.assign(c.D + 1, 0);
   h->stream_ok.assign(c.D, 0);
+  h->stream_bytes.assign(c.D, 0);
   if (h->precision != CFR_P32 || c.int_edge.empty() || c.max_act > 8 || c.I == 0) return;
   h->set_info.resize(c.I);
   for (int64_t d = 0; d < c.D; ++d) {
@@ -237,26 +239,35 @@ static void build_stream(cfr_handle *h) {
     // kernel does not have
     bool ok = d > 0 && is1 > is0 && c.level_wide[d + 1] == c.level_wide[d];
     std::vector<StreamChunk> ch;
+    // a chunk takes several groups only where the depth has enough for every
+    // team of the GPU: a team works through its chunk's groups one by one
+    const int64_t mem = c.iset_mem[is1] - c.iset_mem[is0], kids = c.level_begin[d + 2] - c.level_begin[d + 1];
+    const int64_t pack = std::min<int64_t>(kStreamPackBytes, (12 * mem + 4 * kids) / kStreamSpread);
     for (int32_t I = is0; ok && I < is1;) {
       int32_t J = I + (h->set_info[I].flags & 7);
       if (!stream_fits(stream_layout(make(I, J)))) { ok = false; break; }
       while (J < is1) {  // extend by whole groups while the stage holds them
         const int32_t K = J + (h->set_info[J].flags & 7);
-        if (!stream_fits(stream_layout(make(I, K)))) break;
+        const StreamChunk k = make(I, K);
+        if (!stream_fits(stream_layout(k)) || stream_bytes(k) > pack) break;
         J = K;
       }
       ch.push_back(make(I, J));
+      h->stream_bytes[d] = std::max<int64_t>(h->stream_bytes[d], stream_bytes(ch.back()));
       I = J;
     }
     // then the depth's narrow chance nodes, in chunks of consecutive nodes
     // whose children (consecutive value slots) and chance-array entries fit
     // a stage; each node's child run must lie inside its chunk's
     const int32_t q0 = c.level_chance[d], q1 = c.level_chance[d + 1];
+    const int64_t pack_ch = std::clamp<int64_t>((12 * int64_t(q1 - q0) + 4 * kids) / kStreamSpread, kStreamChanceBytes,
+                                                kStreamPackBytes);
     for (int32_t i = q0; ok && i < q1;) {
       int32_t j = i + 1;
       if (!chance_fits(make_chance(i, j))) { ok = false; break; }
-      while (j < q1 && j - i < kStreamChanceMax && chance_fits(make_chance(i, j + 1))) ++j;
+      while (j < q1 && j - i < kStreamChanceMax && chance_layout(make_chance(i, j + 1)).total <= pack_ch) ++j;
       const StreamChunk k = make_chance(i, j);
+      h->stream_bytes[d] = std::max<int64_t>(h->stream_bytes[d], chance_layout(k).total);
       for (int32_t q = i; q < j; ++q)
         if (c.ch_vb[q] < k.va || (int64_t)c.ch_vb[q] + c.ch_nch[q] > (int64_t)k.va + k.nva) ok = false;
       ch.push_back(k);
@@ -323,6 +334,7 @@ extern "C" int cfr_compile(const cfr_game_spec *spec, const cfr_options *opt, cf
     if (lp == kStreamLanes && h->stream_ok[d]) h->level_lanes[d] = kStreamLanes;
     if ((!lp || (lp == kStreamLanes && !h->stream_ok[d])) && c.level_tiled[d])
       h->level_lanes[d] = std::min(h->level_lanes[d], kTiledLanes);
+    if (!lp && h->stream_ok[d] && c.level_mean_members[d] >= (c.level_tiled[d] ? kStreamAutoTiled : kStreamAutoMembers)) h->level_lanes[d] = kStreamLanes;
     any_tiled = any_tiled || c.level_tiled[d];
     tot_mem += c.level_mean_members[d] * (c.level_iset[2 * d + 2] - c.level_iset[2 * d]);
   }
@@ -739,11 +751,11 @@ extern "C" int cfr_bind(cfr_handle *h, void *arena, size_t bytes, void *stream) 
 // ------------------------------------------------------------ iteration
 // upd: the players whose sets update (bit 0 player 1, bit 1 player 2); the
 // depth-0 launch of the pass that updates player 2 advances t.
-// Streaming CTAs of the streaming backward of depth d: two per SM, never
+// Streaming CTAs of the streaming backward of depth d: one per SM, never
 // more than the depth has chunks.
 static int stream_ctas(const cfr_handle *h, int d) {
   const int n = h->stream_c0[d + 1] - h->stream_c0[d];
-  return std::max(1, std::min(n, 2 * device_sms()));
+  return std::max(1, std::min(n, device_sms()));
 }
 
 // Blocks of the backward launch of depth d (chance blocks, wide chunks, then
@@ -777,7 +789,8 @@ static int launch_bwd(cfr_handle *h, int d, cudaStream_t s, int upd = 3, bool pd
     // of depth d < D - 1 is the backward launch of depth d + 1
     CK(launch_bwd_stream(h->maxa_tier, nb_is, s, game_view(h), state_view<float>(h), h->p<SetInfo>(h->b_set_info),
                          h->p<StreamChunk>(h->b_stream_chunks), h->stream_c0[d], h->stream_c0[d + 1], h->rule, upd,
-                         h->p<int>(h->b_err), pdl, pdl && d + 1 < h->c.D));
+                         h->p<int>(h->b_err), pdl, pdl && d + 1 < h->c.D,
+                         stream_shape(h->stream_bytes[d], h->stream_c0[d + 1] - h->stream_c0[d], device_sms())));
     return CFR_OK;
   }
   // at least one block: the depth-0 launch also advances t
@@ -1600,24 +1613,44 @@ extern "C" int cfr_autotune(cfr_handle *h, int reps, void *stream) {
   rc = h->precision == CFR_P64 ? enqueue_start<double>(h, s) : enqueue_start<float>(h, s);
   if (rc == CFR_OK) rc = run_iter();  // realistic reach and values for the trials
   for (int64_t d = c.D - 1; d > h->top_k && rc == CFR_OK; --d) {  // the near-root kernel has one shape
-    int best = h->level_lanes[d];
+    const int first = h->level_lanes[d];
+    int best = first;
     float best_ms = 1e30f;
     std::vector<int> cd = cand;
-    // the streaming form works on one group of sets at a time with the whole
-    // CTA: a candidate only where sets are long
+    // the streaming form works through a team's sets one group at a time: a
+    // candidate only where sets are long
     if (h->stream_ok[d] && c.level_mean_members[d] >= kStreamMinMembers) cd.push_back(kStreamLanes);
-    for (int L : cd) {
+    auto time = [&](int L, int n, auto &&launch, float *ms) -> int {
       h->level_lanes[d] = L;
-      rc = h->precision == CFR_P64 ? launch_bwd<double>(h, (int)d, s) : launch_bwd<float>(h, (int)d, s);
-      if (rc) break;
       CK(cudaEventRecord(e0, s));
-      for (int r = 0; r < reps && rc == CFR_OK; ++r)
-        rc = h->precision == CFR_P64 ? launch_bwd<double>(h, (int)d, s) : launch_bwd<float>(h, (int)d, s);
+      for (int r = 0; r < n; ++r)
+        if (int e = launch()) return e;
       CK(cudaEventRecord(e1, s));
       CK(cudaEventSynchronize(e1));
+      CK(cudaEventElapsedTime(ms, e0, e1));
+      return CFR_OK;
+    };
+    auto run_depth = [&]() -> int {
+      return h->precision == CFR_P64 ? launch_bwd<double>(h, (int)d, s) : launch_bwd<float>(h, (int)d, s);
+    };
+    for (int L : cd) {  // by itself first: one launch, and more if that was not hopeless
       float ms = 0.f;
-      CK(cudaEventElapsedTime(&ms, e0, e1));
+      rc = time(L, 1, run_depth, &ms);
+      if (rc) break;
+      if (ms * reps > 2.f * best_ms) continue;
+      rc = time(L, reps, run_depth, &ms);
+      if (rc) break;
       if (ms < best_ms) { best_ms = ms; best = L; }
+    }
+    // A depth's launch repeated by itself finds its inputs in L2, which in an
+    // iteration the launches before have left elsewhere (lane groups at two
+    // depths of the 27M-node card game that streams faster: an iteration of
+    // 145 us instead of 131). So the winner has to win in whole iterations too.
+    if (rc == CFR_OK && best != first) {
+      float ms_first = 0.f, ms_best = 0.f;
+      rc = time(first, reps, run_iter, &ms_first);
+      if (rc == CFR_OK) rc = time(best, reps, run_iter, &ms_best);
+      if (ms_best > 0.99f * ms_first) best = first;
     }
     h->level_lanes[d] = best;
   }

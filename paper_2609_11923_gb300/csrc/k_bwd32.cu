@@ -8,9 +8,10 @@ namespace cfr {
 template <int MA>
 static cudaError_t stream_one(int grid, cudaStream_t s, GameView g, StateView<float> st, const SetInfo *info,
                               const StreamChunk *chunks, int c0, int c1, int rule, int upd, int *err, bool pdl,
-                              int early) {
-  return launch_k(bwd_stream_kernel<MA>, grid, kStreamThreads, (size_t)kStreamDynSmem, s, pdl, g, st, info, chunks,
-                  c0, c1, rule, upd, err, early);
+                              int early, StreamShape shape) {
+  const size_t dyn = (size_t)shape.teams * kStreamStages * shape.bytes;
+  return launch_k(bwd_stream_kernel<MA>, grid, 32 * shape.teams * shape.warps, dyn, s, pdl, g, st, info, chunks, c0,
+                  c1, rule, upd, err, early, shape);
 }
 
 cudaError_t prepare_bwd_stream() {
@@ -23,10 +24,10 @@ cudaError_t prepare_bwd_stream() {
 
 cudaError_t launch_bwd_stream(int maxa, int grid, cudaStream_t s, GameView g, StateView<float> st,
                               const SetInfo *info, const StreamChunk *chunks, int c0, int c1, int rule, int upd,
-                              int *err, bool pdl, bool early) {
+                              int *err, bool pdl, bool early, StreamShape shape) {
   const int e = early ? 1 : 0;
-  if (maxa == 4) return stream_one<4>(grid, s, g, st, info, chunks, c0, c1, rule, upd, err, pdl, e);
-  if (maxa == 8) return stream_one<8>(grid, s, g, st, info, chunks, c0, c1, rule, upd, err, pdl, e);
+  if (maxa == 4) return stream_one<4>(grid, s, g, st, info, chunks, c0, c1, rule, upd, err, pdl, e, shape);
+  if (maxa == 8) return stream_one<8>(grid, s, g, st, info, chunks, c0, c1, rule, upd, err, pdl, e, shape);
   return cudaErrorInvalidValue;
 }
 }  // namespace cfr

@@ -34,7 +34,7 @@ inline cudaError_t launch_k(void (*kern)(KArgs...), int grid, int block, size_t 
 // before waiting for that launch.
 cudaError_t launch_bwd_stream(int maxa, int grid, cudaStream_t s, GameView g, StateView<float> st,
                               const SetInfo *info, const StreamChunk *chunks, int c0, int c1, int rule, int upd,
-                              int *err, bool pdl, bool early);
+                              int *err, bool pdl, bool early, StreamShape shape);
 // Allows the streaming kernel its dynamic shared memory (call before the
 // first launch, outside any stream capture; idempotent).
 cudaError_t prepare_bwd_stream();

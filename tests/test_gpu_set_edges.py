@@ -45,3 +45,24 @@ def test_fp64_sums_equal_the_oracle_at_every_group_edge(lanes, a, b):
         np.testing.assert_array_equal(R, o.R, err_msg="m=%d" % m)
         np.testing.assert_array_equal(avg, o.sbar, err_msg="m=%d" % m)
         s.close()
+
+
+@pytest.mark.parametrize("a,b", [(2, 3), (3, 2), (4, 1), (5, 8)])
+@pytest.mark.parametrize("m", [1, 31, 32, 33, 63, 65, 170, 257, 800])
+def test_streamed_sets_at_the_edges_of_teams_and_steps(m, a, b):
+    """One set of the streaming backward, from one member to stages so large
+    that few teams fit. One iteration from the uniform strategy: a regret is a
+    sum of m terms that add up to at most 2 in size (payoffs in [-1, 1] times
+    the deal's probabilities), each with a few roundings, in sums of at most
+    m / 32 + 12 terms one after another."""
+    g = two_level_game(m, a, b)
+    s = cfr.Solver(g, precision=cfr.P32, exec_form=cfr.EXEC_LEVELS, lanes_per_set=cfr.STREAM_LANES)
+    assert cfr.cfr_export_array(s.h, "stream_ok")[1:].all()
+    s.iterate(1)
+    s.synchronize()
+    R, avg, _ = s.get_state()
+    o = oracle.solve(g, 1)
+    tol = 2.0 * (m / 32 + 12 + 12) * 2.0 ** -24
+    assert np.abs(R - o.R).max() <= tol
+    assert (np.abs(avg - o.sbar) <= tol * o.sbar).all()
+    s.close()
