@@ -157,6 +157,8 @@ static void plan(cfr_handle *h) {
   h->plan_bytes = cur;
 }
 
+constexpr int kFewSets = 4 * 152;  // no more than a set for each scheduler of a GB300
+
 // Set descriptors and chunks of the streaming backward (FP32, member order,
 // sets of at most 8 actions). A group is a tile of kTileSets sets (members'
 // reach interleaved) or one untiled set; a chunk is a run of whole groups of
@@ -331,6 +333,10 @@ extern "C" int cfr_compile(const cfr_game_spec *spec, const cfr_options *opt, cf
   build_stream(h);
   for (int64_t d = 0; d < c.D; ++d) {
     h->level_lanes[d] = (lp && lp != kStreamLanes) ? lp : pick(c.level_mean_members[d]);
+    // FP64 with few sets: a warp a set (three depths of 153-459 sets of 120
+    // members in an 11M-node card game: 30 us each by 8 lanes, 13-17 by 32)
+    if (!lp && widest == 8 && c.level_mean_members[d] > 16.0 && c.level_iset[2 * d + 2] - c.level_iset[2 * d] <= kFewSets)
+      h->level_lanes[d] = 32;
     if (lp == kStreamLanes && h->stream_ok[d]) h->level_lanes[d] = kStreamLanes;
     if ((!lp || (lp == kStreamLanes && !h->stream_ok[d])) && c.level_tiled[d])
       h->level_lanes[d] = std::min(h->level_lanes[d], kTiledLanes);
@@ -758,6 +764,13 @@ static int stream_ctas(const cfr_handle *h, int d) {
   return std::max(1, std::min(n, device_sms()));
 }
 
+// Whether depth d has so few warps of sets that each block takes one before any
+// takes two (bwd_level_kernel).
+static bool bwd_spread(const cfr_handle *h, int d) {
+  const int lanes = h->level_lanes[d], nis = h->levels[d].is1 - h->levels[d].is0;
+  return lanes <= 32 && nis > 0 && (nis * (int64_t)lanes + 31) / 32 <= (int64_t)device_sms() * (kThreads / 32);
+}
+
 // Blocks of the backward launch of depth d (chance blocks, wide chunks, then
 // the information-set work; the streaming form has only its CTAs over the
 // depth's set and chance chunks).
@@ -769,6 +782,7 @@ static void bwd_blocks(const cfr_handle *h, int d, int *nb_ch, int *nb_wide, int
   *nb_ch = nch > 0 && lanes != kStreamLanes ? grid_for(nch, kThreads) : 0;
   *nb_wide = d > 0 ? w.wc1 - w.wc0 : 0;
   if (lanes == kStreamLanes) *nb_is = nis > 0 ? stream_ctas(h, d) : 0;
+  else if (bwd_spread(h, d)) *nb_is = std::min((nis * lanes + 31) / 32, device_sms());
   else *nb_is = nis > 0 ? grid_for(nis, kThreads / lanes) : 0;
 }
 
@@ -794,9 +808,10 @@ static int launch_bwd(cfr_handle *h, int d, cudaStream_t s, int upd = 3, bool pd
     return CFR_OK;
   }
   // at least one block: the depth-0 launch also advances t
+  const int flags = (pdl && h->c.D > 1 ? kBwdEarly : 0) |  // (with one depth the launch before may be this one's own)
+                    (bwd_spread(h, d) ? kBwdSpread : 0);
   CK(launch_bwd_level<T>(h->maxa_tier, lanes, std::max(1, nb_ch + nb_wide + nb_is), s, game_view(h), state_view<T>(h),
-                         w, nb_ch, h->rule, upd, (d == 0 && (upd & 2)) ? 1 : 0, pdl,
-                         pdl && h->c.D > 1));  // (with one depth the launch before may be this one's own)
+                         w, nb_ch, h->rule, upd, (d == 0 && (upd & 2)) ? 1 : 0, pdl, flags));
   return CFR_OK;
 }
 

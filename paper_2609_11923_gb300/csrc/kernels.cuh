@@ -764,6 +764,202 @@ __device__ __forceinline__ void load_head(const GameView &g, const StateView<T> 
   }
 }
 
+// A warp's sets in step: its 32 / LANES groups run one set each through the
+// same instructions, shorter sets (and groups without a set: na = 0, no
+// members) idle along. With a loop and sync masks of each group's own the
+// groups of a warp drifted apart and every instruction was issued once per
+// group, which an FP64 pipe that takes 16-19 cycles for a warp instruction
+// feels most. FP64 sets of two and three actions have code of their own
+// where all of a warp's are (the pipe takes as long for a predicated
+// instruction as for another). One iteration: the 11M-node card game in FP64
+// 568 -> 404 us (autotuned 464 -> 350), an 80k-node random tree in two half
+// passes 236 -> 195; in FP32 a 2.8M-node random tree 72 -> 66, a card game of
+// 81k nodes 29.0 -> 26.9.
+
+// FP64: the members of each group's set, none of more than NA actions: their
+// values, and in r[i] and m[i] the totals of slot lane + i * LANES, summed in
+// member order. Members past a set's end add zeros.
+template <int MAXA, int LANES, int NA, int PER>
+__device__ __forceinline__ void warp_chains(const GameView &g, const StateView<double> &st,
+                                            const SetHead<double, MAXA> &hd, bool p2, int lane, int32_t longest,
+                                            double *rows, double (&r)[PER], double (&m)[PER]) {
+  constexpr int C = 2 * NA, ACC = (C + LANES - 1) / LANES;  // chains: regret, then average, by action
+  constexpr int U = LANES <= 8 ? 2 : 1;                     // chunks in flight
+  constexpr bool EXACT = NA < MAXA;                         // every set of the warp has NA actions (or none)
+  const int wl = threadIdx.x & 31, g0 = wl - lane;
+  const int32_t m0 = hd.m0, m1 = hd.m1, M = m1 - m0;
+  double acc[ACC];
+#pragma unroll
+  for (int i = 0; i < ACC; ++i) acc[i] = 0.0;
+  int32_t ps[U], ir[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) member_idx(g, m0 + u * LANES + lane, m1, hd.mr, ps[u], ir[u]);
+  for (int32_t k0 = 0; k0 < longest; k0 += U * LANES) {
+    int32_t qs[U], jr[U];  // the next step's indices
+#pragma unroll
+    for (int u = 0; u < U; ++u) member_idx(g, m0 + k0 + (U + u) * LANES + lane, m1, hd.mr, qs[u], jr[u]);
+    double2 re[U];
+    double vc[U][NA], d[U][NA], mm[U][NA];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const bool in = ps[u] >= 0;
+      const int32_t cb = hd.vb + k0 + u * LANES + lane;
+      re[u] = make_double2(0.0, 0.0);
+      if (in) re[u] = st.reach[ir[u]];
+#pragma unroll
+      for (int a = 0; a < NA; ++a) vc[u][a] = in && (EXACT || a < hd.na) ? st.v[cb + a * M] : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      double vh = hd.sig[0] * vc[u][0];
+#pragma unroll
+      for (int a = 1; a < NA; ++a) vh = vh + hd.sig[a] * vc[u][a];
+      if (ps[u] >= 0) st.v[ps[u]] = vh;
+      const double f = p2 ? -re[u].x : re[u].y;  // opponent's reach, the regret's sign
+      const double pw = p2 ? re[u].y : re[u].x;
+#pragma unroll
+      for (int a = 0; a < NA; ++a) {
+        d[u][a] = f * (vc[u][a] - vh);
+        mm[u][a] = pw * hd.sig[a];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int32_t cnt = longest - k0 - u * LANES;
+      if (cnt <= 0) break;
+#pragma unroll
+      for (int a = 0; a < NA; ++a) {
+        rows[a * kChainRow + wl] = d[u][a];
+        rows[(NA + a) * kChainRow + wl] = mm[u][a];
+      }
+      __syncwarp();
+      const double *row = rows + lane * kChainRow + g0;
+      if (cnt >= LANES) {
+#pragma unroll
+        for (int j = 0; j < LANES; ++j)
+#pragma unroll
+          for (int i = 0; i < ACC; ++i)
+            if (lane + i * LANES < C) acc[i] = acc[i] + row[i * LANES * kChainRow + j];
+      } else {
+#pragma unroll 1
+        for (int j = 0; j < cnt; ++j)
+#pragma unroll
+          for (int i = 0; i < ACC; ++i)
+            if (lane + i * LANES < C) acc[i] = acc[i] + row[i * LANES * kChainRow + j];
+      }
+      __syncwarp();
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) { ps[u] = qs[u]; ir[u] = jr[u]; }
+  }
+#pragma unroll
+  for (int p = 0; p < PER; ++p) {
+    r[p] = p < ACC ? acc[p] : 0.0;
+    m[p] = 0.0;
+#pragma unroll
+    for (int i = 0; i < ACC; ++i) {  // chain NA + lane + p * LANES
+      const int c = NA + lane + p * LANES;
+      const double x = __shfl_sync(0xffffffffu, acc[i], c % LANES, LANES);
+      if (c / LANES == i) m[p] = x;
+    }
+  }
+}
+
+template <typename T, int MAXA, int LANES>
+constexpr bool kInStep = MAXA <= 8 && LANES >= 4 && LANES <= 32;
+
+template <typename T, int MAXA, int LANES>
+__device__ __forceinline__ void bwd_sets(const GameView &g, const StateView<T> &st, const SetHead<T, MAXA> &hd,
+                                         bool p2, int lane, double wt, int rule, int upd, double *rows) {
+  constexpr unsigned full = 0xffffffffu;
+  constexpr int PER = (MAXA + LANES - 1) / LANES;  // slots of a lane: lane, lane + LANES, ...
+  const int32_t sb = hd.sb, na = hd.na;
+  const int most = __reduce_max_sync(full, na);
+  T r[PER], m[PER];
+  if constexpr (sizeof(T) == 8) {
+    const int32_t longest = __reduce_max_sync(full, hd.m1 - hd.m0);
+    if (most == 2 && __all_sync(full, na == 2 || na == 0))
+      warp_chains<MAXA, LANES, 2, PER>(g, st, hd, p2, lane, longest, rows, r, m);
+    else if (most == 3 && __all_sync(full, na == 3 || na == 0))
+      warp_chains<MAXA, LANES, 3, PER>(g, st, hd, p2, lane, longest, rows, r, m);
+    else
+      warp_chains<MAXA, LANES, MAXA, PER>(g, st, hd, p2, lane, longest, rows, r, m);
+  } else {
+    const int32_t m0 = hd.m0, m1 = hd.m1, vb = hd.vb;
+    T racc[MAXA], macc[MAXA];
+#pragma unroll
+    for (int a = 0; a < MAXA; ++a) racc[a] = macc[a] = T(0);
+    auto add = [&](const T(&d)[MAXA], const T(&mm)[MAXA]) {
+#pragma unroll
+      for (int a = 0; a < MAXA; ++a) {
+        racc[a] += d[a];
+        macc[a] += mm[a];
+      }
+    };
+    constexpr int U = LANES <= 8 ? 2 : 1;  // chunks in flight
+    int32_t ps[U], ir[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) member_idx(g, m0 + u * LANES + lane, m1, hd.mr, ps[u], ir[u]);
+    for (int32_t k0 = m0; k0 < m1; k0 += U * LANES) {
+      int32_t qs[U], jr[U];  // the next step's indices
+#pragma unroll
+      for (int u = 0; u < U; ++u) member_idx(g, k0 + (U + u) * LANES + lane, m1, hd.mr, qs[u], jr[u]);
+      T d[U][MAXA], mm[U][MAXA];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        member_data<T, MAXA, false>(g, st, k0 + u * LANES + lane, m0, m1, vb, na, p2, hd.sig, ps[u], ir[u], d[u], mm[u]);
+#pragma unroll
+      for (int u = 0; u < U; ++u) add(d[u], mm[u]);
+#pragma unroll
+      for (int u = 0; u < U; ++u) { ps[u] = qs[u]; ir[u] = jr[u]; }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int a = 0; a < MAXA; ++a) {
+      if (a < most) {
+        racc[a] = group_sum_butterfly<LANES>(racc[a], full);
+        macc[a] = group_sum_butterfly<LANES>(macc[a], full);
+      }
+    }
+#pragma unroll
+    for (int p = 0; p < PER; ++p) {
+      r[p] = m[p] = T(0);
+#pragma unroll
+      for (int a = 0; a < MAXA; ++a)
+        if (a == lane + p * LANES) { r[p] = racc[a]; m[p] = macc[a]; }
+    }
+  }
+  // alternating updates: the other player's sets only pass their values up
+  const bool live = upd & (p2 ? 2 : 1);
+  T pos[PER];
+#pragma unroll
+  for (int p = 0; p < PER; ++p) {
+    const int a = lane + p * LANES;
+    double x = 0.0;
+    if (live && a < na) {
+      if constexpr (LANES >= MAXA) {
+        double Rn, Sn;
+        x = slot_terms(hd.R, hd.S, as_double(r[p]), as_double(m[p]), wt, rule, Rn, Sn);
+        st.R[sb + a] = Rn;
+        st.avg[sb + a] = Sn;
+      } else {
+        x = slot_update(st.R, st.avg, sb + a, as_double(r[p]), as_double(m[p]), wt, rule);
+      }
+    }
+    if constexpr (sizeof(T) == 8) pos[p] = x;
+    else pos[p] = narrow_pos(x);
+  }
+  T tot = T(0);  // in action order; slots past the set's add zero
+#pragma unroll
+  for (int a = 0; a < MAXA; ++a)
+    if (a < most) tot += __shfl_sync(full, pos[a / LANES], a % LANES, LANES);
+#pragma unroll
+  for (int p = 0; p < PER; ++p) {
+    const int a = lane + p * LANES;
+    if (live && a < na) st.sigma[sb + a] = match(pos[p], tot, na);
+  }
+}
+
 template <typename T, int MAXA, int LANES, bool PERSIST>
 __device__ __forceinline__ void bwd_set(const GameView &g, const StateView<T> &st, const SetHead<T, MAXA> &hd, bool p2,
                                         int lane, unsigned mask, double wt, int rule, int upd, double *rows) {
@@ -1015,11 +1211,16 @@ __device__ __forceinline__ void bwd_set_block(const GameView &g, const StateView
 // chunk, then the information-set groups (LANES == kThreads: one set per
 // block). early: the first set of every group is read up before waiting for
 // the launch before, which writes nothing of this depth but its children's
-// values or its members' reach.
+// values or its members' reach. spread: the depth has fewer warps of sets than
+// blocks could hold, and each block takes one warp's sets before any takes two
+// (in FP64 eight warps on an SM wait for its one FP64 pipe: a depth of
+// 153 sets of 120 members 34 us -> 25).
+constexpr int kBwdEarly = 1, kBwdSpread = 2;
 template <typename T, int MAXA, int LANES>
 __global__ void __launch_bounds__(kThreads, MAXA > 8 ? 1 : (MAXA <= 4 ? 4 : 3) - (sizeof(T) == 8 ? 1 : 0)) bwd_level_kernel(GameView g, StateView<T> st, LevelWork w,
                                                             int nb_chance, int rule, int upd, int bump_t,
-                                                            int early) {
+                                                            int flags) {
+  const bool early = flags & kBwdEarly;
   const int nb_wide = w.wc1 - w.wc0;
   if ((int)blockIdx.x < nb_chance) {
     pdl_enter();
@@ -1038,20 +1239,30 @@ __global__ void __launch_bounds__(kThreads, MAXA > 8 ? 1 : (MAXA <= 4 ? 4 : 3) -
   } else {
     constexpr int GPB = kThreads / LANES;
     const int first = nb_chance + nb_wide;
-    const int gid = ((int)blockIdx.x - first) * GPB + (int)threadIdx.x / LANES;
-    const int ngroups = ((int)gridDim.x - first) * GPB;
+    const int blk = (int)blockIdx.x - first, nblk = (int)gridDim.x - first;
+    const int gid = flags & kBwdSpread
+                        ? ((int)threadIdx.x / 32 * nblk + blk) * (32 / LANES) + (int)(threadIdx.x % 32) / LANES
+                        : blk * GPB + (int)threadIdx.x / LANES;
+    const int ngroups = nblk * GPB;
     const int lane = threadIdx.x % LANES;
     const unsigned mask = group_mask<LANES>();
     __shared__ double s_rows[kThreads / 32][kChainDoubles<T, MAXA, LANES>];
     int32_t I = w.is0 + gid;
-    SetHead<T, MAXA> hd;
+    int32_t Iw = I;  // in step: every lane stays while the warp's first set is one
+    if constexpr (kInStep<T, MAXA, LANES>) Iw = I - (int)(threadIdx.x % 32) / LANES;
+    SetHead<T, MAXA> hd = {};
     if (!early) pdl_enter();
     if (I < w.is1) load_head<T, MAXA, LANES, false>(g, st, I, lane, hd);
     if (early) pdl_enter();
     const double wt = avg_weight(*st.t + 1, rule);
-    while (I < w.is1) {
-      bwd_set<T, MAXA, LANES, false>(g, st, hd, I >= w.is2, lane, mask, wt, rule, upd, s_rows[threadIdx.x / 32]);
+    while (Iw < w.is1) {
+      if constexpr (kInStep<T, MAXA, LANES>)
+        bwd_sets<T, MAXA, LANES>(g, st, hd, I >= w.is2, lane, wt, rule, upd, s_rows[threadIdx.x / 32]);
+      else
+        bwd_set<T, MAXA, LANES, false>(g, st, hd, I >= w.is2, lane, mask, wt, rule, upd, s_rows[threadIdx.x / 32]);
       I += ngroups;
+      Iw += ngroups;
+      if (kInStep<T, MAXA, LANES>) hd = {};
       if (I < w.is1) load_head<T, MAXA, LANES, false>(g, st, I, lane, hd);
     }
   }

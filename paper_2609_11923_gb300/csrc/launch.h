@@ -42,7 +42,7 @@ cudaError_t prepare_bwd_stream();
 template <typename T>
 cudaError_t launch_bwd_level(int maxa, int lanes, int grid, cudaStream_t s, GameView g, StateView<T> st,
                              LevelWork w, int nb_chance, int rule, int upd, int bump, bool pdl = false,
-                             bool early = false);
+                             int flags = 0);
 
 // query_occupancy != nullptr: only report resident blocks per SM of the
 // chosen instance (nothing is launched).

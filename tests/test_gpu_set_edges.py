@@ -66,3 +66,34 @@ def test_streamed_sets_at_the_edges_of_teams_and_steps(m, a, b):
     assert np.abs(R - o.R).max() <= tol
     assert (np.abs(avg - o.sbar) <= tol * o.sbar).all()
     s.close()
+
+
+def mixed_sets_game(most):
+    """One depth of player 1's and player 2's sets of 1 to 70 members and 2 to
+    `most` actions, side by side in the same warps; random payoffs."""
+    rng = np.random.default_rng(most)
+    sets = [(m, 2 + (i * 5 + m) % (most - 1)) for i, m in enumerate([1, 2, 5, 9, 33, 3, 70, 4, 8, 17, 1, 31, 32, 6] * 3)]
+    members = [I for I, (m, _) in enumerate(sets) for _ in range(m)]
+    p = rng.gamma(1.0, size=len(members))
+    nodes = [(gg.CHANCE, -1, list(range(1, len(members) + 1)), list(p / p.sum()), 0.0)] + [None] * len(members)
+    for k, I in enumerate(members):
+        leaves = []
+        for _ in range(sets[I][1]):
+            leaves.append(len(nodes))
+            nodes.append((gg.TERMINAL, -1, [], None, float(rng.uniform(-1, 1))))
+        nodes[1 + k] = (gg.P1 if I % 3 else gg.P2, I, leaves, None, 0.0)
+    return gg.from_lists(nodes, [(0 if I % 3 else 1, a) for I, (_, a) in enumerate(sets)])
+
+
+@pytest.mark.parametrize("order", [cfr.ORDER_SIMULTANEOUS, cfr.ORDER_ALTERNATING])
+@pytest.mark.parametrize("lanes", [0, 4, 8, 16, 32])
+@pytest.mark.parametrize("most", [4, 8])
+def test_sets_of_different_sizes_share_a_warp(most, lanes, order):
+    g = mixed_sets_game(most)
+    s = cfr.Solver(g, precision=cfr.P64, exec_form=cfr.EXEC_LEVELS, lanes_per_set=lanes, order=order)
+    s.iterate(30)
+    R, avg, _ = s.get_state()
+    o = oracle.solve(g, 30, order=order)
+    np.testing.assert_array_equal(R, o.R)
+    np.testing.assert_array_equal(avg, o.sbar)
+    s.close()
