@@ -316,7 +316,11 @@ constexpr int kLongSet = 32;
 
 // One set by the LANES lanes of a group: its members' values, and the set's
 // totals into def_r and def_m (see bwd_set, whose sums these are). Every load
-// of a step is issued before the first value is used.
+// of a step is issued before the first value is used. The groups of a warp run
+// in step (see warp_chains): shorter sets, and groups without a set (no
+// members, no actions), idle along, adding zeros. (50 iterations of one-card poker 174 -> 156 us;
+// ten in FP64 of an 80k-node random tree, whose near-root depths these are, by
+// halves 1,970 -> 1,911.)
 struct GroupSet {  // a set's record
   int32_t sb, na, m0, M, vb;
   int2 rk;
@@ -333,8 +337,8 @@ template <typename T, int MODE> __device__ __forceinline__ GroupSet group_record
 }
 
 template <typename T, int MAXA, int LANES, int MODE>
-__device__ __forceinline__ void group_members(const GroupView<T> &g, const GroupSet &s, bool p2, int lane, unsigned mask,
-                                              int upd, double *rows) {
+__device__ __forceinline__ void group_members(const GroupView<T> &g, const GroupSet &s, bool p2, int lane,
+                                              int32_t longest, int upd, double *rows) {
   constexpr bool C = MODE == kCluster, CHAINS = sizeof(T) == 8;
   constexpr int U = LANES <= 8 ? 2 : 1;  // members of a lane in flight
   const int32_t sb = s.sb, na = s.na, m0 = s.m0, M = s.M, vb = s.vb;
@@ -348,7 +352,7 @@ __device__ __forceinline__ void group_members(const GroupView<T> &g, const Group
   }
 #pragma unroll
   for (int i = 0; i < kChainAcc<MAXA, LANES>; ++i) acc[i] = 0.0;
-  for (int32_t k0 = 0; k0 < M; k0 += U * LANES) {
+  for (int32_t k0 = 0; k0 < longest; k0 += U * LANES) {
     int32_t h[U];
     vec2_t<T> r[U];
     T vc[U][MAXA];
@@ -365,7 +369,7 @@ __device__ __forceinline__ void group_members(const GroupView<T> &g, const Group
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      if (k0 + u * LANES >= M) break;  // the same for the whole group
+      if (k0 + u * LANES >= longest) break;
       T vh = T(0);
 #pragma unroll
       for (int a = 0; a < MAXA; ++a)
@@ -385,8 +389,8 @@ __device__ __forceinline__ void group_members(const GroupView<T> &g, const Group
             mm[a] = pw * sig[a];
           }
         }
-        const int32_t left = M - k0 - u * LANES;
-        accumulate_chains<MAXA, LANES>(rows, left < LANES ? left : LANES, na, mask, d, mm, acc);
+        const int32_t left = longest - k0 - u * LANES;
+        accumulate_chains<MAXA, LANES>(rows, left < LANES ? left : LANES, MAXA, 0xffffffffu, d, mm, acc);
       } else {
 #pragma unroll
         for (int a = 0; a < MAXA; ++a)
@@ -395,20 +399,21 @@ __device__ __forceinline__ void group_members(const GroupView<T> &g, const Group
       }
     }
   }
-  if (!(upd & (p2 ? 2 : 1))) return;  // alternating updates: the other player's sets only pass their values up
+  const bool live = upd & (p2 ? 2 : 1);  // alternating updates: the other player's sets only pass their values up
   if constexpr (CHAINS) {
 #pragma unroll
     for (int i = 0; i < kChainAcc<MAXA, LANES>; ++i) {
       const int c = lane + i * LANES;
-      if (c < na) g.def_r[sb + c] = acc[i];
-      else if (c >= MAXA && c - MAXA < na) g.def_m[sb + c - MAXA] = acc[i];
+      if (live && c < na) g.def_r[sb + c] = acc[i];
+      else if (live && c >= MAXA && c - MAXA < na) g.def_m[sb + c - MAXA] = acc[i];
     }
   } else {
-    spw = group_sum_butterfly<LANES>(spw, mask);
-    if (lane == 0) g.def_m[sb] = spw;
-    group_sum_scatter<LANES, MAXA>(racc, lane, mask);
+    __syncwarp();
+    spw = group_sum_butterfly<LANES>(spw, 0xffffffffu);
+    group_sum_scatter<LANES, MAXA>(racc, lane, 0xffffffffu);
+    if (live && na > 0 && lane == 0) g.def_m[sb] = spw;
     constexpr int STEP = MAXA <= LANES ? LANES / MAXA : 1, PER = MAXA <= LANES ? 1 : MAXA / LANES;
-    if (lane % STEP == 0) {
+    if (live && lane % STEP == 0) {
 #pragma unroll
       for (int i = 0; i < PER; ++i)
         if (lane / STEP * PER + i < na) g.def_r[sb + lane / STEP * PER + i] = racc[i];
@@ -423,14 +428,29 @@ __device__ __forceinline__ void group_members(const GroupView<T> &g, const Group
 // card poker and random trees, whose warps mix two to four actions, 3-6%
 // slower that way).
 template <typename T, int MAXA, int LANES, int MODE>
-__device__ __forceinline__ void group_set(const GroupView<T> &g, int32_t I, bool p2, int lane, unsigned mask, int upd,
+__device__ __forceinline__ void group_set(const GroupView<T> &g, int32_t I, bool in, bool p2, int lane, int upd,
                                           double *rows) {
-  const GroupSet s = group_record<T, MODE>(g, I);
+  GroupSet s = {};
+  if (in) s = group_record<T, MODE>(g, I);
+  const int32_t longest = __reduce_max_sync(0xffffffffu, s.M);
   if constexpr (MAXA > 4) {
-    if (s.na <= 2) return group_members<T, 2, LANES, MODE>(g, s, p2, lane, mask, upd, rows);
-    if (s.na <= 4) return group_members<T, 4, LANES, MODE>(g, s, p2, lane, mask, upd, rows);
+    const int most = __reduce_max_sync(0xffffffffu, s.na);
+    if (most <= 2) return group_members<T, 2, LANES, MODE>(g, s, p2, lane, longest, upd, rows);
+    if (most <= 4) return group_members<T, 4, LANES, MODE>(g, s, p2, lane, longest, upd, rows);
   }
-  group_members<T, MAXA, LANES, MODE>(g, s, p2, lane, mask, upd, rows);
+  group_members<T, MAXA, LANES, MODE>(g, s, p2, lane, longest, upd, rows);
+}
+
+// The sets I0 .. I1 (from I2 on player 2's) of one depth by `all` threads,
+// thread ct of them.
+template <typename T, int MAXA, int LANES, int MODE>
+__device__ __forceinline__ void group_sets(const GroupView<T> &g, int32_t I0, int32_t I2, int32_t I1, int ct, int all,
+                                           int upd, double *rows) {
+  const int sub = ct % 32 / LANES, lane = ct % LANES;
+  for (int32_t W = I0 + ct / 32 * (32 / LANES); W < I1; W += all / LANES) {  // the warp's first set
+    const int32_t I = W + sub;
+    group_set<T, MAXA, LANES, MODE>(g, I, I < I1, I >= I2, lane, upd, rows);
+  }
 }
 
 // One long set by a warp with the sums of group_set<.., 8, ..>: lane l of
@@ -537,28 +557,46 @@ __device__ __forceinline__ T slot_write(const GroupView<T> &g, int32_t q, const 
 }
 
 template <typename T, int MAXA, int MODE>
-__device__ __forceinline__ void group_update(const GroupView<T> &g, int32_t I, int a, unsigned mask, double wt,
-                                             int rule) {
+__device__ __forceinline__ void group_update(const GroupView<T> &g, int32_t I, bool in, int a, double wt, int rule) {
   constexpr int L = kUpdateLanes;
-  const int32_t sb = ldk<MODE>(g.iset_slot + I), na = ldk<MODE>(g.iset_slot + I + 1) - sb, q = sb + a;
+  constexpr unsigned full = 0xffffffffu;  // the groups of a warp run in step
+  int32_t sb = 0, na = 0;
+  if (in) {
+    sb = ldk<MODE>(g.iset_slot + I);
+    na = ldk<MODE>(g.iset_slot + I + 1) - sb;
+  }
+  const int32_t q = sb + a;
   T pos = T(0), more = T(0);
   if (a < na) pos = slot_write(g, q, slot_totals<T, MODE>(g, sb, q), wt, rule);
   T tot = T(0);  // positive parts in action order
 #pragma unroll
   for (int b = 0; b < L; ++b) {
-    const T x = __shfl_sync(mask, pos, b, L);
+    const T x = __shfl_sync(full, pos, b, L);
     if (b < na) tot += x;
   }
-  if (MAXA > L && na > L) {  // the same for the whole group
+  if (MAXA > L && __any_sync(full, na > L)) {
     if (a + L < na) more = slot_write(g, q + L, slot_totals<T, MODE>(g, sb, q + L), wt, rule);
 #pragma unroll
     for (int b = 0; b < L; ++b) {
-      const T x = __shfl_sync(mask, more, b, L);
+      const T x = __shfl_sync(full, more, b, L);
       if (b + L < na) tot += x;
     }
     if (a + L < na) g.sigma[q + L] = match(more, tot, na);
   }
   if (a < na) g.sigma[q] = match(pos, tot, na);
+}
+
+// The slots of sets I0 .. I1 by `all` threads, thread ct of them: set I always
+// by the same threads, whatever I0 (their L1 holds its R and avg).
+template <typename T, int MAXA, int MODE>
+__device__ __forceinline__ void group_updates(const GroupView<T> &g, int32_t I0, int32_t I1, int ct, int all,
+                                              double wt, int rule) {
+  constexpr int L = kUpdateLanes;
+  const int sub = ct % 32 / L, groups = all / L;
+  for (int32_t W = I0 - I0 % groups + ct / 32 * (32 / L); W < I1; W += groups) {  // the warp's first set
+    const int32_t I = W + sub;
+    group_update<T, MAXA, MODE>(g, I, I >= I0 && I < I1, ct % L, wt, rule);
+  }
 }
 
 // Every launch of one call's chain may start as soon as the one before it has
@@ -661,11 +699,6 @@ __global__ void __launch_bounds__(NT, 1) batch_iterate_kernel(const InstDesc *ta
     if (n > 0) s_long[tid] = in.g.iset_mem[lw[tid].is1] - in.g.iset_mem[lw[tid].is0] >= kLongSet * n;
   }
   __syncthreads();
-  const int lane = tid % LANES, gid = ct / LANES, ngroups = all / LANES;
-  const unsigned mask = group_mask<LANES>();
-  // slot updates: set I always by the same threads (their L1 holds its R and avg)
-  const int ua = tid % kUpdateLanes, ugid = ct / kUpdateLanes, ugroups = all / kUpdateLanes;
-  const unsigned umask = group_mask<kUpdateLanes>();
   double *rows = s_rows[tid / 32];
   const int halves = in.order ? 2 : 1;  // alternating: player 1's half, then player 2's
   for (long long it = 0; it < n_iter; ++it) {
@@ -698,20 +731,15 @@ __global__ void __launch_bounds__(NT, 1) batch_iterate_kernel(const InstDesc *ta
           if (by_warp)
             for (int32_t I = is0 + ct / 32; I < is1; I += all / 32) group_set_long<MAXA, MODE>(g, I, I >= is2, upd);
         }
-        if (!by_warp) {
-          for (int32_t I = is0 + gid; I < is1; I += ngroups)
-            group_set<T, MAXA, LANES, MODE>(g, I, I >= is2, lane, mask, upd, rows);
-        }
+        if (!by_warp) group_sets<T, MAXA, LANES, MODE>(g, is0, is2, is1, ct, all, upd, rows);
         level_sync<CLUSTERED>();
       }
       if (upd == 3) {
-        for (int32_t I = ugid; I < n_sets; I += ugroups) group_update<T, MAXA, MODE>(g, I, ua, umask, wt, rule);
+        group_updates<T, MAXA, MODE>(g, 0, n_sets, ct, all, wt, rule);
       } else {  // one player's sets
-        for (int d = 0; d < D; ++d) {
-          const int32_t i0 = upd == 1 ? lw[d].is0 : lw[d].is2, i1 = upd == 1 ? lw[d].is2 : lw[d].is1;
-          for (int32_t I = i0 + (ugid + ugroups - i0 % ugroups) % ugroups; I < i1; I += ugroups)
-            group_update<T, MAXA, MODE>(g, I, ua, umask, wt, rule);
-        }
+        for (int d = 0; d < D; ++d)
+          group_updates<T, MAXA, MODE>(g, upd == 1 ? lw[d].is0 : lw[d].is2, upd == 1 ? lw[d].is2 : lw[d].is1, ct, all,
+                                       wt, rule);
       }
       level_sync<CLUSTERED>();
     }

@@ -89,8 +89,6 @@ __global__ void __launch_bounds__(kTopThreads<T, MAXA>, 1) top_kernel(const __gr
     // the root's own value has no reader and no place here
     if (tid == 0 && s_lw[0].is1 > s_lw[0].is0) reinterpret_cast<int32_t *>(s_solve + L.mem_vs)[0] = -1;
     __syncthreads();
-    const int lane = tid % LANES, gid = tid / LANES;
-    const unsigned mask = group_mask<LANES>();
     double *rows = s_rows[tid / 32];
     for (int d = K; d >= 0; --d) {
       const LevelWork &w = s_lw[d];
@@ -104,17 +102,15 @@ __global__ void __launch_bounds__(kTopThreads<T, MAXA>, 1) top_kernel(const __gr
           g.v[g.ch_vs[i]] = s;
         }
       }
-      for (int32_t J = is0 + gid; J < is1; J += NT / LANES)
-        group_set<T, MAXA, LANES, kResident>(g, J, J >= is2, lane, mask, upd, rows);
+      group_sets<T, MAXA, LANES, kResident>(g, is0, is2, is1, tid, NT, upd, rows);
       __syncthreads();
     }
-    const int ua = tid % kUpdateLanes, ugid = tid / kUpdateLanes;
-    const unsigned umask = group_mask<kUpdateLanes>();
-    for (int d = 0; d <= K; ++d) {
-      const int32_t i0 = upd & 1 ? s_lw[d].is0 : s_lw[d].is2, i1 = upd & 2 ? s_lw[d].is1 : s_lw[d].is2;
-      if (upd == 3 && d > 0) break;  // both players' sets: all depths at once
-      for (int32_t J = i0 + ugid; J < (upd == 3 ? (int32_t)I : i1); J += NT / kUpdateLanes)
-        group_update<T, MAXA, kResident>(g, J, ua, umask, wt, in.rule);
+    if (upd == 3) {
+      group_updates<T, MAXA, kResident>(g, 0, (int32_t)I, tid, NT, wt, in.rule);
+    } else {
+      for (int d = 0; d <= K; ++d)
+        group_updates<T, MAXA, kResident>(g, upd & 1 ? s_lw[d].is0 : s_lw[d].is2, upd & 1 ? s_lw[d].is2 : s_lw[d].is1, tid,
+                                          NT, wt, in.rule);
     }
     __syncthreads();
     for (uint32_t q = tid; q < A; q += NT) {
