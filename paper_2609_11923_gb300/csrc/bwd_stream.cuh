@@ -13,7 +13,7 @@
 // whose children are one run of value slots, and their entries of the chance
 // arrays). A CTA's warps form teams (StreamShape), and every team walks its
 // own chunks through its own ring of kStreamStages stages: as soon as its
-// threads are done with a chunk, its first warp starts the cp.async.bulk
+// threads are done with a chunk, one of its warps starts the cp.async.bulk
 // copies of the next chunk but one into the same stage. No team waits for
 // another, so the copies of some teams are in flight while others compute;
 // the loads in flight cost no registers; the one scattered access left is
@@ -34,8 +34,8 @@
 // q = t / G, t / G + n / G, ... of that set (n threads in the team), so a
 // warp reads a tile's reach as one contiguous run. Per-thread FP32 partial
 // sums are finished by a fixed-shape butterfly within the warp and, in the
-// team's first warp, a sum over the team's warps in order (deterministic run
-// to run); that warp then updates the group's slots (one lane per slot) and
+// warp whose turn the group is, a sum over the team's warps in order
+// (deterministic run to run); that warp then updates the group's slots (one lane per slot) and
 // writes sigma^{t+1}. The form pays where sets are long.
 #pragma once
 #include <algorithm>
@@ -52,7 +52,7 @@ constexpr int kStreamSpread = 16 * 152;           // as long as the depth makes 
 constexpr int kStreamChanceBytes = 1024;          // chance nodes are packed up to this size in any case
 constexpr int kStreamSideBytes = 2048;            // bytes of a chunk's R and average sums, and descriptors, at most
 constexpr int kStreamMaxWarps = 16;               // warps of a streaming CTA (one CTA per SM)
-constexpr int kStreamMinWarps = 6;                // of a CTA, unless its stages are so large that even the largest teams are fewer
+constexpr int kStreamMinWarps = 6;                // of a CTA of one-warp teams
 constexpr int kStreamDynSmem = 216 * 1024;        // bytes of all teams' rings
 constexpr int kStreamMinMembers = 32;             // mean members per set below which the autotuner does not try it
 // Mean members per set from which a depth streams by default: of an untiled
@@ -196,21 +196,24 @@ struct StreamShape {
   int32_t teams, warps, bytes;
 };
 
-// The stages take kStreamDynSmem bytes at most. Teams are as small as they can
-// be with kStreamMinWarps warps in a CTA, and larger where the depth has too
-// few chunks to give every team one. (Two warps a team, 14 warps, instead of
-// seven teams of one at depths of 13 KB tiles: 134 us an iteration instead of
-// 131; groups packed into chunks of 6 KB at depths with fewer chunks than
-// teams: 35 us instead of 27 for an endgame of a million edges.)
+// The stages take kStreamDynSmem bytes at most: as many teams as they hold, of
+// one warp where that makes kStreamMinWarps and else of as many as a CTA's
+// warps allow; larger teams too where the depth has too few chunks to give
+// every team one. (Iterations: seven teams of one warp 131 us, of two 132, at
+// depths of 13 KB tiles; three of five 488, two of eight 526, at 26 KB tiles
+// of a 129M-node card game; at 33 KB of the 264M-node one 951 and 935. One
+// warp doing all of a team's updates: 994 there. Groups packed into chunks of
+// 6 KB at depths with fewer chunks than teams: 35 us instead of 27 for an
+// endgame of a million edges.)
 inline StreamShape stream_shape(int64_t largest, int64_t chunks, int sms) {
   StreamShape z;
   z.bytes = (int32_t)((largest + 127) / 128 * 128);
-  const int fit = std::max(1, std::min(kStreamMaxWarps, kStreamDynSmem / (kStreamStages * z.bytes)));
-  auto teams = [&](int t) { return std::min(fit, kStreamMaxWarps / t); };
-  int t = 1;
-  while (t < 8 && (t * teams(t) < kStreamMinWarps || chunks <= (int64_t)sms * teams(2 * t))) t *= 2;
-  z.warps = t;
-  z.teams = teams(t);
+  z.teams = std::max(1, std::min(kStreamMaxWarps, kStreamDynSmem / (kStreamStages * z.bytes)));
+  z.warps = z.teams >= kStreamMinWarps ? 1 : std::min(8, kStreamMaxWarps / z.teams);
+  while (z.warps < 8 && z.teams > 1 && chunks <= (int64_t)sms * (z.teams / 2)) {
+    z.teams /= 2;
+    z.warps = std::min(8, kStreamMaxWarps / z.teams);
+  }
   return z;
 }
 
@@ -438,7 +441,7 @@ __device__ __forceinline__ void stream_chance_chunk(const StreamChunk &d, const 
 //            chance chunk) and have left their partial sums in red
 // A stage is refilled only after every thread of the team is done with its
 // chunk, so a phase cannot complete twice before its waiters see it. red is
-// double-buffered: the first warp has read red[p] of a group before it
+// double-buffered: the warp whose turn a group is has read red[p] before it
 // arrives at the next group's sync, which the others pass before they write
 // red[p] again.
 template <int MAXA>
@@ -488,7 +491,6 @@ __global__ void __launch_bounds__(32 * kStreamMaxWarps, 1)
   // fault-injection hook (err[1], set on the host): issue no copy after the
   // first ones, so that the waits for the next chunk run out
   const bool stall = reinterpret_cast<volatile const int *>(err)[1] != 0;
-  int32_t issued = 0;  // chunks whose copies have been issued (the team's first warp)
   bool ok = true;
   // the first chunks of the team. early: the launch before this one is the
   // backward launch of the next depth, which writes only values of this
@@ -498,13 +500,12 @@ __global__ void __launch_bounds__(32 * kStreamMaxWarps, 1)
   if (tw == 0) {
     for (int i = 0; i < S && ok && first + i * stride < c1; ++i) {
       ok = issue(i, i ? w1 : w0, early ? kIssueRest : kIssueAll);  // a chunk larger than a stage: the waits give up
-      if (ok) ++issued;
     }
   }
   if (early) {
     pdl_enter();
     if (tw == 0)
-      for (int i = 0; i < issued; ++i) issue(i, i ? w1 : w0, kIssueValues);
+      for (int i = 0; i < S && ok && first + i * stride < c1; ++i) issue(i, i ? w1 : w0, kIssueValues);
   }
   const double wt = avg_weight(*st.t + 1, rule);
   uint32_t phase = 0;  // of sync: groups and chance chunks done
@@ -518,11 +519,10 @@ __global__ void __launch_bounds__(32 * kStreamMaxWarps, 1)
     if (!ok) break;
     const StreamChunk d = stream_chunk(w0);
     const unsigned char *stage = ring + s * shape.bytes;
-    auto refill = [&]() {  // every thread of the team is done with the stage
-      if (tw == 0 && c + 2 * stride < c1 && !stall) {
+    auto refill = [&](bool turn) {  // every thread of the team is done with the stage
+      if (turn && c + 2 * stride < c1 && !stall) {
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        if (issue(i + S, w2, kIssueAll)) issued = i + S + 1;
-        else ok = false;
+        ok = issue(i + S, w2, kIssueAll);
       }
     };
     auto team_sync = [&]() {
@@ -536,7 +536,7 @@ __global__ void __launch_bounds__(32 * kStreamMaxWarps, 1)
     if (d.kind == kChunkChance) {
       stream_chance_chunk(d, stage, t, n, st.v);
       team_sync();
-      if (ok) refill();
+      if (ok) refill(tw == 0);
     } else {
       const StreamLayout L = stream_layout(d);
       const SetInfo *sinfo = reinterpret_cast<const SetInfo *>(stage + L.info);
@@ -544,8 +544,10 @@ __global__ void __launch_bounds__(32 * kStreamMaxWarps, 1)
         const int G = sinfo[I - d.I0].flags & 7;
         float racc[MAXA], own;
         stream_members<MAXA>(d, L, stage, I, G, t, n, st.v, racc, own);
+        // the team's warps take turns at the slot updates and the refills
+        const bool turn = shape.warps == 1 || (int)(phase % (uint32_t)shape.warps) == tw;
         StreamSlot z;
-        if (tw == 0) z = stream_slot(d, L, stage, I, G, MAXA, upd);
+        if (turn) z = stream_slot(d, L, stage, I, G, MAXA, upd);
         const int a = lane >> (G == 4 ? 2 : 0), j = lane & (G - 1);
         float r = 0.f;
         if (shape.warps > 1) {
@@ -556,11 +558,11 @@ __global__ void __launch_bounds__(32 * kStreamMaxWarps, 1)
             red[warp][lane][MAXA] = own;
           }
           team_sync();
-          if (ok && tw == 0 && a < MAXA) {
+          if (ok && turn && a < MAXA) {
             own = 0.f;
             for (int w = 0; w < shape.warps; ++w) {  // warps in order
-              r += red[warp + w][j][a];
-              own += red[warp + w][j][MAXA];
+              r += red[warp - tw + w][j][a];
+              own += red[warp - tw + w][j][MAXA];
             }
           }
         } else {
@@ -571,8 +573,8 @@ __global__ void __launch_bounds__(32 * kStreamMaxWarps, 1)
         }
         if (!ok) break;
         I += G;
-        if (I >= d.I1) refill();
-        if (tw == 0) stream_update<MAXA>(z, G, r, own, st.sigma, st.R, st.avg, wt, rule);
+        if (I >= d.I1) refill(turn);
+        if (turn) stream_update<MAXA>(z, G, r, own, st.sigma, st.R, st.avg, wt, rule);
       }
     }
     w0 = w1;
@@ -580,9 +582,9 @@ __global__ void __launch_bounds__(32 * kStreamMaxWarps, 1)
   }
   if (!ok) {
     atomicExch(err, 1);
-    // let every copy in flight land before the warp leaves (bounded)
-    for (int32_t k = max(0, issued - S); k < issued; ++k)
-      if (k >= i) mbar_wait(full0 + 8 * (k % S), (uint32_t)((k / S) & 1));
+    // let the team's copies in flight land before the warp leaves (bounded)
+    for (int32_t k = i; k < i + S && first + k * stride < c1; ++k)
+      mbar_wait(full0 + 8 * (k % S), (uint32_t)((k / S) & 1));
   }
 }
 

@@ -263,11 +263,11 @@ static void build_stream(cfr_handle *h) {
     // a stage; each node's child run must lie inside its chunk's
     const int32_t q0 = c.level_chance[d], q1 = c.level_chance[d + 1];
     const int64_t pack_ch = std::clamp<int64_t>((12 * int64_t(q1 - q0) + 4 * kids) / kStreamSpread, kStreamChanceBytes,
-                                                kStreamPackBytes);
+                                                std::max<int64_t>(kStreamPackBytes, h->stream_bytes[d]));
     for (int32_t i = q0; ok && i < q1;) {
       int32_t j = i + 1;
       if (!chance_fits(make_chance(i, j))) { ok = false; break; }
-      while (j < q1 && j - i < kStreamChanceMax && chance_layout(make_chance(i, j + 1)).total <= pack_ch) ++j;
+      while (j < q1 && j - i < kStreamChanceMax && chance_fits(make_chance(i, j + 1)) && chance_layout(make_chance(i, j + 1)).total <= pack_ch) ++j;
       const StreamChunk k = make_chance(i, j);
       h->stream_bytes[d] = std::max<int64_t>(h->stream_bytes[d], chance_layout(k).total);
       for (int32_t q = i; q < j; ++q)
