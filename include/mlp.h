@@ -60,7 +60,9 @@ size_t mlp_net_image_bytes(int in_dim);
 size_t mlp_net_work_bytes(int in_dim, int rows);
 
 /* prob [rows x 8] = the masked softmax of the logits of X [rows x in_dim].
- * err (device int) is set to 1 if a wait inside the kernel gave up. */
+ * err (an int that the device can write: device or page-locked host memory)
+ * is set to 1 if a wait inside the kernel gave up; rows that it then could not
+ * compute are NaN. It is not cleared: read it once the stream has got there. */
 int mlp_net_predict(const float *X, int in_dim, int rows, const void *img, const float *const *b, const int32_t *nact,
                     float *prob, int *err, void *stream);
 

@@ -135,13 +135,16 @@ __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::be
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
+// A wait gave up. The word may be page-locked host memory: a plain store.
+__device__ __forceinline__ void report(int *err) { *reinterpret_cast<volatile int *>(err) = 1; }
+
 // Bounded wait of a thread that other threads meet at named barriers: when it
 // gives up (or another thread has) it says so and goes on without waiting, so
 // that every such barrier is still reached by all.
 __device__ __forceinline__ void wait_or_go_on(uint32_t bar, uint32_t parity, volatile int *stop, int *err) {
   if (*stop == 0 && !mbar_wait(bar, parity)) {
     *stop = 1;
-    atomicExch(err, 1);
+    report(err);
   }
 }
 
@@ -230,7 +233,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_rows_kernel(const RowArgs a) 
       mbar_init(smem_u32(&sm.act[p]), PT);
     }
     sm.stop = (smem_u32(s_dyn) & 1023u) != 0u;  // the swizzle needs 1,024-byte aligned blocks
-    if (sm.stop) atomicExch(a.err, 1);
+    if (sm.stop) report(a.err);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_smem();
   }
@@ -267,7 +270,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_rows_kernel(const RowArgs a) 
           }
         if (!ok) {
           *stop = 1;
-          atomicExch(a.err, 1);
+          report(a.err);
         }
         for (int i = n > R ? n - R : 0; i < n; ++i)  // no copy is in flight when the CTA leaves
           mbar_wait(smem_u32(&sm.full[i % R]), (uint32_t)((i / R) & 1));
@@ -304,7 +307,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_rows_kernel(const RowArgs a) 
           }
         if (!ok) {
           *stop = 1;
-          atomicExch(a.err, 1);
+          report(a.err);
         }
       }
     } else {
@@ -388,9 +391,11 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_rows_kernel(const RowArgs a) 
               for (int j = 0; j < kOut; ++j)
                 if (j < na) sum += __expf(z[j] - mx);
               const float lse = mx + __logf(sum);
+              // inference after a wait that gave up: no row passes for a result
+              const float failed = !TRAIN && *stop != 0 ? __int_as_float(0x7fc00000) : 0.f;
               float p[kOut];
 #pragma unroll
-              for (int j = 0; j < kOut; ++j) p[j] = j < na ? __expf(z[j] - lse) : 0.f;
+              for (int j = 0; j < kOut; ++j) p[j] = (j < na ? __expf(z[j] - lse) : 0.f) + failed;
               if constexpr (!TRAIN) {
                 if (in) {
                   float4 *o = reinterpret_cast<float4 *>(a.prob + (size_t)(r0 + row) * kOut);
@@ -499,6 +504,10 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_rows_kernel(const RowArgs a) 
         }
       }
     }
+  } else if constexpr (!TRAIN) {
+    for (int t = blockIdx.x; t < a.tiles; t += gridDim.x)
+      for (int i = tid; i < kTile * kOut; i += kThreads)
+        if (t * kTile + i / kOut < a.B) a.prob[(size_t)t * kTile * kOut + i] = __int_as_float(0x7fc00000);
   }
   __syncwarp();
   fence_before();
@@ -535,7 +544,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_wgrad_kernel(const unsigned c
     }
     mbar_init(smem_u32(&sm.acc), 1);
     sm.stop = (smem_u32(s_dyn) & 1023u) != 0u;
-    if (sm.stop) atomicExch(err, 1);
+    if (sm.stop) report(err);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_smem();
   }
@@ -561,7 +570,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_wgrad_kernel(const unsigned c
         }
         if (!ok) {
           *stop = 1;
-          atomicExch(err, 1);
+          report(err);
         }
         for (int i = n > kGradRing ? n - kGradRing : 0; i < n; ++i)
           mbar_wait(smem_u32(&sm.full[i % kGradRing]), (uint32_t)((i / kGradRing) & 1));
@@ -585,14 +594,14 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_wgrad_kernel(const unsigned c
         if (ok) mma_commit(smem_u32(&sm.acc));
         else {
           *stop = 1;
-          atomicExch(err, 1);
+          report(err);
         }
       }
     } else {
       const int wg = warp >> 2, i = wg * 128 + (warp & 3) * 32 + lane;  // this thread's input feature
       if (!mbar_wait(smem_u32(&sm.acc), 0) || *stop) {
         *stop = 1;
-        atomicExch(err, 1);
+        report(err);
       } else {
         fence_after();
         const uint32_t acc = tmem + (uint32_t)wg * 256u + ((uint32_t)((warp & 3) * 32) << 16);

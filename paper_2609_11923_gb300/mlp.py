@@ -92,11 +92,25 @@ class MLP:
         self.img = self.work = None
         if self.fused:
             self.img = torch.zeros(_lib.mlp_net_image_bytes(in_dim), dtype=torch.uint8, device=self.dev)
-            self._err = torch.zeros(1, dtype=torch.int32, device=self.dev)
+            # set to 1 by an inference kernel whose bounded wait gave up
+            # (page-locked: the host reads it without a copy)
+            self._err = torch.zeros(1, dtype=torch.int32).pin_memory()
         self.sync_bf16()
 
     def _s(self) -> int:
         return int(self.torch.cuda.current_stream(self.dev).cuda_stream)
+
+    def _raise_if_failed(self):
+        if self.fused and self._err.numpy()[0] != 0:
+            self._err.zero_()
+            raise RuntimeError("mlp: a bounded wait of an inference kernel gave up; its probabilities are NaN")
+
+    def check(self) -> None:
+        """Waits for the current stream and raises if an inference on it
+        failed (so does the next pass of the network, without waiting)."""
+        if self.fused:
+            self.torch.cuda.current_stream(self.dev).synchronize()
+            self._raise_if_failed()
 
     @property
     def acts(self):
@@ -131,6 +145,7 @@ class MLP:
     def forward(self, X) -> "torch.Tensor":
         """X: [B, in_dim] FP32 on the device. Keeps the activations."""
         torch = self.torch
+        self._raise_if_failed()
         B = X.shape[0]
         self.acts = [X]
         h = X
@@ -167,6 +182,7 @@ class MLP:
 
     def loss_and_grad(self, X, nact, target, weight=None) -> float:
         torch = self.torch
+        self._raise_if_failed()
         B = X.shape[0]
         if self._rows_ok(X):
             need = _lib.mlp_net_work_bytes(self.dims[0], B)
@@ -203,7 +219,10 @@ class MLP:
             _ck(_lib.mlp_adam(_p(b), _p(g), _p(m), _p(v), b.numel(), lr, b1, b2, eps, self.step_no, None, self._s()))
 
     def predict(self, X, nact) -> "torch.Tensor":
+        """Probabilities of the rows. Asynchronous: check() raises if the pass
+        failed, once they are used on the host."""
         torch = self.torch
+        self._raise_if_failed()
         if self._rows_ok(X):
             prob = torch.empty((X.shape[0], N_OUT), dtype=torch.float32, device=self.dev)
             _net_ck(_lib.mlp_net_predict(_p(X), self.dims[0], X.shape[0], _p(self.img), _ptrs(self.b), _p(nact),

@@ -263,6 +263,7 @@ def warm_regrets_many(net: MLP, specs, kappa: float, workers: Optional[int] = No
     X = np.concatenate([f[0] for f in feats])
     na = np.concatenate([f[1] for f in feats])
     prob = net.predict(torch.tensor(X, device=net.dev), torch.tensor(na, device=net.dev)).cpu().numpy()
+    net.check()
     t2 = time.perf_counter()
     out, row = [], 0
     for sp, (_, nag, mass) in zip(specs, feats):

@@ -149,3 +149,16 @@ def test_other_shapes_run_layer_by_layer():
     W, b = net.numpy_params()
     rl, _, _ = mlp_ref.loss_and_grads(W, b, X.astype(np.float64), nact, T.astype(np.float64), bf16=True)
     assert loss == pytest.approx(rl, rel=1e-3)
+
+
+def test_a_failed_inference_is_raised_by_check_and_by_the_next_pass():
+    X, nact, T = (torch.tensor(x, device="cuda") for x in _batch(200, 192, seed=6))
+    net = M.MLP(192, seed=1)
+    p = net.predict(X, nact)
+    net.check()
+    for call in (net.check, lambda: net.predict(X, nact), lambda: net.loss_and_grad(X, nact, T)):
+        net._err.fill_(1)  # what a kernel writes whose wait gave up
+        with pytest.raises(RuntimeError, match="gave up"):
+            call()
+        net.check()
+    assert torch.equal(net.predict(X, nact), p)
