@@ -240,10 +240,18 @@ __host__ __device__ inline ResidentLayout resident_layout(const InstDesc &in, ui
   return L;
 }
 
-// Games of at most this many nodes may be resident (32-bit offsets above
-// cannot overflow below it; the byte count decides).
-constexpr int64_t kResidentNodes = 1 << 16;
+// Only games of at most this many nodes may be resident: the byte count
+// decides, and the 32-bit sums of resident_layout cannot wrap below it (no
+// array has more than a few elements more than the game has nodes).
+constexpr int32_t kResidentNodes = 1 << 16;
 constexpr uint32_t kResidentBytes = 190 * 1024;
+
+// Bytes of shared memory that the arrays take, 0 if they do not fit (host).
+inline uint32_t resident_size(const InstDesc &in, uint32_t T) {
+  if (in.n_nodes > kResidentNodes) return 0;
+  const uint32_t n = resident_layout(in, T).total;
+  return n <= kResidentBytes ? std::max(n, 16u) : 0;
+}
 
 // The arrays that a batched iteration works on (member order).
 template <typename T> struct GroupView {

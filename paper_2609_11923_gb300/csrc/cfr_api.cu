@@ -495,11 +495,10 @@ static InstDesc inst_desc(const cfr_handle *h, int64_t n_iter) {
 // in one CTA, 0 if it cannot be.
 static uint32_t resident_bytes(const cfr_handle *h, const InstDesc &d) {
   const Compiled &c = h->c;
-  if (c.int_edge.empty() || c.N > kResidentNodes) return 0;
+  if (c.int_edge.empty()) return 0;
   for (int64_t l = 1; l < c.D; ++l)
     if (c.level_wide[l + 1] != c.level_wide[l]) return 0;  // wide chance nodes are summed from global memory
-  const uint32_t n = resident_layout(d, h->precision == CFR_P64 ? 8u : 4u).total;
-  return n <= kResidentBytes ? std::max(n, 16u) : 0;
+  return resident_size(d, h->precision == CFR_P64 ? 8u : 4u);
 }
 
 // The part of a game that the near-root kernel holds: depths 0 .. K.
@@ -535,11 +534,11 @@ static void choose_top(cfr_handle *h) {
     if (K > 0 && c.level_wide[K + 1] != c.level_wide[K]) break;  // wide chance nodes: the per-level kernel
     const int64_t sets = c.level_iset[2 * K + 2] - c.level_iset[2 * K];
     if (sets * h->top_lanes > rounds * threads || c.level_int[K + 1] - c.level_int[K] > 4 * threads) break;
-    const uint32_t n = resident_layout(top_desc(h, K), T).total;
-    if (n > kResidentBytes) break;
+    const uint32_t n = resident_size(top_desc(h, K), T);
+    if (n == 0) break;
     if (K > 0) {  // depth 0 alone saves nothing
       h->top_k = (int)K;
-      h->top_smem = std::max(n, 16u);
+      h->top_smem = n;
     }
   }
 }
