@@ -15,8 +15,10 @@ static cudaError_t launch_batch_any(K kern, int threads, const BatchLaunch &l, c
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
   }
+  // The limit belongs to the kernel, not to a launch: every caller sets the
+  // same one, so that a launch from another thread cannot find a lower one.
   if (l.smem > 0) {
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.smem);
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResidentBytes);
     if (e != cudaSuccess) return e;
   }
   cudaLaunchConfig_t cfg = {};

@@ -329,3 +329,35 @@ def test_best_response_at_group_edges_matches_oracle(a, b):
                 np.testing.assert_allclose(cfr.cfr_exploitability(h, s)[1:3], want[:2], rtol=0, atol=1e-14)
     for h in hs:
         cfr.cfr_destroy(h)
+
+
+def test_resident_solves_of_different_sizes_run_from_several_threads():
+    # the same kernel, its shared memory sized by the game: a launch must not
+    # depend on what another thread has just launched
+    import threading
+
+    specs = [gg.random_tree(1, depth=8), gg.random_tree(1, depth=6), gg.random_tree(2, depth=8), gg.random_tree(2, depth=6)]
+    solvers = [cfr.Solver(g, precision=cfr.P32) for g in specs]
+    streams = [torch.cuda.Stream() for _ in specs]
+    torch.cuda.synchronize()
+    errors, start = [], threading.Barrier(len(specs))
+
+    def run(s, st):
+        try:
+            start.wait()
+            for _ in range(2000):
+                cfr.cfr_iterate(s.h, 1, int(st.cuda_stream))
+        except Exception as e:  # noqa: BLE001
+            errors.append(e)
+
+    ts = [threading.Thread(target=run, args=x) for x in zip(solvers, streams)]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    torch.cuda.synchronize()
+    assert not errors, errors[0]
+    for g, s in zip(specs, solvers):
+        one = cfr.Solver(g, precision=cfr.P32)
+        one.iterate(2000)
+        np.testing.assert_array_equal(s.avg_strategy(), one.avg_strategy())
