@@ -823,9 +823,12 @@ __global__ void __launch_bounds__(NT) batch_iterate_push_kernel(const InstDesc *
 // Exploitability of every instance's average strategy (FP64): normalise the
 // average, forward reach under it, then both best responses by depth (the
 // arithmetic of br_level_kernel). CTAs and clusters as batch_iterate_kernel.
+// wide_parts: partial sums of a wide chance node, the caller's and not the
+// CTA's threads (which games of more than four actions in the call lower): the
+// second half of them is the first step of the tree of twice the threads.
 template <int MAXA, int LANES, int THREADS, bool CLUSTERED>
 __global__ void __launch_bounds__(THREADS, 1) batch_br_kernel(const InstDesc *table, const __grid_constant__ InstDesc one,
-                                                           int n_inst) {
+                                                           int n_inst, int wide_parts) {
   __shared__ double sm[THREADS];
   chain_enter();
   const int ncta = CLUSTERED ? (int)cluster_ncta() : 1;
@@ -869,9 +872,15 @@ __global__ void __launch_bounds__(THREADS, 1) batch_br_kernel(const InstDesc *ta
       const int32_t h = __ldg(g.wide_vs + i);
       const int32_t cb = __ldg(g.wide_vb + i), ce = cb + __ldg(g.wide_nch + i);
       double sx = 0.0, sy = 0.0, sa = 0.0;
-      for (int32_t c = cb + threadIdx.x; c < ce; c += THREADS) {
-        const double2 x = ldm<CLUSTERED>(in.vb + c);
-        sx += x.x; sy += x.y; sa += ldm<CLUSTERED>(in.vavg + c);
+      for (int part = threadIdx.x; part < wide_parts; part += THREADS) {  // one or two a thread
+        double px = 0.0, py = 0.0, pa = 0.0;
+        for (int32_t c = cb + part; c < ce; c += wide_parts) {
+          const double2 x = ldm<CLUSTERED>(in.vb + c);
+          px += x.x; py += x.y; pa += ldm<CLUSTERED>(in.vavg + c);
+        }
+        sx = part < THREADS ? px : sx + px;
+        sy = part < THREADS ? py : sy + py;
+        sa = part < THREADS ? pa : sa + pa;
       }
       sx = cta_sum<THREADS>(sx, sm);
       sy = cta_sum<THREADS>(sy, sm);

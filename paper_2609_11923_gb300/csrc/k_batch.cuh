@@ -8,9 +8,9 @@ namespace cfr {
 #define CFR_BATCH_ALL(X) \
   CFR_BATCH_LANES(X, 4, 256) CFR_BATCH_LANES(X, 4, 1024) CFR_BATCH_LANES(X, 8, 256) CFR_BATCH_LANES(X, 8, 1024)
 
-template <typename K>
+template <typename K, typename... More>
 static cudaError_t launch_batch_any(K kern, int threads, const BatchLaunch &l, cudaStream_t s, const InstDesc *table,
-                                    const InstDesc &one) {
+                                    const InstDesc &one, More... more) {
   if (l.cluster > 8) {
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
@@ -40,7 +40,7 @@ static cudaError_t launch_batch_any(K kern, int threads, const BatchLaunch &l, c
     attr[cfg.numAttrs].val.programmaticStreamSerializationAllowed = 1;
     ++cfg.numAttrs;
   }
-  return cudaLaunchKernelEx(&cfg, kern, table, one, l.count);
+  return cudaLaunchKernelEx(&cfg, kern, table, one, l.count, more...);
 }
 
 template <typename T, int MA, int L, int TH>

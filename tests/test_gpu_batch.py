@@ -361,3 +361,19 @@ def test_resident_solves_of_different_sizes_run_from_several_threads():
         one = cfr.Solver(g, precision=cfr.P32)
         one.iterate(2000)
         np.testing.assert_array_equal(s.avg_strategy(), one.avg_strategy())
+
+
+@pytest.mark.parametrize("threads", [256, 1024])
+def test_best_response_of_a_wide_root_does_not_depend_on_the_mix(threads):
+    # a deal of 1,260 outcomes with at most three actions, by itself and beside
+    # a game of seven, whose kernels have half the threads
+    wide, other = gg.large_card(5, 2, 2, 3), gg.endgame(21, 30000)
+    assert wide.iset_nact.max() <= 4 < other.iset_nact.max() <= 8 and wide.child_begin[1] > 1024
+    rows = []
+    for specs in ([wide], [wide, other]):
+        pool, hs, table, tp, tb, s = bound(specs)
+        cfr.cfr_batch_iterate(hs, 20, tp, tb, threads, 8, s)
+        rows.append(cfr.cfr_batch_exploitability(hs, tp, tb, threads, 8, s)[0])
+        for h in hs:
+            cfr.cfr_destroy(h)
+    np.testing.assert_array_equal(rows[0], rows[1])
