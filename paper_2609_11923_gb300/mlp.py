@@ -83,7 +83,7 @@ class MLP:
         self.mb = [torch.zeros_like(b) for b in self.b]
         self.vb = [torch.zeros_like(b) for b in self.b]
         self.step_no = 0
-        self._acts, self._X = None, None
+        self._acts, self._fused_pass = None, None  # (batch, write counters) of the last pass if it was a fused one
         # networks of the warm start's shape run through the fused kernels
         # (mlp_net_*), from packed images of the weights; any other shape
         # runs layer by layer through mlp_gemm
@@ -115,17 +115,35 @@ class MLP:
     @property
     def acts(self):
         """The input, every hidden layer's output and the logits of the last
-        forward pass in FP32. The fused passes keep none: after one of them
-        they are computed here."""
-        if self._acts is None and self._X is not None:
-            self.forward(self._X)
+        pass in FP32. The fused passes keep none: after one of them they are
+        computed here, on first use, from its batch and the weights, and once
+        either has changed (adam_step, sync_bf16, a write into the tensors)
+        they are gone, which raises."""
+        if self._acts is None and self._fused_pass is not None:
+            X, then = self._fused_pass
+            if X is None or then != self._versions(X):
+                raise RuntimeError("mlp: the activations of the last fused pass are gone (its weights or its batch have "
+                                   "changed since); run forward(X)")
+            self.forward(X)
         return self._acts
 
     @acts.setter
     def acts(self, value):
-        self._acts = value
+        self._acts, self._fused_pass = value, None
+
+    def _versions(self, X):
+        """Write counters of what a pass over X reads."""
+        return [0 if t.is_inference() else t._version for t in [X] + self.Wb + self.b]
+
+    def _ran_fused(self, X):
+        self._acts, self._fused_pass = None, (X, self._versions(X))
+
+    def _weights_change(self):  # the kernels write past the counters
+        if self._fused_pass is not None:
+            self._fused_pass = (None, None)
 
     def sync_bf16(self):
+        self._weights_change()
         if self.fused:
             _net_ck(_lib.mlp_net_adam(self._all(self.W, self.b), None, None, None, _ptrs(self.Wb), _p(self.img),
                                       self.dims[0], 0.0, 0.0, 0.0, 0.0, 0, self._s()))
@@ -192,7 +210,7 @@ class MLP:
             _net_ck(_lib.mlp_net_grad(_p(X), self.dims[0], B, _p(self.img), _ptrs(self.b), _p(nact), _p(target),
                                       _p(weight), _ptrs(self.gW), _ptrs(self.gb), _p(self.work), self.work.numel(),
                                       ctypes.byref(loss), self._s()))
-            self._acts, self._X = None, X
+            self._ran_fused(X)
             at = loss.value - self.work.data_ptr()
             got = self.work[at:at + 8].cpu()
             if int(got.view(torch.int32)[1]) != 0:
@@ -208,6 +226,7 @@ class MLP:
 
     def adam_step(self, lr=1e-3, b1=0.9, b2=0.999, eps=1e-8) -> None:
         self.step_no += 1
+        self._weights_change()
         if self.fused:
             _net_ck(_lib.mlp_net_adam(self._all(self.W, self.b), self._all(self.gW, self.gb),
                                       self._all(self.mW, self.mb), self._all(self.vW, self.vb), _ptrs(self.Wb),
@@ -227,7 +246,7 @@ class MLP:
             prob = torch.empty((X.shape[0], N_OUT), dtype=torch.float32, device=self.dev)
             _net_ck(_lib.mlp_net_predict(_p(X), self.dims[0], X.shape[0], _p(self.img), _ptrs(self.b), _p(nact),
                                          _p(prob), _p(self._err), self._s()))
-            self._acts, self._X = None, X
+            self._ran_fused(X)
             return prob
         logits = self.forward(X)
         prob = torch.empty_like(logits)

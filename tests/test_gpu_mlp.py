@@ -162,3 +162,20 @@ def test_a_failed_inference_is_raised_by_check_and_by_the_next_pass():
             call()
         net.check()
     assert torch.equal(net.predict(X, nact), p)
+
+
+def test_activations_after_a_step_are_not_those_of_other_weights():
+    X, nact, T = (torch.tensor(x, device="cuda") for x in _batch(200, 192, seed=8))
+    net = M.MLP(192, seed=2)
+    net.loss_and_grad(X, nact, T)
+    first = [x.clone() for x in net.acts]
+    net.loss_and_grad(X, nact, T)
+    net.adam_step(1e-2)
+    with pytest.raises(RuntimeError, match="gone"):
+        net.acts
+    net.predict(X, nact)
+    X.mul_(2.0)
+    with pytest.raises(RuntimeError, match="gone"):
+        net.backward(torch.zeros(200, 8, device="cuda"))
+    net.forward(X)
+    assert not torch.equal(net.acts[1], first[1])

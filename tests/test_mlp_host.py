@@ -1,5 +1,5 @@
 """Host side of the network (no GPU): a failed inference is reported before its
-probabilities are used."""
+probabilities are used, and activations are never those of another pass."""
 import numpy as np
 import pytest
 import torch
@@ -13,7 +13,8 @@ def bare(err=0):
     net = mlp.MLP.__new__(mlp.MLP)
     net.torch, net.dev, net.fused = torch, torch.device("cpu"), True
     net._err = torch.tensor([err], dtype=torch.int32)
-    net._acts, net._X = None, None
+    net.Wb = net.b = [torch.zeros(3)]
+    net._acts, net._fused_pass = None, None
     return net
 
 
@@ -42,3 +43,25 @@ def test_warm_start_raises_on_a_failed_inference():
 
     with pytest.raises(RuntimeError, match="gave up"):
         warmstart.warm_regrets(Failing(), g, 8.0)
+
+
+@pytest.mark.parametrize("change", [lambda n, x: n._weights_change(), lambda n, x: x.add_(1.0), lambda n, x: n.b[0].zero_()],
+                         ids=["step", "batch", "bias"])
+def test_activations_of_a_fused_pass_are_gone_once_its_inputs_change(change):
+    net, X = bare(), torch.zeros(2, 4)
+    ran = []
+
+    def forward(x):
+        ran.append(x)
+        net.acts = [x]
+
+    net.forward = forward
+    net._ran_fused(X)
+    assert net.acts[0] is X and ran == [X]  # nothing has changed: computed on first use
+    net._ran_fused(X)
+    change(net, X)
+    with pytest.raises(RuntimeError, match="gone"):
+        net.acts
+    forward(X)  # a layer-by-layer pass keeps its own
+    net._weights_change()
+    assert net.acts[0] is X
