@@ -53,8 +53,9 @@ const char *mlp_last_error(void);
  * fan_out] and biases b_l in FP32 (l = 0..3), the same numerics as the calls
  * above layer by layer. `img` holds the weights packed as tensor-core
  * operands: mlp_net_image_bytes(in_dim) bytes (0: the shape is not taken),
- * zeroed once by the caller, written by mlp_net_adam. Returns as above, with
- * mlp_net_last_error(). */
+ * zeroed once by the caller, written by mlp_net_adam. img, prob, work and the
+ * weight gradients have to be 16-byte aligned (else -1). Returns as above,
+ * with mlp_net_last_error(). */
 size_t mlp_net_image_bytes(int in_dim);
 /* Bytes of the workspace of mlp_net_grad for a batch of `rows`. */
 size_t mlp_net_work_bytes(int in_dim, int rows);

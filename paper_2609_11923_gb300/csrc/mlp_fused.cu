@@ -778,6 +778,7 @@ using namespace mlpf;
     if (e_ != cudaSuccess) return fail(-7, std::string(__func__) + ": " + cudaGetErrorString(e_)); \
   } while (0)
 
+static bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 static bool net_shape(int in_dim) { return in_dim >= 4 && in_dim <= kH && in_dim % 4 == 0; }
 static int sm_count(int *n) {
   int dev = 0;
@@ -790,6 +791,7 @@ static int row_args(RowArgs &a, const float *X, int in_dim, int rows, const void
                     const int32_t *nact, int *err) {
   if (!X || !img || !b || !nact || !err || rows <= 0 || !net_shape(in_dim))
     return fail(-1, "mlp_net: bad argument");
+  if (!aligned16(img)) return fail(-1, "mlp_net: img must be 16-byte aligned");  // bulk copies
   a = RowArgs{};
   a.X = X;
   a.img = (const unsigned char *)img;
@@ -800,7 +802,7 @@ static int row_args(RowArgs &a, const float *X, int in_dim, int rows, const void
   a.in_dim = in_dim;
   a.in_blocks = (in_dim + kBlkK - 1) / kBlkK;
   a.tiles = (rows + kTile - 1) / kTile;
-  a.vec = (reinterpret_cast<uintptr_t>(X) & 15u) == 0;
+  a.vec = aligned16(X);
   return 0;
 }
 
@@ -817,7 +819,7 @@ int mlp_net_predict(const float *X, int in_dim, int rows, const void *img, const
   RowArgs a;
   int rc = row_args(a, X, in_dim, rows, img, b, nact, err), sms = 0;
   if (rc) return rc;
-  if (!prob || (reinterpret_cast<uintptr_t>(prob) & 15u)) return fail(-1, "mlp_net_predict: prob must be 16-byte aligned");
+  if (!prob || !aligned16(prob)) return fail(-1, "mlp_net_predict: prob must be 16-byte aligned");
   if ((rc = sm_count(&sms))) return rc;
   a.prob = prob;
   // more tiles than SMs: two in turn on each
@@ -836,6 +838,9 @@ int mlp_net_grad(const float *X, int in_dim, int rows, const void *img, const fl
   if (!target || !gW || !gb || !work || !loss || rows <= 0 || !net_shape(in_dim)) return fail(-1, "mlp_net_grad: bad argument");
   const Work w = work_of(in_dim, rows);
   if (work_bytes < w.bytes) return fail(-1, "mlp_net_grad: the workspace is too small");
+  if (!aligned16(work)) return fail(-1, "mlp_net_grad: work must be 16-byte aligned");
+  for (int l = 0; l < 4; ++l)
+    if (!aligned16(gW[l])) return fail(-1, "mlp_net_grad: the weight gradients must be 16-byte aligned");
   unsigned char *ws = (unsigned char *)work;
   RowArgs a;
   int rc = row_args(a, X, in_dim, rows, img, b, nact, (int *)(ws + w.loss + 4)), sms = 0;

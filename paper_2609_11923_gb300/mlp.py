@@ -202,7 +202,7 @@ class MLP:
         torch = self.torch
         self._raise_if_failed()
         B = X.shape[0]
-        if self._rows_ok(X):
+        if self._rows_ok(X) and all(g.data_ptr() % 16 == 0 for g in self.gW):
             need = _lib.mlp_net_work_bytes(self.dims[0], B)
             if self.work is None or self.work.numel() < need:
                 self.work = torch.empty(need, dtype=torch.uint8, device=self.dev)

@@ -179,3 +179,19 @@ def test_activations_after_a_step_are_not_those_of_other_weights():
         net.backward(torch.zeros(200, 8, device="cuda"))
     net.forward(X)
     assert not torch.equal(net.acts[1], first[1])
+
+
+def test_gradients_in_one_flat_buffer_take_the_layer_by_layer_route():
+    # views that are 4-byte aligned only, as a flat gradient buffer gives them
+    X, nact, T = (torch.tensor(x, device="cuda") for x in _batch(300, 192, seed=9))
+    a, b = M.MLP(192, seed=3), M.MLP(192, seed=3)
+    flat = torch.zeros(1 + sum(g.numel() for g in a.gW), device="cuda")
+    at, views = 1, []
+    for g in a.gW:
+        views.append(flat[at:at + g.numel()].view_as(g))
+        at += g.numel()
+    a.gW = views
+    b.fused = False
+    assert a.loss_and_grad(X, nact, T) == b.loss_and_grad(X, nact, T)
+    for x, y in zip(a.gW + a.gb, b.gW + b.gb):
+        assert torch.equal(x, y)

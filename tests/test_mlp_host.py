@@ -1,6 +1,8 @@
 """Host side of the network (no GPU): a failed inference is reported before its
-probabilities are used, and activations are never those of another pass."""
-import numpy as np
+probabilities are used, activations are never those of another pass, and the C
+entries refuse what their kernels cannot read."""
+import ctypes
+
 import pytest
 import torch
 
@@ -65,3 +67,26 @@ def test_activations_of_a_fused_pass_are_gone_once_its_inputs_change(change):
     forward(X)  # a layer-by-layer pass keeps its own
     net._weights_change()
     assert net.acts[0] is X
+
+
+# addresses that are only looked at: every refusal comes before any launch
+AT = 1 << 20
+
+
+def ptrs(*at):
+    return (ctypes.c_void_p * 4)(*at)
+
+
+@pytest.mark.parametrize("img,prob", [(AT + 2, AT), (AT + 8, AT), (AT, AT + 4)])
+def test_inference_refuses_misaligned_buffers(img, prob):
+    rc = mlp._lib.mlp_net_predict(AT, 64, 5, img, ptrs(AT, AT, AT, AT), AT, prob, AT, None)
+    assert rc == -1 and b"aligned" in mlp._lib.mlp_net_last_error()
+
+
+@pytest.mark.parametrize("bad", ["img", "work", 0, 1, 2, 3])
+def test_training_refuses_misaligned_buffers(bad):
+    at = {k: AT + 4 * (k == bad) for k in ("img", "work", 0, 1, 2, 3)}
+    loss = ctypes.c_void_p()
+    rc = mlp._lib.mlp_net_grad(AT, 64, 5, at["img"], ptrs(AT, AT, AT, AT), AT, AT, None, ptrs(at[0], at[1], at[2], at[3]),
+                               ptrs(AT, AT, AT, AT), at["work"], 1 << 40, ctypes.byref(loss), None)
+    assert rc == -1 and b"aligned" in mlp._lib.mlp_net_last_error()
