@@ -133,12 +133,17 @@ class MLP:
 
     def _versions(self, X):
         """Write counters of what a pass over X reads."""
-        return [0 if t.is_inference() else t._version for t in [X] + self.Wb + self.b]
+        return [self._version(t) for t in [X] + self.Wb + self.b]
+
+    @staticmethod
+    def _version(t) -> int:
+        return 0 if t.is_inference() else t._version
 
     def _ran_fused(self, X):
         self._acts, self._fused_pass = None, (X, self._versions(X))
 
-    def _weights_change(self):  # the kernels write past the counters
+    def _weights_change(self):  # by a kernel, past the counters: Wb and its images together
+        self._images_of = [(w, self._version(w)) for w in self.Wb]
         if self._fused_pass is not None:
             self._fused_pass = (None, None)
 
@@ -155,8 +160,14 @@ class MLP:
     def _all(weights, biases):
         return _ptrs([t for pair in zip(weights, biases) for t in pair])
 
+    def _packed(self) -> bool:
+        """Whether the packed images are those of Wb. A caller's write into Wb,
+        or other tensors in its place, reach only the layer-by-layer passes,
+        until sync_bf16 or a step writes both."""
+        return all(w is x and self._version(w) == v for w, (x, v) in zip(self.Wb, self._images_of))
+
     def _rows_ok(self, X) -> bool:
-        return (self.fused and X.dtype == self.torch.float32 and X.dim() == 2 and X.shape[0] > 0
+        return (self.fused and self._packed() and X.dtype == self.torch.float32 and X.dim() == 2 and X.shape[0] > 0
                 and X.shape[1] == self.dims[0])
 
     # ---------------------------------------------------------------- passes

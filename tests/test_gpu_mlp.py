@@ -195,3 +195,15 @@ def test_gradients_in_one_flat_buffer_take_the_layer_by_layer_route():
     assert a.loss_and_grad(X, nact, T) == b.loss_and_grad(X, nact, T)
     for x, y in zip(a.gW + a.gb, b.gW + b.gb):
         assert torch.equal(x, y)
+
+
+def test_a_write_into_the_bf16_weights_reaches_every_pass():
+    X, nact, T = (torch.tensor(x, device="cuda") for x in _batch(300, 192, seed=10))
+    a, b = M.MLP(192, seed=3), M.MLP(192, seed=3)
+    b.fused = False
+    for net in (a, b):
+        net.Wb[1].mul_(0.5)
+    assert torch.equal(a.predict(X, nact), b.predict(X, nact))
+    assert a.loss_and_grad(X, nact, T) == b.loss_and_grad(X, nact, T)
+    a.sync_bf16()
+    assert a._packed() and torch.equal(a.Wb[1], a.W[1].bfloat16())

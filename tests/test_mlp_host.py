@@ -15,8 +15,10 @@ def bare(err=0):
     net = mlp.MLP.__new__(mlp.MLP)
     net.torch, net.dev, net.fused = torch, torch.device("cpu"), True
     net._err = torch.tensor([err], dtype=torch.int32)
-    net.Wb = net.b = [torch.zeros(3)]
+    net.Wb, net.b = [torch.zeros(3), torch.zeros(2)], [torch.zeros(3)]
+    net.dims = [4, 2]
     net._acts, net._fused_pass = None, None
+    net._weights_change()
     return net
 
 
@@ -67,6 +69,17 @@ def test_activations_of_a_fused_pass_are_gone_once_its_inputs_change(change):
     forward(X)  # a layer-by-layer pass keeps its own
     net._weights_change()
     assert net.acts[0] is X
+
+
+@pytest.mark.parametrize("change", [lambda n: n.Wb[1].add_(1.0), lambda n: n.Wb.__setitem__(0, torch.zeros(3))],
+                         ids=["write", "replace"])
+def test_changed_bf16_weights_leave_the_packed_images(change):
+    net, X = bare(), torch.zeros(2, 4)
+    assert net._rows_ok(X)
+    change(net)
+    assert not net._rows_ok(X)
+    net._weights_change()  # what sync_bf16 and a step do as they write both
+    assert net._rows_ok(X)
 
 
 # addresses that are only looked at: every refusal comes before any launch
