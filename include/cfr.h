@@ -87,12 +87,14 @@ typedef struct cfr_options {
    * barrier between depth levels; CFR_EXEC_AUTO picks by game size: the
    * persistent form up to 768 nodes in CFR_P32 and 350 in CFR_P64 (where
    * it was measured faster than graph replay), the graph form above.
-   * Under CFR_EXEC_AUTO with lanes_per_set, persistent_ctas, graph_iters and
-   * launch_overlap at their defaults, games whose arrays fit one CTA's shared
-   * memory (about 14,000 nodes in CFR_P32; up to 4,000 in CFR_P64) run all
-   * iterations of a call there instead. In the level and graph forms with
-   * lanes_per_set 0, the small depths near the root are one launch of one CTA
-   * that also starts the next iteration's forward pass. */
+   * Under CFR_EXEC_AUTO with lanes_per_set and persistent_ctas at 0, games
+   * whose arrays fit one CTA's shared memory (about 14,000 nodes in CFR_P32;
+   * up to 4,000 in CFR_P64) run all iterations of a cfr_iterate call there
+   * instead ("resident"). In the level and graph forms with lanes_per_set 0,
+   * the small depths near the root are one launch of one CTA that also starts
+   * the next iteration's forward pass. cfr_export_array 37 tells which of
+   * these a handle uses. FP64 results are bitwise the same in every form;
+   * FP32 sums take the form's shape, and its last bits. */
   int exec_form;
   /* Update rule (Section 3, update rules): CFR_RULE_CFR_PLUS (regret clamped
    * at zero, linear averaging w_t = t), CFR_RULE_CFR (no clamp, linear
@@ -118,8 +120,10 @@ typedef struct cfr_options {
    * player 2's with player 1's new strategy; each half accumulates only its
    * player's average (Section 3; Section 4.2 runs the body twice). */
   int order;
-  /* Order of the internal nodes' reach (a layout choice; results are
-   * bitwise the same). CFR_REACH_MEMBERS (default): depth by depth, the
+  /* Order of the internal nodes' reach, a layout choice: results are bitwise
+   * the same in CFR_P64, and in CFR_P32 with lanes_per_set from 1 to 256 (the
+   * resident, near-root and streaming forms, which 0 and 512 may choose, take
+   * member order). CFR_REACH_MEMBERS (default): depth by depth, the
    * members of the depth's information sets in set order, then the depth's
    * chance nodes; the backward pass reads each set's reach as one run and
    * needs no rank table, and the forward pass pulls (every internal node
@@ -170,8 +174,9 @@ typedef struct cfr_counts {
                                   twice that under alternating updates) */
   int64_t upload_bytes;       /* host-to-device bytes cfr_bind copies */
   int64_t iteration;          /* t: iterations completed since bind/reset */
-  int exec_form;              /* resolved execution form */
-  int lanes_per_set;          /* resolved lanes per information set */
+  int exec_form;              /* resolved execution form (of a resident game too: what cfr_profile_iteration,
+                                 cfr_autotune and its lane counts refer to; cfr_export_array 37) */
+  int lanes_per_set;          /* resolved lanes per information set of that form */
   int64_t graph_kernels;      /* kernel nodes in the captured one-iteration graph (0 until captured) */
   int64_t graph_k_kernels;    /* kernel nodes in the captured graph_iters-iteration graph (0 until captured) */
 } cfr_counts;
@@ -215,8 +220,9 @@ int cfr_bind(cfr_handle *h, void *device_arena, size_t bytes, void *stream);
  * forward reach, terminal values, backward values with the fused regret and
  * average update, regret matching), asynchronously on `stream`, in the
  * execution form the options chose: per-level launches, one CUDA graph of an
- * iteration replayed n times (Section 4.3; captured on the first call), or
- * one persistent kernel. The weight w_t of the average comes from a device
+ * iteration replayed n times (Section 4.3; captured on the first call), one
+ * persistent kernel, or (AUTO, small games) one CTA that holds the game in
+ * shared memory. The weight w_t of the average comes from a device
  * counter the iteration itself advances (Section 4.3), so n = 0 is a no-op
  * and split calls give bitwise the same state as one call. CFR_ERR_NOT_BOUND
  * before cfr_bind. If capturing the graph fails, the call warns once on
@@ -226,8 +232,9 @@ int cfr_iterate(cfr_handle *h, int64_t n, void *stream);
 
 /* Waits for `stream` (the synchronisation point of Section 4.3's
  * asynchronous replay) and reports a device-side failure of earlier calls:
- * CFR_ERR_TIMEOUT if a grid barrier of the persistent kernel gave up (the
- * state is then undefined until cfr_reset). */
+ * CFR_ERR_TIMEOUT if a bounded wait gave up: a grid barrier of the persistent
+ * kernel, or a staged copy of the streaming backward (the state is then
+ * undefined until cfr_reset). */
 int cfr_synchronize(cfr_handle *h, void *stream);
 
 /* Average strategy (eq. (rm): the linear-weighted sum normalised per set,
@@ -323,7 +330,11 @@ int cfr_set_state(cfr_handle *h, const double *R, const double *avg, int64_t t, 
  * of at most 8 actions), 36 blocks of each depth's pulling forward launch
  * [D] (member order: one wave, the blocks all SMs hold at once, or fewer
  * where the depth needs fewer; set by cfr_bind; 0 before the first bind and
- * for the deepest depth).
+ * for the deepest depth), 37 what cfr_iterate launches [6]: threads of the
+ * resident form's CTA (0: the game is not resident and the rest holds), its
+ * lanes per set, the deepest depth of the near-root launch (-1: none; level
+ * and graph forms), its lanes per set, whether an iteration's launches overlap
+ * and whether an evaluation's do.
  * Integer arrays are int32. *count receives the element count; out may be
  * NULL to query it. */
 int cfr_export_array(const cfr_handle *h, int which, void *out, int64_t capacity, int64_t *count);
@@ -348,9 +359,10 @@ int cfr_autotune(cfr_handle *h, int reps, void *stream);
  * Section 4.3 discusses the graph-launch floor): the mean time of one
  * iteration's launch structure with no work in it, over n iterations.
  * graph_ms: a CUDA graph of the same launches as the per-level form (2D,
- * or 2D - 1 in member order, whose deepest depth has no forward launch;
- * twice that under alternating updates) with the same grid sizes
- * (depth-first forward, then backward), each an empty kernel. persistent_ms: one
+ * or 2D - 1 in member order, whose deepest depth has no forward launch; with
+ * depths 0 .. K in the near-root launch 2 (D - K) - 1; twice that under
+ * alternating updates) with the same grid sizes (forward, then backward), each
+ * an empty kernel. persistent_ms: one
  * cooperative launch of an empty kernel with the persistent form's grid and
  * its 2D (4D) grid barriers per iteration (bounded
  * waits: CFR_ERR_TIMEOUT if one gives up). The handle must be bound; solver
@@ -421,7 +433,9 @@ int cfr_batch_exploitability(cfr_handle *const *handles, int n, double *out, voi
 int cfr_level_bytes(const cfr_handle *h, int level, int64_t *fwd_bytes, int64_t *bwd_bytes);
 
 /* Measurement: runs ONE iteration (t -> t+1) as per-level launches on
- * `stream` with a CUDA event pair around every launch, and writes each
+ * `stream` with a CUDA event pair around every launch, also of depths that
+ * cfr_iterate puts into the near-root launch and of resident games (in FP32
+ * with the launches' last bits), and writes each
  * launch's device time in milliseconds: fwd_ms[d] and bwd_ms[d] for
  * d = 0 .. D-1 (host arrays of D doubles; under alternating updates the two
  * halves' times of a depth are added). Synchronises `stream`. */

@@ -9,7 +9,7 @@ from __future__ import annotations
 
 import ctypes
 import os
-from typing import Optional, Tuple
+from typing import Dict, Optional, Tuple
 
 import numpy as np
 
@@ -275,6 +275,15 @@ def cfr_export_array(h: int, name: str) -> np.ndarray:
     out = np.empty(n.value, dtype=np.float64 if name in ("tmpl", "tmpl_vs") else np.int32)
     _check(_lib.cfr_export_array(h, which, out.ctypes.data if n.value else None, n.value, ctypes.byref(n)))
     return out
+
+
+def cfr_launch_plan(h: int) -> Dict[str, int]:
+    """What cfr_iterate launches (cfr_export_array 37)."""
+    n = ctypes.c_int64()
+    out = np.empty(6, dtype=np.int32)
+    _check(_lib.cfr_export_array(h, 37, out.ctypes.data, len(out), ctypes.byref(n)))
+    return dict(zip(("resident_threads", "resident_lanes", "near_root_depth", "near_root_lanes", "overlap",
+                     "evaluation_overlap"), out.tolist()))
 
 
 def cfr_debug_set(h: int, key: int, value: int) -> None:

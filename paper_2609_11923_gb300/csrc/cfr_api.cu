@@ -371,12 +371,13 @@ extern "C" int cfr_compile(const cfr_game_spec *spec, const cfr_options *opt, cf
   }
   plan(h);
   choose_top(h);
-  // AUTO with default options: a game that fits one CTA's shared memory runs
-  // there for the whole call (301 nodes: 4.1 us an iteration in FP32, 11.6 in
-  // the persistent form; 4,213: 6.6, 28.8 as a graph; FP64 above about 4,000
-  // nodes is bound by one SM's FP64 pipe and runs as a graph)
-  if (h->opt.exec_form == CFR_EXEC_AUTO && lp == 0 && h->opt.persistent_ctas == 0 && h->opt.graph_iters <= 1 &&
-      h->opt.launch_overlap == CFR_OVERLAP_AUTO && h->maxa_tier <= 8 && c.D > 0 &&
+  // AUTO: a game that fits one CTA's shared memory runs there for the whole
+  // call (301 nodes: 4.1 us an iteration in FP32, 11.6 in the persistent form;
+  // 4,213: 6.6, 28.8 as a graph; FP64 above about 4,000 nodes is bound by one
+  // SM's FP64 pipe and runs as a graph). graph_iters and launch_overlap do not
+  // decide: in FP32 this form's last bits differ from the launches', and those
+  // two options leave the results as they are.
+  if (h->opt.exec_form == CFR_EXEC_AUTO && lp == 0 && h->opt.persistent_ctas == 0 && h->maxa_tier <= 8 && c.D > 0 &&
       (h->precision == CFR_P32 || c.N <= 4000)) {
     h->solo_smem = resident_bytes(h, inst_desc(h, 0));
     h->solo_threads = c.N <= 600 ? 256 : 1024;
@@ -824,6 +825,9 @@ static bool overlap_on(const cfr_handle *h) {
   return h->opt.launch_overlap == CFR_OVERLAP_ON;
 }
 
+// The launches of an evaluation (cfr_exploitability).
+static bool eval_overlap_on(const cfr_handle *) { return true; }
+
 template <typename T>
 static int launch_top_part(cfr_handle *h, cudaStream_t s, int phase, int upd, bool pdl) {
   const InstDesc d = top_desc(h, h->top_k);
@@ -1243,6 +1247,8 @@ extern "C" int cfr_export_array(const cfr_handle *h, int which, void *out, int64
   const void *src = nullptr;
   int64_t n = 0;
   size_t esz = 4;
+  const int32_t plan[6] = {h->solo_smem > 0 ? h->solo_threads : 0, h->solo_lanes, h->top_k, h->top_lanes, overlap_on(h),
+                           eval_overlap_on(h)};
   switch (which) {
     case 0: src = c.child_begin.data(); n = (int64_t)c.child_begin.size(); break;
     case 1: src = c.node_slot.data(); n = (int64_t)c.node_slot.size(); break;
@@ -1281,6 +1287,7 @@ extern "C" int cfr_export_array(const cfr_handle *h, int which, void *out, int64
     case 34: src = h->stream_c0.data(); n = (int64_t)h->stream_c0.size(); break;
     case 35: src = h->stream_ok.data(); n = (int64_t)h->stream_ok.size(); break;
     case 36: src = h->pull_grid.data(); n = (int64_t)h->pull_grid.size(); break;
+    case 37: src = plan; n = sizeof plan / sizeof plan[0]; break;
     default: return set_err(CFR_ERR_ARG, "cfr_export_array: unknown array %d", which);
   }
   *count = n;

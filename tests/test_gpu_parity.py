@@ -525,3 +525,34 @@ def test_launch_count_gate(order, halves):
     assert c["graph_k_kernels"] == 5 * halves * (2 * D - 1)
     p = solve_gpu(g, 3, precision=cfr.P32, form=cfr.EXEC_PERSISTENT, order=order)
     assert p.counts_now()["graph_kernels"] == 0
+
+
+BITS_GAMES = {"tiny": lambda: gg.tiny_card(), "rt8": lambda: gg.random_tree(1, depth=8), "rt10": lambda: gg.random_tree(1, depth=10),
+              "endgame_5k": lambda: gg.endgame(3, 5000), "endgame_300k": lambda: gg.endgame(3, 300000)}
+
+
+def strategies(g, n=30, **kw):
+    s = cfr.Solver(g, **kw)
+    s.iterate(n)
+    out = s.avg_strategy()
+    s.close()
+    return out
+
+
+@pytest.mark.parametrize("precision", [cfr.P32, cfr.P64])
+@pytest.mark.parametrize("name", list(BITS_GAMES))
+def test_launch_options_leave_the_bits_of_the_automatic_form(name, precision):
+    g = BITS_GAMES[name]()
+    ref = strategies(g, precision=precision)
+    for kw in ({"launch_overlap": cfr.OVERLAP_OFF}, {"launch_overlap": cfr.OVERLAP_ON}, {"graph_iters": 7},
+               {"launch_overlap": cfr.OVERLAP_OFF, "graph_iters": 30}):
+        np.testing.assert_array_equal(strategies(g, precision=precision, **kw), ref, err_msg=str(kw))
+
+
+@pytest.mark.parametrize("precision,lanes", [(cfr.P64, 0), (cfr.P32, 8), (cfr.P32, 32), (cfr.P32, 256)])
+@pytest.mark.parametrize("name", list(BITS_GAMES))
+def test_reach_orders_leave_the_bits_where_the_header_says_so(name, precision, lanes):
+    g = BITS_GAMES[name]()
+    ref = strategies(g, precision=precision, lanes_per_set=lanes)
+    for order in (cfr.REACH_BFS, cfr.REACH_SLOTS):
+        np.testing.assert_array_equal(strategies(g, precision=precision, lanes_per_set=lanes, reach_order=order), ref)
