@@ -150,8 +150,8 @@ typedef struct cfr_options {
    * previous launch to complete (so every read sees every earlier write),
    * but its launch and block scheduling overlap the previous kernel's tail
    * (and the FP32 streaming backward copies its first inputs before that
-   * wait). CFR_OVERLAP_OFF: plain stream order. CFR_OVERLAP_AUTO (default):
-   * on in CFR_P32, and in CFR_P64 up to 100,000 nodes (measured on one
+   * wait), and so are an evaluation's. CFR_OVERLAP_OFF: plain stream order.
+   * CFR_OVERLAP_AUTO (default): on in evaluations, in CFR_P32, and in CFR_P64 up to 100,000 nodes (measured on one
    * GB300: the FP64 card game takes 8.5 ms per iteration without it and
    * 10.4 ms with it). Results are bitwise the same. */
   int launch_overlap;

@@ -29,3 +29,13 @@ def test_a_form_or_a_shape_that_is_asked_for_is_the_one_that_runs(kw):
     assert p["resident_threads"] == 0
     if "lanes_per_set" in kw or "reach_order" in kw:
         assert p["near_root_depth"] == -1
+
+
+def test_launches_overlap_where_the_option_says():
+    g, off, on = gg.tiny_card(), cfr.OVERLAP_OFF, cfr.OVERLAP_ON
+    for precision in (cfr.P32, cfr.P64):
+        for overlap, want in ((off, (0, 0)), (on, (1, 1)), (cfr.OVERLAP_AUTO, (1, 1))):
+            p = plan(g, precision=precision, launch_overlap=overlap)
+            assert (p["overlap"], p["evaluation_overlap"]) == want
+    p = plan(gg.random_tree(3, depth=11), precision=cfr.P64)  # more than 100,000 nodes
+    assert (p["overlap"], p["evaluation_overlap"]) == (0, 1)
