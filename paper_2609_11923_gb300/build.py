@@ -15,10 +15,10 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # --fmad=false: no contraction of a*b+c, so FP64 kernels round exactly like
 # the plain definition (bitwise parity in the FP64 mode).
 NVFLAGS = ARCH + ["-O3", "-lineinfo", "--fmad=false", "-std=c++17", "-Xcompiler", "-fPIC"]
-CU_UNITS = ["cfr_api", "k_bwd32", "k_bwd64", "k_pers32", "k_pers64", "k_br", "k_batch32", "k_batch64", "k_batchbr", "k_top32", "k_top64", "mlp", "mlp_fused"]
+CU_UNITS = ["cfr_api", "k_bwd32", "k_bwd64", "k_pers32", "k_pers64", "k_br", "k_batch32", "k_batch64", "k_batchbr", "k_push32", "k_push64", "k_top32", "k_top64", "mlp", "mlp_fused"]
 # FP32-only units may contract a*b+c into one FMA (deterministic, and the
 # FP32 mode is held to the exploitability tolerance, not to bitwise parity).
-FMA_UNITS = {"k_bwd32", "k_pers32", "k_batch32", "k_top32"}
+FMA_UNITS = {"k_bwd32", "k_pers32", "k_batch32", "k_push32", "k_top32"}
 CPP_UNITS = ["compile"]
 
 

@@ -52,19 +52,15 @@ static cudaError_t launch_batch_one(const BatchLaunch &l, cudaStream_t s, const 
 }
 
 // FP64 sums do not depend on the lane count: chains of four or eight lanes.
+template <typename T, int L> constexpr int kBatchLanes = sizeof(T) == 4 ? L : (L <= 4 ? 4 : 8);
+
 template <typename T>
 cudaError_t launch_batch_iterate(int maxa, int lanes, int threads, const BatchLaunch &l, cudaStream_t s,
                                  const InstDesc *table, const InstDesc &one) {
-  if (l.push) {  // the other reach orders: one shape
-    if (maxa == 4)
-      return l.mode == kCluster ? launch_batch_any(batch_iterate_push_kernel<T, 4, 4, 256, kCluster>, 256, l, s, table, one)
-                                : launch_batch_any(batch_iterate_push_kernel<T, 4, 4, 256, kSolo>, 256, l, s, table, one);
-    return l.mode == kCluster ? launch_batch_any(batch_iterate_push_kernel<T, 8, 4, 256, kCluster>, 256, l, s, table, one)
-                              : launch_batch_any(batch_iterate_push_kernel<T, 8, 4, 256, kSolo>, 256, l, s, table, one);
-  }
+  if (l.push) return launch_batch_push<T>(maxa, lanes, threads, l, s, table, one);
 #define IT_CASE(MA, L, TH)                       \
   if (maxa == MA && lanes == L && threads == TH) \
-    return launch_batch_one<T, MA, sizeof(T) == 4 ? L : (L <= 4 ? 4 : 8), TH>(l, s, table, one);
+    return launch_batch_one<T, MA, kBatchLanes<T, L>, TH>(l, s, table, one);
   CFR_BATCH_ALL(IT_CASE)
 #undef IT_CASE
   return cudaErrorInvalidValue;

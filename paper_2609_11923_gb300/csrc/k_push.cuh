@@ -1,0 +1,25 @@
+// k_push.cuh — dispatch of the batched kernels of the pushing reach orders (in
+// files of their own: compiled beside k_batch.cuh's, and loaded when used).
+#pragma once
+#include "k_batch.cuh"
+
+namespace cfr {
+
+template <typename T, int MA, int L, int TH>
+static cudaError_t push_one(const BatchLaunch &l, cudaStream_t s, const InstDesc *table, const InstDesc &one) {
+  constexpr int NT = kBatchThreads<T, MA, TH>;
+  if (l.mode == kCluster) return launch_batch_any(batch_iterate_push_kernel<T, MA, L, NT, kCluster>, NT, l, s, table, one);
+  return launch_batch_any(batch_iterate_push_kernel<T, MA, L, NT, kSolo>, NT, l, s, table, one);
+}
+
+template <typename T>
+cudaError_t launch_batch_push(int maxa, int lanes, int threads, const BatchLaunch &l, cudaStream_t s,
+                              const InstDesc *table, const InstDesc &one) {
+#define PUSH_CASE(MA, L, TH)                     \
+  if (maxa == MA && lanes == L && threads == TH) return push_one<T, MA, kBatchLanes<T, L>, TH>(l, s, table, one);
+  CFR_BATCH_ALL(PUSH_CASE)
+#undef PUSH_CASE
+  return cudaErrorInvalidValue;
+}
+
+}  // namespace cfr

@@ -77,6 +77,10 @@ cudaError_t batch_cluster_room(int cluster, int *clusters);
 template <typename T>
 cudaError_t launch_batch_iterate(int maxa, int lanes, int threads, const BatchLaunch &l, cudaStream_t s,
                                  const InstDesc *table, const InstDesc &one);
+// launch_batch_iterate's launches with l.push.
+template <typename T>
+cudaError_t launch_batch_push(int maxa, int lanes, int threads, const BatchLaunch &l, cudaStream_t s,
+                              const InstDesc *table, const InstDesc &one);
 cudaError_t launch_batch_br(int maxa, int lanes, int threads, const BatchLaunch &l, cudaStream_t s,
                             const InstDesc *table, const InstDesc &one);
 

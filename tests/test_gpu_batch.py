@@ -377,3 +377,30 @@ def test_best_response_of_a_wide_root_does_not_depend_on_the_mix(threads):
         for h in hs:
             cfr.cfr_destroy(h)
     np.testing.assert_array_equal(rows[0], rows[1])
+
+
+@pytest.mark.parametrize("threads", [256, 1024])
+def test_pushing_orders_take_the_callers_shape(threads):
+    specs = [gg.endgame(5, 4000), gg.tiny_card(), gg.random_tree(3, depth=8)]  # up to seven actions, and up to four
+    specs = [specs, specs[1:]]
+    for games in specs:
+        want = [oracle.solve(sp, 40).avg_strategy() for sp in games]
+        fp32 = {}
+        for lanes in (2, 4, 8, 32):
+            for cluster in (1, 2):
+                for precision in (cfr.P64, cfr.P32):
+                    pool, hs, table, tp, tb, s = bound(games, precision, cfr.REACH_BFS)
+                    cfr.cfr_batch_iterate(hs, 40, tp, tb, threads, lanes, s, cluster=cluster)
+                    got = []
+                    for h in hs:
+                        got.append(np.empty(cfr.cfr_get_counts(h)["n_slots"]))
+                        cfr.cfr_avg_strategy(h, got[-1], False, s)
+                        cfr.cfr_destroy(h)
+                    if precision == cfr.P64:
+                        for x, y in zip(got, want):
+                            np.testing.assert_array_equal(x, y)
+                    else:  # the shape of the sums follows the lanes, not the CTAs
+                        fp32.setdefault(lanes, got)
+                        for x, y in zip(got, fp32[lanes]):
+                            np.testing.assert_array_equal(x, y)
+        assert any(not np.array_equal(x, y) for x, y in zip(fp32[4], fp32[32]))
