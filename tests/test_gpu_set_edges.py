@@ -97,3 +97,29 @@ def test_sets_of_different_sizes_share_a_warp(most, lanes, order):
     np.testing.assert_array_equal(R, o.R)
     np.testing.assert_array_equal(avg, o.sbar)
     s.close()
+
+
+def seconds(s, n=20):
+    s.iterate(n)
+    torch.cuda.synchronize()
+    best = 1e9
+    for _ in range(5):
+        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        e0.record()
+        s.iterate(n)
+        e1.record()
+        torch.cuda.synchronize()
+        best = min(best, e0.elapsed_time(e1))
+    return best
+
+
+def test_short_sets_do_not_pay_for_the_lanes_of_a_group():
+    # sets of one member by groups of 32 lanes: no slower than by groups of 4
+    from tests.test_gpu_batch import chain_game
+
+    took = {}
+    for lanes in (4, 32):
+        s = cfr.Solver(chain_game(40), precision=cfr.P64, exec_form=cfr.EXEC_PERSISTENT, lanes_per_set=lanes)
+        took[lanes] = seconds(s)
+        s.close()
+    assert took[32] < 1.12 * took[4], took
