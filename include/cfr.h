@@ -344,12 +344,16 @@ int cfr_export_array(const cfr_handle *h, int which, void *out, int64_t capacity
  * (1, 2, 4, 8, 16, 32, and 256 = one block per set when sets have at most 8
  * actions, and 512 = the streaming backward at depths that can stream;
  * `reps` launches each; 512 only where sets have at least 32 members on
- * average) and takes the fastest where `reps` whole iterations are faster with
- * it than with the present choice; in the
- * persistent form it also times whole persistent iterations per lane count.
+ * average) and takes the fastest (in games whose iteration moves more than 32
+ * MB only where `reps` whole iterations are faster with it than with the
+ * present choice; in smaller ones all depths' winners stay only if whole
+ * iterations are no slower with them); in the persistent form it also times
+ * whole persistent iterations per lane count. Then the near-root launch and
+ * the resident form stay only where calls of `reps` iterations are not slower
+ * with them (cfr_export_array 37).
  * Trial launches overwrite the solver state, so the call ends by resetting it
  * (as cfr_reset) and dropping a captured graph. The chosen counts are
- * exported as array 12. In the FP32 mode the lane count fixes the shape of
+ * exported as array 12. In the FP32 mode the lane count and the form fix the shape of
  * the member reductions, so a different choice changes the last bits of the
  * iterates; pin it with cfr_options.lanes_per_set for bitwise repeatability
  * across processes. Synchronises `stream`. */

@@ -1617,6 +1617,150 @@ extern "C" int cfr_launch_floor(cfr_handle *h, int64_t n, void *stream, double *
   return rc;
 }
 
+// Iterations of fewer bytes than this keep most of their state in L2.
+constexpr int64_t kDuelBytes = int64_t(32) << 20;
+
+struct TuneClock {
+  cudaStream_t s;
+  cudaEvent_t e0 = nullptr, e1 = nullptr;
+  ~TuneClock() {
+    if (e0) cudaEventDestroy(e0);
+    if (e1) cudaEventDestroy(e1);
+  }
+  int start() {
+    CK(cudaEventCreate(&e0));
+    CK(cudaEventCreate(&e1));
+    return CFR_OK;
+  }
+  template <typename F> int time(int n, F &&launch, float *ms) {
+    CK(cudaEventRecord(e0, s));
+    for (int r = 0; r < n; ++r)
+      if (int e = launch()) return e;
+    CK(cudaEventRecord(e1, s));
+    CK(cudaEventSynchronize(e1));
+    CK(cudaEventElapsedTime(ms, e0, e1));
+    return CFR_OK;
+  }
+};
+
+// Lanes per set of every depth's backward launch (the near-root and resident
+// forms are off).
+template <typename T>
+static int tune_levels(cfr_handle *h, int reps, TuneClock &clock) {
+  const Compiled &c = h->c;
+  cudaStream_t s = clock.s;
+  const std::vector<int32_t> first = h->level_lanes;
+  // kThreads = one set per block
+  const std::vector<int> cand = h->maxa_tier <= 8 ? std::vector<int>{1, 2, 4, 8, 16, 32, kThreads} : std::vector<int>{4, 8, 16, 32};
+  auto run_iter = [&]() { return enqueue_iteration<T>(h, s); };
+  int rc = run_iter();  // realistic reach and values for the trials
+  if (rc) return rc;
+  const bool duel = algo_bytes_per_iter(c, h->precision) > kDuelBytes;
+  for (int64_t d = c.D - 1; d >= 0; --d) {
+    int best = first[d];
+    float best_ms = 1e30f;
+    std::vector<int> cd = cand;
+    // the streaming form works through a team's sets one group at a time: a
+    // candidate only where sets are long
+    if (h->stream_ok[d] && c.level_mean_members[d] >= kStreamMinMembers) cd.push_back(kStreamLanes);
+    auto run_depth = [&]() { return launch_bwd<T>(h, (int)d, s); };
+    for (int L : cd) {  // by itself first: once (the launch before may load the kernel), and more if that was not hopeless
+      float ms = 0.f;
+      h->level_lanes[d] = L;
+      if ((rc = run_depth()) || (rc = clock.time(1, run_depth, &ms))) return rc;
+      if (ms * reps > 2.f * best_ms) continue;
+      if ((rc = clock.time(reps, run_depth, &ms))) return rc;
+      if (ms < best_ms) { best_ms = ms; best = L; }
+    }
+    // A depth's launch repeated by itself finds its inputs in L2, which in an
+    // iteration the launches before have left elsewhere (lane groups at two
+    // depths of the 27M-node card game that streams faster: an iteration of
+    // 145 us instead of 131). So in large games the winner has to win in whole
+    // iterations too.
+    if (duel && best != first[d]) {
+      float ms_first = 0.f, ms_best = 0.f;
+      h->level_lanes[d] = first[d];
+      if ((rc = clock.time(reps, run_iter, &ms_first))) return rc;
+      h->level_lanes[d] = best;
+      if ((rc = clock.time(reps, run_iter, &ms_best))) return rc;
+      if (ms_best > 0.99f * ms_first) best = first[d];
+    }
+    h->level_lanes[d] = best;
+  }
+  if (!duel && h->level_lanes != first) {  // in small games all winners together
+    float ms_first = 0.f, ms_best = 0.f;
+    const std::vector<int32_t> best = h->level_lanes;
+    if ((rc = clock.time(reps, run_iter, &ms_best))) return rc;
+    h->level_lanes = first;
+    if ((rc = run_iter()) || (rc = clock.time(reps, run_iter, &ms_first))) return rc;
+    if (ms_best <= ms_first) h->level_lanes = best;
+  }
+  return CFR_OK;
+}
+
+template <typename T>
+static int tune_persistent(cfr_handle *h, int reps, TuneClock &clock) {
+  // groups of at most a warp
+  const std::vector<int> cand = h->maxa_tier <= 8 ? std::vector<int>{1, 2, 4, 8, 16, 32} : std::vector<int>{4, 8, 16, 32};
+  int best = h->persist_lanes, rc = CFR_OK;
+  float best_ms = 1e30f;
+  for (int L : cand) {
+    float ms = 0.f;
+    h->persist_lanes = L;
+    h->persist_grid = 0;
+    if ((rc = launch_persistent_form<T>(h, 1, clock.s))) break;
+    if ((rc = clock.time(1, [&]() { return launch_persistent_form<T>(h, reps, clock.s); }, &ms))) break;
+    if (ms < best_ms) { best_ms = ms; best = L; }
+  }
+  h->persist_lanes = best;
+  h->persist_grid = 0;
+  return rc;
+}
+
+// Tunes the launches of every depth, then keeps the near-root launch and the
+// resident form only where a call of `reps` iterations is not slower with them
+// (a set of 300 members of five actions in FP64: near-root 125 us an
+// iteration, by blocks of their own 74).
+template <typename T>
+static int tune(cfr_handle *h, int reps, cudaStream_t s) {
+  const int near_root = h->top_k;
+  const uint32_t solo = h->solo_smem;
+  TuneClock clock{s};
+  h->top_k = -1;
+  h->solo_smem = 0;
+  int rc = clock.start();
+  if (rc == CFR_OK) rc = tune_levels<T>(h, reps, clock);
+  if (rc == CFR_OK && h->exec_form == CFR_EXEC_PERSISTENT) rc = tune_persistent<T>(h, reps, clock);
+  auto call = [&](float *ms) {
+    drop_graphs(h);
+    int e = iterate_t<T>(h, reps, s);  // captures
+    *ms = 1e30f;
+    for (int k = 0; k < 3 && e == CFR_OK; ++k) {
+      float one = 0.f;
+      e = clock.time(1, [&]() { return iterate_t<T>(h, reps, s); }, &one);
+      *ms = std::min(*ms, one);
+    }
+    return e;
+  };
+  const bool launches = h->exec_form != CFR_EXEC_PERSISTENT && near_root >= 0;
+  float ms = 0.f, with = 0.f;
+  if (rc == CFR_OK && (launches || solo)) rc = call(&ms);
+  if (rc == CFR_OK && launches) {
+    h->top_k = near_root;
+    rc = call(&with);
+    if (rc == CFR_OK && with > 1.02f * ms) h->top_k = -1;
+    else ms = with;
+  }
+  if (rc == CFR_OK && solo) {
+    h->solo_smem = solo;
+    rc = call(&with);
+    if (rc == CFR_OK && with > 1.02f * ms) h->solo_smem = 0;
+  }
+  if (h->exec_form == CFR_EXEC_PERSISTENT || rc) h->top_k = near_root;
+  if (rc) h->solo_smem = solo;
+  return rc;
+}
+
 extern "C" int cfr_autotune(cfr_handle *h, int reps, void *stream) {
   if (!h) return set_err(CFR_ERR_ARG, "cfr_autotune: null handle");
   if (!h->bound) return set_err(CFR_ERR_NOT_BOUND, "cfr_autotune: call cfr_bind first");
@@ -1624,81 +1768,7 @@ extern "C" int cfr_autotune(cfr_handle *h, int reps, void *stream) {
   const Compiled &c = h->c;
   if (c.D == 0) return CFR_OK;
   cudaStream_t s = (cudaStream_t)stream;
-  // per-level candidates (kThreads = one set per block); the persistent kernel takes groups of at most a warp
-  std::vector<int> cand = h->maxa_tier <= 8 ? std::vector<int>{1, 2, 4, 8, 16, 32, kThreads} : std::vector<int>{4, 8, 16, 32};
-  std::vector<int> cand_p = h->maxa_tier <= 8 ? std::vector<int>{1, 2, 4, 8, 16, 32} : std::vector<int>{4, 8, 16, 32};
-  cudaEvent_t e0, e1;
-  CK(cudaEventCreate(&e0));
-  CK(cudaEventCreate(&e1));
-  int rc = CFR_OK;
-  auto run_iter = [&]() -> int {
-    return h->precision == CFR_P64 ? enqueue_iteration<double>(h, s) : enqueue_iteration<float>(h, s);
-  };
-  rc = h->precision == CFR_P64 ? enqueue_start<double>(h, s) : enqueue_start<float>(h, s);
-  if (rc == CFR_OK) rc = run_iter();  // realistic reach and values for the trials
-  for (int64_t d = c.D - 1; d > h->top_k && rc == CFR_OK; --d) {  // the near-root kernel has one shape
-    const int first = h->level_lanes[d];
-    int best = first;
-    float best_ms = 1e30f;
-    std::vector<int> cd = cand;
-    // the streaming form works through a team's sets one group at a time: a
-    // candidate only where sets are long
-    if (h->stream_ok[d] && c.level_mean_members[d] >= kStreamMinMembers) cd.push_back(kStreamLanes);
-    auto time = [&](int L, int n, auto &&launch, float *ms) -> int {
-      h->level_lanes[d] = L;
-      CK(cudaEventRecord(e0, s));
-      for (int r = 0; r < n; ++r)
-        if (int e = launch()) return e;
-      CK(cudaEventRecord(e1, s));
-      CK(cudaEventSynchronize(e1));
-      CK(cudaEventElapsedTime(ms, e0, e1));
-      return CFR_OK;
-    };
-    auto run_depth = [&]() -> int {
-      return h->precision == CFR_P64 ? launch_bwd<double>(h, (int)d, s) : launch_bwd<float>(h, (int)d, s);
-    };
-    for (int L : cd) {  // by itself first: one launch, and more if that was not hopeless
-      float ms = 0.f;
-      rc = time(L, 1, run_depth, &ms);
-      if (rc) break;
-      if (ms * reps > 2.f * best_ms) continue;
-      rc = time(L, reps, run_depth, &ms);
-      if (rc) break;
-      if (ms < best_ms) { best_ms = ms; best = L; }
-    }
-    // A depth's launch repeated by itself finds its inputs in L2, which in an
-    // iteration the launches before have left elsewhere (lane groups at two
-    // depths of the 27M-node card game that streams faster: an iteration of
-    // 145 us instead of 131). So the winner has to win in whole iterations too.
-    if (rc == CFR_OK && best != first) {
-      float ms_first = 0.f, ms_best = 0.f;
-      rc = time(first, reps, run_iter, &ms_first);
-      if (rc == CFR_OK) rc = time(best, reps, run_iter, &ms_best);
-      if (ms_best > 0.99f * ms_first) best = first;
-    }
-    h->level_lanes[d] = best;
-  }
-  if (rc == CFR_OK && h->exec_form == CFR_EXEC_PERSISTENT) {
-    int best = h->persist_lanes;
-    float best_ms = 1e30f;
-    for (int L : cand_p) {
-      h->persist_lanes = L;
-      h->persist_grid = 0;
-      rc = h->precision == CFR_P64 ? launch_persistent_form<double>(h, 1, s) : launch_persistent_form<float>(h, 1, s);
-      if (rc) break;
-      CK(cudaEventRecord(e0, s));
-      rc = h->precision == CFR_P64 ? launch_persistent_form<double>(h, reps, s) : launch_persistent_form<float>(h, reps, s);
-      CK(cudaEventRecord(e1, s));
-      CK(cudaEventSynchronize(e1));
-      float ms = 0.f;
-      CK(cudaEventElapsedTime(&ms, e0, e1));
-      if (ms < best_ms) { best_ms = ms; best = L; }
-    }
-    h->persist_lanes = best;
-    h->persist_grid = 0;
-  }
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
+  int rc = h->precision == CFR_P64 ? tune<double>(h, reps, s) : tune<float>(h, reps, s);
   if (rc) return rc;
   drop_graphs(h);
   CK(cudaMemsetAsync(h->arena + h->b_err.off, 0, 16, s));

@@ -123,3 +123,22 @@ def test_short_sets_do_not_pay_for_the_lanes_of_a_group():
         took[lanes] = seconds(s)
         s.close()
     assert took[32] < 1.12 * took[4], took
+
+
+@pytest.mark.parametrize("g", [two_level_game(300, 5, 8), two_level_game(1000, 2, 2), gg.random_tree(1, depth=8)],
+                         ids=["300x5x8", "1000x2x2", "rt8"])
+def test_tuning_is_not_slower_than_a_shape_that_it_tries(g):
+    # long sets near the root, and a game at the edge of the resident form
+    fixed = []
+    for lanes in (8, 32, 256):
+        s = cfr.Solver(g, precision=cfr.P64, exec_form=cfr.EXEC_GRAPH, lanes_per_set=lanes)
+        fixed.append(seconds(s))
+        s.close()
+    s = cfr.Solver(g, precision=cfr.P64)
+    s.autotune()
+    tuned = seconds(s)
+    s.reset()
+    s.iterate(9)
+    np.testing.assert_array_equal(s.avg_strategy(), oracle.solve(g, 9).avg_strategy())
+    s.close()
+    assert tuned < 1.2 * min(fixed), (tuned, fixed)
