@@ -1,10 +1,13 @@
 """The streaming backward's teams, checked on the CPU: a model of one team
 (its warps, the copies in flight, the stage barriers and the barrier at the
-end of a group) under random interleavings. No stage is refilled while a warp
-still reads it, no partial sums are overwritten before the first warp has
-added them, no parity wait sees its barrier two phases ahead, and every warp
-finishes. A team whose first warp refills before the group's barrier shows the
-checker at work.
+end of a group) under random interleavings. The warps take turns: the one whose
+turn a group is (its number in the team's sequence modulo the warps) adds the
+partial sums, refills the stage after a chunk's last group and updates the
+slots; after a chance chunk warp 0 refills. No stage is refilled while a warp
+still reads it, no partial sums are overwritten before their warp has added
+them, no parity wait sees its barrier two phases ahead, and every warp
+finishes. A warp that refills before the group's barrier, and partial sums in
+one buffer, show the checker at work.
 """
 import random
 
@@ -17,14 +20,14 @@ class Hazard(AssertionError):
     pass
 
 
-def run(groups, warps, seed, refill_early=False):
+def run(groups, warps, seed, refill_early=False, buffers=2):
     """groups[i]: groups of chunk i (0: a chance chunk, which has one barrier
     too). Returns once every warp has finished."""
     rng = random.Random(seed)
     full, sync, arrived = [0] * STAGES, [0], [0]  # phases completed; arrivals of the phase under way
     holds = [None] * STAGES                       # the chunk whose copies a stage takes or holds
     reading = [set() for _ in range(STAGES)]
-    red = [None, None]                            # the group whose sums red[p] holds until warp 0 has read them
+    red = [None] * buffers                        # the group whose sums red[p] holds until their warp has read them
     copies = []                                   # stages with copies in flight
 
     def issue(i):
@@ -50,12 +53,13 @@ def run(groups, warps, seed, refill_early=False):
             for q in range(max(n, 1)):
                 yield  # the members, from the stage
                 last = q == max(n, 1) - 1
-                if refill_early and last and w == 0 and i + STAGES < len(groups):
+                turn = w == (phase % warps if n else 0)  # adds the sums, refills, updates
+                if refill_early and last and turn and i + STAGES < len(groups):
                     issue(i + STAGES)
-                if n and red[phase % 2] not in (None, phase):
-                    raise Hazard("partial sums overwritten")
                 if n:
-                    red[phase % 2] = phase
+                    if red[phase % buffers] not in (None, phase):
+                        raise Hazard("partial sums overwritten")
+                    red[phase % buffers] = phase
                 if last:
                     reading[s].discard(w)
                 if warps > 1:
@@ -65,11 +69,15 @@ def run(groups, warps, seed, refill_early=False):
                         sync[0] += 1
                     while not ready(sync[0], phase):
                         yield
-                if w == 0:
+                if turn:
+                    if n:
+                        yield  # the sums of the warps in order
+                        if red[phase % buffers] != phase:
+                            raise Hazard("partial sums of another group")
+                        red[phase % buffers] = None
                     if last and i + STAGES < len(groups) and not refill_early:
                         issue(i + STAGES)
-                    yield  # the sums and the update
-                    red[phase % 2] = None
+                    yield  # the update
                 phase += 1
 
     for i in range(min(STAGES, len(groups))):
@@ -100,3 +108,18 @@ def test_a_refill_before_the_barrier_is_caught():
     with pytest.raises(Hazard):
         for seed in range(150):
             run([1, 2, 1, 2, 1, 2], 4, seed, refill_early=True)
+
+
+def test_one_buffer_of_partial_sums_is_caught():
+    # the next group's first warp can be there while this group's warp, another
+    # one, has not read them yet
+    with pytest.raises(Hazard):
+        for seed in range(150):
+            run([1, 2, 1, 2, 1, 2], 4, seed, buffers=1)
+
+
+@pytest.mark.parametrize("groups", [[], [0], [1], [0] * 9, [3] * 9, [1, 0, 2, 0, 0, 3, 1]])
+def test_sequences_at_the_edges(groups):
+    for warps in (1, 3, 5, 8):
+        for seed in range(30):
+            run(groups, warps, seed)
