@@ -10,6 +10,7 @@ layer is h_out = relu(h_in @ W + b).
 from __future__ import annotations
 
 import ctypes
+from operator import attrgetter
 from typing import List, Optional
 
 import numpy as np
@@ -41,6 +42,7 @@ for _f in ("mlp_gemm", "mlp_softmax_xent", "mlp_relu_grad", "mlp_colsum", "mlp_a
 _lib.mlp_last_error.restype = ctypes.c_char_p
 
 N_OUT = 8
+_VERSION = attrgetter("_version")
 
 
 def _ck(rc):
@@ -95,14 +97,15 @@ class MLP:
             # set to 1 by an inference kernel whose bounded wait gave up
             # (page-locked: the host reads it without a copy)
             self._err = torch.zeros(1, dtype=torch.int32).pin_memory()
+            self._err_host = self._err.numpy()
         self.sync_bf16()
 
     def _s(self) -> int:
         return int(self.torch.cuda.current_stream(self.dev).cuda_stream)
 
     def _raise_if_failed(self):
-        if self.fused and self._err.numpy()[0] != 0:
-            self._err.zero_()
+        if self.fused and self._err_host[0] != 0:
+            self._err_host[0] = 0
             raise RuntimeError("mlp: a bounded wait of an inference kernel gave up; its probabilities are NaN")
 
     def check(self) -> None:
@@ -121,7 +124,7 @@ class MLP:
         they are gone, which raises."""
         if self._acts is None and self._fused_pass is not None:
             X, then = self._fused_pass
-            if X is None or then != self._versions(X):
+            if X is None or then != self._counters([X, *self.b]) or not self._packed():
                 raise RuntimeError("mlp: the activations of the last fused pass are gone (its weights or its batch have "
                                    "changed since); run forward(X)")
             self.forward(X)
@@ -131,21 +134,31 @@ class MLP:
     def acts(self, value):
         self._acts, self._fused_pass = value, None
 
-    def _versions(self, X):
-        """Write counters of what a pass over X reads."""
-        return [self._version(t) for t in [X] + self.Wb + self.b]
-
+    # A pass over X reads X, the biases, and Wb or its images; the write
+    # counters of tensors tell whether a caller has written into them since
+    # (inference tensors have none and count as never written).
     @staticmethod
-    def _version(t) -> int:
-        return 0 if t.is_inference() else t._version
+    def _counters(ts):
+        try:
+            return [*map(_VERSION, ts)]
+        except RuntimeError:
+            return [-1 if t.is_inference() else t._version for t in ts]
 
     def _ran_fused(self, X):
-        self._acts, self._fused_pass = None, (X, self._versions(X))
+        self._acts, self._fused_pass = None, (X, self._counters([X, *self.b]))
 
     def _weights_change(self):  # by a kernel, past the counters: Wb and its images together
-        self._images_of = [(w, self._version(w)) for w in self.Wb]
+        wb = self.Wb.copy()  # held, so that no other tensor can have their ids
+        self._images_of = (wb, [*map(id, wb)], self._counters(wb))
         if self._fused_pass is not None:
             self._fused_pass = (None, None)
+
+    def _packed(self) -> bool:
+        """Whether the packed images are those of Wb. A caller's write into Wb,
+        or other tensors in its place, reach only the layer-by-layer passes,
+        until sync_bf16 or a step writes both."""
+        _, ids, then = self._images_of
+        return [*map(id, self.Wb)] == ids and self._counters(self.Wb) == then
 
     def sync_bf16(self):
         self._weights_change()
@@ -159,12 +172,6 @@ class MLP:
     @staticmethod
     def _all(weights, biases):
         return _ptrs([t for pair in zip(weights, biases) for t in pair])
-
-    def _packed(self) -> bool:
-        """Whether the packed images are those of Wb. A caller's write into Wb,
-        or other tensors in its place, reach only the layer-by-layer passes,
-        until sync_bf16 or a step writes both."""
-        return all(w is x and self._version(w) == v for w, (x, v) in zip(self.Wb, self._images_of))
 
     def _rows_ok(self, X) -> bool:
         return (self.fused and self._packed() and X.dtype == self.torch.float32 and X.dim() == 2 and X.shape[0] > 0
@@ -209,18 +216,26 @@ class MLP:
                 _ck(_lib.mlp_relu_grad(_p(dh), _p(h_in), dh.numel(), self._s()))
                 d = dh
 
+    def _fused_grad(self, X, B, nact, target, weight, loss) -> bool:
+        """Launches the fused pass; False, and nothing launched, if its kernels
+        cannot write the gradient tensors (views that are not 16-byte aligned)."""
+        need = _lib.mlp_net_work_bytes(self.dims[0], B)
+        if self.work is None or self.work.numel() < need:
+            self.work = self.torch.empty(need, dtype=self.torch.uint8, device=self.dev)
+        rc = _lib.mlp_net_grad(_p(X), self.dims[0], B, _p(self.img), _ptrs(self.b), _p(nact), _p(target), _p(weight),
+                               _ptrs(self.gW), _ptrs(self.gb), _p(self.work), self.work.numel(), ctypes.byref(loss),
+                               self._s())
+        if rc != 0 and any(g.data_ptr() % 16 for g in self.gW):
+            return False
+        _net_ck(rc)
+        return True
+
     def loss_and_grad(self, X, nact, target, weight=None) -> float:
         torch = self.torch
         self._raise_if_failed()
         B = X.shape[0]
-        if self._rows_ok(X) and all(g.data_ptr() % 16 == 0 for g in self.gW):
-            need = _lib.mlp_net_work_bytes(self.dims[0], B)
-            if self.work is None or self.work.numel() < need:
-                self.work = torch.empty(need, dtype=torch.uint8, device=self.dev)
-            loss = _vp()
-            _net_ck(_lib.mlp_net_grad(_p(X), self.dims[0], B, _p(self.img), _ptrs(self.b), _p(nact), _p(target),
-                                      _p(weight), _ptrs(self.gW), _ptrs(self.gb), _p(self.work), self.work.numel(),
-                                      ctypes.byref(loss), self._s()))
+        loss = _vp()
+        if self._rows_ok(X) and self._fused_grad(X, B, nact, target, weight, loss):
             self._ran_fused(X)
             at = loss.value - self.work.data_ptr()
             got = self.work[at:at + 8].cpu()

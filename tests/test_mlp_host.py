@@ -15,6 +15,7 @@ def bare(err=0):
     net = mlp.MLP.__new__(mlp.MLP)
     net.torch, net.dev, net.fused = torch, torch.device("cpu"), True
     net._err = torch.tensor([err], dtype=torch.int32)
+    net._err_host = net._err.numpy()
     net.Wb, net.b = [torch.zeros(3), torch.zeros(2)], [torch.zeros(3)]
     net.dims = [4, 2]
     net._acts, net._fused_pass = None, None
