@@ -766,7 +766,7 @@ __global__ void __launch_bounds__(NT, 1) batch_iterate_kernel(const InstDesc *ta
 // Breadth-first and value-slot reach orders (layout options): the same
 // iteration with the pushing forward of kernels.cuh.
 template <typename T, int MAXA, int LANES, int NT, int MODE>
-__global__ void __launch_bounds__(NT, 1) batch_iterate_push_kernel(const InstDesc *table,
+__global__ void __launch_bounds__(NT) batch_iterate_push_kernel(const InstDesc *table,
                                                                 const __grid_constant__ InstDesc one, int n_inst) {
   constexpr bool CLUSTERED = MODE == kCluster;
   __shared__ double sm[NT];
