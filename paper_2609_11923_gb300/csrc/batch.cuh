@@ -37,34 +37,47 @@ struct ClusterRoom {
 };
 
 // CTAs for every instance of a batch (host): 1, 2, 4, 8 or 16, at least
-// `least`. Estimated cycles of an iteration, from solves of endgames: in one
-// CTA 8,000 + 1.6 a node from shared memory (`alone`), 12,000 + 2 a node from
-// global memory; in a cluster 45,000 (2 D - 1 barriers of 1,900 with stores in
-// flight, and every read through L2) + 1.5 a node and CTA. The instance that
+// `least`, by an estimate of an iteration's time (batch_ns). The instance that
 // takes longest gets twice its CTAs as long as all of them run at the same
 // time (a cluster too many waits for a whole instance: ten large endgames with
 // six of 16 took 89 us an iteration, with four 64); a batch that does not run
 // at the same time anyway, while it takes longer than an even share of it.
 struct BatchLoad {
-  int64_t nodes;
-  double share;  // of the longest run's iterations
-  bool alone;
+  int64_t nodes, sets, depths;
+  int64_t chain;  // members of each depth's largest set, summed
+  bool resident;  // by one CTA, from shared memory
+  bool fp64;
+  double share;   // of the longest run's iterations
 };
+
+// An iteration by c CTAs in ns: what every depth costs (barriers and chains of
+// loads, both ways), what the CTAs share, and the largest sets, each walked by
+// one group. Least squares over 38 games alone, 1,024 threads and 8 lanes, 1 to
+// 16 CTAs: endgames of 10,000 to 920,000 nodes (5 depths), random trees of 122
+// to 275,000 (4 to 11), two-round card games of 2,800 to 350,000 (8), chains of
+// 10 to 100 depths, sets of 300 and 3,000 members; within 20% in FP32 (7 to 10%
+// on average), 36% in FP64 (13%). By nodes alone, fitted to endgames, a game of
+// 300 chains of 100 depths side by side got 16 CTAs: 881 us an iteration, by
+// one 696.
+inline double batch_ns(const BatchLoad &l, int c) {
+  const double D = (double)l.depths, I = (double)l.sets / c, N = (double)l.nodes / c, L = (double)l.chain;
+  if (l.fp64) return c > 1 ? 2500.0 + 3300.0 * D + 68.0 * I + 3.4 * N + 200.0 * L : 1340.0 * D + 61.0 * I + 3.3 * N + 137.0 * L;
+  if (c > 1) return 1800.0 + 2570.0 * D + 19.0 * I + 0.53 * N + 9.0 * L;
+  return l.resident ? 1700.0 + 580.0 * D + 10.5 * I + 0.13 * N + 6.6 * L : 580.0 * D + 19.0 * I + 0.39 * N + 8.3 * L;
+}
+
 inline std::vector<int> plan_clusters(const std::vector<BatchLoad> &load, int least, const ClusterRoom &room) {
   const int n = (int)load.size();
-  auto cycles = [&](int i, int c) {
-    const double N = (double)load[i].nodes;
-    const double t = c > 1 ? 45000.0 + 1.5 * N / c : load[i].alone ? 8000.0 + 1.6 * N : 12000.0 + 2.0 * N;
-    return t * load[i].share;
-  };
+  auto time = [&](int i, int c) { return batch_ns(load[i], c) * load[i].share; };
+  auto exists = [&](int c) { return c == 16 ? room.sixteen > 0 : c == 8 ? room.eight > 0 : c == 4 ? room.four > 0 : true; };
   std::vector<int> cta(n, least);
   int count[17] = {0};  // instances by CTAs
-  double work = 0.0;    // CTA cycles
-  std::priority_queue<std::pair<double, int>> longest;  // (cycles, instance)
+  double work = 0.0;    // CTA ns
+  std::priority_queue<std::pair<double, int>> longest;  // (ns, instance)
   for (int i = 0; i < n; ++i) {
     ++count[least];
-    work += least * cycles(i, least);
-    longest.push({cycles(i, least), -i});
+    work += least * time(i, least);
+    longest.push({time(i, least), -i});
   }
   auto fits = [&]() {
     const int eights = 2 * count[16] + count[8];
@@ -76,7 +89,7 @@ inline std::vector<int> plan_clusters(const std::vector<BatchLoad> &load, int le
     const double t = longest.top().first;
     const int i = -longest.top().second, c = cta[i];
     longest.pop();
-    if (c == 16 || cycles(i, 2 * c) >= t) continue;
+    if (c == 16 || !exists(2 * c) || time(i, 2 * c) >= t) continue;
     --count[c];
     ++count[2 * c];
     if (!fits() && !(waves && t > work / room.sms)) {
@@ -84,9 +97,9 @@ inline std::vector<int> plan_clusters(const std::vector<BatchLoad> &load, int le
       --count[2 * c];
       continue;
     }
-    work += 2 * c * cycles(i, 2 * c) - c * t;
+    work += 2 * c * time(i, 2 * c) - c * t;
     cta[i] = 2 * c;
-    longest.push({cycles(i, 2 * c), -i});
+    longest.push({time(i, 2 * c), -i});
   }
   return cta;
 }

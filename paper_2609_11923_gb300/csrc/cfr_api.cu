@@ -73,6 +73,7 @@ struct cfr_handle {
   Buf b_set_info, b_stream_chunks;
   // CFR_EXEC_AUTO, small games: the whole game resident in one CTA (0: not)
   uint32_t solo_smem = 0;
+  int64_t chain = 0;  // members of each depth's largest set, summed
   int solo_threads = 256, solo_lanes = 8;
   // per-level forms: depths 0 .. top_k near the root as one launch (-1: none)
   int top_k = -1, top_lanes = 8;
@@ -368,6 +369,12 @@ extern "C" int cfr_compile(const cfr_game_spec *spec, const cfr_options *opt, cf
       const uint32_t m = c.int_mask[q];
       if (c.int_slot[q] < 0 && m != 0u && ((m & kBigNode) || __builtin_popcount(m) > kFanLight)) w.fan = 1;
     }
+  }
+  for (int64_t d = 0; d < c.D; ++d) {
+    int64_t longest = 0;
+    for (int32_t I = c.level_iset[2 * d]; I < c.level_iset[2 * d + 2]; ++I)
+      longest = std::max<int64_t>(longest, c.iset_mem[I + 1] - c.iset_mem[I]);
+    h->chain += longest;
   }
   plan(h);
   choose_top(h);
@@ -1843,8 +1850,12 @@ static int batch_plan(cfr_handle *const *hs, int n, const int64_t *iters, int64_
     e[i].d = inst_desc(hs[i], iters ? iters[i] : n_iter);
     e[i].smem = iterate && cluster == 1 ? resident_bytes(hs[i], e[i].d) : 0;
     load[i].nodes = hs[i]->c.N;
+    load[i].sets = hs[i]->c.I;
+    load[i].depths = hs[i]->c.D;
+    load[i].chain = hs[i]->chain;
+    load[i].resident = e[i].smem > 0;
+    load[i].fp64 = !iterate || bp.precision == CFR_P64;  // a best response is in FP64
     load[i].share = iters ? (double)iters[i] / (double)longest : 1.0;
-    load[i].alone = e[i].smem > 0 && bp.precision == CFR_P32;
   }
   ClusterRoom room;
   int rc = cluster_room(&room);
