@@ -1627,6 +1627,8 @@ extern "C" int cfr_launch_floor(cfr_handle *h, int64_t n, void *stream, double *
 // Iterations of fewer bytes than this keep most of their state in L2.
 constexpr int64_t kDuelBytes = int64_t(32) << 20;
 
+static bool tune_duel(const cfr_handle *h) { return algo_bytes_per_iter(h->c, h->precision) > kDuelBytes; }
+
 struct TuneClock {
   cudaStream_t s;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -1662,7 +1664,7 @@ static int tune_levels(cfr_handle *h, int reps, TuneClock &clock) {
   auto run_iter = [&]() { return enqueue_iteration<T>(h, s); };
   int rc = run_iter();  // realistic reach and values for the trials
   if (rc) return rc;
-  const bool duel = algo_bytes_per_iter(c, h->precision) > kDuelBytes;
+  const bool duel = tune_duel(h);
   for (int64_t d = c.D - 1; d >= 0; --d) {
     int best = first[d];
     float best_ms = 1e30f;
@@ -1671,10 +1673,11 @@ static int tune_levels(cfr_handle *h, int reps, TuneClock &clock) {
     // candidate only where sets are long
     if (h->stream_ok[d] && c.level_mean_members[d] >= kStreamMinMembers) cd.push_back(kStreamLanes);
     auto run_depth = [&]() { return launch_bwd<T>(h, (int)d, s); };
-    for (int L : cd) {  // by itself first: once (the launch before may load the kernel), and more if that was not hopeless
+    for (int L : cd) {  // by itself: once, again if that was hopeless (it may have loaded the kernel), and more if not
       float ms = 0.f;
       h->level_lanes[d] = L;
-      if ((rc = run_depth()) || (rc = clock.time(1, run_depth, &ms))) return rc;
+      if ((rc = clock.time(1, run_depth, &ms))) return rc;
+      if (ms * reps > 2.f * best_ms && (rc = clock.time(1, run_depth, &ms))) return rc;
       if (ms * reps > 2.f * best_ms) continue;
       if ((rc = clock.time(reps, run_depth, &ms))) return rc;
       if (ms < best_ms) { best_ms = ms; best = L; }
@@ -1693,14 +1696,6 @@ static int tune_levels(cfr_handle *h, int reps, TuneClock &clock) {
       if (ms_best > 0.99f * ms_first) best = first[d];
     }
     h->level_lanes[d] = best;
-  }
-  if (!duel && h->level_lanes != first) {  // in small games all winners together
-    float ms_first = 0.f, ms_best = 0.f;
-    const std::vector<int32_t> best = h->level_lanes;
-    if ((rc = clock.time(reps, run_iter, &ms_best))) return rc;
-    h->level_lanes = first;
-    if ((rc = run_iter()) || (rc = clock.time(reps, run_iter, &ms_first))) return rc;
-    if (ms_best <= ms_first) h->level_lanes = best;
   }
   return CFR_OK;
 }
@@ -1724,20 +1719,24 @@ static int tune_persistent(cfr_handle *h, int reps, TuneClock &clock) {
   return rc;
 }
 
-// Tunes the launches of every depth, then keeps the near-root launch and the
-// resident form only where a call of `reps` iterations is not slower with them
-// (a set of 300 members of five actions in FP64: near-root 125 us an
-// iteration, by blocks of their own 74).
+// Tunes the launches of every depth, then keeps what it found (small games),
+// the near-root launch and the resident form only where calls of `reps`
+// iterations are not slower with them (a set of 300 members of five actions in
+// FP64: near-root 125 us an iteration, by blocks of their own 70).
 template <typename T>
 static int tune(cfr_handle *h, int reps, cudaStream_t s) {
+  const std::vector<int> first = h->level_lanes;
   const int near_root = h->top_k;
   const uint32_t solo = h->solo_smem;
+  const bool launches = h->exec_form != CFR_EXEC_PERSISTENT;
   TuneClock clock{s};
   h->top_k = -1;
   h->solo_smem = 0;
   int rc = clock.start();
   if (rc == CFR_OK) rc = tune_levels<T>(h, reps, clock);
-  if (rc == CFR_OK && h->exec_form == CFR_EXEC_PERSISTENT) rc = tune_persistent<T>(h, reps, clock);
+  if (rc == CFR_OK && !launches) rc = tune_persistent<T>(h, reps, clock);
+  const std::vector<int> found = h->level_lanes;
+  float best_ms = 1e30f;
   auto call = [&](float *ms) {
     drop_graphs(h);
     int e = iterate_t<T>(h, reps, s);  // captures
@@ -1749,22 +1748,30 @@ static int tune(cfr_handle *h, int reps, cudaStream_t s) {
     }
     return e;
   };
-  const bool launches = h->exec_form != CFR_EXEC_PERSISTENT && near_root >= 0;
-  float ms = 0.f, with = 0.f;
-  if (rc == CFR_OK && (launches || solo)) rc = call(&ms);
-  if (rc == CFR_OK && launches) {
+  // whether the handle as it is now is not clearly slower than the best so far
+  auto stays = [&]() {
+    float ms = 0.f;
+    if (rc || (rc = call(&ms))) return false;
+    const bool ok = ms <= 1.02f * best_ms;
+    if (ok) best_ms = ms;
+    return ok;
+  };
+  const bool check = launches && !tune_duel(h) && found != first;
+  if (rc == CFR_OK && (solo || (launches && (near_root >= 0 || check)))) stays();
+  if (check) {
+    h->level_lanes = first;
+    const float ms = best_ms;
+    if (!stays() || best_ms > 0.98f * ms) h->level_lanes = found;
+  }
+  h->top_k = near_root;
+  if (launches && near_root >= 0 && !stays()) h->top_k = -1;
+  h->solo_smem = solo;
+  if (solo && !stays()) h->solo_smem = 0;
+  if (rc) {
+    h->level_lanes = first;
     h->top_k = near_root;
-    rc = call(&with);
-    if (rc == CFR_OK && with > 1.02f * ms) h->top_k = -1;
-    else ms = with;
-  }
-  if (rc == CFR_OK && solo) {
     h->solo_smem = solo;
-    rc = call(&with);
-    if (rc == CFR_OK && with > 1.02f * ms) h->solo_smem = 0;
   }
-  if (h->exec_form == CFR_EXEC_PERSISTENT || rc) h->top_k = near_root;
-  if (rc) h->solo_smem = solo;
   return rc;
 }
 
