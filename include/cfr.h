@@ -89,7 +89,7 @@ typedef struct cfr_options {
    * it was measured faster than graph replay), the graph form above.
    * Under CFR_EXEC_AUTO with lanes_per_set and persistent_ctas at 0, games
    * whose arrays fit one CTA's shared memory (about 14,000 nodes in CFR_P32;
-   * up to 4,000 in CFR_P64) run all iterations of a cfr_iterate call there
+   * up to 3,000 in CFR_P64) run all iterations of a cfr_iterate call there
    * instead ("resident"). In the level and graph forms with lanes_per_set 0,
    * the small depths near the root are one launch of one CTA that also starts
    * the next iteration's forward pass. cfr_export_array 37 tells which of

@@ -380,12 +380,14 @@ extern "C" int cfr_compile(const cfr_game_spec *spec, const cfr_options *opt, cf
   choose_top(h);
   // AUTO: a game that fits one CTA's shared memory runs there for the whole
   // call (301 nodes: 4.1 us an iteration in FP32, 11.6 in the persistent form;
-  // 4,213: 6.6, 28.8 as a graph; FP64 above about 4,000 nodes is bound by one
-  // SM's FP64 pipe and runs as a graph). graph_iters and launch_overlap do not
+  // 4,213: 6.6, 28.8 as a graph). In FP64 one SM's pipe bounds it: up to 3,000
+  // nodes (random trees of 1,105 and 3,385: 23.9 and 52.6 us resident, 27.0 and
+  // 38.5 as a graph with the near-root launch; a card game of 2,791 33.2 and
+  // 33.1, one-card poker of 2,341 18.1 and 24.8). graph_iters and launch_overlap do not
   // decide: in FP32 this form's last bits differ from the launches', and those
   // two options leave the results as they are.
   if (h->opt.exec_form == CFR_EXEC_AUTO && lp == 0 && h->opt.persistent_ctas == 0 && h->maxa_tier <= 8 && c.D > 0 &&
-      (h->precision == CFR_P32 || c.N <= 4000)) {
+      (h->precision == CFR_P32 || c.N <= 3000)) {
     h->solo_smem = resident_bytes(h, inst_desc(h, 0));
     h->solo_threads = c.N <= 600 ? 256 : 1024;
     const double mean = c.I > 0 ? tot_mem / (double)c.I : 1.0;
