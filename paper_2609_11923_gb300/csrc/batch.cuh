@@ -8,17 +8,17 @@
 // The CTAs of a cluster share each depth's work, meet at the hardware cluster
 // barrier (barrier.cluster, release/acquire) between depths, and read the
 // state arrays through L2 because their L1s are not coherent. Each instance's
-// arithmetic depends only on its own arrays and on (THREADS, LANES), not on
-// the number of its CTAs: a solve gives bitwise the same result alone and
-// inside any mix run with the same shape. Wide chance nodes are summed by one
-// CTA in a fixed order.
+// arithmetic depends only on its own arrays and on the caller's threads and
+// lanes, not on the number of its CTAs or on the other instances: a solve gives
+// bitwise the same result alone and inside any mix run with the same shape.
+// Wide chance nodes are summed by one CTA in a fixed order.
 //
-// One CTA for every instance left the largest alone on one SM: a round of 64
-// endgames of 1e3 to 2e5 edges (50 iterations, exploitability, strategies)
-// 13.2 -> 5.0 ms; of ten of 2e5 to 1e6 edges, 8 CTAs each before, 11.9 -> 9.2.
-// Small solves in shared memory, loads issued together, slot updates by lanes
-// and enough registers: 5.0 -> 2.9 and 9.2 -> 5.4 ms; an iteration of 10,400
-// nodes in one CTA 28 -> 13 us (33 with the updates inside the depths).
+// What it gave, step by step, for a round of 64 endgames of 1e3 to 2e5 edges
+// (50 iterations, exploitability, strategies) and one of ten of 2e5 to 1e6: one
+// CTA each (8 for the ten) 13.2 and 11.9 ms; CTAs by size 5.0 and 9.2; small
+// solves in shared memory, loads issued together, slot updates by lanes 2.9 and
+// 5.4; code for two and four actions and cluster sizes by what the GPU holds 2.7
+// and 4.0. An iteration of 10,400 nodes in one CTA 28 -> 10.7 us.
 #pragma once
 #include <algorithm>
 #include <queue>

@@ -48,9 +48,11 @@ constexpr int kStreamLanes = 512;                 // lanes_per_set code of this 
 constexpr int kStreamStages = 2;                  // a team's ring
 constexpr int kStreamStageBytes = 48 * 1024;      // bytes one chunk may stage at most
 constexpr int kStreamPackBytes = 6 * 1024;        // groups are packed into a chunk up to this size,
-constexpr int kStreamSpread = 16 * 152;           // as long as the depth makes this many chunks (one for each of a GB300's warps)
+constexpr int kStreamSpread = 16 * 152;           // as long as the depth makes this many chunks (one for each warp of a GB300's
+                                                  // 152 SMs; games are compiled on hosts without a GPU to ask)
 constexpr int kStreamChanceBytes = 1024;          // chance nodes are packed up to this size in any case
-constexpr int kStreamSideBytes = 2048;            // bytes of a chunk's R and average sums, and descriptors, at most
+constexpr int kStreamSideBytes = 2048;            // bytes of a chunk's R, average sums and descriptors: bounds its sets (32 of
+                                                  // two actions), which a team updates one group after another
 constexpr int kStreamMaxWarps = 16;               // warps of a streaming CTA (one CTA per SM)
 constexpr int kStreamMinWarps = 6;                // of a CTA of one-warp teams
 constexpr int kStreamDynSmem = 216 * 1024;        // bytes of all teams' rings
@@ -98,7 +100,7 @@ static_assert(sizeof(StreamChunk) == 64, "StreamChunk is 64 bytes");
 // Byte offsets of the staged arrays: what the members' work reads, then
 // (from total on) what the slot updates read besides: R, then the average
 // sums, 8 bytes a slot each. (s_*: the latter's sizes together with the
-// descriptors', which kStreamSideBytes bounds.)
+// descriptors', which kStreamSideBytes bounds; nothing is laid out by them.)
 struct StreamLayout {
   uint32_t reach, val, mem, info, sig, total;
   uint32_t s_info, s_R, s_avg, s_total;

@@ -158,7 +158,9 @@ static void plan(cfr_handle *h) {
   h->plan_bytes = cur;
 }
 
-constexpr int kFewSets = 4 * 152;  // no more than a set for each scheduler of a GB300
+// No more than a set for each scheduler of a GB300's 152 SMs (games are compiled
+// on hosts without a GPU to ask).
+constexpr int kFewSets = 4 * 152;
 
 // Set descriptors and chunks of the streaming backward (FP32, member order,
 // sets of at most 8 actions). A group is a tile of kTileSets sets (members'

@@ -3,17 +3,16 @@
 Requests (game specs with arrival times) are compiled on arrival by worker
 threads, admitted into a device memory pool by their footprint (cfr_plan)
 whenever a slot and enough pool memory are free, and solved together: every
-round is ONE batched launch that runs `check_every` iterations of every
-active solve (one CTA per solve), followed by ONE batched exploitability
-launch. Solves that reach `target * pot` exploitability (or `max_iters`)
+round is a batched call that runs `check_every` iterations of every active
+solve, followed by ONE batched exploitability call. Solves that reach `target * pot` exploitability (or `max_iters`)
 retire, free their memory, and the next arrivals are admitted before the
 next round, so work that arrives while others are on the GPU overlaps with
-them. Requests of at least `big_edges` edges run as thread-block clusters of
-`cluster` CTAs (a second batched launch on a side stream, concurrent with
-the one-CTA launch of the rest), so one large subgame no longer holds every
-round to the speed of a single SM. Whether a request is large depends only
-on the request, so a solve's iterates do not depend on what else is in the
-batch.
+them. The library gives every solve as many CTAs as its size asks for.
+Requests of at least `big_edges` edges go out as a second batched call on a
+side stream, concurrent with the rest, with a shape of their own
+(`big_threads`, `big_lanes`) and at least `cluster` CTAs each. Whether a
+request is large depends only on the request, so a solve's iterates do not
+depend on what else is in the batch.
 
 Admission (``admit``): requests are taken in arrival order. A request whose
 footprint exceeds the whole pool can never be admitted and is answered at
@@ -284,12 +283,12 @@ class Server:
                 nxt = pending[0].arrival if pending else now + 1e-3
                 time.sleep(max(0.0, min(nxt - (time.perf_counter() - t0), 2e-3)))
                 continue
-            active.sort(key=lambda a: a.big)  # one-CTA solves first, clusters after
+            active.sort(key=lambda a: a.big)
             hs = [a.h for a in active]
             iters = [min(self.check_every, self.max_iters - a.done) for a in active]
             nb = sum(1 for a in active if a.big)
             ns = len(active) - nb
-            if nb:  # the large solves as clusters on the side stream, concurrently
+            if nb:  # the large solves on the side stream, concurrently
                 self.side.wait_stream(self.torch.cuda.current_stream())
                 cfr.cfr_batch_iterate(hs[ns:], 0, self.table2_ptr, self.table_bytes, self.big_threads, self.big_lanes,
                                       int(self.side.cuda_stream), iters=iters[ns:], cluster=self.cluster)

@@ -16,8 +16,8 @@ import pytest
 import gamegen as gg
 from paper_2609_11923_gb300 import cfr
 
-STAGE = 48 * 1024  # bytes of a stage (the compute threads' data)
-SIDE = 2048  # bytes of a side slot (the control warp's data)
+STAGE = 48 * 1024  # bytes of a stage without R and the average sums
+SIDE = 2048  # bytes of a chunk's R, average sums and descriptors
 
 GAMES = {
     "tiny": lambda: gg.tiny_card(),
