@@ -444,10 +444,15 @@ def run_ours(args):
 
     # the launch structure alone (empty kernels, same grids / same barriers), for comparison with ms_per_step
     floor_graph, floor_pers = cfr.cfr_launch_floor(solver.h, 200, s)
+    # per depth one forward and one backward launch; in member order the deepest
+    # depth has no forward launch (no internal node below it pulls), and depths
+    # 0 .. K of the near-root launch have one together
+    K = cfr.cfr_launch_plan(solver.h)["near_root_depth"]
+    iter_launches = 2 * (D - K) - 1 if K >= 0 else (D - 1 if args.reach_order == "members" else D) + D
     launch_floor = {"graph_ms": floor_graph, "persistent_ms": floor_pers,
                     "what": "per iteration: a graph of the same %d launches (same grids) of an empty kernel; one "
                             "cooperative empty kernel with the persistent form's grid and %d grid barriers"
-                            % ((D - 1 if args.reach_order == "members" else D) + D, 2 * D)}
+                            % (iter_launches, 2 * D)}
 
     # end to end through the public API: upload (bind) + K iterations + average strategy to host
     e2e = None
@@ -486,11 +491,8 @@ def run_ours(args):
         batched = serving_leg(args.batched_requests, args.max_iters, args.batched_baseline)
     barrier()
 
-    # kernels of the captured iteration (graph form); otherwise per depth one
-    # forward and one backward launch (in member order the deepest depth has
-    # no forward launch: no internal node below it pulls)
-    fwd_launches = D - 1 if args.reach_order == "members" else D
-    per_iter_launches = graph_kernels or {cfr.EXEC_LEVELS: fwd_launches + D}.get(counts["exec_form"], 0)
+    # kernels of the captured iteration (graph form)
+    per_iter_launches = graph_kernels or {cfr.EXEC_LEVELS: iter_launches}.get(counts["exec_form"], 0)
     gpu_launches = args.steps * per_iter_launches if per_iter_launches else 1
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,

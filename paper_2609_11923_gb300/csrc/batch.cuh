@@ -38,8 +38,8 @@ struct ClusterRoom {
 
 // CTAs for every instance of a batch (host): 1, 2, 4, 8 or 16, at least
 // `least`, by an estimate of an iteration's time (batch_ns). The instance that
-// takes longest gets twice its CTAs as long as all of them run at the same
-// time (a cluster too many waits for a whole instance: ten large endgames with
+// takes longest gets twice its CTAs, or more, as long as all of them run at the
+// same time (a cluster too many waits for a whole instance: ten large endgames with
 // six of 16 took 89 us an iteration, with four 64); a batch that does not run
 // at the same time anyway, while it takes longer than an even share of it.
 struct BatchLoad {
@@ -89,17 +89,19 @@ inline std::vector<int> plan_clusters(const std::vector<BatchLoad> &load, int le
     const double t = longest.top().first;
     const int i = -longest.top().second, c = cta[i];
     longest.pop();
-    if (c == 16 || !exists(2 * c) || time(i, 2 * c) >= t) continue;
+    int more = 2 * c;  // the next size that is faster: a cluster of two may lose more to its barriers than it shares
+    while (more <= 16 && exists(more) && time(i, more) >= t) more *= 2;
+    if (more > 16 || !exists(more)) continue;
     --count[c];
-    ++count[2 * c];
+    ++count[more];
     if (!fits() && !(waves && t > work / room.sms)) {
       ++count[c];
-      --count[2 * c];
+      --count[more];
       continue;
     }
-    work += 2 * c * time(i, 2 * c) - c * t;
-    cta[i] = 2 * c;
-    longest.push({time(i, 2 * c), -i});
+    work += more * time(i, more) - c * t;
+    cta[i] = more;
+    longest.push({time(i, more), -i});
   }
   return cta;
 }

@@ -80,6 +80,8 @@ def test_depths_are_paid_for_in_every_ctas_barriers(lib):
     assert ctas(lib, [(920440, 4380, 5, 532, 0, 0)]) == ctas(lib, [(275507, 33629, 11, 140, 0, 0)]) == [16]
     # FP64 is worth a cluster far earlier (10,000 nodes: 142 us, by 16 CTAs 50)
     assert ctas(lib, [(10241, 1334, 8, 90, 1, 1)])[0] >= 8 and ctas(lib, [(10414, 400, 5, 41, 1, 0)]) == [1]
+    # a cluster of two loses more to its barriers than it shares, one of 16 gains (23 us, 26, 18)
+    assert ctas(lib, [(21178, 620, 5, 60, 0, 0)]) == [16]
     # long sets are walked by a group each wherever its CTA is
     assert ctas(lib, [(13801, 6, 3, 600, 0, 1)]) == [1]
 
