@@ -10,6 +10,7 @@ layer is h_out = relu(h_in @ W + b).
 from __future__ import annotations
 
 import ctypes
+import struct
 from operator import attrgetter
 from typing import List, Optional
 
@@ -238,10 +239,10 @@ class MLP:
         if self._rows_ok(X) and self._fused_grad(X, B, nact, target, weight, loss):
             self._ran_fused(X)
             at = loss.value - self.work.data_ptr()
-            got = self.work[at:at + 8].cpu()
-            if int(got.view(torch.int32)[1]) != 0:
+            total, failed = struct.unpack("=fi", self.work[at:at + 8].cpu().numpy().tobytes())
+            if failed:
                 raise RuntimeError("mlp: a bounded wait of the training kernels gave up")
-            return float(got.view(torch.float32)[0]) / B
+            return total / B
         logits = self.forward(X)
         dlog = torch.empty_like(logits)
         rows = torch.empty(B, dtype=torch.float32, device=self.dev)
