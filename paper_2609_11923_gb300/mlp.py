@@ -11,7 +11,8 @@ from __future__ import annotations
 
 import ctypes
 import struct
-from operator import attrgetter
+from itertools import chain
+from operator import is_, methodcaller
 from typing import List, Optional
 
 import numpy as np
@@ -43,7 +44,7 @@ for _f in ("mlp_gemm", "mlp_softmax_xent", "mlp_relu_grad", "mlp_colsum", "mlp_a
 _lib.mlp_last_error.restype = ctypes.c_char_p
 
 N_OUT = 8
-_VERSION = attrgetter("_version")
+_DATA_PTR = methodcaller("data_ptr")
 
 
 def _ck(rc):
@@ -56,12 +57,31 @@ def _net_ck(rc):
         raise RuntimeError("mlp: " + (_lib.mlp_net_last_error() or b"").decode())
 
 
+def _writes(t) -> int:
+    """A tensor's write counter (an inference tensor has none: never written)."""
+    try:
+        return t._version
+    except RuntimeError:
+        return -1
+
+
 def _p(t) -> int:
     return 0 if t is None else int(t.data_ptr())
 
 
+_ARRAYS = {}
+
+
 def _ptrs(ts):
-    return (_vp * len(ts))(*[t.data_ptr() for t in ts])
+    """The tensors' addresses as a C array (kept by its contents: building one
+    takes as long as a launch)."""
+    at = tuple(map(_DATA_PTR, ts))
+    a = _ARRAYS.get(at)
+    if a is None:
+        if len(_ARRAYS) >= 64:
+            _ARRAYS.clear()
+        a = _ARRAYS[at] = (_vp * len(at))(*at)
+    return a
 
 
 class MLP:
@@ -72,13 +92,18 @@ class MLP:
         self.dev = torch.device(device)
         self.dims = [in_dim] + list(hidden) + [out]
         rng = np.random.default_rng(seed)
-        self.W, self.b, self.Wb = [], [], []
-        for fi, fo in zip(self.dims[:-1], self.dims[1:]):
+        # the biases, and the BF16 weights, are views of one tensor each: the
+        # write counter that a tensor shares with its views then tells at once
+        # whether a caller has written into any of them (_packed, acts)
+        shapes = list(zip(self.dims[:-1], self.dims[1:]))
+        self._flat_b, self.b = self._views([(fo,) for _, fo in shapes], torch.float32)
+        self._flat_wb, self.Wb = self._views(shapes, torch.bfloat16)
+        self._own_b, self._own_wb = tuple(self.b), tuple(self.Wb)
+        self.W = []
+        for fi, fo in shapes:
             lim = np.sqrt(6.0 / fi)  # He-uniform for ReLU layers
             w = rng.uniform(-lim, lim, size=(fi, fo)).astype(np.float32)
             self.W.append(torch.tensor(w, device=self.dev))
-            self.b.append(torch.zeros(fo, dtype=torch.float32, device=self.dev))
-            self.Wb.append(torch.empty((fi, fo), dtype=torch.bfloat16, device=self.dev))
         self.gW = [torch.zeros_like(w) for w in self.W]
         self.gb = [torch.zeros_like(b) for b in self.b]
         self.mW = [torch.zeros_like(w) for w in self.W]
@@ -98,15 +123,24 @@ class MLP:
             # set to 1 by an inference kernel whose bounded wait gave up
             # (page-locked: the host reads it without a copy)
             self._err = torch.zeros(1, dtype=torch.int32).pin_memory()
-            self._err_host = self._err.numpy()
+            self._failed = ctypes.c_int32.from_address(self._err.data_ptr())
         self.sync_bf16()
+
+    def _views(self, shapes, dtype):
+        """Zeros of these shapes, 512 bytes aligned as tensors of their own
+        would be, in one tensor: that tensor and its views."""
+        at = [0]
+        for s in shapes:
+            at.append(at[-1] + (int(np.prod(s)) + 255) // 256 * 256)
+        flat = self.torch.zeros(at[-1], dtype=dtype, device=self.dev)
+        return flat, [flat[a:a + int(np.prod(s))].view(s) for a, s in zip(at, shapes)]
 
     def _s(self) -> int:
         return int(self.torch.cuda.current_stream(self.dev).cuda_stream)
 
     def _raise_if_failed(self):
-        if self.fused and self._err_host[0] != 0:
-            self._err_host[0] = 0
+        if self.fused and self._failed.value:
+            self._failed.value = 0
             raise RuntimeError("mlp: a bounded wait of an inference kernel gave up; its probabilities are NaN")
 
     def check(self) -> None:
@@ -121,11 +155,11 @@ class MLP:
         """The input, every hidden layer's output and the logits of the last
         pass in FP32. The fused passes keep none: after one of them they are
         computed here, on first use, from its batch and the weights, and once
-        either has changed (adam_step, sync_bf16, a write into the tensors)
-        they are gone, which raises."""
+        either has changed (adam_step, sync_bf16, a write into the tensors,
+        other tensors in their place) they are gone, which raises."""
         if self._acts is None and self._fused_pass is not None:
-            X, then = self._fused_pass
-            if X is None or then != self._counters([X, *self.b]) or not self._packed():
+            X, x, b = self._fused_pass
+            if X is None or x != _writes(X) or b != _writes(self._flat_b) or not self._own(self.b, self._own_b) or not self._packed():
                 raise RuntimeError("mlp: the activations of the last fused pass are gone (its weights or its batch have "
                                    "changed since); run forward(X)")
             self.forward(X)
@@ -135,31 +169,23 @@ class MLP:
     def acts(self, value):
         self._acts, self._fused_pass = value, None
 
-    # A pass over X reads X, the biases, and Wb or its images; the write
-    # counters of tensors tell whether a caller has written into them since
-    # (inference tensors have none and count as never written).
     @staticmethod
-    def _counters(ts):
-        try:
-            return [*map(_VERSION, ts)]
-        except RuntimeError:
-            return [-1 if t.is_inference() else t._version for t in ts]
+    def _own(now, own) -> bool:
+        return all(map(is_, now, own))
 
     def _ran_fused(self, X):
-        self._acts, self._fused_pass = None, (X, self._counters([X, *self.b]))
+        self._acts, self._fused_pass = None, (X, _writes(X), _writes(self._flat_b))
 
     def _weights_change(self):  # by a kernel, past the counters: Wb and its images together
-        wb = self.Wb.copy()  # held, so that no other tensor can have their ids
-        self._images_of = (wb, [*map(id, wb)], self._counters(wb))
+        self._packed_at = _writes(self._flat_wb) if self._own(self.Wb, self._own_wb) else None
         if self._fused_pass is not None:
-            self._fused_pass = (None, None)
+            self._fused_pass = (None, 0, 0)
 
     def _packed(self) -> bool:
-        """Whether the packed images are those of Wb. A caller's write into Wb,
-        or other tensors in its place, reach only the layer-by-layer passes,
-        until sync_bf16 or a step writes both."""
-        _, ids, then = self._images_of
-        return [*map(id, self.Wb)] == ids and self._counters(self.Wb) == then
+        """Whether the packed images are those of Wb. A caller's write into Wb
+        reaches only the layer-by-layer passes, until sync_bf16 or a step writes
+        both; with other tensors in Wb's place those passes run for good."""
+        return _writes(self._flat_wb) == self._packed_at and self._own(self.Wb, self._own_wb)
 
     def sync_bf16(self):
         self._weights_change()
@@ -172,7 +198,7 @@ class MLP:
 
     @staticmethod
     def _all(weights, biases):
-        return _ptrs([t for pair in zip(weights, biases) for t in pair])
+        return _ptrs(chain.from_iterable(zip(weights, biases)))
 
     def _rows_ok(self, X) -> bool:
         return (self.fused and self._packed() and X.dtype == self.torch.float32 and X.dim() == 2 and X.shape[0] > 0

@@ -11,12 +11,14 @@ from paper_2609_11923_gb300 import mlp, warmstart
 
 
 def bare(err=0):
-    """A network without its tensors, in the state that its fused passes leave."""
+    """A network without most of its tensors, in the state that its fused passes leave."""
     net = mlp.MLP.__new__(mlp.MLP)
     net.torch, net.dev, net.fused = torch, torch.device("cpu"), True
     net._err = torch.tensor([err], dtype=torch.int32)
-    net._err_host = net._err.numpy()
-    net.Wb, net.b = [torch.zeros(3), torch.zeros(2)], [torch.zeros(3)]
+    net._failed = ctypes.c_int32.from_address(net._err.data_ptr())
+    net._flat_wb, net._flat_b = torch.zeros(5), torch.zeros(4)
+    net.Wb, net.b = list(net._flat_wb.split([3, 2])), list(net._flat_b.split([1, 3]))
+    net._own_wb, net._own_b = tuple(net.Wb), tuple(net.b)
     net.dims = [4, 2]
     net._acts, net._fused_pass = None, None
     net._weights_change()
@@ -50,8 +52,9 @@ def test_warm_start_raises_on_a_failed_inference():
         warmstart.warm_regrets(Failing(), g, 8.0)
 
 
-@pytest.mark.parametrize("change", [lambda n, x: n._weights_change(), lambda n, x: x.add_(1.0), lambda n, x: n.b[0].zero_()],
-                         ids=["step", "batch", "bias"])
+@pytest.mark.parametrize("change", [lambda n, x: n._weights_change(), lambda n, x: x.add_(1.0), lambda n, x: n.b[0].zero_(),
+                                    lambda n, x: n.b.__setitem__(1, torch.zeros(3)), lambda n, x: n.Wb[1].zero_()],
+                         ids=["step", "batch", "bias", "other bias", "weights"])
 def test_activations_of_a_fused_pass_are_gone_once_its_inputs_change(change):
     net, X = bare(), torch.zeros(2, 4)
     ran = []
@@ -77,10 +80,12 @@ def test_activations_of_a_fused_pass_are_gone_once_its_inputs_change(change):
 def test_changed_bf16_weights_leave_the_packed_images(change):
     net, X = bare(), torch.zeros(2, 4)
     assert net._rows_ok(X)
+    net.b[0].add_(1.0)  # biases are read as they are
+    assert net._rows_ok(X)
     change(net)
     assert not net._rows_ok(X)
     net._weights_change()  # what sync_bf16 and a step do as they write both
-    assert net._rows_ok(X)
+    assert net._rows_ok(X) == (net.Wb[0] is net._own_wb[0])
 
 
 # addresses that are only looked at: every refusal comes before any launch
