@@ -1726,7 +1726,7 @@ static int tune_persistent(cfr_handle *h, int reps, TuneClock &clock) {
 // Tunes the launches of every depth, then keeps what it found (small games),
 // the near-root launch and the resident form only where calls of `reps`
 // iterations are not slower with them (a set of 300 members of five actions in
-// FP64: near-root 125 us an iteration, by blocks of their own 70).
+// FP64: near-root 125 us an iteration, by blocks of their own 50).
 template <typename T>
 static int tune(cfr_handle *h, int reps, cudaStream_t s) {
   const std::vector<int> first = h->level_lanes;
