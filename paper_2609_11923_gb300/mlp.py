@@ -210,7 +210,7 @@ class MLP:
         torch = self.torch
         self._raise_if_failed()
         B = X.shape[0]
-        self.acts = [X]
+        acts = self.acts = [X]
         h = X
         L = len(self.W)
         for l in range(L):
@@ -219,7 +219,7 @@ class MLP:
             # A(m, k) = h[m, k]; B(k, n) = Wb[k, n]
             _ck(_lib.mlp_gemm(_p(h), 0, h.shape[1], 1, _p(self.Wb[l]), 1, fo, 1, _p(out), None, fo, B, fo,
                               self.dims[l], _p(self.b[l]), 1 if l < L - 1 else 0, 0, self._s()))
-            self.acts.append(out)
+            acts.append(out)
             h = out
         return h
 
@@ -227,10 +227,10 @@ class MLP:
         """Gradients of every weight and bias given d loss / d logits."""
         torch = self.torch
         B = dlogits.shape[0]
-        d = dlogits
+        d, acts = dlogits, self.acts
         for l in range(len(self.W) - 1, -1, -1):
             fi, fo = self.dims[l], self.dims[l + 1]
-            h_in = self.acts[l]
+            h_in = acts[l]
             # gW = h_in^T d : A(m=i, k=b) = h_in[b, i]; B(k=b, n=j) = d[b, j]
             _ck(_lib.mlp_gemm(_p(h_in), 0, 1, fi, _p(d), 0, fo, 1, _p(self.gW[l]), None, fo, fi, fo, B, None, 0, 0,
                               self._s()))
