@@ -639,7 +639,7 @@ __device__ __forceinline__ void chain_leave() {
 // hold every depth back by a dependent chain of FP64 instructions that serve
 // a few lanes each.
 template <typename T, int MAXA, int LANES, int NT, int MODE>
-__global__ void __launch_bounds__(NT, 1) batch_iterate_kernel(const InstDesc *table, const __grid_constant__ InstDesc one,
+__global__ void __launch_bounds__(NT, MODE == kSolo && NT <= 256 && MAXA <= 4 ? 2 : 1) batch_iterate_kernel(const InstDesc *table, const __grid_constant__ InstDesc one,
                                                            int n_inst) {
   constexpr bool CLUSTERED = MODE == kCluster;
   extern __shared__ __align__(128) unsigned char s_solve[];
