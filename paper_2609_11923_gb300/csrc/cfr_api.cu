@@ -1677,11 +1677,14 @@ static int tune_levels(cfr_handle *h, int reps, TuneClock &clock) {
     // candidate only where sets are long
     if (h->stream_ok[d] && c.level_mean_members[d] >= kStreamMinMembers) cd.push_back(kStreamLanes);
     auto run_depth = [&]() { return launch_bwd<T>(h, (int)d, s); };
-    for (int L : cd) {  // by itself: once, again if that was hopeless (it may have loaded the kernel), and more if not
+    // by itself, after one launch (which may load the kernel); sets are long
+    // enough for a candidate to be hopeless: not again if once was
+    const bool probe = c.level_mean_members[d] > 32.0;
+    for (int L : cd) {
       float ms = 0.f;
       h->level_lanes[d] = L;
-      if ((rc = clock.time(1, run_depth, &ms))) return rc;
-      if (ms * reps > 2.f * best_ms && (rc = clock.time(1, run_depth, &ms))) return rc;
+      if ((rc = run_depth())) return rc;
+      if (probe && (rc = clock.time(1, run_depth, &ms))) return rc;
       if (ms * reps > 2.f * best_ms) continue;
       if ((rc = clock.time(reps, run_depth, &ms))) return rc;
       if (ms < best_ms) { best_ms = ms; best = L; }
