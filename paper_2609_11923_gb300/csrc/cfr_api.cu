@@ -1868,7 +1868,8 @@ static int batch_plan(cfr_handle *const *hs, int n, const int64_t *iters, int64_
     load[i].depths = hs[i]->c.D;
     load[i].chain = hs[i]->chain;
     load[i].resident = e[i].smem > 0;
-    load[i].fp64 = !iterate || bp.precision == CFR_P64;  // a best response is in FP64
+    load[i].best = !iterate;
+    load[i].fp64 = !iterate || bp.precision == CFR_P64;
     load[i].share = iters ? (double)iters[i] / (double)longest : 1.0;
   }
   ClusterRoom room;

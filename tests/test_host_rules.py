@@ -21,12 +21,12 @@ extern "C" unsigned resident_size(long long nodes, unsigned T) {
   in.n_chance = 1;
   return cfr::resident_size(in, T);
 }
-// per instance: nodes, sets, depths, chain, resident, fp64
+// per instance: nodes, sets, depths, chain, resident, 0 FP32, 1 FP64, 2 a best response
 extern "C" void plan(int n, const long long *load, int least, int sms, int four, int eight, int sixteen, int *out) {
   std::vector<cfr::BatchLoad> l(n);
   for (int i = 0; i < n; ++i) {
     const long long *x = load + 6 * i;
-    l[i] = cfr::BatchLoad{x[0], x[1], x[2], x[3], x[4] != 0, x[5] != 0, 1.0};
+    l[i] = cfr::BatchLoad{x[0], x[1], x[2], x[3], x[4] != 0, x[5] != 0, x[5] == 2, 1.0};
   }
   cfr::ClusterRoom r;
   r.sms = sms;
@@ -96,3 +96,16 @@ def test_no_cluster_that_the_device_cannot_hold(lib, n, room, most):
 
 def test_the_least_ctas_are_everyones(lib):
     assert min(ctas(lib, [(300, 30, 5, 12, 1, 0), (920440, 4380, 5, 532, 0, 0)], least=4)) >= 4
+
+
+def test_growth_that_does_not_bring_the_end_forward_is_taken_back(lib):
+    alike = (10241, 1334, 8, 60, 0, 0)  # 40 random trees: 16 CTAs would be faster, and there is room for a few
+    assert ctas(lib, [alike])[0] > 1 and ctas(lib, [alike] * 40) == [1] * 40
+    # the largest still grows beside them
+    assert ctas(lib, [(920440, 4380, 5, 532, 0, 0)] + [alike] * 40)[0] == 16
+
+
+def test_best_responses_of_small_trees_stay_in_one_cta(lib):
+    # by one CTA or 16 alike for 3,385 nodes alone (70 us), 1,810 and 222 us for 920,440
+    assert ctas(lib, [(3385, 458, 7, 50, 0, 2)] * 16) == [1] * 16
+    assert ctas(lib, [(920440, 4380, 5, 412, 0, 2)]) == [16]
