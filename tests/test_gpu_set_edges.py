@@ -141,4 +141,4 @@ def test_tuning_is_not_slower_than_a_shape_that_it_tries(g):
     s.iterate(9)
     np.testing.assert_array_equal(s.avg_strategy(), oracle.solve(g, 9).avg_strategy())
     s.close()
-    assert tuned < 1.2 * min(fixed), (tuned, fixed)
+    assert tuned < 1.35 * min(fixed), (tuned, fixed)  # 1.0 measured, 1.5 to 2.5 with the forms untried
